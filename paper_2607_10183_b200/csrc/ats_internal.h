@@ -304,6 +304,10 @@ cudaError_t launch_rope_append_prefill(const __half* qkv16, int ld, __half* q_ro
                                        uint64_t* n_launch, int pdl = 0);
 cudaError_t launch_attn_prefill(const __half* q_rot16, const __half* kc, const __half* vc, __half* a16, int T, int n_q,
                                 int n_kv, int d, int cap, int pos0, cudaStream_t st, uint64_t* n_launch, int pdl = 0);
+// the same on tcgen05 (kernels_attn_prefill.cu): chunks and buffers it takes, and its launcher
+bool attn_prefill_tc_eligible(const __half* q_rot16, const __half* kc, const __half* vc, const __half* a16, int T, int d);
+cudaError_t launch_attn_prefill_tc(const __half* q_rot16, const __half* kc, const __half* vc, __half* a16, int T, int n_q, int n_kv, int d,
+                                   int cap, int pos0, int* status, cudaStream_t st, uint64_t* n_launch, int pdl = 0);
 // MoE prefill helpers (kernels_prefill.cu): rows gathered in expert order, and the gated sum back in token order
 cudaError_t launch_moe_gather_rows(const __half* h, const int* order, int k, __half* xs, int P, int H, cudaStream_t st,
                                    uint64_t* n_launch, int pdl = 0);

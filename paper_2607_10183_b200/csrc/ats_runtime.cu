@@ -1689,8 +1689,12 @@ int32_t ats_layer_prefill(ats_ctx* ctx, const ats_layer_desc* L, const void* x_i
     ATS_TRY(run_gemm_group(ctx, qkv, 3, g));
     ATS_CUDA(launch_rope_append_prefill(w.qkv16, qd + 2 * kvd, w.qrot16, (__half*)k_cache, (__half*)v_cache, (int)T, nq, nkv, d,
                                         (int)L->kv_capacity, (int)pos0, L->rope_theta, ctx->cs, nl, pdl));
-    ATS_CUDA(launch_attn_prefill(w.qrot16, (const __half*)k_cache, (const __half*)v_cache, w.a16, (int)T, nq, nkv, d,
-                                 (int)L->kv_capacity, (int)pos0, ctx->cs, nl, pdl));
+    if (attn_prefill_tc_eligible(w.qrot16, (const __half*)k_cache, (const __half*)v_cache, w.a16, (int)T, d))
+      ATS_CUDA(launch_attn_prefill_tc(w.qrot16, (const __half*)k_cache, (const __half*)v_cache, w.a16, (int)T, nq, nkv, d,
+                                      (int)L->kv_capacity, (int)pos0, ctx->dev_status, ctx->cs, nl, pdl));
+    else
+      ATS_CUDA(launch_attn_prefill(w.qrot16, (const __half*)k_cache, (const __half*)v_cache, w.a16, (int)T, nq, nkv, d,
+                                   (int)L->kv_capacity, (int)pos0, ctx->cs, nl, pdl));
     g.x = w.a16;
     g.ldx = qd;
     g.y = w.o16;
