@@ -355,12 +355,19 @@ struct GemmParams {
   int grp_max_rows;         // the largest expert's row count (sizes the grid)
   uint64_t grp_stride;
   const uint8_t* const* grp_tab[3];
+  // optional fused SwiGLU (launch_gemm_ts only): act[t][f] = rn16(silu(y[t][f]) * y[t][n_rows + f]) of segments gate, up;
+  // y itself is written only where it is not null
+  __half* act;
+  int ldact;
+  int* counters;  // kAttnMaxCounters ints, zero between launches (launch_gemm_ts: arrival counts of split tiles)
 };
+// The dequantizing GEMM with the weights in tensor memory (kernels_gemm_ts.cu): operands it takes, scratch it likes to have
+// (it runs with any), and its launcher
+bool gemm_ts_eligible(const GemmParams& p);
+uint64_t gemm_ts_scratch_bytes(int T, int n_total, int K);
+cudaError_t launch_gemm_ts(const GemmParams& p, int sm_count, cudaStream_t st, uint64_t* n_launch, std::string* err);
 uint64_t gemm_scratch_bytes(int T, int n_total, int K);
 cudaError_t launch_gemm(const GemmParams& p, cudaStream_t st, uint64_t* n_launch, std::string* err);
-// y = rn16(sum over splits of partial[s][T][ldy]) (+ optional residual into y2), splits in ascending order (kernels_gemm.cu)
-cudaError_t launch_gemm_splitk_reduce(const float* partial, __half* y, int T, int n_cols, int ldy, int splits, const __half* res, __half* y2,
-                                      int pdl, cudaStream_t st, uint64_t* n_launch);
 // GEMMs as pairs of CTAs (kernels_gemm_pair.cu): shapes they take, and their launcher
 bool gemm_pair_eligible(const GemmParams& p);
 cudaError_t launch_gemm_pair(const GemmParams& p, cudaStream_t st, uint64_t* n_launch, std::string* err);

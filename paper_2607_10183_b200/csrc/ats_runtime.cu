@@ -341,12 +341,33 @@ static int32_t run_gemv_group(ats_ctx* ctx, Operand* ops, int n, GemvParams p) {
   return ATS_OK;
 }
 
+// One GEMM launch: the 4-bit formats on the kernel that keeps the weights in tensor memory, fp16 matrices as CTA pairs where
+// they have enough tiles, else the single-CTA kernel (slice address tables; ATS_FLAG_NO_GEMM_PAIR).  A SwiGLU that was asked for
+// runs in the epilogue or as a launch of its own.
+static int32_t launch_gemm_any(ats_ctx* ctx, GemmParams p) {
+  std::string err;
+  cudaError_t e;
+  __half* act = p.act;
+  p.counters = reinterpret_cast<int*>(ctx->ws) + 64;  // (the attention's: zero between launches, and launches follow one another)
+  const bool pairs = !(ctx->cfg.flags & ATS_FLAG_NO_GEMM_PAIR);
+  if (pairs && gemm_ts_eligible(p)) {
+    e = launch_gemm_ts(p, ctx->sm_count, ctx->cs, &ctx->stats.kernel_launches, &err);
+    act = nullptr;
+  } else if (pairs && gemm_pair_eligible(p)) {
+    e = launch_gemm_pair(p, ctx->cs, &ctx->stats.kernel_launches, &err);
+  } else {
+    e = launch_gemm(p, ctx->cs, &ctx->stats.kernel_launches, &err);
+  }
+  if (e != cudaSuccess) return check_cuda(ctx, e, err.empty() ? "launch_gemm" : err.c_str());
+  if (act) ATS_CUDA(launch_swiglu16(p.y, p.ldy, p.ldact, act, p.T, ctx->cs, &ctx->stats.kernel_launches, p.pdl));
+  return ATS_OK;
+}
+
 static int32_t run_gemm_group(ats_ctx* ctx, Operand* ops, int n, GemmParams p) {
   p.K = (int)ops[0].t->d.k_in;
   p.status = ctx->dev_status;
   p.w16 = ops[0].t->d.fmt == ATS_FMT_W16;  // a group shares one format (check_layer)
   p.mx = ops[0].t->d.fmt == ATS_FMT_MXFP4;
-  std::string err;
   // fp16 weight tiles come through one tensor map per matrix: such a group always runs matrix by matrix
   if ((count_streamed(ops, n) <= (int)ctx->cfg.ring_slots && !p.w16) || n == 1) {
     ATS_TRY(acquire_ops(ctx, ops, n));
@@ -356,15 +377,10 @@ static int32_t run_gemm_group(ats_ctx* ctx, Operand* ops, int n, GemmParams p) {
       p.seg[i] = GemvSeg{ops[i].ptr, (int)ops[i].t->d.n_out};
       rows += ops[i].t->d.n_out;
     }
-    cudaError_t e;
     {
       TimedLaunch tl(ctx, 2, 2ull * (uint64_t)p.T * rows * (uint64_t)p.K);
-      if (!(ctx->cfg.flags & ATS_FLAG_NO_GEMM_PAIR) && gemm_pair_eligible(p))
-        e = launch_gemm_pair(p, ctx->cs, &ctx->stats.kernel_launches, &err);
-      else
-        e = launch_gemm(p, ctx->cs, &ctx->stats.kernel_launches, &err);
+      ATS_TRY(launch_gemm_any(ctx, p));
     }
-    if (e != cudaSuccess) return check_cuda(ctx, e, err.empty() ? "launch_gemm" : err.c_str());
     return release_ops(ctx, ops, n);
   }
   int row0 = 0;
@@ -374,18 +390,15 @@ static int32_t run_gemm_group(ats_ctx* ctx, Operand* ops, int n, GemmParams p) {
     q.n_seg = 1;
     q.seg[0] = GemvSeg{ops[i].ptr, (int)ops[i].t->d.n_out};
     q.y += row0;
-    cudaError_t e;
+    q.act = nullptr;
     {
       TimedLaunch tl(ctx, 2, 2ull * (uint64_t)q.T * (uint64_t)q.seg[0].n_rows * (uint64_t)q.K);
-      if (!(ctx->cfg.flags & ATS_FLAG_NO_GEMM_PAIR) && gemm_pair_eligible(q))
-        e = launch_gemm_pair(q, ctx->cs, &ctx->stats.kernel_launches, &err);
-      else
-        e = launch_gemm(q, ctx->cs, &ctx->stats.kernel_launches, &err);
+      ATS_TRY(launch_gemm_any(ctx, q));
     }
-    if (e != cudaSuccess) return check_cuda(ctx, e, err.empty() ? "launch_gemm" : err.c_str());
     ATS_TRY(release_ops(ctx, ops + i, 1));
     row0 += (int)ops[i].t->d.n_out;
   }
+  if (p.act) ATS_CUDA(launch_swiglu16(p.y, p.ldy, p.ldact, p.act, p.T, ctx->cs, &ctx->stats.kernel_launches, p.pdl));
   return ATS_OK;
 }
 
@@ -468,6 +481,7 @@ static LayerWs layout_prefill(const ats_layer_desc& L, uint32_t T, uint8_t* base
   b.take(kWsReserved);
   const uint64_t H = L.hidden, qd = (uint64_t)L.n_q_heads * L.head_dim, kvd = (uint64_t)L.n_kv_heads * L.head_dim;
   uint64_t scratch = 0;
+  auto gemm_want = [&](int n, int k) { return std::max(gemm_scratch_bytes((int)T, n, k), gemm_ts_scratch_bytes((int)T, n, k)); };
   if (L.wq >= 0) {
     w.h16 = (__half*)b.take(T * H * 2);
     w.qkv16 = (__half*)b.take(T * (qd + 2 * kvd) * 2);
@@ -475,8 +489,8 @@ static LayerWs layout_prefill(const ats_layer_desc& L, uint32_t T, uint8_t* base
     w.a16 = (__half*)b.take(T * qd * 2);
     w.o16 = (__half*)b.take(T * H * 2);
     w.x1_16 = (__half*)b.take(T * H * 2);
-    scratch = std::max(scratch, gemm_scratch_bytes((int)T, (int)(qd + 2 * kvd), (int)H));
-    scratch = std::max(scratch, gemm_scratch_bytes((int)T, (int)H, (int)qd));
+    scratch = std::max(scratch, gemm_want((int)(qd + 2 * kvd), (int)H));
+    scratch = std::max(scratch, gemm_want((int)H, (int)qd));
   }
   w.h2_16 = (__half*)b.take(T * H * 2);
   if (L.n_experts) {
@@ -495,8 +509,8 @@ static LayerWs layout_prefill(const ats_layer_desc& L, uint32_t T, uint8_t* base
     w.gu16 = (__half*)b.take((uint64_t)T * 2 * L.ffn * 2);
     w.act16 = (__half*)b.take((uint64_t)T * L.ffn * 2);
     w.d16 = (__half*)b.take(T * H * 2);
-    scratch = std::max(scratch, gemm_scratch_bytes((int)T, (int)(2 * L.ffn), (int)H));
-    scratch = std::max(scratch, gemm_scratch_bytes((int)T, (int)H, (int)L.ffn));
+    scratch = std::max(scratch, gemm_want((int)(2 * L.ffn), (int)H));
+    scratch = std::max(scratch, gemm_want((int)H, (int)L.ffn));
   }
   w.gemm_scratch = b.take(scratch);
   w.gemm_scratch_bytes = scratch;
@@ -1020,16 +1034,17 @@ int32_t ats_linear(ats_ctx* ctx, int32_t id, const void* x, void* y, uint32_t M)
     return run_gemv_group(ctx, &op, 1, p);
   }
   GemmParams g{};
+  g.pdl = (ctx->cfg.flags & ATS_FLAG_NO_PDL) ? 0 : 1;
   g.T = (int)M;
   g.x = (const __half*)x;
   g.ldx = (int)t->d.k_in;
   g.y = (__half*)y;
   g.ldy = (int)t->d.n_out;
-  g.scratch_bytes = gemm_scratch_bytes((int)M, (int)t->d.n_out, (int)t->d.k_in);
-  if (g.scratch_bytes + kWsReserved > align_up(ctx->cfg.workspace_bytes))
-    return fail(ctx, ATS_ERR_NOMEM, "workspace too small for the GEMM: need %llu bytes",
-                (unsigned long long)(g.scratch_bytes + kWsReserved));
+  const uint64_t need = gemm_scratch_bytes((int)M, (int)t->d.n_out, (int)t->d.k_in);
+  if (need + kWsReserved > align_up(ctx->cfg.workspace_bytes))
+    return fail(ctx, ATS_ERR_NOMEM, "workspace too small for the GEMM: need %llu bytes", (unsigned long long)(need + kWsReserved));
   g.scratch = ctx->ws + kWsReserved;
+  g.scratch_bytes = align_up(ctx->cfg.workspace_bytes) - kWsReserved;
   return run_gemm_group(ctx, &op, 1, g);
 }
 
@@ -1202,6 +1217,7 @@ int32_t ats_linear_static_scratch(ats_ctx* ctx, int32_t id, const void* x, void*
   void* scratch = nullptr;
   ATS_CUDA(gemm_static_scratch(&scratch));
   GemmParams g{};
+  g.pdl = (ctx->cfg.flags & ATS_FLAG_NO_PDL) ? 0 : 1;
   g.T = (int)M;
   g.x = (const __half*)x;
   g.ldx = (int)t->d.k_in;
@@ -1778,7 +1794,6 @@ int32_t ats_layer_prefill(ats_ctx* ctx, const ats_layer_desc* L, const void* x_i
         ctx->stats.streamed_bytes += need;
       }
     }
-    std::string err;
     GemmParams m{};
     m.T = P;
     m.pdl = pdl;
@@ -1799,9 +1814,10 @@ int32_t ats_layer_prefill(ats_ctx* ctx, const ats_layer_desc* L, const void* x_i
     m.ldx = H;
     m.y = w.gu16;
     m.ldy = 2 * F;
-    cudaError_t ce = launch_gemm(m, ctx->cs, nl, &err);
-    if (ce != cudaSuccess) return check_cuda(ctx, ce, err.empty() ? "launch_gemm (expert gate/up)" : err.c_str());
-    ATS_CUDA(launch_swiglu16(w.gu16, 2 * F, F, w.act16, P, ctx->cs, nl, pdl));
+    m.act = w.act16;
+    m.ldact = F;
+    ATS_TRY(launch_gemm_any(ctx, m));
+    m.act = nullptr;
     m.n_seg = 1;
     m.K = F;
     m.seg[0] = GemvSeg{slice0(td), H};
@@ -1812,8 +1828,7 @@ int32_t ats_layer_prefill(ats_ctx* ctx, const ats_layer_desc* L, const void* x_i
     m.ldx = F;
     m.y = w.d16;
     m.ldy = H;
-    ce = launch_gemm(m, ctx->cs, nl, &err);
-    if (ce != cudaSuccess) return check_cuda(ctx, ce, err.empty() ? "launch_gemm (expert down)" : err.c_str());
+    ATS_TRY(launch_gemm_any(ctx, m));
     ATS_CUDA(launch_moe_combine_sorted(resid, w.gates, w.d16, w.pos, (__half*)x_out, (int)T, k, H, ctx->cs, nl, pdl));
     return ATS_OK;
   }
@@ -1821,8 +1836,10 @@ int32_t ats_layer_prefill(ats_ctx* ctx, const ats_layer_desc* L, const void* x_i
   g.ldx = H;
   g.y = w.gu16;
   g.ldy = 2 * (int)L->ffn;
+  g.act = w.act16;
+  g.ldact = (int)L->ffn;
   ATS_TRY(run_gemm_group(ctx, gu, 2, g));
-  ATS_CUDA(launch_swiglu16(w.gu16, 2 * (int)L->ffn, (int)L->ffn, w.act16, (int)T, ctx->cs, nl, pdl));
+  g.act = nullptr;
   g.x = w.act16;
   g.ldx = (int)L->ffn;
   g.y = w.d16;

@@ -2,7 +2,7 @@
 // over the cache (tensor cores), fp16 residual add and SwiGLU.  Every intermediate of the prefill path is stored as fp16 (the
 // operands of the tensor-core GEMMs), so these kernels read and write fp16 and compute in fp32.
 #include "ats_internal.h"
-#include "sm100_sync.cuh"
+#include "sm100_umma.cuh"
 
 namespace ats {
 
@@ -308,7 +308,7 @@ __global__ void swiglu16_kernel(const __half* __restrict__ gu, int ld, int ffn, 
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       const float2 g = __half22float2(bits_as_half2(gw[q])), u = __half22float2(bits_as_half2(uw[q]));
-      const __half2 r = __floats2half2_rn(g.x / (1.0f + expf(-g.x)) * u.x, g.y / (1.0f + expf(-g.y)) * u.y);
+      const __half2 r = __floats2half2_rn(silu_times(g.x, u.x), silu_times(g.y, u.y));  // (the fused form's arithmetic)
       ow[q] = *reinterpret_cast<const uint32_t*>(&r);
     }
     *reinterpret_cast<uint4*>(act + t * ffn + c) = make_uint4(ow[0], ow[1], ow[2], ow[3]);

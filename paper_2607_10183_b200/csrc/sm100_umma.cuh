@@ -109,6 +109,14 @@ __device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, i
       : "memory");
 }
 
+// silu(g) u.  exp2 and reciprocal approximations are good to a few units of the 24th bit; the result is rounded to 11.
+__device__ __forceinline__ float silu_times(float g, float u) {
+  float e, r;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(g * -1.4426950408889634f));
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(1.0f + e));
+  return g * r * u;
+}
+
 // One lane polls for its warp (hundreds of threads polling one barrier word slow its arrivals down).
 __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, int lane) {
   int got = 1;

@@ -1,0 +1,40 @@
+"""The dequantizing GEMM with the weights in tensor memory at the edges of its tiles, units and work ranges, against the oracle."""
+import numpy as np
+import pytest
+
+from oracle import ats_oracle as O
+from paper_2607_10183_b200 import workloads as W
+from tests import helpers as H
+
+pytestmark = pytest.mark.gpu
+MB = 1 << 20
+
+
+# K: one 32-wide block, a 64-k step and its neighbours, a 128-k unit and its neighbours, an odd number of blocks per row (scales
+# read from 4-byte boundaries); N around one CTA's 128 and the pair's 256 features; T around 32, the tiles of 128 and 256 and
+# their multiples; long reductions of few tiles (a tile summed by two to four CTA pairs, each in several parts, with one
+# accumulator and with two) and many tiles (ranges that begin and end inside tiles).
+@pytest.mark.parametrize("fmt", ["q4", "mxfp4"])
+@pytest.mark.parametrize("N,K,T", [(1, 32, 9), (127, 64, 31), (129, 96, 33), (255, 160, 255), (257, 224, 256), (256, 256, 257), (300, 288, 513),
+                                   (128, 16384, 10), (200, 4128, 65), (513, 2080, 300), (9600, 512, 12), (6001, 1056, 270), (8192, 1024, 600)])
+def test_gemm_edges_match_oracle(fmt, N, K, T):
+    import torch
+    from paper_2607_10183_b200 import binding as B
+    packed, scales = (W.q4_packed if fmt == "q4" else W.mxfp4_packed)(91, 0, W.ROLE_UP, N, K)
+    x = W.activations(91, 0, (T, K))
+    ws = 8 * T * N * 4 + 2 * MB
+    ctx = B.Context(ws + W.q4_bytes(N, K) + 2 * MB, workspace_bytes=ws)
+    tid = ctx.register_q4(packed, scales)
+    ctx.set_placement([(tid, -1, B.ATS_GPU)])
+    xd = H.to_dev(x)
+    outs = []
+    for _ in range(2):  # the second call finds the arrival counters as the first left them
+        y = torch.full((T + 1, N), 7.0, dtype=torch.float16, device="cuda")
+        ctx.linear(tid, xd, y, T)
+        ctx.sync()
+        outs.append(y.cpu().numpy())
+    ctx.close()
+    rows = np.unique(np.r_[0, T // 2, T - 1, np.arange(max(0, T - 3), T), np.arange(min(T, 256) - 2, min(T, 256)), np.arange(0, T, 97)])
+    H.assert_close(outs[0][rows], O.linear(x[rows], packed, scales, O.WEIGHT_F16, round_out=True), what=f"{fmt} {N}x{K} T={T}")
+    assert np.all(outs[0][T] == 7.0)
+    assert np.array_equal(outs[0].view(np.uint16), outs[1].view(np.uint16))
