@@ -832,7 +832,7 @@ cudaError_t launch_attn_decode_fused(AttnDecodeParams p, int d, int pdl, cudaStr
 // Warp 0 extracts the k largest logits (equal logits: lower index first) and their gates from logit[Epad] in shared memory.
 __device__ __forceinline__ void router_select(const float* logit, int m, int E, int Epad, int k, int renorm,
                                               int32_t* __restrict__ ids, float* __restrict__ gates) {
-  const int lane = threadIdx.x;
+  const int lane = threadIdx.x & 31;
   const int per = Epad / 32;  // candidates per lane: e = lane + 32*j
   uint32_t taken = 0;
   float sel_v = 0.f;  // lane j (< k) keeps the j-th selected logit
@@ -1139,6 +1139,114 @@ __global__ void __launch_bounds__(kRouterClThreads) router_topk_cluster_kernel(c
   router_select(logit, m, E, Epad, k, renorm, ids, gates);
 }
 
+// The same routing for many tokens: a CTA takes four tokens and streams the whole router matrix through shared memory (16-byte
+// asynchronous copies, stages of 32 KB), so that a weight is read from L2 and converted once for four tokens.  Thread (row
+// group, four experts) sums its chain of rows in each of the eight ranges, and the chains and ranges are added up in
+// router_topk_cluster_kernel's order, so a token's logits have the same bits whichever kernel ran.  Bound by instruction issue
+// (16 multiply-adds, 4 conversions and 2 shared-memory loads per row and thread).  512 tokens of 2048 through 128 experts: 71.7 ->
+// 24.8 us, 512 of 2048 through 256: 140 -> 39 us.
+constexpr int kRouterTok = 4;
+constexpr int kRouterTokThreads = 512;   // 4 experts each: E / 4 x (2048 / E) row groups
+constexpr int kRouterStageRows = 8;      // rows of a chain per stage
+constexpr int kRouterStageElems = kRouterStageRows * 2048;  // ... of all R = 2048 / E chains: contiguous rows of W_r
+// One wave of CTAs takes 23 us (128 experts of 2048) to 45 us (512 of 1024) whatever the tokens, the cluster kernel 14.5 and 31 us for 64
+// tokens, 22.9 and 48.5 us for 128.
+constexpr int kRouterManyTokens = 128;
+
+__global__ void __launch_bounds__(kRouterTokThreads) router_topk_tokens_kernel(const __half* __restrict__ h, const __half* __restrict__ wr, int M,
+                                                                               int H, int E, int Epad, int k, int renorm, int stages,
+                                                                               int32_t* __restrict__ ids, float* __restrict__ gates) {
+  extern __shared__ __align__(16) float smem[];
+  const int Hc = H / kRouterCluster, R = 2048 / E, per_range = Hc / R / kRouterStageRows, n_st = kRouterCluster * per_range;
+  __half* w_s = reinterpret_cast<__half*>(smem);                                   // [stages][8 R rows][E]
+  float4* h_s = reinterpret_cast<float4*>(w_s + (size_t)stages * kRouterStageElems);  // [H]: the row's element of the four tokens
+  float* part = reinterpret_cast<float*>(h_s + H);                                 // [R][kRouterTok][E]
+  float* logit = part + (size_t)2048 * kRouterTok;                                 // [kRouterTok][Epad]
+  const int tid = threadIdx.x, m0 = blockIdx.x * kRouterTok, live = min(kRouterTok, M - m0);
+  const int lanes = E / 4, grp = tid / lanes, e0 = (tid % lanes) * 4;
+  int ld_st = 0, ld_at = 0;  // next stage to load and its place in the ring
+  const __half* src = wr;
+  const uint32_t ring = (uint32_t)__cvta_generic_to_shared(w_s);
+  auto load = [&] {
+    if (ld_st < n_st) {
+      const uint32_t dst = ring + (uint32_t)(ld_at * kRouterStageElems * 2);
+#pragma unroll
+      for (int q = 0; q < kRouterStageElems / 8 / kRouterTokThreads; ++q) {
+        const int c = (tid + q * kRouterTokThreads) * 8;
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + 2u * c), "l"(src + c) : "memory");
+      }
+      src += kRouterStageElems;
+      ++ld_st;
+      if (++ld_at == stages) ld_at = 0;
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  load();  // (the router matrix does not depend on the preceding kernel)
+  load();
+  if (stages == 4) load();
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  for (int j = tid; j < kRouterTok * (H / 8); j += kRouterTokThreads) {
+    const int t = j & 3, i = (j >> 2) * 8;
+    const uint4 v = t < live ? *reinterpret_cast<const uint4*>(h + (size_t)(m0 + t) * H + i) : make_uint4(0, 0, 0, 0);
+    const uint32_t vs[4] = {v.x, v.y, v.z, v.w};
+    float* d = reinterpret_cast<float*>(h_s + i) + t;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const float2 f = __half22float2(u32_as_half2(vs[q]));
+      d[8 * q] = f.x;
+      d[8 * q + 4] = f.y;
+    }
+  }
+  for (int j = tid; j < kRouterTok * Epad; j += kRouterTokThreads) logit[j] = 0.f;
+  float acc[kRouterTok][4];
+  int at = 0, in_range = 0;  // place in the ring, stage of the range
+  const __half* w0 = w_s + (size_t)grp * E + e0;
+  const float4* xr = h_s + grp;
+  for (int st = 0; st < n_st; ++st) {
+    if (stages == 4) asm volatile("cp.async.wait_group 2;" ::: "memory");
+    else asm volatile("cp.async.wait_group 1;" ::: "memory");
+    __syncthreads();  // stage st is there, and everybody has read stage st - 1: its place is free
+    load();
+    if (in_range == 0) {
+#pragma unroll
+      for (int t = 0; t < kRouterTok; ++t)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[t][q] = 0.f;
+    }
+    const __half* w = w0 + at * kRouterStageElems;
+#pragma unroll
+    for (int b = 0; b < kRouterStageRows; ++b) {
+      const float4 x = xr[b * R];
+      const uint2 wv = *reinterpret_cast<const uint2*>(w + b * 2048);
+      const float2 wa = __half22float2(u32_as_half2(wv.x)), wb = __half22float2(u32_as_half2(wv.y));
+      const float xs[kRouterTok] = {x.x, x.y, x.z, x.w}, ws[4] = {wa.x, wa.y, wb.x, wb.y};
+#pragma unroll
+      for (int t = 0; t < kRouterTok; ++t)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[t][q] = fmaf(xs[t], ws[q], acc[t][q]);
+    }
+    xr += kRouterStageRows * R;
+    if (++at == stages) at = 0;
+    if (++in_range == per_range) {  // the range's chains are complete
+      in_range = 0;
+#pragma unroll
+      for (int t = 0; t < kRouterTok; ++t)
+        *reinterpret_cast<float4*>(part + ((size_t)grp * kRouterTok + t) * E + e0) = make_float4(acc[t][0], acc[t][1], acc[t][2], acc[t][3]);
+      __syncthreads();
+      for (int j = tid; j < kRouterTok * E; j += kRouterTokThreads) {
+        float v = 0.f;
+#pragma unroll 8
+        for (int g = 0; g < R; ++g) v += part[g * kRouterTok * E + j];
+        logit[j] += v;  // (E >= 32 is a power of two: E = Epad)
+      }
+    }
+  }
+  __syncthreads();
+  const int t = tid >> 5;  // one warp per token
+  if (t < live) router_select(logit + t * Epad, m0 + t, E, Epad, k, renorm, ids, gates);
+}
+
 cudaError_t launch_router_topk(const __half* h, const __half* wr, int M, int H, int E, int k, int renorm, int32_t* ids,
                                float* gates, cudaStream_t st, uint64_t* n_launch, int pdl) {
   return launch_router_topk_norm(h, wr, M, H, E, k, renorm, ids, gates, nullptr, 0, nullptr, 0.f, st, n_launch, pdl);
@@ -1154,6 +1262,19 @@ cudaError_t launch_router_topk_norm(const __half* h, const __half* wr, int M, in
   if (E % 8 == 0 && H % (8 * kRouterCluster) == 0 && H <= 8 * kRouterClThreads * kRouterCluster && (((uintptr_t)wr | (uintptr_t)h) & 15) == 0) {
     const int L = E / 8, R = kRouterClThreads / L;
     const size_t smem_cl = ((size_t)H / kRouterCluster + (size_t)R * E + (size_t)(kRouterCluster + 1) * Epad) * sizeof(float);
+    auto smem_tok = [&](int stages) {
+      return (size_t)stages * kRouterStageElems * 2 + ((size_t)4 * H + 2048 * kRouterTok + (size_t)kRouterTok * Epad) * sizeof(float);
+    };
+    constexpr size_t kMost = 227 * 1024 - 2048;
+    // (chains of a multiple of eight rows: 2048 / E of them in each range)
+    if (M >= kRouterManyTokens && !norm_gain && E == Epad && 2048 % E == 0 && H / kRouterCluster % (kRouterStageRows * R) == 0 && smem_tok(3) <= kMost) {
+      const int stages = smem_tok(4) <= kMost ? 4 : 3;
+      const cudaError_t e = cudaFuncSetAttribute(router_topk_tokens_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_tok(stages));
+      if (e != cudaSuccess) return e;
+      ++*n_launch;
+      return launch_dep(router_topk_tokens_kernel, dim3((M + kRouterTok - 1) / kRouterTok), dim3(kRouterTokThreads), smem_tok(stages), st, pdl, 1,
+                        h, wr, M, H, E, Epad, k, renorm, stages, ids, gates);
+    }
     if (smem_cl <= 160 * 1024) {
       if (smem_cl > 48 * 1024) {  // (cheap; set on every call because the size depends on the shape)
         cudaError_t e = cudaFuncSetAttribute(router_topk_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_cl);

@@ -737,6 +737,34 @@ def test_route_topk_bit_exact_with_ties(B, torch, Hd, E, k):
     ctx.close()
 
 
+# Many tokens (the kernel that takes four tokens per CTA): the last CTA with one to four tokens, the shortest chains it takes (eight
+# rows), 32 experts and as many as 1024, three stages instead of four; and the neighbours it leaves to the cluster kernel.
+@pytest.mark.parametrize("Hd,E,k,M", [(512, 256, 8, 128), (2048, 128, 8, 129), (4096, 32, 4, 130), (4096, 64, 6, 131), (256, 1024, 32, 132),
+                                      (6144, 128, 8, 128), (2048, 128, 8, 127), (2048, 96, 8, 128)])
+def test_route_topk_many_tokens(B, torch, Hd, E, k, M):
+    rng = np.random.default_rng(13)
+    Wr = rng.normal(0, 0.02, size=(Hd, E)).astype(np.float16)
+    Wr[:, 9] = Wr[:, 30] = Wr[:, 2]
+    h = rng.normal(size=(M, Hd)).astype(np.float16)
+    h[M - 1] = (Wr[:, 2].astype(np.float32) * 50).astype(np.float16)
+    ids_ref, gates_ref, logits = O.route_topk(h, Wr, k)
+    assert ids_ref[M - 1, :3].tolist() == [2, 9, 30]
+    top = -np.sort(-logits, axis=1)[:, :k + 1]
+    clear = np.array([np.all((d > 1e-5) | (d == 0)) for d in top[:, :-1] - top[:, 1:]])  # fp32 sums of O(1) logits: 1e-6
+    assert clear.mean() > 0.9
+    ctx = make_ctx(B, 4 * MB)
+    rid = ctx.register_f16(Wr)
+    ctx.set_placement([])
+    ids = torch.full((M + 1, k), -7, dtype=torch.int32, device="cuda")
+    gates = torch.empty((M, k), dtype=torch.float32, device="cuda")
+    ctx.route_topk(rid, H.to_dev(h), M, k, ids, gates)
+    ctx.sync()
+    got = ids.cpu().numpy()
+    ctx.close()
+    assert np.array_equal(got[:M][clear], ids_ref[clear]) and np.all(got[M] == -7)
+    assert np.max(np.abs(gates.cpu().numpy()[clear] - gates_ref[clear])) <= 1e-5  # gates move by at most the logits' error
+
+
 def run_moe(B, torch, shape, cfg, M, host_experts, ring_slots=8, chunk=MB, flags=0, ws=4 * MB):
     Bk = W.moe_block(cfg, 0, shape)
     sl = W.q4_bytes(shape.ffn, shape.hidden)
