@@ -111,7 +111,8 @@ __device__ __forceinline__ void attn_decode_compute(const AttnDecodeParams& p, c
   constexpr int CH = D * 2 / 16;       // 16-byte chunks per cache row
   constexpr int KROW = D * 2 + 16;     // key row pitch in shared memory: the 16-byte pad makes lane-per-row reads conflict-free
   constexpr int VROW = D * 2;
-  constexpr int EPT = D / 64;          // output elements per thread in the merges (64 threads per head)
+  constexpr int TPH = POS < D ? POS : D;  // threads per head in the merges (of the head's POS)
+  constexpr int EPT = D / TPH;            // output elements of each
   uint8_t* k_s = dyn_s;                              // [POS][KROW]
   uint8_t* v_s = dyn_s + (size_t)POS * KROW;    // [POS][VROW]
   float (&q_s)[kAttnMaxGroup][kAttnMaxD] = as.q_s;
@@ -229,10 +230,10 @@ __device__ __forceinline__ void attn_decode_compute(const AttnDecodeParams& p, c
   for (int v = 0; v < V; ++v) w_acc[warp][lane * V + v] = acc[v];
   ATS_ATR(4);
   job_sync();
-  // merge each head's warps (ascending) into this split's partial: 64 threads per head
-  const int g2 = tid / 64, j = tid % 64;
+  // merge each head's warps (ascending) into this split's partial
+  const int g2 = g, j = tid % POS;
   const int hq2 = hbase + g2;
-  if (g2 < G) {
+  if (j < TPH) {
     float* part = p.part + ((size_t)hq2 * n_splits + split) * (D + 2);
     float mx = -INFINITY;
 #pragma unroll
@@ -246,10 +247,10 @@ __device__ __forceinline__ void attn_decode_compute(const AttnDecodeParams& p, c
       const float f = m > -INFINITY ? expf(m - mx) : 0.f;
       l = fmaf(w_l[g2 * SUB + w], f, l);
 #pragma unroll
-      for (int q = 0; q < EPT; ++q) o[q] = fmaf(w_acc[g2 * SUB + w][j + 64 * q], f, o[q]);
+      for (int q = 0; q < EPT; ++q) o[q] = fmaf(w_acc[g2 * SUB + w][j + TPH * q], f, o[q]);
     }
 #pragma unroll
-    for (int q = 0; q < EPT; ++q) part[j + 64 * q] = o[q];
+    for (int q = 0; q < EPT; ++q) part[j + TPH * q] = o[q];
     if (j == 0) {
       part[D] = mx;
       part[D + 1] = l;
@@ -269,34 +270,36 @@ __device__ __forceinline__ void attn_decode_compute(const AttnDecodeParams& p, c
   }
   job_sync();
   ATS_ATR(6);
-  if (!is_last || g2 >= G) return;
+  if (!is_last || j >= TPH) return;
   const float* base = p.part + (size_t)hq2 * n_splits * (D + 2);
   float mx = -INFINITY, l = 0.f, o[EPT];
 #pragma unroll
   for (int q = 0; q < EPT; ++q) o[q] = 0.f;
-  constexpr int NB = 16;  // splits per round trip: all of a batch's loads are issued before any is used
+  // A batch of splits per round trip: lane u fetches the maximum and the sum of split u, every thread its elements of all of
+  // them.  (Every thread fetching all three for 16 splits took 80 registers: one CTA of 512 threads per SM, two waves of them
+  // for 4091 positions of 8 kv heads.  At 64 registers two share an SM: a decode step there 55.6 -> 52.1 us, at 1025 positions,
+  // where all threads of a head's warps merge now, 36.1 -> 35.8.)
+  constexpr int NB = 32 / EPT;
   for (int s0 = 0; s0 < n_splits; s0 += NB) {
-    float m[NB], ls[NB], v[NB][EPT];
+    const bool mine = lane < NB && s0 + lane < n_splits;
+    const float* ps = base + (size_t)s0 * (D + 2);
+    const float m_u = mine ? __ldcg(ps + (size_t)lane * (D + 2) + D) : -INFINITY;
+    const float l_u = mine ? __ldcg(ps + (size_t)lane * (D + 2) + D + 1) : 0.f;
+    float v[NB][EPT];
 #pragma unroll
-    for (int u = 0; u < NB; ++u) {
-      const bool in = s0 + u < n_splits;
-      const float* ps = base + (size_t)(s0 + u) * (D + 2);
-      m[u] = in ? __ldcg(ps + D) : -INFINITY;
-      ls[u] = in ? __ldcg(ps + D + 1) : 0.f;
+    for (int u = 0; u < NB; ++u)
 #pragma unroll
-      for (int q = 0; q < EPT; ++q) v[u][q] = in ? __ldcg(ps + j + 64 * q) : 0.f;
-    }
-    float bm = mx;
-#pragma unroll
-    for (int u = 0; u < NB; ++u) bm = fmaxf(bm, m[u]);
+      for (int q = 0; q < EPT; ++q) v[u][q] = s0 + u < n_splits ? __ldcg(ps + (size_t)u * (D + 2) + j + TPH * q) : 0.f;
+    const float bm = fmaxf(mx, ad_warp_max(m_u));
     const float rs = mx > -INFINITY ? expf(mx - bm) : 0.f;  // rescale what earlier batches accumulated
+    const float f_u = m_u > -INFINITY ? expf(m_u - bm) : 0.f;
     l *= rs;
 #pragma unroll
     for (int q = 0; q < EPT; ++q) o[q] *= rs;
 #pragma unroll
     for (int u = 0; u < NB; ++u) {
-      const float f = m[u] > -INFINITY ? expf(m[u] - bm) : 0.f;
-      l = fmaf(ls[u], f, l);
+      const float f = __shfl_sync(0xffffffffu, f_u, u);
+      l = fmaf(__shfl_sync(0xffffffffu, l_u, u), f, l);
 #pragma unroll
       for (int q = 0; q < EPT; ++q) o[q] = fmaf(v[u][q], f, o[q]);
     }
@@ -304,7 +307,7 @@ __device__ __forceinline__ void attn_decode_compute(const AttnDecodeParams& p, c
   }
   const float inv = 1.0f / l;
 #pragma unroll
-  for (int q = 0; q < EPT; ++q) p.a16[(size_t)hq2 * D + j + 64 * q] = __float2half_rn(o[q] * inv);
+  for (int q = 0; q < EPT; ++q) p.a16[(size_t)hq2 * D + j + TPH * q] = __float2half_rn(o[q] * inv);
   ATS_ATR(7);
 }
 

@@ -761,7 +761,7 @@ cudaError_t launch_rmsnorm(const void* x, int x_is_f32, const __half* gain, __ha
 // there, so the cache crosses the L2-to-SM fabric once instead of once per query head; that traffic, not DRAM, bounds
 // this kernel.  Warp (head, sub-block) owns 32 positions, one per lane.
 // Positions per CTA: 64, or 128 for contexts beyond 1024 so that the final merge still reads all splits of a head in
-// one round trip (16 splits) up to 2048 positions.  (64 positions up to 2048, with both kernels' registers capped so that
+// one round trip (16 splits of 64 positions, 32 of 128) up to 4096 positions.  (64 positions up to 2048, with both kernels' registers capped so that
 // a CTA of this kernel fits an SM beside a CTA of the streaming GEMV, was measured and lost: the GEMV slows down by 0.5 us
 // per launch at 80 registers and this kernel by 2.9 us with 17 splits to merge, and nothing is gained back.)
 // (A tensor-core form, scores as Q K^T and outputs as V^T P^T by mma.sync m16n8k16 with the group's heads as operand rows,
@@ -780,7 +780,7 @@ size_t attn_decode_scratch_floats(int n_q, int d, int n_ctx) {
 }
 
 template <int D, int SUB>
-__global__ void __launch_bounds__(512) attn_decode_fused_kernel(const AttnDecodeParams p) {
+__global__ void __launch_bounds__(512, 2) attn_decode_fused_kernel(const AttnDecodeParams p) {
   extern __shared__ __align__(16) uint8_t dyn_s[];
   __shared__ AttnShared as;
   attn_decode_body<D, SUB, true>(p, (int)blockIdx.x, (int)blockIdx.y, (int)gridDim.x, (int)threadIdx.x, (int)blockDim.x, dyn_s, as);

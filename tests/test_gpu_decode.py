@@ -737,6 +737,20 @@ def test_route_topk_bit_exact_with_ties(B, torch, Hd, E, k):
     ctx.close()
 
 
+# The merge of the splits takes 32 of them (two output elements per thread: 16) in one round trip: contexts of exactly that many
+# splits, one more, and three round trips, for both head dimensions and with 64 and 128 positions per split.
+@pytest.mark.parametrize("d,group,pos", [(64, 2, 2047), (64, 2, 4095), (64, 2, 4096), (64, 2, 8300), (128, 1, 4096), (128, 4, 8191),
+                                         (128, 8, 1023), (128, 8, 1024), (128, 8, 2048)])
+def test_attention_merge_round_trips(B, torch, d, group, pos):
+    shape = W.DenseShape(hidden=256, n_q_heads=2 * group, n_kv_heads=2, head_dim=d, ffn=448)
+    dbg = {}
+    ys, kg, vg, st, (edges, wmode) = run_dense_decode(B, torch, shape, 97, pos, pos + 1, ALL_GPU, debug=dbg)
+    L = W.dense_layer(97, 0, shape)
+    kc, vc = W.kv_cache(97, 0, 2, pos + 1, d, pos)
+    want = O.dense_layer(W.activations(97, 0, (1, 256)), H.oracle_dense_tensors(L), shape, kc, vc, pos, edges, wmode)
+    H.assert_close(ys[0], want, what=f"layer, {pos + 1} positions")
+
+
 # Many tokens (the kernel that takes four tokens per CTA): the last CTA with one to four tokens, the shortest chains it takes (eight
 # rows), 32 experts and as many as 1024, three stages instead of four; and the neighbours it leaves to the cluster kernel.
 @pytest.mark.parametrize("Hd,E,k,M", [(512, 256, 8, 128), (2048, 128, 8, 129), (4096, 32, 4, 130), (4096, 64, 6, 131), (256, 1024, 32, 132),
