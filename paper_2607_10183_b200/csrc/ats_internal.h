@@ -355,22 +355,18 @@ struct GemmParams {
   int grp_max_rows;         // the largest expert's row count (sizes the grid)
   uint64_t grp_stride;
   const uint8_t* const* grp_tab[3];
-  // optional fused SwiGLU (launch_gemm_ts only): act[t][f] = rn16(silu(y[t][f]) * y[t][n_rows + f]) of segments gate, up;
+  // optional fused SwiGLU (launch_gemm_pair only): act[t][f] = rn16(silu(y[t][f]) * y[t][n_rows + f]) of segments gate, up;
   // y itself is written only where it is not null
   __half* act;
   int ldact;
-  int* counters;  // kAttnMaxCounters ints, zero between launches (launch_gemm_ts: arrival counts of split tiles)
+  int* counters;  // kAttnMaxCounters ints, zero between launches (launch_gemm_pair: arrival counts of split tiles)
 };
-// The dequantizing GEMM with the weights in tensor memory (kernels_gemm_ts.cu): operands it takes, scratch it likes to have
-// (it runs with any), and its launcher
-bool gemm_ts_eligible(const GemmParams& p);
-uint64_t gemm_ts_scratch_bytes(int T, int n_total, int K);
-cudaError_t launch_gemm_ts(const GemmParams& p, int sm_count, cudaStream_t st, uint64_t* n_launch, std::string* err);
+// GEMMs on pairs of CTAs (kernels_gemm_pair.cu): operands they take, scratch they like to have (they run with any), and their launcher
+bool gemm_pair_eligible(const GemmParams& p);
+uint64_t gemm_pair_scratch_bytes(int T, int n_total, int K);
+cudaError_t launch_gemm_pair(const GemmParams& p, int sm_count, cudaStream_t st, uint64_t* n_launch, std::string* err);
 uint64_t gemm_scratch_bytes(int T, int n_total, int K);
 cudaError_t launch_gemm(const GemmParams& p, cudaStream_t st, uint64_t* n_launch, std::string* err);
-// GEMMs as pairs of CTAs (kernels_gemm_pair.cu): shapes they take, and their launcher
-bool gemm_pair_eligible(const GemmParams& p);
-cudaError_t launch_gemm_pair(const GemmParams& p, cudaStream_t st, uint64_t* n_launch, std::string* err);
 // fixed split-K scratch inside the library's device image (no allocation): capacity, and its address on the current device
 uint64_t gemm_static_scratch_capacity();
 cudaError_t gemm_static_scratch(void** out);

@@ -341,20 +341,17 @@ static int32_t run_gemv_group(ats_ctx* ctx, Operand* ops, int n, GemvParams p) {
   return ATS_OK;
 }
 
-// One GEMM launch: the 4-bit formats on the kernel that keeps the weights in tensor memory, fp16 matrices as CTA pairs where
-// they have enough tiles, else the single-CTA kernel (slice address tables; ATS_FLAG_NO_GEMM_PAIR).  A SwiGLU that was asked for
-// runs in the epilogue or as a launch of its own.
+// One GEMM launch: on pairs of CTAs, or the single-CTA kernel (slice address tables; ATS_FLAG_NO_GEMM_PAIR).  A SwiGLU that was
+// asked for runs in the epilogue or as a launch of its own.
 static int32_t launch_gemm_any(ats_ctx* ctx, GemmParams p) {
   std::string err;
   cudaError_t e;
   __half* act = p.act;
   p.counters = reinterpret_cast<int*>(ctx->ws) + 64;  // (the attention's: zero between launches, and launches follow one another)
   const bool pairs = !(ctx->cfg.flags & ATS_FLAG_NO_GEMM_PAIR);
-  if (pairs && gemm_ts_eligible(p)) {
-    e = launch_gemm_ts(p, ctx->sm_count, ctx->cs, &ctx->stats.kernel_launches, &err);
+  if (pairs && gemm_pair_eligible(p)) {
+    e = launch_gemm_pair(p, ctx->sm_count, ctx->cs, &ctx->stats.kernel_launches, &err);
     act = nullptr;
-  } else if (pairs && gemm_pair_eligible(p)) {
-    e = launch_gemm_pair(p, ctx->cs, &ctx->stats.kernel_launches, &err);
   } else {
     e = launch_gemm(p, ctx->cs, &ctx->stats.kernel_launches, &err);
   }
@@ -368,8 +365,15 @@ static int32_t run_gemm_group(ats_ctx* ctx, Operand* ops, int n, GemmParams p) {
   p.status = ctx->dev_status;
   p.w16 = ops[0].t->d.fmt == ATS_FMT_W16;  // a group shares one format (check_layer)
   p.mx = ops[0].t->d.fmt == ATS_FMT_MXFP4;
-  // fp16 weight tiles come through one tensor map per matrix: such a group always runs matrix by matrix
-  if ((count_streamed(ops, n) <= (int)ctx->cfg.ring_slots && !p.w16) || n == 1) {
+  bool together = n == 1 || count_streamed(ops, n) <= (int)ctx->cfg.ring_slots;
+  if (together && p.w16 && n > 1) {  // (the single-CTA kernel takes fp16 matrices one by one)
+    GemmParams probe = p;
+    probe.counters = reinterpret_cast<int*>(ctx->ws) + 64;
+    probe.n_seg = n;
+    for (int i = 0; i < n; ++i) probe.seg[i] = GemvSeg{nullptr, (int)ops[i].t->d.n_out};
+    together = !(ctx->cfg.flags & ATS_FLAG_NO_GEMM_PAIR) && gemm_pair_eligible(probe);
+  }
+  if (together) {
     ATS_TRY(acquire_ops(ctx, ops, n));
     p.n_seg = n;
     uint64_t rows = 0;
@@ -481,7 +485,7 @@ static LayerWs layout_prefill(const ats_layer_desc& L, uint32_t T, uint8_t* base
   b.take(kWsReserved);
   const uint64_t H = L.hidden, qd = (uint64_t)L.n_q_heads * L.head_dim, kvd = (uint64_t)L.n_kv_heads * L.head_dim;
   uint64_t scratch = 0;
-  auto gemm_want = [&](int n, int k) { return std::max(gemm_scratch_bytes((int)T, n, k), gemm_ts_scratch_bytes((int)T, n, k)); };
+  auto gemm_want = [&](int n, int k) { return std::max(gemm_scratch_bytes((int)T, n, k), gemm_pair_scratch_bytes((int)T, n, k)); };
   if (L.wq >= 0) {
     w.h16 = (__half*)b.take(T * H * 2);
     w.qkv16 = (__half*)b.take(T * (qd + 2 * kvd) * 2);

@@ -1,304 +1,1094 @@
-// fp16-weight GEMM as a pair of CTAs on two SMs (tcgen05 cta_group::2): Y[T][N] = X[T][K] * W^T, W an unquantized fp16 matrix.
+// GEMM of prompts on pairs of CTAs (sm_100a, tcgen05 cta_group::2): Y[T][N] = X[T][K] W^T for the two 4-bit block formats and for
+// fp16 matrices; fp16 operands (4-bit: w = rn16(scale * code), one rounding), fp32 accumulation.
 //
-// A single CTA that computes 256 tokens x 256 features reads 96 bytes of operands per cycle from shared memory while
-// the tensor pipe is busy and refills 64 more: above the SM's 128.  As a pair, the instruction computes 256 tokens
-// (128 from each CTA's shared memory) x 256 features (128 weight rows from each CTA's shared memory), so every CTA
-// reads 64 bytes per cycle and refills 47.  Pair tile: 512 tokens (two 128-token blocks per CTA, one accumulator each,
-// all 512 tensor-memory columns of both SMs) x 256 features.
+// The weights are the A operand (M = 256 features, 128 per CTA), the tokens are the instruction's N (32..256, chosen from T).
+// 4-bit weights are expanded into tensor memory: a thread of the sixteen dequantization warps turns 32-weight blocks of one
+// feature (its lane) into sixteen columns each; nothing is stored to shared memory, no swizzle, no proxy fence.  (With the
+// weights as a shared-memory operand a 64-k step of 256 features took about 1700 cycles, whatever the number of tokens, for the
+// chain wait - store - fence - arrive that every warp went through in every step.)  fp16 weights go to shared memory by TMA.
 //
-// Roles in each CTA: warp 0 = TMA producer (activations of its 256 tokens and its 128 weight rows, boxes of 64 rows x 64 k,
-// 128-byte swizzle), warp 1 = tensor-memory allocation (both CTAs, cta_group::2) and, in the leader (even rank) only,
-// MMA issue; warps 2..9 = epilogue (tcgen05.ld of the CTA's own accumulators, fp16 stores).
-// Barriers: the loads of BOTH CTAs complete on the leader's full barrier (loads carry cta_group::2 and name that barrier:
-// the own barrier's address with the peer bit cleared), for which the leader posts the byte count of both; the leader's
-// tcgen05.commit releases a stage in both CTAs (one commit per CTA: its own barrier, then the peer's through mapa).
-// Every mbarrier wait is bounded; a CTA that gives up raises the status word and skips its work, but every thread still
-// reaches the closing cluster barrier, so that no CTA leaves while its partner may still signal it.
+// Unit of work: 128 k of a tile.  4-bit: codes and scales of a unit stream through a ring in shared memory by TMA (rows whose
+// scales are not 16-byte aligned: 4-byte asynchronous copies), activations through another (each CTA loads half of the
+// tokens), the expanded weights through `stages` slots of 64 tensor-memory columns.  fp16: one ring of 64-k steps, activations and
+// weights together.  The leader's MMA warp issues for both CTAs.  Eight epilogue warps move the accumulator through shared memory
+// to 16-byte stores (optionally + residual, or SwiGLU of 64 gate and 64 up features per CTA).  Two accumulators take turns where
+// tensor memory has room (fp16 weights; tiles of at most 128 tokens), so that the epilogue of one runs under the MMAs of the next.
+// The tensor core truncates what it adds to an accumulator, so long chains drift: where units_at_once says so, a stretch is
+// added up in parts, rounding, in words of the scratch that belong to the thread that reads them back.
+//
+// Work division: the (feature tile, token tile) tiles go to the pairs (one CTA per SM, persistent) in waves of neighbours, which
+// read the same weights and tokens from L2 at the same time (contiguous ranges of tiles per pair instead: 2048 tokens, fp16 gate
+// and up 447 us against 346, 4096 x 14336 254 against 196).  The units of the tiles that are left for the last wave form one line
+// of work that is cut into equal contiguous ranges.  A tile that falls into several of them is summed through fp32 partials in
+// the scratch: every contributor but the last to arrive leaves its part there; the last adds the parts in ascending k order (so
+// the result does not depend on who that is) and writes the tile.  Nobody waits for anybody.
+//
+// What bounds it: 4-bit, up to about 128 tokens, the expansion (about 900 cycles per unit and CTA: 3500 warp instructions at
+// close to one per cycle and scheduler); fp16 there the weights' way from memory; beyond that the MMAs and the power limit.
+// Back to back on new weights, before -> now (before: weights as a shared-memory operand, 256-token tiles, with reduction,
+// residual and SwiGLU launches):
+//   77 tokens MXFP4: 28672 x 4096 with SwiGLU 66 -> 41 us, 6144 x 4096 25 -> 21, 4096 x 14336 41 -> 34
+//   512 tokens Q4: gate and up 143 -> 103-107 us, 4096 x 14336 78 -> 71;  2048 tokens: gate and up 462 -> 360 (1335 TFLOP/s)
+//   2048 tokens fp16: q, k, v 152 -> 78 us, o 66 -> 59, gate and up 451 -> 346 (1390 TFLOP/s), 4096 x 14336 189 -> 196
+//
+// Roles per CTA: warp 0 = activation loads (fp16: and weights), warp 1 = tensor-memory allocation and (leader) MMA issue, warps 2, 3
+// = code and scale loads, warps 4..11 = epilogue, warps 12..27 = dequantization: four groups of four.  Every mbarrier wait is
+// bounded; on expiry the CTA raises the status word, skips the rest, and every thread still reaches the closing cluster barrier.
 #include <cuda.h>
 
 #include "ats_internal.h"
-#include "sm100_sync.cuh"
+#include "sm100_umma.cuh"
 
 namespace ats {
 
 namespace {
 
-constexpr int BM = 128, BK = 64, BOXR = 64;
-constexpr int kTokPerCta = 256, kFeatPerCta = 128;           // per CTA: two token blocks, half of the pair's 256 features
-constexpr int kXBytes = kTokPerCta * BK * 2;                 // 32 KB
-constexpr int kWBytes = kFeatPerCta * BK * 2;                // 16 KB
-constexpr int kStageBytes = kXBytes + kWBytes;               // 48 KB
-constexpr int kStages = 4;
-constexpr int kThreads = 10 * 32;
-constexpr uint32_t kPeerBitMask = 0xFEFFFFFFu;               // clears the CTA-rank bit of a shared::cluster address
+constexpr int kFeat = 128;                 // features per CTA
+constexpr int kUnitK = 128;                // k per unit of work: 64 bytes of codes per row
+constexpr int kMaxCodes = 12, kMaxX = 12;  // ring depths at most
+constexpr int kCodeBytes = kFeat * 64;     // 8 KB
+constexpr int kScaleBytes = kFeat * 16;    // per row: the eight scales of the 256-k line (or, unaligned, six halves)
+constexpr int kStagePitch = 272;           // bytes per token of the output staging: 128 halves + 16
+constexpr int kW16Bytes = kFeat * 128;     // fp16 weights of a 64-k step: 16 KB
+constexpr int kW16StageTok = 64;           // tokens staged at a time with fp16 weights (the ring has the rest of shared memory)
+enum { kFmtQ4 = 0, kFmtMx = 1, kFmtW16 = 2 };
+constexpr int kPairThreads = 28 * 32;
+constexpr int kMaxA = 4;                   // weight stages in tensor memory at most
+constexpr int kMaxParts = 4;               // contributors of a split tile at most
+constexpr uint32_t kColA = 256;            // tensor-memory columns: accumulator 0..255, weight stages from 256 on
+constexpr uint32_t kClearPeer = 0xFEFFFFFFu;
 
+struct PairSeg {
+  const uint8_t* base;
+  int n_rows;
+  int tile0;  // first feature tile of the segment
+  int col0;   // first output column of the segment
+};
 struct PairParams {
-  int K, T, N;
-  int ksteps;
+  PairSeg seg[3];
+  int n_seg;
+  int K, T;
+  int n_ft, n_tt;     // feature tiles, token tiles
+  int nt;             // tokens per tile
+  int units, ksteps;  // per tile: 128-k units, 64-k steps
+  int pairs;
+  int n_whole;        // tiles that a pair has to itself; the units of the others are divided over ...
+  int split_pairs;    // ... this many pairs
+  int stages, codes, xs;  // depths of the rings: weights in tensor memory, codes (a multiple of it), activations
+  int sc16;           // scale rows are 16-byte aligned
   __half* y;
   int ldy;
+  const __half* res;  // optional: y2 = rn16(res + y)
+  __half* y2;
+  __half* act;        // optional: SwiGLU of segments 0 (gate) and 1 (up); y may then be null
+  int ldact;
+  float* partial;     // slots of 2 * 128 features x slot_tok tokens
+  int slot_tok;
+  int slots2;         // a pair may leave a part of two tiles (ranges not cut at equal fractions of a tile)
+  float* own;         // a further slot per pair: sums of a stretch in several parts
+  int stage_tok;      // tokens that the staging holds: a multiple of 64, or all
+  int max_units;      // units that one accumulator adds up at most
+  int* counters;      // [2 * pairs], zero between launches
   int* status;
+  const int* grp_off;  // grouped form: row offsets per expert
+  int ft_per;          // ... feature tiles per expert
+  unsigned long long grp_stride;
 };
 
-__device__ __forceinline__ uint32_t cluster_rank() {
+__device__ __forceinline__ uint32_t cta_rank() {
   uint32_t r;
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
   return r;
 }
-__device__ __forceinline__ uint32_t map_to_cta(uint32_t saddr, uint32_t rank) {
-  uint32_t r;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(saddr), "r"(rank));
-  return r;
-}
-__device__ __forceinline__ void cluster_sync_all() {
+__device__ __forceinline__ void pair_sync() {
   asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
-// the load of one 64-row x 64-k box; its bytes complete on the pair leader's barrier
-__device__ __forceinline__ void tma_load_pair(void* dst, const CUtensorMap* map, int x, int y, uint64_t* own_bar) {
+// arrival on the leader's copy of a barrier (from either CTA)
+__device__ __forceinline__ void arrive_leader(uint64_t* own) {
+  uint32_t a;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(a) : "r"(smem_u32(own)));
+  asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(a) : "memory");
+}
+// Loads are issued like MMAs: by all lanes of a warp, in flow that is the same for the warp, with the instruction left to one.
+__device__ __forceinline__ void tma_pair_2d(uint32_t one, uint32_t dst, const CUtensorMap* map, int x, int y, uint64_t* own_bar) {
   asm volatile(
-      "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(
-          smem_u32(dst)),
-      "l"(map), "r"(x), "r"(y), "r"(smem_u32(own_bar) & kPeerBitMask)
+      "{\n.reg .pred q;\nsetp.ne.b32 q, %5, 0;\n@q cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes "
+      "[%0], [%1, {%2, %3}], [%4];\n}" ::"r"(dst),
+      "l"(map), "r"(x), "r"(y), "r"(smem_u32(own_bar) & kClearPeer), "r"(one)
       : "memory");
 }
-__device__ __forceinline__ uint64_t umma_desc(uint32_t saddr) {
-  uint64_t d = 0;
-  d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);
-  d |= (uint64_t)1 << 16;
-  d |= (uint64_t)(1024 >> 4) << 32;
-  d |= (uint64_t)1 << 46;
-  d |= (uint64_t)2 << 61;  // 128-byte swizzle
+__device__ __forceinline__ void tma_pair_3d(uint32_t one, uint32_t dst, const CUtensorMap* map, int x, int y, uint64_t* own_bar) {
+  asm volatile(
+      "{\n.reg .pred q;\nsetp.ne.b32 q, %6, 0;\n@q cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes "
+      "[%0], [%1, {%2, %3, %4}], [%5];\n}" ::"r"(dst),
+      "l"(map), "r"(x), "r"(y), "r"(0), "r"(smem_u32(own_bar) & kClearPeer), "r"(one)
+      : "memory");
+}
+__device__ __forceinline__ void tma_3d_one(uint32_t one, uint32_t dst, const CUtensorMap* map, int x, int y, int z, uint64_t* bar) {
+  asm volatile(
+      "{\n.reg .pred q;\nsetp.ne.b32 q, %6, 0;\n@q cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, "
+      "{%2, %3, %4}], [%5];\n}" ::"r"(dst),
+      "l"(map), "r"(x), "r"(y), "r"(z), "r"(smem_u32(bar)), "r"(one)
+      : "memory");
+}
+__device__ __forceinline__ void expect_tx_one(uint32_t one, uint64_t* bar, uint32_t bytes) {
+  asm volatile("{\n.reg .pred q;\nsetp.ne.b32 q, %2, 0;\n@q mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n}" ::"r"(smem_u32(bar)),
+               "r"(bytes), "r"(one)
+               : "memory");
+}
+// The value of any lane (all hold the same) as one the compiler knows to be the same for the warp.
+__device__ __forceinline__ int uniform(int v) { return (int)__reduce_max_sync(0xffffffffu, (unsigned)v); }
+__device__ __forceinline__ void umma_ts_pair(uint32_t one, uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
+  asm volatile(
+      "{\n.reg .pred p, q;\nsetp.ne.b32 p, %4, 0;\nsetp.ne.b32 q, %5, 0;\n@q tcgen05.mma.cta_group::2.kind::f16 [%0], [%1], %2, %3, p;\n}" ::"r"(
+          d_tmem),
+      "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(one)
+      : "memory");
+}
+__device__ __forceinline__ void umma_ss_pair(uint32_t one, uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
+  asm volatile(
+      "{\n.reg .pred p, q;\nsetp.ne.b32 p, %4, 0;\nsetp.ne.b32 q, %5, 0;\n@q tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(
+          d_tmem),
+      "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(one)
+      : "memory");
+}
+// arrives on the same barrier of both CTAs when the pair's MMAs issued so far are done
+__device__ __forceinline__ void umma_commit_both(uint32_t one, uint64_t* bar) {
+  asm volatile(
+      "{\n.reg .pred q;\n.reg .b16 m;\nmov.b16 m, 3;\nsetp.ne.b32 q, %1, 0;\n@q "
+      "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], m;\n}" ::"r"(smem_u32(bar)),
+      "r"(one)
+      : "memory");
+}
+__device__ __forceinline__ void cp_async4z(uint32_t dst, const void* src, bool live) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(live ? 4 : 0) : "memory");
+}
+__device__ __forceinline__ void cp_async_arrive(uint64_t* bar) {
+  asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+__device__ __forceinline__ __half2 as_h2(uint32_t v) {
+  __half2 h;
+  *reinterpret_cast<uint32_t*>(&h) = v;
+  return h;
+}
+__device__ __forceinline__ uint32_t as_u32(__half2 h) { return *reinterpret_cast<uint32_t*>(&h); }
+// (v & mask) | or_bits in one instruction (left to itself the compiler takes eight logic operations per word, not five)
+__device__ __forceinline__ uint32_t and_or(uint32_t v, uint32_t mask, uint32_t or_bits) {
+  uint32_t d;
+  asm("lop3.b32 %0, %1, %2, %3, 0xEA;" : "=r"(d) : "r"(v), "r"(mask), "r"(or_bits));
   return d;
 }
-// kind::f16, fp16 x fp16 -> fp32, both operands K-major, M = 256 over the pair, N = 256
-__device__ __forceinline__ uint32_t umma_idesc_pair() { return (1u << 4) | ((uint32_t)(256 >> 3) << 17) | ((uint32_t)(256 >> 4) << 24); }
-__device__ __forceinline__ void umma_f16_pair(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\ntcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(d_tmem),
-      "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
-      : "memory");
+// One code word (8 codes, internal nibble order) times the block scale -> 8 fp16 weights, k ascending.
+template <bool MX>
+__device__ __forceinline__ void expand_word(uint32_t w, __half2 s2, uint32_t* o) {
+  if (MX) {
+    const __half2 k2p14 = as_h2(0x74007400u);
+    const uint32_t kMag = 0x0E000E00u, kSgn = 0x80008000u;
+    o[0] = as_u32(__hmul2(__hmul2(as_h2(and_or(w << 9, kMag, (w << 12) & kSgn)), k2p14), s2));
+    o[1] = as_u32(__hmul2(__hmul2(as_h2(and_or(w << 5, kMag, (w << 8) & kSgn)), k2p14), s2));
+    o[2] = as_u32(__hmul2(__hmul2(as_h2(and_or(w << 1, kMag, (w << 4) & kSgn)), k2p14), s2));
+    o[3] = as_u32(__hmul2(__hmul2(as_h2(and_or(w >> 3, kMag, w & kSgn)), k2p14), s2));
+  } else {
+    const uint32_t kMagic = 0x64006400u, w8 = w >> 8;
+    const __half2 k1032 = as_h2(0x64086408u), k16th = as_h2(0x2C002C00u), kM72 = as_h2(0xD480D480u);
+    o[0] = as_u32(__hmul2(__hsub2(as_h2(and_or(w, 0x000F000Fu, kMagic)), k1032), s2));
+    o[1] = as_u32(__hmul2(__hfma2(as_h2(and_or(w, 0x00F000F0u, kMagic)), k16th, kM72), s2));
+    o[2] = as_u32(__hmul2(__hsub2(as_h2(and_or(w8, 0x000F000Fu, kMagic)), k1032), s2));
+    o[3] = as_u32(__hmul2(__hfma2(as_h2(and_or(w8, 0x00F000F0u, kMagic)), k16th, kM72), s2));
+  }
 }
-// arrives on the barrier at shared::cluster address `bar_addr` when the pair's MMAs issued so far are done
-__device__ __forceinline__ void umma_commit_pair(uint32_t bar_addr) {
-  asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar_addr) : "memory");
+// A warp waits with all its lanes; try_wait lets the hardware park it, so that the many waiting warps leave the issue slots
+// and the barrier unit to those that work (polling with test_wait cost 3 to 20 %).
+__device__ __forceinline__ bool wait_warp(uint64_t* bar, uint32_t parity) {
+  return __all_sync(0xffffffffu, mbar_wait_suspending(bar, parity));
 }
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&v)[32]) {
+// A test whose result is looked at later: its latency (about 200 cycles here) passes under other work.
+__device__ __forceinline__ bool peek(uint64_t* bar, uint32_t parity) { return mbar_test_wait(bar, parity); }
+
+__device__ __forceinline__ void tmem_ld_x16(uint32_t taddr, uint32_t* v) {
   asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, %17, "
-      "%18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
       : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]), "=r"(v[9]),
-        "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]), "=r"(v[16]), "=r"(v[17]), "=r"(v[18]),
-        "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]), "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]),
-        "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
+        "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
       : "r"(taddr)
       : "memory");
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void tmem_ld_wait_x16(uint32_t* v) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]), "+r"(v[6]), "+r"(v[7]), "+r"(v[8]), "+r"(v[9]),
+                 "+r"(v[10]), "+r"(v[11]), "+r"(v[12]), "+r"(v[13]), "+r"(v[14]), "+r"(v[15])::"memory");
+}
+template <int N>
+struct Int {
+  static constexpr int value = N;
+};
+struct PairMaps {
+  CUtensorMap codes[3], scales[3];  // of the segments (scales: where their rows are 16-byte aligned)
+};
+// One stretch of a pair's work: units u0 .. u1-1 of a tile.
+struct Stretch {
+  int tile, u0, u1;
+};
+// Walks a pair's stretches; the same sequence in every role of both CTAs.
+struct Walk {
+  int tile, step, n_whole;  // whole tiles: pair, pair + pairs, ... (neighbours in L2 run at the same time)
+  int units;
+  long long at, end;        // the pair's range of the last tiles' units, counted from tile n_whole on
+  __device__ __forceinline__ Walk(const PairParams& p, int pair) {
+    units = p.units;
+    tile = pair;
+    step = p.pairs;
+    n_whole = p.n_whole;
+    const long long n = (long long)(p.n_ft * p.n_tt - n_whole) * units;
+    at = pair < p.split_pairs ? n * pair / p.split_pairs : 0;
+    end = pair < p.split_pairs ? n * (pair + 1) / p.split_pairs : 0;
+  }
+  __device__ __forceinline__ bool next(Stretch& s) {
+    if (tile < n_whole) {
+      s.tile = tile;
+      s.u0 = 0;
+      s.u1 = units;
+      tile += step;
+      return true;
+    }
+    if (at >= end) return false;
+    const int t = (int)(at / units);
+    s.tile = n_whole + t;
+    s.u0 = (int)(at - (long long)t * units);
+    s.u1 = (int)min((long long)units, s.u0 + (end - at));
+    at += s.u1 - s.u0;
+    return true;
+  }
+};
+// Which rows, tokens and expert a tile stands for.
+struct Tile {
+  int sg, row0;        // segment, first feature row of the PAIR within it (SwiGLU: first feature of the 128)
+  int t0, T, rowoff;   // first token, tokens of the (expert's) matrix, its first row
+  int expert;
+  bool empty;
+};
+__device__ __forceinline__ Tile tile_of(const PairParams& p, int tile) {
+  Tile r;
+  int ft = tile / p.n_tt;
+  const int tt = tile - ft * p.n_tt;
+  r.expert = 0;
+  r.T = p.T;
+  r.rowoff = 0;
+  if (p.grp_off) {  // feature tiles of one expert after another
+    r.expert = ft / p.ft_per;
+    ft -= r.expert * p.ft_per;
+    r.rowoff = p.grp_off[r.expert];
+    r.T = p.grp_off[r.expert + 1] - r.rowoff;
+  }
+  r.t0 = tt * p.nt;
+  r.empty = r.t0 >= r.T;
+  r.sg = 0;
+  if (p.act) {
+    r.row0 = ft * kFeat;
+  } else {
+    while (r.sg + 1 < p.n_seg && ft >= p.seg[r.sg + 1].tile0) ++r.sg;
+    r.row0 = (ft - p.seg[r.sg].tile0) * 2 * kFeat;
+  }
+  return r;
 }
 
-__global__ void __launch_bounds__(kThreads, 1)
-    gemm_w16_pair_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUtensorMap wmap, const PairParams p) {
+// Units that go into an accumulator before it is handed over: a stretch in equal parts of p.max_units at most.
+__device__ __forceinline__ int seg_units(const PairParams& p, int n) { return (n + (n - 1) / p.max_units) / ((n + p.max_units - 1) / p.max_units); }
+
+template <int FMT>
+__global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ PairMaps wmap,
+                                                                const __grid_constant__ PairParams p) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  __shared__ uint64_t full[kStages], empty[kStages], acc_full;
-  __shared__ uint32_t tmem_base_s;
+  __shared__ uint64_t afull[kMaxA], aempty[kMaxA], xfull[kMaxX], xempty[kMaxX], cfull[kMaxCodes], cempty[kMaxCodes], acc_full[2], d_empty[2];
+  __shared__ uint32_t tmem_s;
+  __shared__ int last_s;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const uint32_t rank = cluster_rank();     // 0 = leader
-  const int pair = blockIdx.x >> 1;          // feature tile of the pair
-  const int n0 = pair * 256 + (int)rank * kFeatPerCta;             // first weight row this CTA loads
-  const int t0 = blockIdx.y * 512 + (int)rank * kTokPerCta;        // first token of this CTA
-  const int nks = p.ksteps;
+  const uint32_t rank = cta_rank();
+  const int pair = blockIdx.x >> 1;
+  const int S = p.stages, NC = p.codes, NX = p.xs;
+  const int xbytes = p.nt / 2 * 128;                 // this CTA's activation bytes of a 64-k step
+  uint8_t* x_s = smem;                               // [NX][2][nt / 2 rows][128 bytes], swizzled
+  const int step_bytes = xbytes + kW16Bytes;         // (fp16 weights: [NX] of a step's activations and weights, nothing else)
+  uint8_t* code_s = x_s + (size_t)NX * (FMT == kFmtW16 ? step_bytes : 2 * xbytes);   // [NC][128 rows][64 bytes], 16-byte pieces swizzled by row pair
+  uint8_t* scale_s = code_s + (size_t)NC * kCodeBytes;
+  uint8_t* out_s = scale_s + (size_t)NC * kScaleBytes;  // [nt][kStagePitch]
+  // two accumulators that take turns: of 128 columns beside the weights, of 256 where those are not in tensor memory
+  const bool two = FMT == kFmtW16 || p.nt <= 128;
+  constexpr uint32_t kAcc = FMT == kFmtW16 ? 256 : 128;
+  const int sc_pitch = p.sc16 ? 16 : 12;
+
   if (threadIdx.x == 0) {
-    for (int s = 0; s < kStages; ++s) {
-      mbar_init(&full[s], 1);   // the leader's own arrive.expect_tx; the bytes of both CTAs' loads complete on it
-      mbar_init(&empty[s], 1);  // one commit from the leader's MMA thread
+    for (int s = 0; s < S; ++s) {
+      mbar_init(&afull[s], 8);      // (leader) four dequantization warps of each CTA
+      mbar_init(&aempty[s], 1);
     }
-    mbar_init(&acc_full, 1);
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    for (int s = 0; s < NX; ++s) {
+      mbar_init(&xfull[s], 1);      // (leader) expect_tx
+      mbar_init(&xempty[s], 1);
+    }
+    for (int s = 0; s < 2; ++s) {
+      mbar_init(&acc_full[s], 1);
+      mbar_init(&d_empty[s], 16);   // (leader) eight epilogue warps of each CTA
+    }
+    mbar_fence_init();
   }
-  if (warp == 1) {  // one warp of each CTA, same shared-memory offset and column count in both
-    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_s)), "r"(512u) : "memory");
+  if (warp == 2 && lane == 0) {     // (the loaders' own barriers: they start before the CTAs have met)
+    for (int s = 0; s < NC; ++s) {
+      mbar_init(&cfull[s], p.sc16 ? 1 : 1 + 64);
+      mbar_init(&cempty[s], 4);     // the warps of the stage's group
+    }
+    mbar_fence_init();
+  }
+  // ---- code and scale loads (warp 2; warp 3 too where the scales' rows are not 16-byte aligned).  Weights depend on nothing:
+  // the first units are requested before the CTAs of the pair meet, the rest by the loaders' own branch below.
+  bool ok = true;
+  Stretch st;
+  Walk ld_walk(p, pair);
+  int ld_n = 0, ld_u = 0, ld_end = 0, ld_cs = 0;   // units requested; next and last unit of the current stretch; ring place
+  int ld_first = 0, ld_e = 0, ld_sa = 0, ld_sb = 0;
+  uint32_t ld_par = 1;
+  auto load_units = [&](int upto) {
+    const uint32_t one = elect_one();
+    const int half_k = p.K / 2, nblk = p.K / 32;
+    while (ld_n < upto) {
+      if (ld_u == ld_end) {
+        if (!uniform(ld_walk.next(st))) return;
+        const Tile tl = tile_of(p, st.tile);
+        if (uniform(tl.empty)) continue;
+        ld_u = uniform(st.u0);
+        ld_end = uniform(st.u1);
+        ld_e = uniform(tl.expert);
+        ld_sa = p.act ? 0 : uniform(tl.sg);
+        ld_sb = p.act ? 1 : ld_sa;
+        ld_first = uniform(p.act ? tl.row0 + (int)rank * 64 : tl.row0 + (int)rank * kFeat);
+      }
+      if (ld_n >= NC) {
+        ok = wait_warp(&cempty[ld_cs], ld_par);
+        if (!ok) return;
+      }
+      uint64_t* bar = &cfull[ld_cs];
+      const uint32_t sdst = smem_u32(scale_s) + (uint32_t)(ld_cs * kScaleBytes);
+      const int second = p.act ? ld_first : ld_first + 64;
+      if (warp == 2) {  // rows beyond the matrix and k beyond its end read as zeros
+        const uint32_t dst = smem_u32(code_s) + (uint32_t)(ld_cs * kCodeBytes);
+        expect_tx_one(one, bar, (uint32_t)(kCodeBytes + (p.sc16 ? kScaleBytes : 0)));
+        tma_3d_one(one, dst, &wmap.codes[ld_sa], ld_u * 64, ld_first, ld_e, bar);
+        tma_3d_one(one, dst + kCodeBytes / 2, &wmap.codes[ld_sb], ld_u * 64, second, ld_e, bar);
+        if (p.sc16) {  // (a line of eight scales serves two units: 16 bytes are the least that a copy takes)
+          tma_3d_one(one, sdst, &wmap.scales[ld_sa], (ld_u >> 1) * 8, ld_first, ld_e, bar);
+          tma_3d_one(one, sdst + kScaleBytes / 2, &wmap.scales[ld_sb], (ld_u >> 1) * 8, second, ld_e, bar);
+        }
+      }
+      if (!p.sc16) {
+        // six halves of each row from the 4-byte boundary at or below the unit's first scale; the reader skips the odd one.
+        // Words that begin beyond the matrix's scales are not read.
+        const int l = (warp - 2) * 32 + lane, rows = p.seg[ld_sa].n_rows;
+        const size_t hi = (size_t)rows * nblk * 2;
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+          const int gr = (j ? second : ld_first) + l;
+          const bool live = gr < rows;
+          const uint8_t* sc = p.seg[j ? ld_sb : ld_sa].base + (unsigned long long)ld_e * p.grp_stride + (size_t)rows * half_k;
+          const size_t lo = (((size_t)(live ? gr : 0) * nblk + ld_u * 4) * 2) & ~(size_t)3;
+#pragma unroll
+          for (int q = 0; q < 3; ++q) {
+            const bool in = live && lo + 4 * q < hi;
+            cp_async4z(sdst + (uint32_t)((l + 64 * j) * 12 + 4 * q), sc + (in ? lo + 4 * q : 0), in);
+          }
+        }
+        cp_async_arrive(bar);
+      }
+      ++ld_n;
+      ++ld_u;
+      if (++ld_cs == NC) ld_cs = 0, ld_par ^= 1u;
+    }
+  };
+  if (FMT != kFmtW16 && (warp == 2 || (warp == 3 && !p.sc16))) {
+    if (!p.sc16) asm volatile("bar.sync 2, 64;" ::: "memory");  // the barriers are initialised
+    __syncwarp();
+    if (p.grp_off) asm volatile("griddepcontrol.wait;" ::: "memory");
+    load_units(min(4, NC));
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_s)), "r"(512u) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
   }
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-  cluster_sync_all();  // both CTAs' barriers are initialised and their tensor memory allocated before anyone signals the other
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  const uint32_t tmem_base = tmem_base_s;
-  if (warp == 0) asm volatile("griddepcontrol.wait;" ::: "memory");  // the activations come from the preceding kernel
+  tc_fence_before();
+  pair_sync();
+  tc_fence_after();
+  const uint32_t tmem = tmem_s;
+  // The weights do not depend on the preceding kernel; the activations (and the grouped form's row offsets) do.  What the
+  // epilogue touches is ordered behind the activation loads.
+  if (warp == 0 || p.grp_off) asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
-  bool failed = false;
-  if (warp == 0) {
-    if (lane == 0) {
-      for (int i = 0; i < nks; ++i) {
-        const int s = i % kStages;
-        if (i >= kStages && !mbar_wait(&empty[s], ((i / kStages) - 1) & 1)) {
-          failed = true;
-          break;
+  // 72 registers a thread at launch; the epilogue's sums need more: 56 + 4 x 64 + 2 x 96 = 7 x 72
+  if (warp < 4) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
+    if (warp == 0) {
+      // ------------------------------------------------------------ activations
+      const uint32_t one = elect_one();
+      Walk mine(p, pair);
+      const uint32_t x0 = smem_u32(x_s);
+      int s = 0, n = 0;
+      uint32_t par = 1;
+      while (uniform(ok && mine.next(st))) {
+        const Tile tl = tile_of(p, st.tile);
+        const int u0 = uniform(st.u0), u1 = uniform(tl.empty ? 0 : st.u1);
+        const int row = uniform(tl.rowoff + tl.t0 + (int)rank * (p.nt / 2));
+        if constexpr (FMT == kFmtW16) {
+          const int sa = p.act ? 0 : uniform(tl.sg), sb = p.act ? 1 : sa;
+          const int wa = uniform(tl.row0 + (int)rank * (p.act ? 64 : kFeat)), wb = p.act ? wa : wa + 64;
+          const int k1 = min(2 * u1, p.ksteps);
+          for (int ks = 2 * u0; ks < k1; ++ks) {
+            if (n >= NX && !wait_warp(&xempty[s], par)) {
+              ok = false;
+              break;
+            }
+            ++n;
+            const uint32_t dst = x0 + (uint32_t)(s * step_bytes), dw = dst + (uint32_t)xbytes;
+            if (rank == 0) expect_tx_one(one, &xfull[s], (uint32_t)(2 * step_bytes));
+            tma_pair_2d(one, dst, &xmap, ks * 64, row, &xfull[s]);
+            tma_pair_3d(one, dw, &wmap.codes[sa], ks * 64, wa, &xfull[s]);
+            tma_pair_3d(one, dw + kW16Bytes / 2, &wmap.codes[sb], ks * 64, wb, &xfull[s]);
+            if (++s == NX) s = 0, par ^= 1u;
+          }
+          continue;
         }
-        uint8_t* st = smem + (size_t)s * kStageBytes;
-        if (rank == 0) mbar_expect_tx(&full[s], 2u * kStageBytes);
-        for (int b = 0; b < kTokPerCta / BOXR; ++b) tma_load_pair(st + kWBytes + (size_t)b * BOXR * BK * 2, &xmap, i * BK, t0 + b * BOXR, &full[s]);
-        for (int b = 0; b < kFeatPerCta / BOXR; ++b) tma_load_pair(st + (size_t)b * BOXR * BK * 2, &wmap, i * BK, n0 + b * BOXR, &full[s]);
+        for (int u = u0; u < u1; ++u) {
+          if (n >= NX && !wait_warp(&xempty[s], par)) {
+            ok = false;
+            break;
+          }
+          ++n;
+          const bool two = 2 * u + 1 < p.ksteps;
+          const uint32_t dst = x0 + (uint32_t)(s * 2 * xbytes);
+          if (rank == 0) expect_tx_one(one, &xfull[s], (uint32_t)((two ? 4 : 2) * xbytes));
+          tma_pair_2d(one, dst, &xmap, u * 128, row, &xfull[s]);
+          if (two) tma_pair_2d(one, dst + (uint32_t)xbytes, &xmap, u * 128 + 64, row, &xfull[s]);
+          if (++s == NX) s = 0, par ^= 1u;
+        }
       }
-    }
-  } else if (warp == 1) {
-    if (lane == 0 && rank == 0) {
-      const uint32_t idesc = umma_idesc_pair();
-      const uint64_t desc0 = umma_desc(smem_u32(smem));
-      uint32_t empty_peer[kStages];
+    } else if (warp == 1) {
+      // ------------------------------------------------------------ MMA issue (leader)
+      if (rank == 0) {
+        const uint32_t one = elect_one();
+        const uint32_t idesc = umma_idesc_f16(2 * kFeat, p.nt);
+        const uint64_t xd = umma_desc_sw128(smem_u32(x_s));
+        Walk mine(p, pair);
+        int s = 0, sx = 0, seg = 0;  // places in the rings, accumulator segments so far
+        uint32_t par = 0, parx = 0;
+        bool ready = false, readyx = false;
+        while (uniform(ok && mine.next(st))) {
+          const Tile tl = tile_of(p, st.tile);
+          const int u0 = uniform(st.u0), u1 = uniform(tl.empty ? 0 : st.u1);
+          int left = 0;  // units until the accumulator is handed over
+          uint32_t d = 0, accumulate = 0;
+          if (u1 == 0) continue;
+          const int part = seg_units(p, u1 - u0);
+          for (int u = u0; u < u1; ++u) {
+            if (left == 0) {
+              left = min(part, u1 - u);
+              accumulate = 0;
+              const int b = two ? seg & 1 : 0, use = two ? seg >> 1 : seg;
+              d = kAcc * b;
+              if (use > 0 && !wait_warp(&d_empty[b], (use - 1) & 1)) {
+                ok = false;
+                break;
+              }
+            }
+            if constexpr (FMT == kFmtW16) {
+              for (int ks = 2 * u; ok && ks < min(2 * u + 2, p.ksteps); ++ks) {
+                if (!__all_sync(0xffffffffu, readyx) && !wait_warp(&xfull[sx], parx)) {
+                  ok = false;
+                  break;
+                }
+                tc_fence_after();
+                const int sxn = sx + 1 == NX ? 0 : sx + 1;
+                const uint32_t parxn = sx + 1 == NX ? parx ^ 1u : parx;
+                readyx = peek(&xfull[sxn], parxn);
+                const uint64_t bd = xd + (uint64_t)((uint32_t)sx * (uint32_t)(step_bytes >> 4)), ad = bd + (uint64_t)(xbytes >> 4);
 #pragma unroll
-      for (int s = 0; s < kStages; ++s) empty_peer[s] = map_to_cta(smem_u32(&empty[s]), 1);
-      uint32_t accum = 0, par = 0;
-      int s = 0;
-      bool ok = true;
-      for (int i = 0; i < nks; ++i) {
-        if (!mbar_wait(&full[s], par)) {
+                for (int kk = 0; kk < 4; ++kk)
+                  umma_ss_pair(one, d, ad + (uint64_t)(2 * kk), bd + (uint64_t)(2 * kk), idesc, kk > 0 ? 1u : accumulate);
+                accumulate = 1;
+                umma_commit_both(one, &xempty[sx]);
+                sx = sxn, parx = parxn;
+              }
+              if (!ok) break;
+              if (--left == 0) {
+                umma_commit_both(one, &acc_full[seg & 1]);
+                ++seg;
+              }
+              continue;
+            }
+            if ((!__all_sync(0xffffffffu, ready) && !wait_warp(&afull[s], par)) ||
+                (!__all_sync(0xffffffffu, readyx) && !wait_warp(&xfull[sx], parx))) {
+              ok = false;
+              break;
+            }
+            tc_fence_after();
+            const int sn = s + 1 == S ? 0 : s + 1, sxn = sx + 1 == NX ? 0 : sx + 1;
+            const uint32_t parn = s + 1 == S ? par ^ 1u : par, parxn = sx + 1 == NX ? parx ^ 1u : parx;
+            ready = peek(&afull[sn], parn);
+            readyx = peek(&xfull[sxn], parxn);
+            const uint64_t bd = xd + (uint64_t)((uint32_t)sx * 2u * (uint32_t)(xbytes >> 4));
+            const uint32_t at = kColA + 64u * s;  // (all 512 columns are this CTA's: the allocation starts at 0)
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk) umma_ts_pair(one, d, at + 8u * kk, bd + (uint64_t)(2 * kk), idesc, kk > 0 ? 1u : accumulate);
+            if (2 * u + 1 < p.ksteps) {
+#pragma unroll
+              for (int kk = 0; kk < 4; ++kk)
+                umma_ts_pair(one, d, at + 32u + 8u * kk, bd + (uint64_t)((uint32_t)(xbytes >> 4) + 2 * kk), idesc, 1);
+            }
+            accumulate = 1;
+            umma_commit_both(one, &aempty[s]);
+            umma_commit_both(one, &xempty[sx]);
+            if (--left == 0) {
+              umma_commit_both(one, &acc_full[two ? seg & 1 : 0]);
+              ++seg;
+            }
+            s = sn, par = parn;
+            sx = sxn, parx = parxn;
+          }
+        }
+      }
+    } else {
+      // ------------------------------------------------------------ code and scale loaders, continued
+      if (FMT != kFmtW16 && (warp == 2 || !p.sc16)) load_units(0x7fffffff);
+      asm volatile("cp.async.wait_all;" ::: "memory");
+    }
+  } else if (warp >= 12) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 64;");
+    // ------------------------------------------------------------ dequantization: thread = (feature, one 32-k block of a step)
+    // Four groups of four warps, one for each weight stage, so that four of these chains of latencies (barrier, shared memory,
+    // arithmetic, tensor-memory store, barrier) run side by side.  A group takes every S-th unit; the code ring's depth is a
+    // multiple of S, so every barrier belongs to one group (a phase's parity says which one it is only to a waiter that has
+    // seen the one before).
+    const int quarter = warp & 3, grp = (warp - 12) >> 2;
+    const int row = quarter * 32 + lane;
+    const int nblk = p.K / 32;
+    const uint32_t a_col = tmem + ((uint32_t)(quarter * 32) << 16) + kColA + 64u * grp;
+    const uint8_t* code_row = code_s + row * 64;
+    const uint8_t* scale_row = scale_s + row * sc_pitch;
+    const uint32_t swz = (uint32_t)((row >> 1) & 3) << 4;
+    Walk mine(p, pair);
+    int skip = grp;               // units until this group's next
+    int cs = grp;                 // its place in the code ring
+    uint32_t cpar = 0, apar = 1;  // (the first wait for an empty stage passes at once)
+    while (FMT != kFmtW16 && ok && grp < S && mine.next(st)) {
+      const Tile tl = tile_of(p, st.tile);
+      if (tl.empty) continue;
+      const int first = p.act ? tl.row0 + (int)rank * 64 + (row & 63) : tl.row0 + (int)rank * kFeat + row;
+      const int odd = p.sc16 ? 0 : (int)(((long long)first * nblk) & 1);  // units start at even offsets: the row decides
+      int u = st.u0 + skip;
+      for (; u < st.u1; u += S) {
+        if (!wait_warp(&cfull[cs], cpar)) {
           ok = false;
           break;
         }
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint64_t wdesc = desc0 + (uint64_t)((uint32_t)s * (uint32_t)(kStageBytes >> 4));  // weight rows: the B operand (N)
-        const uint64_t xdesc = wdesc + (uint64_t)(kWBytes >> 4);                                // activation rows: the A operand (M)
-#pragma unroll
-        for (int kk = 0; kk < BK / 16; ++kk) {
-#pragma unroll
-          for (int mb = 0; mb < 2; ++mb)
-            umma_f16_pair(tmem_base + (uint32_t)(mb * 256), xdesc + (uint64_t)(mb * ((BM * BK * 2) >> 4) + 2 * kk), wdesc + (uint64_t)(2 * kk),
-                          idesc, kk > 0 ? 1u : accum);
+        const bool free_seen = peek(&aempty[grp], apar);
+        const uint8_t* cr = code_row + (uint32_t)(cs * kCodeBytes);
+        const uint8_t* sr = scale_row + (uint32_t)(cs * kScaleBytes);
+        uint2 sw;  // four scales
+        if (p.sc16) {
+          sw = *reinterpret_cast<const uint2*>(sr + (u & 1) * 8);
+        } else {
+          const uint32_t w0 = *reinterpret_cast<const uint32_t*>(sr), w1 = *reinterpret_cast<const uint32_t*>(sr + 4),
+                         w2 = *reinterpret_cast<const uint32_t*>(sr + 8);
+          sw = odd ? make_uint2(__byte_perm(w0, w1, 0x5432), __byte_perm(w1, w2, 0x5432)) : make_uint2(w0, w1);
+          const int left = nblk - u * 4;  // blocks that exist; what follows belongs to the next row
+          if (left < 4) sw.y &= left < 3 ? 0u : 0x0000FFFFu;
+          if (left < 2) sw.x &= 0x0000FFFFu;
         }
-        accum = 1;
-        umma_commit_pair(smem_u32(&empty[s]));  // this CTA's producer may refill the stage ...
-        umma_commit_pair(empty_peer[s]);        // ... and so may the partner's
-        if (++s == kStages) {
-          s = 0;
-          par ^= 1;
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+          uint32_t o[32];
+          const uint32_t pairs = c ? sw.y : sw.x;
+#pragma unroll
+          for (int b = 0; b < 2; ++b) {
+            const uint4 q = *reinterpret_cast<const uint4*>(cr + (((uint32_t)(2 * c + b) << 4) ^ swz));
+            const __half2 sc = as_h2(__byte_perm(pairs, 0, b ? 0x3232 : 0x1010));
+            expand_word<FMT == kFmtMx>(q.x, sc, o + 16 * b);
+            expand_word<FMT == kFmtMx>(q.y, sc, o + 16 * b + 4);
+            expand_word<FMT == kFmtMx>(q.z, sc, o + 16 * b + 8);
+            expand_word<FMT == kFmtMx>(q.w, sc, o + 16 * b + 12);
+          }
+          if (c == 0) {
+            if (!__all_sync(0xffffffffu, free_seen) && !wait_warp(&aempty[grp], apar)) {
+              ok = false;
+              break;
+            }
+            tc_fence_after();
+          }
+          tmem_st_x32(a_col + 32u * c, o);
         }
+        if (!ok) break;
+        tmem_st_wait();
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) {
+          arrive_leader(&afull[grp]);
+          mbar_arrive(&cempty[cs]);
+        }
+        apar ^= 1u;
+        cs += S;
+        if (cs >= NC) cs -= NC, cpar ^= 1u;
       }
-      if (ok) {
-        umma_commit_pair(smem_u32(&acc_full));
-        umma_commit_pair(map_to_cta(smem_u32(&acc_full), 1));
-      } else {
-        failed = true;
-      }
+      skip = u - st.u1;
     }
   } else {
-    // ------------------------------------------------------------ epilogue: this CTA's 256 tokens x 256 features
-    const int w2 = warp - 2;           // 0..7
-    const int q = warp & 3;            // tensor-memory lane quarter this warp may read
-    const int half = w2 >> 2;          // which half of the 256 feature columns
-    int ready = 0;
-    if (nks > 0) {
-      if (lane == 0) ready = mbar_wait(&acc_full, 0) ? 1 : 0;
-      ready = __shfl_sync(0xffffffffu, ready, 0);
-    }
-    if (ready) {
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const int nbase = pair * 256;
+    // ------------------------------------------------------------ epilogue
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 96;");
+    const int quarter = warp & 3;
+    const int half = (warp - 4) >> 2;        // two warps per quarter: even and odd runs of 32 tokens
+    const int tid = threadIdx.x - 128;       // 0..255
+    const int feat = quarter * 32 + lane;    // this thread's feature of the CTA's 128
+    const uint32_t d_col = tmem + ((uint32_t)(quarter * 32) << 16);
+    auto epi_sync = [] { asm volatile("bar.sync 1, 256;" ::: "memory"); };
+    auto epi_all = [](bool v) {
+      uint32_t r;
+      asm volatile("{\n.reg .pred a, b;\nsetp.ne.u32 a, %1, 0;\nbarrier.cta.red.and.pred b, 1, 256, a;\nselp.u32 %0, 1, 0, b;\n}"
+                   : "=r"(r)
+                   : "r"((uint32_t)v)
+                   : "memory");
+      return r != 0;
+    };
+    Walk mine(p, pair);
+    int seg = 0;
+    while (ok && mine.next(st)) {
+      const Tile tl = tile_of(p, st.tile);
+      if (tl.empty) continue;
+      const int ntok = min(p.nt, tl.T - tl.t0);
+      // ---- all parts but the last of the stretch: added up in this thread's own words of the scratch
+      const int n = st.u1 - st.u0, part = seg_units(p, n), n_part = (n + part - 1) / part;
+      uint32_t col = 0;
+      float* own = p.own + (size_t)blockIdx.x * kFeat * p.slot_tok + feat;
+      auto add_own = [&](float* v, int c0, auto n_tok) {  // (all loads before the first addition)
+        constexpr int NT = decltype(n_tok)::value;
+        float w[NT];
+#pragma unroll
+        for (int i = 0; i < NT; ++i) w[i] = c0 + i < ntok ? __ldcg(own + (size_t)(c0 + i) * kFeat) : 0.f;
+#pragma unroll
+        for (int i = 0; i < NT; ++i) v[i] += w[i];
+      };
+      for (int g = 0; g < n_part; ++g, ++seg) {
+        const int b = two ? seg & 1 : 0, use = two ? seg >> 1 : seg;
+        const bool got = wait_warp(&acc_full[b], use & 1);
+        ok = g + 1 == n_part || !got ? epi_all(got) : got;  // (the eight warps give up together: they share barriers)
+        if (!ok) break;
+        tc_fence_after();
+        col = d_col + kAcc * b;
+        if (g + 1 == n_part) break;
 #pragma unroll 1
-      for (int mb = 0; mb < 2; ++mb) {
-        const int t = t0 + mb * BM + q * 32 + lane;
+        for (int c0 = 32 * half; c0 < ntok; c0 += 64) {
+          float v[32];
+          tmem_ld_x32(col + c0, reinterpret_cast<uint32_t*>(v));
+          tmem_ld_wait_x32(reinterpret_cast<uint32_t*>(v));
+          if (g) add_own(v, c0, Int<32>{});
+#pragma unroll
+          for (int i = 0; i < 32; ++i)
+            if (c0 + i < ntok) __stcg(own + (size_t)(c0 + i) * kFeat, v[i]);
+        }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) arrive_leader(&d_empty[b]);
+      }
+      if (!ok) break;
+      const int last_b = two ? seg & 1 : 0;
+      ++seg;
+      const bool split = st.u0 > 0 || st.u1 < p.units;
+      bool write = true;
+      // contributors of a split tile: the pairs whose ranges meet it.  Pair q holds units n q / P .. n (q + 1) / P - 1, so
+      // unit u lies with q = ((u + 1) P - 1) / n.
+      int first = pair, n_con = 1;
+      auto part_of = [&](int q) {  // this CTA's half of what pair q leaves of the tile
+        // (the first contributor begins the tile, the others come upon it at the start of their range)
+        return p.partial + ((size_t)(p.slots2 && q == first ? p.split_pairs + q : q) * 2 + rank) * kFeat * p.slot_tok;
+      };
+      if (split) {
+        const long long n_units = (long long)(p.n_ft * p.n_tt - p.n_whole) * p.units, lo = (long long)(st.tile - p.n_whole) * p.units;
+        first = (int)(((lo + 1) * p.split_pairs - 1) / n_units);
+        n_con = (int)(((lo + p.units) * p.split_pairs - 1) / n_units) - first + 1;
+        int* cnt = p.counters + 2 * first + rank;
+        if (tid == 0) {
+          int v;
+          asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(cnt) : "memory");
+          last_s = v == n_con - 1;
+        }
+        epi_sync();
+        write = last_s != 0;
+        if (!write) {
+          float* dst = part_of(pair) + feat;
 #pragma unroll 1
-        for (int c0 = half * 128; c0 < half * 128 + 128; c0 += 32) {
-          uint32_t v[32];
-          tmem_ld32(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(mb * 256 + c0), v);
-          if (t < p.T) {
-            __half* dst = p.y + (size_t)t * p.ldy + nbase + c0;
-            if (nbase + c0 + 32 <= p.N && (p.ldy % 8 == 0) && ((reinterpret_cast<uintptr_t>(p.y) & 15) == 0)) {
+          for (int c0 = 32 * half; c0 < ntok; c0 += 64) {
+            float v[32];
+            tmem_ld_x32(col + c0, reinterpret_cast<uint32_t*>(v));
+            tmem_ld_wait_x32(reinterpret_cast<uint32_t*>(v));
+            if (n_part > 1) add_own(v, c0, Int<32>{});
 #pragma unroll
-              for (int e = 0; e < 32; e += 8) {
-                uint32_t o[4];
+            for (int i = 0; i < 32; ++i)
+              if (c0 + i < ntok) __stcg(dst + (size_t)(c0 + i) * kFeat, v[i]);
+          }
+          epi_sync();  // every part is written (and last_s read) before the arrival that releases them
+          if (tid == 0) {
+            int prev;
+            asm volatile("atom.add.acq_rel.gpu.global.s32 %0, [%1], 1;" : "=r"(prev) : "l"(cnt) : "memory");
+            last_s = prev == n_con - 1;
+          }
+          epi_sync();
+          write = last_s != 0;  // all the others arrived in the meantime
+        }
+        epi_sync();
+        if (write && tid == 0) *cnt = 0;  // ready for the next launch
+      }
+      const int me = pair - first;
+      // the other contributors' parts (NO of them at most) come in batches of NT tokens and are added in the order of the pairs
+      auto add_parts = [&](auto tokens, auto others, int c0, float (&v)[16]) {
+        constexpr int NT = decltype(tokens)::value, NO = decltype(others)::value;
 #pragma unroll
-                for (int h = 0; h < 4; ++h) {
-                  const __half2 hh = __floats2half2_rn(__uint_as_float(v[e + 2 * h]), __uint_as_float(v[e + 2 * h + 1]));
-                  o[h] = *reinterpret_cast<const uint32_t*>(&hh);
-                }
-                *reinterpret_cast<uint4*>(dst + e) = make_uint4(o[0], o[1], o[2], o[3]);
-              }
-            } else {
+        for (int h = 0; h < 16; h += NT) {
+          float w[NO][NT];
 #pragma unroll
-              for (int e = 0; e < 32; ++e)
-                if (nbase + c0 + e < p.N) dst[e] = __float2half_rn(__uint_as_float(v[e]));
+          for (int c = 0; c < NO; ++c) {
+            const float* src = part_of(first + (c + 1 < n_con ? c + (c >= me) : 0)) + (size_t)(c0 + h) * kFeat + feat;
+#pragma unroll
+            for (int i = 0; i < NT; ++i) w[c][i] = c + 1 < n_con && c0 + h + i < ntok ? __ldcg(src + i * kFeat) : 0.f;
+          }
+#pragma unroll
+          for (int i = 0; i < NT; ++i) {
+            float acc = 0.f;
+#pragma unroll
+            for (int c = 0; c <= NO; ++c) {
+              if (c == me) acc += v[h + i];
+              if (c < NO) acc += w[c][i];
+            }
+            v[h + i] = acc;
+          }
+        }
+      };
+      for (int h0 = 0; h0 < ntok; h0 += p.stage_tok) {  // as many tokens at a time as the staging holds
+      const int h1 = min(h0 + p.stage_tok, ntok);
+      auto stage16 = [&](const float* v, int c0) {
+        __half* o = reinterpret_cast<__half*>(out_s + (size_t)(c0 - h0) * kStagePitch) + feat;
+#pragma unroll
+        for (int i = 0; i < 16; ++i) o[i * (kStagePitch / 2)] = __float2half_rn(v[i]);
+      };
+      if (write) {
+#pragma unroll 1
+        for (int c0 = h0 + 32 * half; c0 < h1; c0 += 64) {
+          if (!split) {
+            float v[32];
+            tmem_ld_x32(col + c0, reinterpret_cast<uint32_t*>(v));
+            tmem_ld_wait_x32(reinterpret_cast<uint32_t*>(v));
+            if (n_part > 1) add_own(v, c0, Int<32>{});
+            stage16(v, c0);
+            stage16(v + 16, c0 + 16);
+          } else {
+#pragma unroll 1
+            for (int h = c0; h < min(c0 + 32, h1); h += 16) {
+              float v[16];
+              tmem_ld_x16(col + h, reinterpret_cast<uint32_t*>(v));
+              tmem_ld_wait_x16(reinterpret_cast<uint32_t*>(v));
+              if (n_part > 1) add_own(v, h, Int<16>{});
+              if (n_con == 2) add_parts(Int<16>{}, Int<1>{}, h, v);
+              else add_parts(Int<8>{}, Int<kMaxParts - 1>{}, h, v);
+              stage16(v, h);
             }
           }
         }
       }
-    } else if (nks > 0) {
-      failed = true;
+      if (h1 == ntok) {
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) arrive_leader(&d_empty[last_b]);  // the accumulator may be overwritten
+      }
+      if (!write) continue;
+      epi_sync();
+      const size_t trow = (size_t)tl.rowoff + tl.t0;
+      if (p.act) {
+        const int F = p.seg[0].n_rows, f0 = tl.row0 + (int)rank * 64;
+        const int c = (tid & 7) * 8;
+        const int live = F - f0 - c;  // F is a multiple of 8: a run of eight is live or not
+        if (live > 0) {
+#pragma unroll 2
+          for (int t = h0 + (tid >> 3); t < h1; t += 32) {
+            const uint4 g4 = *reinterpret_cast<const uint4*>(out_s + (size_t)(t - h0) * kStagePitch + c * 2);
+            const uint4 u4 = *reinterpret_cast<const uint4*>(out_s + (size_t)(t - h0) * kStagePitch + 128 + c * 2);
+            const uint32_t gw[4] = {g4.x, g4.y, g4.z, g4.w}, uw[4] = {u4.x, u4.y, u4.z, u4.w};
+            uint32_t a[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+              const float2 g = __half22float2(as_h2(gw[q])), u = __half22float2(as_h2(uw[q]));
+              a[q] = as_u32(__floats2half2_rn(silu_times(g.x, u.x), silu_times(g.y, u.y)));
+            }
+            *reinterpret_cast<uint4*>(p.act + (trow + t) * p.ldact + f0 + c) = make_uint4(a[0], a[1], a[2], a[3]);
+            if (p.y) {
+              *reinterpret_cast<uint4*>(p.y + (trow + t) * p.ldy + f0 + c) = g4;
+              *reinterpret_cast<uint4*>(p.y + (trow + t) * p.ldy + F + f0 + c) = u4;
+            }
+          }
+        }
+      } else {
+        const int r0 = tl.row0 + (int)rank * kFeat;
+        const int live = min(kFeat, p.seg[tl.sg].n_rows - r0);
+        const int colbase = p.seg[tl.sg].col0 + r0;
+        const bool vec = (p.ldy % 8 == 0) && (colbase % 8 == 0) &&
+                         (((reinterpret_cast<uintptr_t>(p.y) | reinterpret_cast<uintptr_t>(p.res) | reinterpret_cast<uintptr_t>(p.y2)) & 15) == 0);
+        const int c = (tid & 15) * 8;
+        if (vec && c + 8 <= live) {
+          for (int tb = h0 + (tid >> 4); tb < h1; tb += 64) {
+            // four tokens at a time, their residuals requested before anything is stored
+            uint4 r4[4];
+            if (p.res) {
+#pragma unroll
+              for (int q = 0; q < 4; ++q)
+                if (tb + 16 * q < h1) r4[q] = __ldg(reinterpret_cast<const uint4*>(p.res + (trow + tb + 16 * q) * p.ldy + colbase + c));
+            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+              const int t = tb + 16 * q;
+              if (t >= h1) break;
+              const uint4 o4 = *reinterpret_cast<const uint4*>(out_s + (size_t)(t - h0) * kStagePitch + c * 2);
+              const size_t off = (trow + t) * p.ldy + colbase + c;
+              *reinterpret_cast<uint4*>(p.y + off) = o4;
+              if (p.res) {
+                const uint32_t ow[4] = {o4.x, o4.y, o4.z, o4.w}, rw[4] = {r4[q].x, r4[q].y, r4[q].z, r4[q].w};
+                uint32_t z[4];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                  const float2 a = __half22float2(as_h2(ow[e])), b = __half22float2(as_h2(rw[e]));
+                  z[e] = as_u32(__floats2half2_rn(b.x + a.x, b.y + a.y));
+                }
+                *reinterpret_cast<uint4*>(p.y2 + off) = make_uint4(z[0], z[1], z[2], z[3]);
+              }
+            }
+          }
+        } else if (c < live) {
+          for (int t = h0 + (tid >> 4); t < h1; t += 16) {
+            const __half* o = reinterpret_cast<const __half*>(out_s + (size_t)(t - h0) * kStagePitch) + c;
+            const size_t off = (trow + t) * p.ldy + colbase + c;
+            for (int q = 0; q < min(8, live - c); ++q) {
+              p.y[off + q] = o[q];
+              if (p.res) p.y2[off + q] = __float2half_rn(__half2float(p.res[off + q]) + __half2float(o[q]));
+            }
+          }
+        }
+      }
+      epi_sync();  // the staging may be filled again
+      }
     }
   }
-  if (failed && p.status) raise_status(p.status, 2);
-  // nobody leaves, frees tensor memory or lets its shared memory go while the partner may still read or signal it
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-  cluster_sync_all();
-  if (warp == 1) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512u) : "memory");
+  __syncwarp();
+  if (!ok && lane == 0) raise_status(p.status, 3);
+  __syncwarp();
+  // nobody leaves or frees tensor memory while the partner may still read or signal it
+  tc_fence_before();
+  pair_sync();
+  if (warp == 1) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u) : "memory");
 }
 
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
-                                  const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
-                                  CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-EncodeTiledFn encode_fn() {
-  static EncodeTiledFn fn = nullptr;
-  if (!fn) {
-    void* ptr = nullptr;
-    cudaDriverEntryPointQueryResult qres;
-    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &ptr, cudaEnableDefault, &qres) == cudaSuccess && qres == cudaDriverEntryPointSuccess)
-      fn = reinterpret_cast<EncodeTiledFn>(ptr);
+// ------------------------------------------------------------------------------------------------- host side
+// Units that one accumulator adds up at most.  The tensor core truncates each sum, and what a chain drops grows with its
+// length: of the fp16 results 0.5 % differ from the exact sum's rounding after 1024 k, 1.7 % after 4096, 2.7 % after 7168.  A
+// prompt of 512 through a layer of 4096 features has 5.1e-4 of its outputs more than 2e-3 off with q, k, v in chains of 2048 k at
+// most (the softmax multiplies their errors), 9.8e-4 with 4096.  Wide matrices (gate and up) make no difference up to 4096, where a part
+// costs the most: 104 us against 118 in parts of 2048.  From 1024 tokens on a chain is the stretch.
+int units_at_once(int n_ft, int T, int K) { return T >= 1024 ? (K + kUnitK - 1) / kUnitK : (n_ft > 32 ? 4096 : 1536) / kUnitK; }
+
+struct PairPlan {
+  int nt, n_tt, pairs, n_whole, split_pairs, slots2, own;
+  uint64_t scratch;
+};
+// Cost in SM cycles of the ways to divide the work (see the kernel's comment).  A unit costs its MMAs, the expansion of its weights
+// or their way from memory, whichever is longest; a tile its epilogue; a split tile the parts' way through L2; a stretch that is
+// added up in several parts theirs, unless the MMAs go on meanwhile in the other accumulator.
+PairPlan pair_plan(const int* ft_of_seg, int n_seg, int T, int K, bool w16, int max_pairs, uint64_t scratch_bytes) {
+  PairPlan best{};
+  double best_cost = 1e300;
+  int n_ft = 0;
+  for (int i = 0; i < n_seg; ++i) n_ft += ft_of_seg[i];
+  const int units = (K + kUnitK - 1) / kUnitK, max_units = units_at_once(n_ft, T, K);
+  int last = 0;
+  for (int most : {256, 192, 128}) {
+    const int n_tt = (T + most - 1) / most;
+    if (n_tt == last) continue;
+    last = n_tt;
+    const int nt = ((T + n_tt - 1) / n_tt + 31) / 32 * 32;
+    const uint64_t slot = 2ull * kFeat * std::min(nt, T) * 4;
+    const double unit = std::max(w16 ? 1400.0 : 825.0 + 1.25 * nt, 6.65 * nt), tile = w16 ? 500.0 : 12.0 * nt;
+    const double flush = w16 || nt <= 128 ? 1500.0 : 100.0 * (nt - 110);
+    auto stretch = [&](double len) { return len * unit + (std::ceil(len / max_units) - 1) * flush; };
+    // whole tiles in waves of one per pair; the rest, `rem`, whole in a wave of its own or divided over n pairs, `len` units each
+    const int tiles = n_ft * n_tt, waves = tiles / max_pairs, rem = tiles % max_pairs;
+    auto take = [&](double cost, double len, int n, int slots) {
+      const bool parts = std::max(len, waves || !slots ? (double)units : 0.0) > max_units;
+      const int pairs = waves ? max_pairs : slots ? n : rem;
+      const uint64_t need = ((uint64_t)n * slots + (parts ? pairs : 0)) * slot;
+      if (need > scratch_bytes && (slots || nt > 128)) return;  // (whole tiles of one token tile do without, in one part)
+      cost += waves * (stretch(units) + tile);
+      if (cost >= best_cost) return;
+      best_cost = cost;
+      best = PairPlan{nt, n_tt, pairs, slots ? tiles - rem : tiles, n, slots == 2, parts && need <= scratch_bytes, need > scratch_bytes ? 0 : need};
+    };
+    take(rem ? stretch(units) + tile : 0.0, units, 0, 0);
+    auto red = [&](double con) { return 5000.0 + (con - 1) * nt * 32.0; };
+    for (int s = 2; s <= kMaxParts && s <= units && rem && rem * s <= max_pairs; ++s)
+      if (units % s == 0 || units > 4 * s) take(stretch((units + s - 1) / s) + red(s), (units + s - 1) / s, rem * s, 1);
+    const double per = (double)rem * units / max_pairs;
+    if (per >= 1 && units <= per * (kMaxParts - 2))  // (a tile meets at most units / per + 2 ranges)
+      take(stretch(std::ceil(per)) + tile + 4000.0 + red(std::ceil(units / per) + 1), std::ceil(per), max_pairs, 2);
   }
-  return fn;
+  return best;
 }
+
+int pairs_of_device(int sm_count) { return std::min(sm_count / 2, kAttnMaxCounters / 2); }
 
 }  // namespace
 
-// Shapes the pair kernel takes: one fp16 matrix, no residual, operands aligned for TMA, and enough tiles to occupy three
-// quarters of the SMs (it has no split-K: with fewer tiles the single-CTA kernel, which splits K, is faster; measured
-// cross-over: 112 CTAs even, 128 and more 8 to 17 % faster, 64 and fewer slower).
-bool gemm_pair_eligible(const GemmParams& g) {
-  if (!g.w16 || g.grp_off || g.n_seg != 1 || g.T < 384 || g.ldx % 8 || g.K < BK || (reinterpret_cast<uintptr_t>(g.x) & 15)) return false;
-  if (g.res || g.y2 || g.K % 8 || (reinterpret_cast<uintptr_t>(g.seg[0].base) & 15)) return false;
-  return 2L * ((g.seg[0].n_rows + 255) / 256) * ((g.T + 511) / 512) >= 112;
+uint64_t gemm_pair_scratch_bytes(int T, int n_total, int K) {
+  const int ft = (n_total + 2 * kFeat - 1) / (2 * kFeat);
+  return std::max(pair_plan(&ft, 1, T, K, false, 74, ~0ull).scratch, pair_plan(&ft, 1, T, K, true, 74, ~0ull).scratch) + 256;
 }
 
-cudaError_t launch_gemm_pair(const GemmParams& g, cudaStream_t st, uint64_t* n_launch, std::string* err) {
-  if (!gemm_pair_eligible(g)) return cudaErrorInvalidValue;
-  EncodeTiledFn enc = encode_fn();
+bool gemm_pair_eligible(const GemmParams& g) {
+  if ((g.w16 && g.grp_off) || g.n_seg < 1 || g.n_seg > 3 || !g.counters || g.K % (g.w16 ? 8 : 32) || g.ldx % 8) return false;
+  if (reinterpret_cast<uintptr_t>(g.x) & 15) return false;
+  if ((g.res != nullptr) != (g.y2 != nullptr)) return false;
+  for (int i = 0; i < g.n_seg; ++i) {
+    if (reinterpret_cast<uintptr_t>(g.seg[i].base) & 15) return false;
+    if (g.grp_tab[i]) return false;
+  }
+  if (g.act && (g.n_seg != 2 || g.seg[0].n_rows != g.seg[1].n_rows || g.seg[0].n_rows % 8 || g.ldact % 8 || g.ldy % 8 || g.res ||
+                ((reinterpret_cast<uintptr_t>(g.act) | reinterpret_cast<uintptr_t>(g.y)) & 15)))
+    return false;
+  if (g.grp_off && ((g.n_seg != 1 && !g.act) || g.grp_stride % 16 || g.res)) return false;
+  return true;
+}
+
+cudaError_t launch_gemm_pair(const GemmParams& g, int sm_count, cudaStream_t st, uint64_t* n_launch, std::string* err) {
+  TensorMapEncodeFn enc = tensor_map_encode();
   if (!enc) {
     if (err) *err = "cuTensorMapEncodeTiled is not available from the driver";
     return cudaErrorNotSupported;
   }
-  CUtensorMap xmap, wmap;
-  const cuuint32_t box[2] = {BK, BOXR}, estr[2] = {1, 1};
-  const cuuint64_t xdims[2] = {(cuuint64_t)g.K, (cuuint64_t)g.T}, xstr[1] = {(cuuint64_t)g.ldx * 2};
-  if (enc(&xmap, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, const_cast<__half*>(g.x), xdims, xstr, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+  PairParams p{};
+  p.n_seg = g.n_seg;
+  int ft_of_seg[3] = {0, 0, 0}, n_ft = 0, col = 0;
+  for (int i = 0; i < g.n_seg; ++i) {
+    const int ft = g.act ? (i ? 0 : (g.seg[0].n_rows + kFeat - 1) / kFeat) : (g.seg[i].n_rows + 2 * kFeat - 1) / (2 * kFeat);
+    p.seg[i] = PairSeg{g.seg[i].base, g.seg[i].n_rows, n_ft, col};
+    ft_of_seg[i] = ft;
+    n_ft += ft;
+    col += g.seg[i].n_rows;
+  }
+  p.K = g.K;
+  p.T = g.T;
+  p.units = (g.K + kUnitK - 1) / kUnitK;
+  p.ksteps = (g.K + 63) / 64;
+  const int max_pairs = pairs_of_device(sm_count);
+  bool own = false;
+  if (g.grp_off) {
+    if (g.n_groups <= 0 || g.grp_max_rows <= 0) return cudaErrorInvalidValue;
+    p.n_tt = (g.grp_max_rows + 255) / 256;
+    p.nt = ((g.grp_max_rows + p.n_tt - 1) / p.n_tt + 31) / 32 * 32;
+    p.ft_per = n_ft;
+    p.n_ft = n_ft * g.n_groups;
+    p.pairs = (int)std::min<long long>((long long)p.n_ft * p.n_tt, max_pairs);
+    p.n_whole = p.n_ft * p.n_tt;
+  } else {
+    const PairPlan pl = pair_plan(ft_of_seg, g.n_seg, g.T, g.K, g.w16, max_pairs, g.scratch ? g.scratch_bytes : 0);
+    p.nt = pl.nt;
+    p.n_tt = pl.n_tt;
+    p.n_ft = n_ft;
+    p.pairs = pl.pairs;
+    p.n_whole = pl.n_whole;
+    p.split_pairs = pl.split_pairs;
+    p.slots2 = pl.slots2;
+    own = pl.own;
+  }
+  p.sc16 = !g.w16 && g.K % 256 == 0;
+  p.y = g.y;
+  p.ldy = g.ldy;
+  p.res = g.res;
+  p.y2 = g.y2;
+  p.act = g.act;
+  p.ldact = g.ldact;
+  p.partial = (float*)g.scratch;
+  p.slot_tok = std::min(p.nt, g.T);
+  p.own = p.partial + (size_t)(p.split_pairs * (p.slots2 ? 2 : 1)) * 2 * kFeat * p.slot_tok;
+  p.max_units = own ? units_at_once(n_ft, g.T, g.K) : p.units;
+  p.counters = g.counters;
+  p.status = g.status;
+  p.grp_off = g.grp_off;
+  p.grp_stride = g.grp_stride;
+  CUtensorMap xmap;
+  const cuuint64_t dims[2] = {(cuuint64_t)g.K, (cuuint64_t)g.T}, strides[1] = {(cuuint64_t)g.ldx * 2};
+  const cuuint32_t box[2] = {64, (cuuint32_t)(p.nt / 2)}, es[2] = {1, 1};
+  if (enc(&xmap, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, const_cast<__half*>(g.x), dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
           CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS) {
     if (err) *err = "cuTensorMapEncodeTiled failed for the activation tile";
     return cudaErrorInvalidValue;
   }
-  const size_t smem = (size_t)kStages * kStageBytes + 1024;
+  PairMaps maps;
+  for (int i = 0; i < 3; ++i) {
+    if (i >= g.n_seg) {
+      maps.codes[i] = maps.codes[0];
+      maps.scales[i] = maps.scales[0];
+      continue;
+    }
+    const GemvSeg& sg = g.seg[i];
+    const cuuint64_t row = g.w16 ? (cuuint64_t)g.K * 2 : (cuuint64_t)g.K / 2, groups = g.grp_off ? (cuuint64_t)g.n_groups : 1;
+    const cuuint64_t wd[3] = {g.w16 ? (cuuint64_t)g.K : row, (cuuint64_t)sg.n_rows, groups};
+    const cuuint64_t ws[2] = {row, g.grp_off ? (cuuint64_t)g.grp_stride : row * sg.n_rows};
+    const cuuint32_t wb[3] = {64, 64, 1}, we[3] = {1, 1, 1};
+    if (enc(&maps.codes[i], g.w16 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_UINT8, 3, const_cast<uint8_t*>(sg.base), wd, ws, wb, we,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, g.w16 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B,
+            g.w16 ? CU_TENSOR_MAP_L2_PROMOTION_L2_256B : CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS) {
+      if (err) *err = "cuTensorMapEncodeTiled failed for the weights";
+      return cudaErrorInvalidValue;
+    }
+    maps.scales[i] = maps.codes[i];
+    if (p.sc16) {  // scales: [n_rows][K / 32] halves behind the codes, eight at a time
+      const cuuint64_t sd[3] = {(cuuint64_t)g.K / 32, wd[1], wd[2]}, ss[2] = {(cuuint64_t)g.K / 16, ws[1]};
+      const cuuint32_t sb[3] = {8, 64, 1};
+      if (enc(&maps.scales[i], CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3, const_cast<uint8_t*>(sg.base) + (size_t)sg.n_rows * (g.K / 2), sd, ss, sb, we,
+              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) !=
+          CUDA_SUCCESS) {
+        if (err) *err = "cuTensorMapEncodeTiled failed for the scales";
+        return cudaErrorInvalidValue;
+      }
+    }
+  }
+  constexpr size_t kMost = 227 * 1024 - 1024;
+  size_t smem;
+  if (g.w16) {  // a ring of steps, as deep as a staging of 64 tokens leaves room for
+    p.stage_tok = kW16StageTok;
+    const size_t fixed = 1024 + (size_t)kW16StageTok * kStagePitch, step = (size_t)p.nt * 64 + kW16Bytes;
+    p.xs = (int)std::min<size_t>(kMaxX, (kMost - fixed) / step);
+    smem = fixed + p.xs * step;
+  } else {  // three activation stages and a code ring twice as deep as the weight stages, then more activations
+    p.stage_tok = p.nt;
+    const size_t fixed = 1024 + (size_t)p.nt * kStagePitch, xs = (size_t)p.nt * 128, cs = kCodeBytes + kScaleBytes;
+    p.stages = fixed + 3 * xs + 8 * cs <= kMost ? 4 : 3;
+    p.codes = 2 * p.stages;
+    p.xs = (int)std::min<size_t>(kMaxX, (kMost - fixed - p.codes * cs) / xs);
+    while (p.codes + p.stages <= kMaxCodes && fixed + p.xs * xs + (p.codes + p.stages) * cs <= kMost) p.codes += p.stages;
+    smem = fixed + p.xs * xs + p.codes * cs;
+  }
   static uint64_t attr_done = 0;
   if (first_use_on_device(&attr_done)) {
-    cudaError_t e1 = cudaFuncSetAttribute(gemm_w16_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e1 != cudaSuccess) return e1;
+    for (const void* k : {reinterpret_cast<const void*>(gemm_pair_kernel<kFmtQ4>), reinterpret_cast<const void*>(gemm_pair_kernel<kFmtMx>),
+                          reinterpret_cast<const void*>(gemm_pair_kernel<kFmtW16>)}) {
+      const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMost);
+      if (e != cudaSuccess) return e;
+    }
   }
-  const int tchunks = (g.T + 511) / 512;
   ++*n_launch;
-  const int N = g.seg[0].n_rows;
-  const cuuint64_t wdims[2] = {(cuuint64_t)g.K, (cuuint64_t)N}, wstr[1] = {(cuuint64_t)g.K * 2};
-  if (enc(&wmap, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, const_cast<uint8_t*>(g.seg[0].base), wdims, wstr, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-          CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS) {
-    if (err) *err = "cuTensorMapEncodeTiled failed for the weight tile";
-    return cudaErrorInvalidValue;
-  }
-  PairParams p{};
-  p.K = g.K;
-  p.T = g.T;
-  p.N = N;
-  p.ksteps = (g.K + BK - 1) / BK;
-  p.y = g.y;
-  p.ldy = g.ldy;
-  p.status = g.status;
-  const dim3 grid(2 * ((N + 255) / 256), tchunks);
-  return launch_dep(gemm_w16_pair_kernel, grid, dim3(kThreads), smem, st, g.pdl, 2, xmap, wmap, p);
+  auto run = [&](auto* kernel) { return launch_dep(kernel, dim3(2 * p.pairs), dim3(kPairThreads), smem, st, g.pdl, 2, xmap, maps, p); };
+  return g.w16 ? run(gemm_pair_kernel<kFmtW16>) : g.mx ? run(gemm_pair_kernel<kFmtMx>) : run(gemm_pair_kernel<kFmtQ4>);
 }
 
 }  // namespace ats

@@ -1,4 +1,4 @@
-"""The dequantizing GEMM with the weights in tensor memory at the edges of its tiles, units and work ranges, against the oracle."""
+"""The GEMMs on pairs of CTAs at the edges of their tiles, units and work ranges, against the oracle."""
 import numpy as np
 import pytest
 
@@ -36,5 +36,32 @@ def test_gemm_edges_match_oracle(fmt, N, K, T):
     ctx.close()
     rows = np.unique(np.r_[0, T // 2, T - 1, np.arange(max(0, T - 3), T), np.arange(min(T, 256) - 2, min(T, 256)), np.arange(0, T, 97)])
     H.assert_close(outs[0][rows], O.linear(x[rows], packed, scales, O.WEIGHT_F16, round_out=True), what=f"{fmt} {N}x{K} T={T}")
+    assert np.all(outs[0][T] == 7.0)
+    assert np.array_equal(outs[0].view(np.uint16), outs[1].view(np.uint16))
+
+
+# fp16 weights: K around the 64-k step and the 128-k unit (multiples of 8), the same edges of N and T, tiles of up to 256 tokens in
+# two accumulators, in several parts and with several contributors, and more tiles than pairs with a remainder
+@pytest.mark.parametrize("N,K,T", [(1, 8, 9), (127, 56, 31), (129, 72, 33), (255, 136, 255), (257, 200, 256), (256, 256, 257), (300, 1000, 513),
+                                   (128, 8192, 10), (513, 4104, 300), (9600, 264, 12), (6001, 520, 270), (4352, 512, 1300)])
+def test_gemm_w16_edges_match_oracle(N, K, T):
+    import torch
+    from paper_2607_10183_b200 import binding as B
+    w = W.w16_matrix(92, 0, W.ROLE_UP, N, K)
+    x = W.activations(92, 0, (T, K))
+    ws = 8 * T * N * 4 + 2 * MB
+    ctx = B.Context(ws + 2 * N * K + 2 * MB, workspace_bytes=ws)
+    tid = ctx.register_w16(w)
+    ctx.set_placement([(tid, -1, B.ATS_GPU)])
+    xd = H.to_dev(x)
+    outs = []
+    for _ in range(2):
+        y = torch.full((T + 1, N), 7.0, dtype=torch.float16, device="cuda")
+        ctx.linear(tid, xd, y, T)
+        ctx.sync()
+        outs.append(y.cpu().numpy())
+    ctx.close()
+    rows = np.unique(np.r_[0, T // 2, T - 1, np.arange(max(0, T - 3), T), np.arange(min(T, 256) - 2, min(T, 256)), np.arange(0, T, 97)])
+    H.assert_close(outs[0][rows], O.linear_w16(x[rows], w, round_out=True), what=f"w16 {N}x{K} T={T}")
     assert np.all(outs[0][T] == 7.0)
     assert np.array_equal(outs[0].view(np.uint16), outs[1].view(np.uint16))
