@@ -75,4 +75,12 @@ __device__ __forceinline__ bool mbar_wait_suspending(uint64_t* bar, uint32_t par
 }
 
 }  // namespace
+// Eight 4-bit floats (sign, two exponent bits, one mantissa bit) as fp16, exactly: o[j] = (low, high) nibble of byte j.
+__device__ __forceinline__ void cvt_e2m1x8(uint32_t w, uint32_t (&o)[4]) {
+  asm("{\n.reg .b8 a, b, c, d;\nmov.b32 {a, b, c, d}, %4;\ncvt.rn.f16x2.e2m1x2 %0, a;\ncvt.rn.f16x2.e2m1x2 %1, b;\n"
+      "cvt.rn.f16x2.e2m1x2 %2, c;\ncvt.rn.f16x2.e2m1x2 %3, d;\n}"
+      : "=r"(o[0]), "=r"(o[1]), "=r"(o[2]), "=r"(o[3])
+      : "r"(w));
+}
+
 }  // namespace ats
