@@ -150,12 +150,6 @@ __device__ __forceinline__ int f2i_magic(float x, float up) {
 // low half): the operands of dp2a.lo / dp2a.hi against the two masked words.  Words 16 and 17 hold mul = 2^-sh and
 // corr = -8 * sum(xi) * mul; both are NaN when the block holds an Inf or a NaN (fp32 exponent field 255), so that the
 // block's term, and with it the output, is NaN.
-//
-// Microscaling 4-bit floats (MX): twice an element is an integer in [-12, 12]; the kernel looks the biased byte
-// 2 e + 16 up per nibble (see mx_bytes) and uses the same unsigned dot products: sum xi (2 e + 16) = 2 sum xi e + 16 sum xi,
-// so mul is halved and the correction stays -8 * sum(xi) * mul.  The lookup yields the bytes of a word's even k
-// (0,2,4,6) and odd k (1,3,5,7), so for this format words 4w..4w+3 hold the pairs (xi_0, xi_2), (xi_4, xi_6), (xi_1, xi_3),
-// (xi_5, xi_7) of the run.
 constexpr int kXqWords = 20;  // 18 used; the 80-byte pitch keeps the 128-bit reads of consecutive blocks conflict-free
 
 // The shift of a block from the largest fp32 exponent field m among its (fp16-valued) elements.
@@ -169,26 +163,17 @@ __device__ __forceinline__ void block_scale(uint32_t m, float& up, float& mul) {
 }
 
 // One run of 8 consecutive elements (one code word's worth) -> its four words of the block.
-template <bool MX>
 __device__ __forceinline__ uint4 pack_run(const int (&xi)[8]) {
   uint4 o;
-  if (MX) {
-    o.x = __byte_perm((uint32_t)xi[0], (uint32_t)xi[2], 0x5410u);
-    o.y = __byte_perm((uint32_t)xi[4], (uint32_t)xi[6], 0x5410u);
-    o.z = __byte_perm((uint32_t)xi[1], (uint32_t)xi[3], 0x5410u);
-    o.w = __byte_perm((uint32_t)xi[5], (uint32_t)xi[7], 0x5410u);
-  } else {
-    o.x = __byte_perm((uint32_t)xi[0], (uint32_t)xi[4], 0x5410u);
-    o.y = __byte_perm((uint32_t)xi[1], (uint32_t)xi[5], 0x5410u);
-    o.z = __byte_perm((uint32_t)xi[2], (uint32_t)xi[6], 0x5410u);
-    o.w = __byte_perm((uint32_t)xi[3], (uint32_t)xi[7], 0x5410u);
-  }
+  o.x = __byte_perm((uint32_t)xi[0], (uint32_t)xi[4], 0x5410u);
+  o.y = __byte_perm((uint32_t)xi[1], (uint32_t)xi[5], 0x5410u);
+  o.z = __byte_perm((uint32_t)xi[2], (uint32_t)xi[6], 0x5410u);
+  o.w = __byte_perm((uint32_t)xi[3], (uint32_t)xi[7], 0x5410u);
   return o;
 }
 
 // Four adjacent lanes each hold one run of a 32-element block; exponent maximum and integer sum are shared by two
 // butterfly shuffles.  Lane w of the group writes words 4w..4w+3 (and lane 0 the two scalars).
-template <bool MX>
 __device__ __forceinline__ void quantize_run4(const float (&x)[8], int w, uint32_t* blk) {
   uint32_t m = 0;
 #pragma unroll
@@ -206,22 +191,26 @@ __device__ __forceinline__ void quantize_run4(const float (&x)[8], int w, uint32
   }
   sx += __shfl_xor_sync(0xffffffffu, sx, 1);
   sx += __shfl_xor_sync(0xffffffffu, sx, 2);
-  *reinterpret_cast<uint4*>(blk + 4 * w) = pack_run<MX>(xi);
-  if (w == 0) *reinterpret_cast<float2*>(blk + 16) = make_float2(MX ? 0.5f * mul : mul, -8.0f * (float)sx * mul);
+  *reinterpret_cast<uint4*>(blk + 4 * w) = pack_run(xi);
+  if (w == 0) *reinterpret_cast<float2*>(blk + 16) = make_float2(mul, -8.0f * (float)sx * mul);
 }
 
-// Four nibbles (the low 16 bits of sel: sign bit, three magnitude bits each) -> the bytes 2 e + 16 of their elements.
-// Twice the magnitudes are v = 0 1 2 3 4 6 8 12.  Two eight-byte tables for prmt: 16 - v, looked up with the sign bits
-// masked out, and 2 v, looked up with the sign bit left in the selector, where prmt returns the sign of the table byte
-// (0: every entry is positive) instead of the byte.  Their sum is 16 + v for a non-negative element and 16 - v for a
-// negative one; no byte exceeds 40, so one 32-bit addition adds the four bytes without carries.
-__device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel) {
-  uint32_t d;
-  asm("prmt.b32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(sel));  // generic form: selector bit 3 = replicate the byte's sign
-  return d;
+// Microscaling 4-bit floats: the elements convert to fp16 exactly and meet the fp16 activations in mma.m16n8k16 (exact products,
+// fp32 sums within a block, the block's scale applied in fp32).  One activation row would fill one of the instruction's eight
+// columns; instead the columns are eight blocks of the row and the sixteen rows of the weight operand are the same eight blocks of
+// two weight rows, of which the products of a block with itself, the diagonal, are wanted.  Lane 4 g + t holds word t of block g
+// of both rows (a warp's 128 bytes of a weight row: no bank conflicts) and run t of the activation block g; word and run are
+// dealt to the two instructions of a block in the order in which cvt_e2m1x8 unpacks a word's bytes.  Per 512 weights: 8
+// conversions, 2 mma, 10 loads, selections and multiply-adds; table look-ups and dp2a, both at half rate, took about 52.
+__device__ __forceinline__ uint4 mx_run(const uint4 h) {  // eight fp16 activations -> pairs (0, 2), (4, 6), (1, 3), (5, 7)
+  return make_uint4(__byte_perm(h.x, h.y, 0x5410u), __byte_perm(h.z, h.w, 0x5410u), __byte_perm(h.x, h.y, 0x7632u),
+                    __byte_perm(h.z, h.w, 0x7632u));
 }
-__device__ __forceinline__ uint32_t mx_bytes(uint32_t sel) {
-  return prmt(0x0D0E0F10u, 0x04080A0Cu, sel & 0x7777u) + prmt(0x06040200u, 0x18100C08u, sel);
+__device__ __forceinline__ void mma16816(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
 struct StreamSeg {
@@ -395,8 +384,10 @@ __device__ __forceinline__ bool stream_consume(const StreamParams& p, const int 
   const int part = wg % PARTS, rsub = wg / PARTS;
   const int pblk = (nblk + PARTS - 1) / PARTS;
   const int b0 = part * pblk, b1 = min(nblk, b0 + pblk);
-  uint32_t xr[J][16];
+  uint32_t xr[J][16];       // integer codes: this lane's blocks; microscaling: [4 j + i] = its run of block group i
   float xm[J], xc[J];
+  constexpr int NG = 4 * J;  // microscaling: groups of eight blocks of the part
+  const int g8 = lane >> 2, t4 = lane & 3;
   ATS_TR(0);
   {
     // Thread t owns the runs of 8 consecutive elements r = t + 512 j (one run when K <= 4096, up to four for K = 16384);
@@ -451,7 +442,10 @@ __device__ __forceinline__ bool stream_consume(const StreamParams& p, const int 
           xv[2 * q + 1] = f.y;
         }
         if (p.h_out && bx == 0) *reinterpret_cast<uint4*>(p.h_out + i0) = make_uint4(o4[0], o4[1], o4[2], o4[3]);
-        quantize_run4<MX>(xv, tid & 3, xq_s + (size_t)(tid >> 2) * kXqWords);
+        if (MX)
+          reinterpret_cast<uint4*>(xq_s)[tid] = mx_run(make_uint4(o4[0], o4[1], o4[2], o4[3]));
+        else
+          quantize_run4(xv, tid & 3, xq_s + (size_t)(tid >> 2) * kXqWords);
       }
     } else {
       if (!dep_resolved) asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -468,16 +462,31 @@ __device__ __forceinline__ bool stream_consume(const StreamParams& p, const int 
       for (int j = 0; j < 4; ++j) {
         const int r = tid + kConsumerThreads * j;
         if (r * 8 < K) {
-          float xv[8];
-          unpack_h8(raw[j], xv);
-          quantize_run4<MX>(xv, r & 3, xq_s + (size_t)(r >> 2) * kXqWords);
+          if (MX) {
+            reinterpret_cast<uint4*>(xq_s)[r] = mx_run(raw[j]);
+          } else {
+            float xv[8];
+            unpack_h8(raw[j], xv);
+            quantize_run4(xv, r & 3, xq_s + (size_t)(r >> 2) * kXqWords);
+          }
         }
       }
     }
     ATS_TR(2);
     consumer_sync_all();
+    if constexpr (MX) {
 #pragma unroll
-    for (int j = 0; j < J; ++j) {
+      for (int i = 0; i < NG; ++i) {
+        const int b = b0 + 8 * i + g8;
+        const uint4 v = b < b1 ? reinterpret_cast<const uint4*>(xq_s)[4 * b + t4] : make_uint4(0, 0, 0, 0);
+        xr[i / 4][4 * (i % 4)] = v.x;
+        xr[i / 4][4 * (i % 4) + 1] = v.y;
+        xr[i / 4][4 * (i % 4) + 2] = v.z;
+        xr[i / 4][4 * (i % 4) + 3] = v.w;
+      }
+    }
+#pragma unroll
+    for (int j = 0; !MX && j < J; ++j) {
       const int b = b0 + lane + 32 * j;
       if (b < b1) {
         const uint4* src = reinterpret_cast<const uint4*>(xq_s + (size_t)b * kXqWords);
@@ -532,62 +541,100 @@ __device__ __forceinline__ bool stream_consume(const StreamParams& p, const int 
       if (li == 0) ATS_TR(4);
       ATS_TR(100 + it);
       const uint8_t* st = stages + (size_t)s * stage_bytes;
-      uint4 cw[RPW][J];
-      float sc[RPW][J];
-#pragma unroll
-      for (int r = 0; r < RPW; ++r) {
-        const int row = r * (ROWS / RPW) + rsub;  // stage row of this warp's r-th row
-        const uint4* codes = reinterpret_cast<const uint4*>(st + (size_t)row * row_codes);
-        const __half* scp = reinterpret_cast<const __half*>(st + (size_t)ROWS * row_codes + (size_t)row * row_scales);
-#pragma unroll
-        for (int j = 0; j < J; ++j) {
-          const int b = b0 + lane + 32 * j;
-          const bool in = b < b1;
-          cw[r][j] = in ? codes[b] : make_uint4(0, 0, 0, 0);
-          sc[r][j] = in ? __half2float(scp[b]) : 0.f;
-        }
-      }
-      // The stage is released as soon as its words are in registers, not after the arithmetic on them: a stage that is
-      // held while it is being computed on is a stage that is not in flight, and the ring is what keeps HBM busy.  The
-      // fold below makes the release wait for every load (an instruction issues only when its operands have arrived).
-      {
-        uint32_t fold = 0;
-#pragma unroll
-        for (int r = 0; r < RPW; ++r)
-#pragma unroll
-          for (int j = 0; j < J; ++j) fold ^= cw[r][j].x ^ cw[r][j].y ^ cw[r][j].z ^ cw[r][j].w ^ __float_as_uint(sc[r][j]);
-        asm volatile("" ::"r"(fold) : "memory");
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&sh.empty[s]);
-      }
-      if (have_prev) reduce_store(prev, li - 1 - li0);
       float acc[RPW];
+      if constexpr (MX) {
+        uint32_t cw[RPW][NG];
+        unsigned short sc[RPW][NG];
 #pragma unroll
-      for (int r = 0; r < RPW; ++r) {
-        acc[r] = 0.f;
+        for (int r = 0; r < RPW; ++r) {
+          const int row = r * (ROWS / RPW) + rsub;
+          const uint32_t* codes = reinterpret_cast<const uint32_t*>(st + (size_t)row * row_codes) + 4 * (b0 + g8) + t4;
+          const unsigned short* scp = reinterpret_cast<const unsigned short*>(st + (size_t)ROWS * row_codes + (size_t)row * row_scales) + b0 + g8;
 #pragma unroll
-        for (int j = 0; j < J; ++j) {
-          const uint32_t ws[4] = {cw[r][j].x, cw[r][j].y, cw[r][j].z, cw[r][j].w};
-          int dl = 0, dh = 0;
+          for (int i = 0; i < NG; ++i) {
+            const bool in = b0 + 8 * i + g8 < b1;
+            cw[r][i] = in ? codes[32 * i] : 0u;
+            sc[r][i] = in ? scp[8 * i] : (unsigned short)0;
+          }
+        }
+        {
+          uint32_t fold = 0;  // (see below)
 #pragma unroll
-          for (int w = 0; w < 4; ++w) {
-            if (MX) {
-              const uint32_t ev = mx_bytes(ws[w]), od = mx_bytes(ws[w] >> 16);  // k = 0 2 4 6 and k = 1 3 5 7 of the word
-              dl = dp2a_lo(xr[j][4 * w], ev, dl);
-              dl = dp2a_hi(xr[j][4 * w + 1], ev, dl);
-              dh = dp2a_lo(xr[j][4 * w + 2], od, dh);
-              dh = dp2a_hi(xr[j][4 * w + 3], od, dh);
-            } else {
+          for (int r = 0; r < RPW; ++r)
+#pragma unroll
+            for (int i = 0; i < NG; ++i) fold ^= cw[r][i] ^ sc[r][i];
+          asm volatile("" ::"r"(fold) : "memory");
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&sh.empty[s]);
+        }
+        if (have_prev) reduce_store(prev, li - 1 - li0);
+        const bool odd = g8 & 1, diagonal = t4 == g8 >> 1;
+#pragma unroll
+        for (int r = 0; r < RPW; r += 2) {
+          float s0 = 0.f, s1 = 0.f;
+#pragma unroll
+          for (int i = 0; i < NG; ++i) {
+            uint32_t a0[4], a1[4];
+            cvt_e2m1x8(cw[r][i], a0);
+            cvt_e2m1x8(cw[r + 1][i], a1);
+            const uint32_t* x = &xr[i / 4][4 * (i % 4)];
+            float c[4] = {0.f, 0.f, 0.f, 0.f};
+            mma16816(c, a0[0], a1[0], a0[1], a1[1], x[0], x[1]);
+            mma16816(c, a0[2], a1[2], a0[3], a1[3], x[2], x[3]);
+            s0 = fmaf(__half2float(__ushort_as_half(sc[r][i])), odd ? c[1] : c[0], s0);
+            s1 = fmaf(__half2float(__ushort_as_half(sc[r + 1][i])), odd ? c[3] : c[2], s1);
+          }
+          acc[r] = diagonal ? s0 : 0.f;
+          acc[r + 1] = diagonal ? s1 : 0.f;
+        }
+      } else {
+        uint4 cw[RPW][J];
+        float sc[RPW][J];
+#pragma unroll
+        for (int r = 0; r < RPW; ++r) {
+          const int row = r * (ROWS / RPW) + rsub;  // stage row of this warp's r-th row
+          const uint4* codes = reinterpret_cast<const uint4*>(st + (size_t)row * row_codes);
+          const __half* scp = reinterpret_cast<const __half*>(st + (size_t)ROWS * row_codes + (size_t)row * row_scales);
+#pragma unroll
+          for (int j = 0; j < J; ++j) {
+            const int b = b0 + lane + 32 * j;
+            const bool in = b < b1;
+            cw[r][j] = in ? codes[b] : make_uint4(0, 0, 0, 0);
+            sc[r][j] = in ? __half2float(scp[b]) : 0.f;
+          }
+        }
+        // The stage is released as soon as its words are in registers, not after the arithmetic on them: a stage that is
+        // held while it is being computed on is a stage that is not in flight, and the ring is what keeps HBM busy.  The
+        // fold below makes the release wait for every load (an instruction issues only when its operands have arrived).
+        {
+          uint32_t fold = 0;
+#pragma unroll
+          for (int r = 0; r < RPW; ++r)
+#pragma unroll
+            for (int j = 0; j < J; ++j) fold ^= cw[r][j].x ^ cw[r][j].y ^ cw[r][j].z ^ cw[r][j].w ^ __float_as_uint(sc[r][j]);
+          asm volatile("" ::"r"(fold) : "memory");
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&sh.empty[s]);
+        }
+        if (have_prev) reduce_store(prev, li - 1 - li0);
+#pragma unroll
+        for (int r = 0; r < RPW; ++r) {
+          acc[r] = 0.f;
+#pragma unroll
+          for (int j = 0; j < J; ++j) {
+            const uint32_t ws[4] = {cw[r][j].x, cw[r][j].y, cw[r][j].z, cw[r][j].w};
+            int dl = 0, dh = 0;
+#pragma unroll
+            for (int w = 0; w < 4; ++w) {
               const uint32_t lo = ws[w] & 0x0F0F0F0Fu, hi = ws[w] & 0xF0F0F0F0u;  // hi carries 16 * code
               dl = dp2a_lo(xr[j][4 * w], lo, dl);
               dl = dp2a_hi(xr[j][4 * w + 1], lo, dl);
               dh = dp2a_lo(xr[j][4 * w + 2], hi, dh);
               dh = dp2a_hi(xr[j][4 * w + 3], hi, dh);
             }
+            const float dot = (float)(dl + (dh >> 4));  // dh is a multiple of 16, |dot| < 2^24: exact
+            acc[r] = fmaf(sc[r][j], fmaf(dot, xm[j], xc[j]), acc[r]);
           }
-          // integer codes: dh is a multiple of 16; either way |dot| < 2^24: exact
-          const float dot = MX ? (float)(dl + dh) : (float)(dl + (dh >> 4));
-          acc[r] = fmaf(sc[r][j], fmaf(dot, xm[j], xc[j]), acc[r]);
         }
       }
       ATS_TR(200 + it);

@@ -65,6 +65,23 @@ def test_dequant_every_element_pair_times_every_accepted_scale(B, torch):
     ctx.close()
 
 
+# One row on the streaming GEMV, where the blocks of a row are dealt to the warps in eights: parts of the row that end inside an eight
+# (K = 2816: two parts of 44 blocks, 8448: eight of 33), a single eight, the short-row form up to 1024, the longest row.
+@pytest.mark.parametrize("K", [256, 768, 1024, 1280, 2816, 4096, 8448, 14336, 16384])
+def test_linear_one_row_parts_of_a_row(B, torch, K):
+    N = 96
+    packed, sb = W.mxfp4_packed(91, 0, W.ROLE_Q, N, K)
+    x = W.activations(91, 0, (1, K))
+    ctx = ctx_for(B, W.q4_bytes(N, K))
+    tid = ctx.register_mxfp4(packed, sb)
+    ctx.set_placement([(tid, -1, B.ATS_GPU)])
+    y = torch.empty((1, N), dtype=torch.float16, device="cuda")
+    ctx.linear(tid, H.to_dev(x), y, 1)
+    ctx.sync()
+    H.assert_close(y.cpu().numpy(), O.linear(x, packed, sb, round_out=True), what=f"K={K}")
+    ctx.close()
+
+
 @pytest.mark.parametrize("N,K,M", [(8, 32, 1), (37, 96, 3), (130, 1024, 8), (4096, 4096, 1), (256, 14336, 2), (300, 4096, 20), (1024, 1024, 129), (2048, 768, 1), (64, 256, 1)])
 def test_linear_matches_oracle_gemv_and_gemm(B, torch, N, K, M):
     """Up to 8 rows: the generic GEMV (fp32 accumulation of exact products); more: the tcgen05 GEMM with the weight tile
