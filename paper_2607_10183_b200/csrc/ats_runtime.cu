@@ -259,8 +259,8 @@ static int count_streamed(const Operand* ops, int n) {
   return c;
 }
 
-// One GEMV: the streaming kernel where the shapes allow it (one row of a 4-bit format; two rows as two launches), else the
-// fp16-weight kernel, the mma.sync kernel (4-bit formats, three to eight rows) or the generic kernel, preceded by a
+// One GEMV: the streaming kernel where the shapes allow it (one row of a 4-bit format), else the fp16-weight kernel, the
+// mma.sync kernel (4-bit formats, two or three to eight rows) or the generic kernel, preceded by a
 // separate RMSNorm launch when a norm prologue was asked for.  Which kernel runs depends on format and shapes only, never on placement.
 static int32_t launch_gemv_any(ats_ctx* ctx, GemvParams p) {
   p.pdl = (ctx->cfg.flags & ATS_FLAG_NO_PDL) ? 0 : 1;
@@ -270,27 +270,6 @@ static int32_t launch_gemv_any(ats_ctx* ctx, GemvParams p) {
     TimedLaunch tl(ctx, 0, gemv_work_bytes(p));
     ATS_CUDA(launch_gemv_stream(p, ctx->dev_status, ctx->sm_count, ctx->cs, &ctx->stats.kernel_launches));
     return ATS_OK;
-  }
-  if (p.M == 2 && !p.w16) {
-    // Two rows: the single-row streaming kernel once per row is faster than the generic kernel over both (two launches at
-    // about 8 us against one of 19 us for 14336 x 4096), and each row gets exactly the single-row result.
-    GemvParams q = p;
-    q.M = 1;
-    if (gemv_stream_eligible(q)) {
-      for (int r = 0; r < 2; ++r) {
-        TimedLaunch tl(ctx, 0, gemv_work_bytes(q));
-        ATS_CUDA(launch_gemv_stream(q, ctx->dev_status, ctx->sm_count, ctx->cs, &ctx->stats.kernel_launches));
-        if (q.x) q.x += q.ldx;
-        if (q.norm_x16) q.norm_x16 += q.K;
-        if (q.norm_x32) q.norm_x32 += q.K;
-        if (q.norm_out) q.norm_out += q.K;
-        if (q.y32) q.y32 += q.ldy;
-        if (q.y16) q.y16 += q.ldy;
-        if (q.res32) q.res32 += q.ldres;
-        if (q.res16) q.res16 += q.ldres;
-      }
-      return ATS_OK;
-    }
   }
   if (p.norm_gain) {
     if (!p.norm_out) return fail(ctx, ATS_ERR_INVALID, "internal: norm prologue without an output buffer");
@@ -302,7 +281,10 @@ static int32_t launch_gemv_any(ats_ctx* ctx, GemvParams p) {
   TimedLaunch tl(ctx, 0, gemv_work_bytes(p));
   if (p.w16)
     ATS_CUDA(launch_gemv_w16(p, ctx->cs, &ctx->stats.kernel_launches));
-  else if (p.M >= 3 && gemv_mma_eligible(p))  // from three rows on the tensor-core form is the faster one (its cost does not grow with M)
+  else if (p.M >= (p.K % 256 ? 3 : 2) && gemv_mma_eligible(p))
+    // From three rows on the tensor-core form is the faster one (its cost does not grow with M); streamed through its ring
+    // (K a multiple of 256) from two (4096 x 4096, two launches of the streaming kernel against one: MXFP4 9.7 and 5.4 us, Q4 7.9
+    // and 5.4; 14336 x 4096: 18.2 and 10, 14.5 and 11.8).
     ATS_CUDA(launch_gemv_mma(p, ctx->cs, &ctx->stats.kernel_launches));
   else
     ATS_CUDA(launch_gemv(p, ctx->cs, &ctx->stats.kernel_launches));

@@ -65,6 +65,25 @@ def test_dequant_every_element_pair_times_every_accepted_scale(B, torch):
     ctx.close()
 
 
+# Two to eight rows through the ring of the few-row GEMV (K a multiple of 256): one step of K, parts of unequal length (11 and 56
+# steps over eight), tiles of 16 rows that are not full, one unit and more units than the grid has places for.
+@pytest.mark.parametrize("fmt", ["q4", "mxfp4"])
+@pytest.mark.parametrize("N,K,M", [(1, 256, 2), (17, 512, 3), (130, 2816, 8), (96, 14336, 5), (4999, 1024, 4), (40000, 256, 2)])
+def test_linear_few_rows_ring(B, torch, fmt, N, K, M):
+    packed, scales = (W.q4_packed if fmt == "q4" else W.mxfp4_packed)(91, 0, W.ROLE_UP, N, K)
+    x = W.activations(91, 0, (M, K))
+    ctx = ctx_for(B, W.q4_bytes(N, K))
+    tid = ctx.register_q4(packed, scales) if fmt == "q4" else ctx.register_mxfp4(packed, scales)
+    ctx.set_placement([(tid, -1, B.ATS_GPU)])
+    y = torch.full((M + 1, N), 7.0, dtype=torch.float16, device="cuda")
+    ctx.linear(tid, H.to_dev(x), y, M)
+    ctx.sync()
+    got = y.cpu().numpy()
+    ctx.close()
+    H.assert_close(got[:M], O.linear(x, packed, scales, round_out=True), what=f"{fmt} {N}x{K} M={M}")
+    assert np.all(got[M] == 7.0)
+
+
 # One row on the streaming GEMV, where the blocks of a row are dealt to the warps in eights: parts of the row that end inside an eight
 # (K = 2816: two parts of 44 blocks, 8448: eight of 33), a single eight, the short-row form up to 1024, the longest row.
 @pytest.mark.parametrize("K", [256, 768, 1024, 1280, 2816, 4096, 8448, 14336, 16384])
