@@ -382,12 +382,13 @@ __device__ __forceinline__ bool stream_consume(const StreamParams& p, const int 
   const int wg = warp % kGroupWarps;          // warp within the group
   const int tg = tid % (kGroupWarps * 32);    // thread within the group
   const int part = wg % PARTS, rsub = wg / PARTS;
-  const int pblk = (nblk + PARTS - 1) / PARTS;
-  const int b0 = part * pblk, b1 = min(nblk, b0 + pblk);
+  // (microscaling: parts of whole groups of eight blocks; there are K / 256 of them)
+  const int pblk = MX ? ((nblk + PARTS - 1) / PARTS + 7) / 8 * 8 : (nblk + PARTS - 1) / PARTS;
+  const int b0 = min(nblk, part * pblk), b1 = min(nblk, b0 + pblk);
   uint32_t xr[J][16];       // integer codes: this lane's blocks; microscaling: [4 j + i] = its run of block group i
   float xm[J], xc[J];
   constexpr int NG = 4 * J;  // microscaling: groups of eight blocks of the part
-  const int g8 = lane >> 2, t4 = lane & 3;
+  const int g8 = lane >> 2, t4 = lane & 3, ng = (b1 - b0) / 8;
   ATS_TR(0);
   {
     // Thread t owns the runs of 8 consecutive elements r = t + 512 j (one run when K <= 4096, up to four for K = 16384);
@@ -478,7 +479,7 @@ __device__ __forceinline__ bool stream_consume(const StreamParams& p, const int 
 #pragma unroll
       for (int i = 0; i < NG; ++i) {
         const int b = b0 + 8 * i + g8;
-        const uint4 v = b < b1 ? reinterpret_cast<const uint4*>(xq_s)[4 * b + t4] : make_uint4(0, 0, 0, 0);
+        const uint4 v = i < ng ? reinterpret_cast<const uint4*>(xq_s)[4 * b + t4] : make_uint4(0, 0, 0, 0);
         xr[i / 4][4 * (i % 4)] = v.x;
         xr[i / 4][4 * (i % 4) + 1] = v.y;
         xr[i / 4][4 * (i % 4) + 2] = v.z;
@@ -545,18 +546,21 @@ __device__ __forceinline__ bool stream_consume(const StreamParams& p, const int 
       if constexpr (MX) {
         uint32_t cw[RPW][NG];
         unsigned short sc[RPW][NG];
+        auto fetch = [&](auto all) {  // all: the part has NG groups
 #pragma unroll
-        for (int r = 0; r < RPW; ++r) {
-          const int row = r * (ROWS / RPW) + rsub;
-          const uint32_t* codes = reinterpret_cast<const uint32_t*>(st + (size_t)row * row_codes) + 4 * (b0 + g8) + t4;
-          const unsigned short* scp = reinterpret_cast<const unsigned short*>(st + (size_t)ROWS * row_codes + (size_t)row * row_scales) + b0 + g8;
+          for (int r = 0; r < RPW; ++r) {
+            const int row = r * (ROWS / RPW) + rsub;
+            const uint32_t* codes = reinterpret_cast<const uint32_t*>(st + (size_t)row * row_codes) + 4 * (b0 + g8) + t4;
+            const unsigned short* scp = reinterpret_cast<const unsigned short*>(st + (size_t)ROWS * row_codes + (size_t)row * row_scales) + b0 + g8;
 #pragma unroll
-          for (int i = 0; i < NG; ++i) {
-            const bool in = b0 + 8 * i + g8 < b1;
-            cw[r][i] = in ? codes[32 * i] : 0u;
-            sc[r][i] = in ? scp[8 * i] : (unsigned short)0;
+            for (int i = 0; i < NG; ++i) {
+              cw[r][i] = all || i < ng ? codes[32 * i] : 0u;
+              sc[r][i] = all || i < ng ? scp[8 * i] : (unsigned short)0;
+            }
           }
-        }
+        };
+        if (ng == NG) fetch(true);
+        else fetch(false);
         {
           uint32_t fold = 0;  // (see below)
 #pragma unroll
@@ -571,7 +575,7 @@ __device__ __forceinline__ bool stream_consume(const StreamParams& p, const int 
         const bool odd = g8 & 1, diagonal = t4 == g8 >> 1;
 #pragma unroll
         for (int r = 0; r < RPW; r += 2) {
-          float s0 = 0.f, s1 = 0.f;
+          float s0[2] = {0.f, 0.f}, s1[2] = {0.f, 0.f};  // even and odd column of this lane: one of them may be on the diagonal
 #pragma unroll
           for (int i = 0; i < NG; ++i) {
             uint32_t a0[4], a1[4];
@@ -581,11 +585,14 @@ __device__ __forceinline__ bool stream_consume(const StreamParams& p, const int 
             float c[4] = {0.f, 0.f, 0.f, 0.f};
             mma16816(c, a0[0], a1[0], a0[1], a1[1], x[0], x[1]);
             mma16816(c, a0[2], a1[2], a0[3], a1[3], x[2], x[3]);
-            s0 = fmaf(__half2float(__ushort_as_half(sc[r][i])), odd ? c[1] : c[0], s0);
-            s1 = fmaf(__half2float(__ushort_as_half(sc[r + 1][i])), odd ? c[3] : c[2], s1);
+            const float f0 = __half2float(__ushort_as_half(sc[r][i])), f1 = __half2float(__ushort_as_half(sc[r + 1][i]));
+            s0[0] = fmaf(f0, c[0], s0[0]);
+            s0[1] = fmaf(f0, c[1], s0[1]);
+            s1[0] = fmaf(f1, c[2], s1[0]);
+            s1[1] = fmaf(f1, c[3], s1[1]);
           }
-          acc[r] = diagonal ? s0 : 0.f;
-          acc[r + 1] = diagonal ? s1 : 0.f;
+          acc[r] = diagonal ? (odd ? s0[1] : s0[0]) : 0.f;
+          acc[r + 1] = diagonal ? (odd ? s1[1] : s1[0]) : 0.f;
         }
       } else {
         uint4 cw[RPW][J];
