@@ -27,8 +27,8 @@
 // close to one per cycle and scheduler); fp16 there the weights' way from memory; beyond that the MMAs and the power limit.
 // Back to back on new weights, before -> now (before: weights as a shared-memory operand, 256-token tiles, with reduction,
 // residual and SwiGLU launches):
-//   77 tokens MXFP4: 28672 x 4096 with SwiGLU 66 -> 37 us, 6144 x 4096 25 -> 21, 4096 x 14336 41 -> 33
-//   512 tokens Q4: gate and up 143 -> 103-107 us, 4096 x 14336 78 -> 71;  2048 tokens: gate and up 462 -> 360 (1335 TFLOP/s)
+//   77 tokens MXFP4: 28672 x 4096 with SwiGLU 66 -> 36 us, 6144 x 4096 25 -> 21, 4096 x 14336 41 -> 33
+//   512 tokens Q4: gate and up 143 -> 103-107 us, 4096 x 14336 78 -> 69;  2048 tokens: gate and up 462 -> 351 (1372 TFLOP/s)
 //   2048 tokens fp16: q, k, v 152 -> 78 us, o 66 -> 59, gate and up 451 -> 346 (1390 TFLOP/s), 4096 x 14336 189 -> 196
 //
 // Roles per CTA: warp 0 = activation loads (fp16: and weights), warp 1 = tensor-memory allocation and (leader) MMA issue, warps 2, 3
@@ -338,12 +338,12 @@ __global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid
   }
   if (warp == 2 && lane == 0) {     // (the loaders' own barriers: they start before the CTAs have met)
     for (int s = 0; s < NC; ++s) {
-      mbar_init(&cfull[s], p.sc16 ? 1 : 1 + 64);
+      mbar_init(&cfull[s], p.sc16 ? 2 : 1 + 64);
       mbar_init(&cempty[s], 4);     // the warps of the stage's group
     }
     mbar_fence_init();
   }
-  // ---- code and scale loads (warp 2; warp 3 too where the scales' rows are not 16-byte aligned).  Weights depend on nothing:
+  // ---- code loads (warp 2) and scale loads (warp 3; both where the scales' rows are not 16-byte aligned).  Weights depend on nothing:
   // the first units are requested before the CTAs of the pair meet, the rest by the loaders' own branch below.
   bool ok = true;
   Stretch st;
@@ -373,15 +373,17 @@ __global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid
       uint64_t* bar = &cfull[ld_cs];
       const uint32_t sdst = smem_u32(scale_s) + (uint32_t)(ld_cs * kScaleBytes);
       const int second = p.act ? ld_first : ld_first + 64;
+      // (two warps: one alone needed 770 cycles per unit for its four loads, as long as the unit takes at 16 tokens; 18944 x 14336
+      // 59.8 -> 56.7 us)
       if (warp == 2) {  // rows beyond the matrix and k beyond its end read as zeros
         const uint32_t dst = smem_u32(code_s) + (uint32_t)(ld_cs * kCodeBytes);
-        expect_tx_one(one, bar, (uint32_t)(kCodeBytes + (p.sc16 ? kScaleBytes : 0)));
+        expect_tx_one(one, bar, (uint32_t)kCodeBytes);
         tma_3d_one(one, dst, &wmap.codes[ld_sa], ld_u * 64, ld_first, ld_e, bar);
         tma_3d_one(one, dst + kCodeBytes / 2, &wmap.codes[ld_sb], ld_u * 64, second, ld_e, bar);
-        if (p.sc16) {  // (a line of eight scales serves two units: 16 bytes are the least that a copy takes)
-          tma_3d_one(one, sdst, &wmap.scales[ld_sa], (ld_u >> 1) * 8, ld_first, ld_e, bar);
-          tma_3d_one(one, sdst + kScaleBytes / 2, &wmap.scales[ld_sb], (ld_u >> 1) * 8, second, ld_e, bar);
-        }
+      } else if (p.sc16) {  // (a line of eight scales serves two units: 16 bytes are the least that a copy takes)
+        expect_tx_one(one, bar, (uint32_t)kScaleBytes);
+        tma_3d_one(one, sdst, &wmap.scales[ld_sa], (ld_u >> 1) * 8, ld_first, ld_e, bar);
+        tma_3d_one(one, sdst + kScaleBytes / 2, &wmap.scales[ld_sb], (ld_u >> 1) * 8, second, ld_e, bar);
       }
       if (!p.sc16) {
         // six halves of each row from the 4-byte boundary at or below the unit's first scale; the reader skips the odd one.
@@ -407,8 +409,8 @@ __global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid
       if (++ld_cs == NC) ld_cs = 0, ld_par ^= 1u;
     }
   };
-  if (FMT != kFmtW16 && (warp == 2 || (warp == 3 && !p.sc16))) {
-    if (!p.sc16) asm volatile("bar.sync 2, 64;" ::: "memory");  // the barriers are initialised
+  if (FMT != kFmtW16 && (warp == 2 || warp == 3)) {
+    asm volatile("bar.sync 2, 64;" ::: "memory");  // the barriers are initialised
     __syncwarp();
     if (p.grp_off) asm volatile("griddepcontrol.wait;" ::: "memory");
     load_units(min(4, NC));
@@ -559,7 +561,7 @@ __global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid
       }
     } else {
       // ------------------------------------------------------------ code and scale loaders, continued
-      if (FMT != kFmtW16 && (warp == 2 || !p.sc16)) load_units(0x7fffffff);
+      if (FMT != kFmtW16) load_units(0x7fffffff);
       asm volatile("cp.async.wait_all;" ::: "memory");
     }
   } else if (warp >= 12) {
