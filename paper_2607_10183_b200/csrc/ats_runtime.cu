@@ -484,7 +484,7 @@ static LayerWs layout_prefill(const ats_layer_desc& L, uint32_t T, uint8_t* base
     const uint64_t P = (uint64_t)T * L.top_k;
     w.ids = (int32_t*)b.take(P * 4);
     w.gates = (float*)b.take(P * 4);
-    w.order = (int*)b.take(P * 4);
+    w.order = (int*)b.take(P * 4);  // (order, pos and grp_off follow one another: one copy writes them)
     w.pos = (int*)b.take(P * 4);
     w.grp_off = (int*)b.take(((uint64_t)L.n_experts + 1) * 4);
     w.xs16 = (__half*)b.take(P * H * 2);
@@ -1718,15 +1718,14 @@ int32_t ats_layer_prefill(ats_ctx* ctx, const ats_layer_desc* L, const void* x_i
     ATS_CUDA(launch_router_topk(w.h2_16, (const __half*)ctx->tensors[L->router].f16_dev, (int)T, H, E, k,
                                 (L->flags & ATS_LAYER_NO_TOPK_RENORM) ? 0 : 1, w.ids, w.gates, ctx->cs, nl, pdl));
     ATS_TRY(fetch_ids(ctx, w.ids, P, E));
-    int32_t* order_h = ctx->ids_host + kMaxPairs;       // sorted position -> pair
-    int32_t* pos_h = ctx->ids_host + 2 * kMaxPairs;     // pair -> sorted position
-    int32_t* off_h = ctx->ids_host + 3 * kMaxPairs;     // expert -> first sorted position; [E] = P
+    // the sort's arrays, laid out as the workspace has them, so that one copy takes all three
+    int32_t* order_h = ctx->ids_host + kMaxPairs;              // sorted position -> pair
+    int32_t* pos_h = order_h + (w.pos - w.order);              // pair -> sorted position
+    int32_t* off_h = order_h + (w.grp_off - w.order);          // expert -> first sorted position; [E] = P
     int max_rows = 0;
     if (ats_host_group_pairs(ctx->ids_host, (uint32_t)P, (uint32_t)E, order_h, pos_h, off_h, &max_rows) != ATS_OK)
       return fail(ctx, ATS_ERR_INVALID, "routing ids out of range");
-    ATS_CUDA(cudaMemcpyAsync(w.order, order_h, (size_t)P * 4, cudaMemcpyHostToDevice, ctx->cs));
-    ATS_CUDA(cudaMemcpyAsync(w.pos, pos_h, (size_t)P * 4, cudaMemcpyHostToDevice, ctx->cs));
-    ATS_CUDA(cudaMemcpyAsync(w.grp_off, off_h, (size_t)(E + 1) * 4, cudaMemcpyHostToDevice, ctx->cs));
+    ATS_CUDA(cudaMemcpyAsync(w.order, order_h, (size_t)(off_h + E + 1 - order_h) * 4, cudaMemcpyHostToDevice, ctx->cs));
     ATS_CUDA(launch_moe_gather_rows(w.h2_16, w.order, k, w.xs16, P, H, ctx->cs, nl, pdl));
     const Tensor &tg = ctx->tensors[L->w_gate], &tu = ctx->tensors[L->w_up], &td = ctx->tensors[L->w_down];
     auto slice0 = [](const Tensor& t) -> const uint8_t* { return t.contiguous_dev ? t.slices[0].dev : nullptr; };
