@@ -240,6 +240,7 @@ struct MoeGemvParams {
   const uint8_t* const* tab1;
   int x_div;           // activation row of pair p is p / x_div (k when one x per token, 1 when one per slot)
   int P;
+  int M;               // tokens the pairs belong to
   int n_experts;       // ids outside [0, n_experts) are replaced by 0 and raise *status (implicit addressing)
   int* status;
   // common
@@ -258,6 +259,10 @@ cudaError_t launch_moe_gemv(const MoeGemvParams& p, const MoeJobs* jobs /*null =
 bool moe_gemv_stream_eligible(const MoeGemvParams& p);
 cudaError_t launch_moe_gemv_stream(const MoeGemvParams& p, const MoeJobs* jobs /*null = implicit*/, int* status, int sm_count,
                                    int pdl, cudaStream_t st, uint64_t* n_launch);
+// several tokens, pairs grouped by expert (kernels_gemv_mma.cu)
+bool moe_gemv_mma_eligible(const MoeGemvParams& p);
+cudaError_t launch_moe_gemv_mma(const MoeGemvParams& p, const MoeJobs* jobs /*null = implicit*/, int sm_count, int pdl, cudaStream_t st,
+                                uint64_t* n_launch);
 
 // reads `bytes` of device memory once with the streaming GEMV's access pattern and drops them (kernels_gemv_stream.cu)
 cudaError_t launch_hbm_read_probe(const uint8_t* src, uint64_t bytes, int* status, int sm_count, cudaStream_t st);

@@ -597,9 +597,10 @@ static int32_t apply_placement(ats_ctx* ctx) {
 // in groups that fit the ring.
 // One grouped-expert GEMV launch: the streaming kernel where the shapes allow it, else the generic one.
 static cudaError_t launch_moe_gemv_any(ats_ctx* ctx, const MoeGemvParams& p, const MoeJobs* jobs) {
+  const int pdl = (ctx->cfg.flags & ATS_FLAG_NO_PDL) ? 0 : 1;
+  if (moe_gemv_mma_eligible(p)) return launch_moe_gemv_mma(p, jobs, ctx->sm_count, pdl, ctx->cs, &ctx->stats.kernel_launches);
   if (moe_gemv_stream_eligible(p))
-    return launch_moe_gemv_stream(p, jobs, ctx->dev_status, ctx->sm_count, (ctx->cfg.flags & ATS_FLAG_NO_PDL) ? 0 : 1, ctx->cs,
-                                  &ctx->stats.kernel_launches);
+    return launch_moe_gemv_stream(p, jobs, ctx->dev_status, ctx->sm_count, pdl, ctx->cs, &ctx->stats.kernel_launches);
   return launch_moe_gemv(p, jobs, ctx->cs, &ctx->stats.kernel_launches);
 }
 
@@ -1259,6 +1260,7 @@ int32_t ats_moe_linear(ats_ctx* ctx, int32_t id, const void* x, const int32_t* i
   if (P > 256) return fail(ctx, ATS_ERR_SHAPE, "M*k = %u exceeds 256", P);
   MoeGemvParams p{};
   p.P = (int)P;
+  p.M = (int)M;
   p.x_div = x_per_slot ? 1 : (int)k;
   p.x = (const __half*)x;
   p.ldx = (int)t->d.k_in;
@@ -1541,6 +1543,7 @@ int32_t ats_layer_decode(ats_ctx* ctx, const ats_layer_desc* L, const void* x_in
   }
   MoeGemvParams s1{};
   s1.P = P;
+  s1.M = (int)M;
   s1.x_div = k;
   s1.x = w.h2_16;
   s1.ldx = H;
@@ -1550,6 +1553,7 @@ int32_t ats_layer_decode(ats_ctx* ctx, const ats_layer_desc* L, const void* x_in
   if (!(mskip & 64)) ATS_TRY(run_moe_stage(ctx, L->w_gate, L->w_up, w.ids, ids_host, s1, call_tab[0], call_tab[1]));
   MoeGemvParams s2{};
   s2.P = P;
+  s2.M = (int)M;
   s2.x_div = 1;
   s2.x = w.act16;
   s2.ldx = (int)L->ffn;

@@ -263,6 +263,58 @@ constexpr int kRingWarps = 8;
 // Four stages are in flight per warp, two with gate and up; a fifth takes from the L1 what the activations need (11.3 us for 10.2).
 constexpr int kRingStages = 4, kRingStagesSw = 2;
 
+// Asynchronous copies of step k's tile: codes of rows lane / 8 + 4 q (piece lane % 8), scales of row lane (lanes 0..15).
+__device__ __forceinline__ void ring_request(uint32_t dst, const uint8_t* const (&cp)[4], const uint8_t* sp, int k, int lane) {
+#pragma unroll
+  for (int q = 0; q < 4; ++q)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + (uint32_t)(((lane >> 3) + 4 * q) * kRingPitch + (lane & 7) * 16)),
+                 "l"(cp[q] + (size_t)k * 128)
+                 : "memory");
+  if (lane < 16)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + (uint32_t)(16 * kRingPitch + lane * 16)), "l"(sp + (size_t)k * 16) : "memory");
+}
+
+// A stage's 256 k of NT tiles: lane (g, t) holds rows g, g + 8 of column pair t and gives the activations xv of column g.
+template <bool MX, int NT>
+__device__ __forceinline__ void ring_step(const uint8_t* st, int g, int t, const uint4 (&xv)[8], float (&acc)[NT][4]) {
+  uint4 sc[NT][2];
+#pragma unroll
+  for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+    for (int h = 0; h < 2; ++h) sc[nt][h] = *reinterpret_cast<const uint4*>(st + nt * kRingTile + 16 * kRingPitch + (g + 8 * h) * 16);
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    uint4 x = xv[j];
+    if (MX)
+      x = make_uint4(__byte_perm(x.x, x.y, 0x5410u), __byte_perm(x.z, x.w, 0x5410u), __byte_perm(x.x, x.y, 0x7632u),
+                     __byte_perm(x.z, x.w, 0x7632u));
+#pragma unroll
+    for (int nt = 0; nt < NT; ++nt) {
+      const uint8_t* tile = st + nt * kRingTile + j * 16 + t * 4;
+      const uint32_t q0 = *reinterpret_cast<const uint32_t*>(tile + g * kRingPitch);
+      const uint32_t q1 = *reinterpret_cast<const uint32_t*>(tile + (g + 8) * kRingPitch);
+      uint32_t a0[4], a1[4];
+      if (MX) {
+        cvt_e2m1x8(q0, a0);
+        cvt_e2m1x8(q1, a1);
+      } else {
+        decode_word<false>(q0, a0);
+        decode_word<false>(q1, a1);
+      }
+      float c[4] = {0.f, 0.f, 0.f, 0.f};
+      const uint32_t f0[4] = {a0[0], a1[0], a0[1], a1[1]}, f1[4] = {a0[2], a1[2], a0[3], a1[3]};
+      mma16816(c, f0, x.x, x.y);
+      mma16816(c, f1, x.z, x.w);
+      const uint32_t w0[4] = {sc[nt][0].x, sc[nt][0].y, sc[nt][0].z, sc[nt][0].w}, w1[4] = {sc[nt][1].x, sc[nt][1].y, sc[nt][1].z, sc[nt][1].w};
+      const float s0 = scale_of(w0, j), s1 = scale_of(w1, j);
+      acc[nt][0] = fmaf(s0, c[0], acc[nt][0]);
+      acc[nt][1] = fmaf(s0, c[1], acc[nt][1]);
+      acc[nt][2] = fmaf(s1, c[2], acc[nt][2]);
+      acc[nt][3] = fmaf(s1, c[3], acc[nt][3]);
+    }
+  }
+}
+
 template <bool MX, bool SW>
 __global__ void __launch_bounds__(32 * kRingWarps, 2) gemv_mma_ring_kernel(const MmaGemvParams p) {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -315,17 +367,7 @@ __global__ void __launch_bounds__(32 * kRingWarps, 2) gemv_mma_ring_kernel(const
         }
       }
 #pragma unroll
-      for (int nt = 0; nt < NT; ++nt) {
-        const uint32_t dst = my_u + (uint32_t)((rs * NT + nt) * kRingTile);
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-          asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + (uint32_t)(((lane >> 3) + 4 * q) * kRingPitch + (lane & 7) * 16)),
-                       "l"(cp[nt][q] + (size_t)rk * 128)
-                       : "memory");
-        if (lane < 16)
-          asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + (uint32_t)(16 * kRingPitch + lane * 16)), "l"(sp[nt] + (size_t)rk * 16)
-                       : "memory");
-      }
+      for (int nt = 0; nt < NT; ++nt) ring_request(my_u + (uint32_t)((rs * NT + nt) * kRingTile), cp[nt], sp[nt], rk, lane);
       if (++rk == k_hi) rk = k_lo, ru += gridDim.x * upc;
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
@@ -353,42 +395,7 @@ __global__ void __launch_bounds__(32 * kRingWarps, 2) gemv_mma_ring_kernel(const
         request();
         const uint8_t* st = my + (size_t)cs * NT * kRingTile;
         if (++cs == S) cs = 0;
-        uint4 sc[NT][2];
-#pragma unroll
-        for (int nt = 0; nt < NT; ++nt)
-#pragma unroll
-          for (int h = 0; h < 2; ++h) sc[nt][h] = *reinterpret_cast<const uint4*>(st + nt * kRingTile + 16 * kRingPitch + (g + 8 * h) * 16);
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          uint4 x = xv[j];
-          if (MX)
-            x = make_uint4(__byte_perm(x.x, x.y, 0x5410u), __byte_perm(x.z, x.w, 0x5410u), __byte_perm(x.x, x.y, 0x7632u),
-                           __byte_perm(x.z, x.w, 0x7632u));
-#pragma unroll
-          for (int nt = 0; nt < NT; ++nt) {
-            const uint8_t* tile = st + nt * kRingTile + j * 16 + t * 4;
-            const uint32_t q0 = *reinterpret_cast<const uint32_t*>(tile + g * kRingPitch);
-            const uint32_t q1 = *reinterpret_cast<const uint32_t*>(tile + (g + 8) * kRingPitch);
-            uint32_t a0[4], a1[4];
-            if (MX) {
-              cvt_e2m1x8(q0, a0);
-              cvt_e2m1x8(q1, a1);
-            } else {
-              decode_word<false>(q0, a0);
-              decode_word<false>(q1, a1);
-            }
-            float c[4] = {0.f, 0.f, 0.f, 0.f};
-            const uint32_t f0[4] = {a0[0], a1[0], a0[1], a1[1]}, f1[4] = {a0[2], a1[2], a0[3], a1[3]};
-            mma16816(c, f0, x.x, x.y);
-            mma16816(c, f1, x.z, x.w);
-            const uint32_t w0[4] = {sc[nt][0].x, sc[nt][0].y, sc[nt][0].z, sc[nt][0].w}, w1[4] = {sc[nt][1].x, sc[nt][1].y, sc[nt][1].z, sc[nt][1].w};
-            const float s0 = scale_of(w0, j), s1 = scale_of(w1, j);
-            acc[nt][0] = fmaf(s0, c[0], acc[nt][0]);
-            acc[nt][1] = fmaf(s0, c[1], acc[nt][1]);
-            acc[nt][2] = fmaf(s1, c[2], acc[nt][2]);
-            acc[nt][3] = fmaf(s1, c[3], acc[nt][3]);
-          }
-        }
+        ring_step<MX, NT>(st, g, t, xv, acc);
       }
     }
 #pragma unroll
@@ -399,6 +406,178 @@ __global__ void __launch_bounds__(32 * kRingWarps, 2) gemv_mma_ring_kernel(const
     __syncthreads();
     write_units<SW, NT>(p, red_s[buf], u0, upc, ks, n_rows);
     buf ^= 1;  // (the next unit's sums go to the other half: one barrier a unit)
+  }
+  asm volatile("cp.async.wait_all;" ::: "memory");
+}
+
+// Routed experts for several tokens: the (token, slot) pairs grouped by expert, up to eight pairs of an expert as the columns, so
+// that an expert's weights are read and decoded once for them instead of once per pair.  Every CTA groups the pairs for itself from
+// the ids (at most 256: a pair's place is the number of earlier pairs of its expert; no sort, no launch of its own); a unit
+// is 16 rows (SwiGLU: 16 gate and 16 up rows) of a group, and the units of all groups form one line that the warps of a grid of two
+// CTAs per SM go through as above.  The K split depends on K alone and a column's sums on its own activations alone, so a
+// pair's result has the same bits whatever it is grouped with.  What bounds it: the activations (their
+// rows come through the L1 as often as the weights) and the grouping (its loop unrolled: 10 us less
+// for 256 pairs).  FFN half of a layer, 2048 x 768 experts, 8 per token, 32 tokens, streaming -> grouped: Q4 16 experts 130 -> 60 us,
+// 64 130 -> 85; MXFP4 16 191 -> 53, 64 192 -> 74, 128 193 -> 106.
+constexpr int kMoePairs = 256, kMoeCols = 8;
+// A part of K has at least two steps: with one the 32-token blocks above take 5 to 12 % longer, with four up to 2 %.
+constexpr int kMoeSplitSteps = 2;
+struct MoeMmaParams {
+  const uint8_t *base0, *base1;
+  uint64_t stride;
+  const int32_t* ids;  // null: pairs and weights from MoeJobs
+  const uint8_t *const *tab0, *const *tab1;
+  int x_div, P, n_experts;
+  int* status;
+  int n_rows, K, mode, ksplit;
+  const __half* x;
+  int ldx;
+  float* y32;
+  __half* y16;
+  int ldy;
+};
+
+template <bool MX, bool SW>
+__global__ void __launch_bounds__(32 * kRingWarps, 2) moe_mma_ring_kernel(const MoeMmaParams p, const __grid_constant__ MoeJobs jobs) {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  constexpr int NT = SW ? 2 : 1;
+  constexpr int S = SW ? kRingStagesSw : kRingStages;
+  extern __shared__ __align__(16) uint8_t ring[];
+  __shared__ float red_s[kRingWarps][NT][16][kMoeCols + 1];
+  __shared__ const uint8_t* w_s[NT][kMoePairs];        // a group's weights
+  __shared__ uint16_t row_s[kMoePairs][kMoeCols];      // its pairs (output rows); 0xFFFF: none
+  __shared__ unsigned long long key_s[kMoePairs];
+  __shared__ uint8_t group_s[kMoePairs];               // of a group's first pair: the group
+  __shared__ int warp_groups[kRingWarps];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int g = lane >> 2, t = lane & 3;
+  asm volatile("griddepcontrol.wait;" ::: "memory");  // ids, activations and gathered weights come from the kernels before
+  // ---- groups: thread q places pair q
+  int n_groups = 0;
+  {
+    const int q = threadIdx.x, n = p.ids ? p.P : jobs.n;
+    const uint8_t *w0 = nullptr, *w1 = nullptr;
+    unsigned long long key = ~0ull;
+    if (q < n) {
+      if (p.ids) {
+        size_t e = (size_t)(unsigned)p.ids[q];
+        if (e >= (size_t)p.n_experts) {  // an id that names no expert: expert 0 stands in and the status word says so
+          if (blockIdx.x == 0) raise_status(p.status, 7);
+          e = 0;
+        }
+        key = e;
+        w0 = p.tab0 ? p.tab0[e] : p.base0 + e * p.stride;
+        if (SW) w1 = p.tab1 ? p.tab1[e] : p.base1 + e * p.stride;
+      } else {
+        w0 = jobs.w0[q];
+        if (SW) w1 = jobs.w1[q];
+        key = (unsigned long long)w0;
+      }
+    }
+    key_s[q] = key;
+    *reinterpret_cast<uint4*>(row_s[q]) = make_uint4(~0u, ~0u, ~0u, ~0u);
+    __syncthreads();
+    int place = 0, first = q;  // earlier pairs of the expert; first pair of the group
+    if (32 * w < n) {
+#pragma unroll 16
+      for (int i = 0; i < 32 * w + 32; ++i) {
+        const bool same = key_s[i] == key && i < q;
+        if (same && place % kMoeCols == 0) first = i;
+        place += same;
+      }
+    }
+    const bool opens = q < n && place % kMoeCols == 0;
+    const unsigned open = __ballot_sync(0xFFFFFFFFu, opens);
+    if (lane == 0) warp_groups[w] = __popc(open);
+    __syncthreads();
+    int gi = __popc(open & ((1u << lane) - 1));
+#pragma unroll
+    for (int i = 0; i < kRingWarps; ++i) {
+      if (i < w) gi += warp_groups[i];
+      n_groups += warp_groups[i];
+    }
+    if (opens) {
+      first = q;
+      group_s[q] = (uint8_t)gi;
+      w_s[0][gi] = w0;
+      if (SW) w_s[NT - 1][gi] = w1;
+    }
+    __syncthreads();
+    if (q < n) row_s[group_s[first]][place % kMoeCols] = (uint16_t)(p.ids ? q : jobs.orow[q]);
+    __syncthreads();
+  }
+  const int K = p.K, nblk = K / 32, n_step = K / 256, n_rows = p.n_rows;
+  const int per_group = (n_rows + 15) / 16, n_units = n_groups * per_group;
+  const int ks = p.ksplit, upc = kRingWarps / ks, part = w % ks, slot = w / ks;
+  const int per = (n_step + ks - 1) / ks, k_lo = min(part * per, n_step), k_hi = min(k_lo + per, n_step);
+  uint8_t* my = ring + (size_t)w * S * NT * kRingTile;
+  const uint32_t my_u = (uint32_t)__cvta_generic_to_shared(my);
+  int ru = blockIdx.x * upc + slot, rk = k_lo, rs = 0;
+  const uint8_t *cp[NT][4], *sp[NT];
+  auto request = [&] {
+    if (ru < n_units && k_lo < k_hi) {
+      if (rk == k_lo) {
+        const int gr = ru / per_group, r0 = 16 * (ru - gr * per_group);
+#pragma unroll
+        for (int nt = 0; nt < NT; ++nt) {  // rows beyond the last: the last (their sums are not written)
+          const uint8_t* base = w_s[nt][gr];
+#pragma unroll
+          for (int q = 0; q < 4; ++q) cp[nt][q] = base + (size_t)min(r0 + (lane >> 3) + 4 * q, n_rows - 1) * (K / 2) + (lane & 7) * 16;
+          sp[nt] = base + (size_t)n_rows * (K / 2) + (size_t)min(r0 + (lane & 15), n_rows - 1) * nblk * 2;
+        }
+      }
+#pragma unroll
+      for (int nt = 0; nt < NT; ++nt) ring_request(my_u + (uint32_t)((rs * NT + nt) * kRingTile), cp[nt], sp[nt], rk, lane);
+      if (++rk == k_hi) rk = k_lo, ru += gridDim.x * upc;
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    if (++rs == S) rs = 0;
+  };
+#pragma unroll
+  for (int i = 0; i < S - 1; ++i) request();
+  int cs = 0;
+  for (int u0 = blockIdx.x * upc; u0 < n_units; u0 += gridDim.x * upc) {
+    float acc[NT][4];
+#pragma unroll
+    for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) acc[nt][i] = 0.f;
+    if (u0 + slot < n_units) {
+      const int row = row_s[(u0 + slot) / per_group][g];
+      const bool xlive = row != 0xFFFF;
+      const __half* xrow = p.x + (size_t)(xlive ? row / p.x_div : 0) * p.ldx + 8 * t;
+      for (int k = k_lo; k < k_hi; ++k) {
+        uint4 xv[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) xv[j] = xlive ? __ldg(reinterpret_cast<const uint4*>(xrow + k * 256 + j * 32)) : make_uint4(0, 0, 0, 0);
+        asm volatile("cp.async.wait_group %0;" ::"n"(S - 2) : "memory");
+        __syncwarp();  // the stage is there for every lane, and the last one has been read by all: its place is free
+        request();
+        ring_step<MX, NT>(my + (size_t)cs * NT * kRingTile, g, t, xv, acc);
+        if (++cs == S) cs = 0;
+      }
+    }
+#pragma unroll
+    for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) red_s[w][nt][g + 8 * (i >> 1)][2 * t + (i & 1)] = acc[nt][i];
+    __syncthreads();
+    for (int e = threadIdx.x; e < upc * 16 * kMoeCols; e += blockDim.x) {
+      const int row = e % 16, m = e / 16 % kMoeCols, sl = e / (16 * kMoeCols), u = u0 + sl;
+      if (u >= n_units) break;
+      const int gr = u / per_group, r = 16 * (u - gr * per_group) + row, o = row_s[gr][m];
+      if (o == 0xFFFF || r >= n_rows) continue;
+      float s0 = 0.f, s1 = 0.f;
+      for (int q = 0; q < ks; ++q) {
+        s0 += red_s[sl * ks + q][0][row][m];
+        if (SW) s1 += red_s[sl * ks + q][NT - 1][row][m];
+      }
+      const size_t at = (size_t)o * p.ldy + r;
+      if (SW) p.y16[at] = __float2half_rn(s0 / (1.0f + expf(-s0)) * s1);
+      else if (p.mode == GEMV_OUT_F32) p.y32[at] = s0;
+      else p.y16[at] = __float2half_rn(s0);
+    }
+    __syncthreads();
   }
   asm volatile("cp.async.wait_all;" ::: "memory");
 }
@@ -465,6 +644,50 @@ cudaError_t launch_gemv_mma(const GemvParams& g, cudaStream_t st, uint64_t* n_la
   }
   return sw ? launch_dep(gemv_mma_kernel<false, true>, grid, block, 0, st, g.pdl, 1, p)
             : launch_dep(gemv_mma_kernel<false, false>, grid, block, 0, st, g.pdl, 1, p);
+}
+
+// The streaming kernel takes a pair at the rate of its weights, whoever else reads them, and is the faster one while the pairs share
+// few experts.  Pairs per expert, streaming against grouped, us for the FFN half of a layer of 2048 x 768 experts: Q4 2: 43 / 49
+// (32 experts), 70 / 70 (64), 132 / 123 (128), 4: 42.6 / 37.0 (16), 73 / 53 (32), 130 / 85 (64); MXFP4 0.5: 23 / 23.5 (16), 1:
+// 38 / 37 (32), 59 / 53 (64), 104 / 81 (128), 2: 38 / 30 (16).  A function of the call's shapes, not of where experts are.
+bool moe_gemv_mma_eligible(const MoeGemvParams& g) {
+  return g.M > 1 && g.P >= (g.mx ? 1 : 3) * g.n_experts && g.P <= kMoePairs && g.K % 256 == 0 && !(g.ldx & 7) && !(reinterpret_cast<uintptr_t>(g.x) & 15) &&
+         (g.mode == GEMV_SWIGLU_F16 || g.mode == GEMV_OUT_F32 || g.mode == GEMV_OUT_F16);
+}
+
+cudaError_t launch_moe_gemv_mma(const MoeGemvParams& g, const MoeJobs* jobs, int sm_count, int pdl, cudaStream_t st, uint64_t* n_launch) {
+  const int pairs = jobs ? jobs->n : g.P;
+  if (pairs <= 0) return cudaSuccess;
+  if (!moe_gemv_mma_eligible(g)) return cudaErrorInvalidValue;
+  const bool sw = g.mode == GEMV_SWIGLU_F16;
+  MoeMmaParams p{};
+  p.base0 = g.base0; p.base1 = g.base1; p.stride = g.stride; p.ids = jobs ? nullptr : g.ids;
+  p.tab0 = g.tab0; p.tab1 = g.tab1; p.x_div = g.x_div; p.P = g.P; p.n_experts = g.n_experts; p.status = g.status;
+  p.n_rows = g.n_rows; p.K = g.K; p.mode = g.mode; p.x = g.x; p.ldx = g.ldx;
+  p.y32 = g.y32; p.y16 = g.y16; p.ldy = g.ldy;
+  int ks = 1;
+  while (ks < kRingWarps && g.K / 256 >= 2 * kMoeSplitSteps * ks) ks *= 2;
+  p.ksplit = ks;
+  MoeJobs none;
+  none.n = 0;
+  const size_t smem = (size_t)kRingWarps * (sw ? 2 * kRingStagesSw : kRingStages) * kRingTile;
+  const long ctas = ((long)pairs * ((g.n_rows + 15) / 16) * ks + kRingWarps - 1) / kRingWarps;
+  static uint64_t attr_done = 0;
+  if (first_use_on_device(&attr_done)) {
+    const int most = kRingWarps * std::max(kRingStages, 2 * kRingStagesSw) * kRingTile;
+    const void* kernels[4] = {reinterpret_cast<const void*>(moe_mma_ring_kernel<false, false>), reinterpret_cast<const void*>(moe_mma_ring_kernel<true, false>),
+                              reinterpret_cast<const void*>(moe_mma_ring_kernel<false, true>), reinterpret_cast<const void*>(moe_mma_ring_kernel<true, true>)};
+    for (const void* k : kernels) {
+      const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+      if (e != cudaSuccess) return e;
+    }
+  }
+  ++*n_launch;
+  auto run = [&](auto* k) {
+    return launch_dep(k, dim3((unsigned)std::min<long>(ctas, 2L * sm_count)), dim3(32 * kRingWarps), smem, st, pdl, 1, p, jobs ? *jobs : none);
+  };
+  if (g.mx) return sw ? run(moe_mma_ring_kernel<true, true>) : run(moe_mma_ring_kernel<true, false>);
+  return sw ? run(moe_mma_ring_kernel<false, true>) : run(moe_mma_ring_kernel<false, false>);
 }
 
 }  // namespace ats

@@ -925,6 +925,33 @@ def test_route_and_moe_linear_standalone(B, torch):
     ctx.close()
 
 
+@pytest.mark.parametrize("fmt,n,k_in,E,M,k,per_slot", [
+    ("q4", 16, 256, 1, 3, 1, 0),       # the smallest: one group of three pairs, one unit of one step
+    ("q4", 33, 256, 3, 9, 1, 1),       # a last unit of one row; groups of more and fewer than eight
+    ("mx", 100, 768, 5, 7, 3, 0),      # steps that do not divide
+    ("mx", 48, 2048, 1, 32, 8, 1),     # 256 pairs of one expert: 32 full groups
+    ("mx", 80, 2048, 200, 32, 8, 0),   # many groups of one or two
+    ("q4", 24, 1280, 4, 17, 2, 1),     # five steps in two parts
+])
+def test_moe_linear_groups_pairs_by_expert(B, torch, fmt, n, k_in, E, M, k, per_slot):
+    """Several tokens: pairs of one expert are the columns of one product, whatever their order."""
+    rng = np.random.default_rng(n + k_in + M)
+    packed, scales = (W.mxfp4_packed if fmt == "mx" else W.q4_packed)(96, 0, 0, n, k_in, E)
+    packed, scales = packed.reshape(E, n, -1), scales.reshape(E, n, -1)
+    ids = rng.integers(0, E, (M, k)).astype(np.int32)
+    x = W.activations(96, M, (M, k, k_in) if per_slot else (M, k_in))
+    ctx = make_ctx(B, packed.nbytes + 2 * (k_in // 32) * n * E + 512 * E + MB)
+    tid = ctx.register_q4(packed, scales)
+    ctx.set_placement([(tid, -1, B.ATS_GPU)])
+    y = torch.empty((M, k, n), dtype=torch.float16, device="cuda")
+    ctx.moe_linear(tid, H.to_dev(x), H.to_dev(ids), y, M, k, per_slot)
+    ctx.sync()
+    want = O.moe_linear(x, ids, packed, scales, x_per_slot=bool(per_slot))
+    # one fp16 rounding (4.9e-4) and fp32 sums of at most 2048 products (far below it): the file's gate
+    H.assert_close(y.cpu().numpy().reshape(M * k, n), want.reshape(M * k, n))
+    ctx.close()
+
+
 # ------------------------------------------------------------------------------------------------- errors (host-made)
 def test_errors_are_statuses_and_context_stays_usable(B, torch):
     ctx = make_ctx(B, 4 * MB, ring_slots=1, slot_bytes=1024)
