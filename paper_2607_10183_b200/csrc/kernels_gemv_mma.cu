@@ -321,7 +321,7 @@ __global__ void __launch_bounds__(32 * kRingWarps, 2) gemv_mma_ring_kernel(const
   constexpr int NT = SW ? 2 : 1;     // weight tiles per unit
   constexpr int S = SW ? kRingStagesSw : kRingStages;
   extern __shared__ __align__(16) uint8_t ring[];
-  __shared__ float red_s[2][kRingWarps][NT][16][8];
+  __shared__ __align__(16) float red_s[2][kRingWarps][NT][16][8];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int g = lane >> 2, t = lane & 3;
   const int K = p.K, nblk = K / 32, M = p.M, n_step = K / 256;
@@ -445,7 +445,7 @@ __global__ void __launch_bounds__(32 * kRingWarps, 2) moe_mma_ring_kernel(const 
   extern __shared__ __align__(16) uint8_t ring[];
   __shared__ float red_s[kRingWarps][NT][16][kMoeCols + 1];
   __shared__ const uint8_t* w_s[NT][kMoePairs];        // a group's weights
-  __shared__ uint16_t row_s[kMoePairs][kMoeCols];      // its pairs (output rows); 0xFFFF: none
+  __shared__ __align__(16) uint16_t row_s[kMoePairs][kMoeCols];  // its pairs (output rows); 0xFFFF: none
   __shared__ unsigned long long key_s[kMoePairs];
   __shared__ uint8_t group_s[kMoePairs];               // of a group's first pair: the group
   __shared__ int warp_groups[kRingWarps];
