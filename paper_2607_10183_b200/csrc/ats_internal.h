@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+#include <initializer_list>
 #include <string>
 #include <vector>
 
@@ -185,14 +187,27 @@ cudaError_t launch_gemv_stream(const GemvParams& p, int* status, int sm_count, c
 // Grouped-expert GEMV: job j multiplies the slice w0[j] (and w1[j] for SwiGLU) with activation row xrow[j] and
 // writes output row j_out[j].  Implicit mode (n_jobs_explicit == 0): job p = 0..P-1 uses expert ids[p] of a
 // contiguous resident tensor.
-// Function attributes (the dynamic shared-memory limit) are per device: a launcher sets them the first time it runs on
-// each device.  `done` holds one bit per device ordinal; setting an attribute twice is harmless, so no lock is needed.
-inline bool first_use_on_device(uint64_t* done) {
+// Function attributes (the dynamic shared-memory limit) are per device and belong to the kernel, whoever launches it: a launcher
+// sets them to the largest value that any of its shapes asks for, the first time that it runs on each device.  `done` holds one
+// bit per device ordinal; it is set after the attributes are, so a thread that sees it may launch (two threads may both set them,
+// to the same values).
+template <typename Set>
+inline cudaError_t once_per_device(std::atomic<uint64_t>* done, Set set) {
   int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return true;
-  if ((*done >> dev) & 1ull) return false;
-  *done |= 1ull << dev;
-  return true;
+  const bool known = cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 64;
+  if (known && ((done->load(std::memory_order_acquire) >> dev) & 1ull)) return cudaSuccess;
+  const cudaError_t e = set();
+  if (e == cudaSuccess && known) done->fetch_or(1ull << dev, std::memory_order_release);
+  return e;
+}
+// ... where the shared-memory limit is all there is to set.
+inline cudaError_t smem_limit_once(std::atomic<uint64_t>* done, std::initializer_list<const void*> kernels, size_t bytes) {
+  return once_per_device(done, [&] {
+    cudaError_t e = cudaSuccess;
+    for (const void* k : kernels)
+      if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    return e;
+  });
 }
 
 // Launch with the programmatic-dependent-launch attribute: the kernel may start while its predecessor in the stream is

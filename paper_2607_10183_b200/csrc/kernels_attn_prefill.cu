@@ -318,11 +318,9 @@ template <int D>
 cudaError_t launch_tc(const CUtensorMap& qm, const CUtensorMap& km, const CUtensorMap& vm, const AttnTcParams& p, int grid, cudaStream_t st,
                       int pdl) {
   constexpr size_t smem = (size_t)(2 * kQRows + kRing * kKeys) * D * 2 + 1024;
-  static uint64_t attr_done = 0;
-  if (first_use_on_device(&attr_done)) {
-    cudaError_t e = cudaFuncSetAttribute(attn_prefill_tc_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
+  static std::atomic<uint64_t> attr_done;
+  const cudaError_t e = smem_limit_once(&attr_done, {reinterpret_cast<const void*>(attn_prefill_tc_kernel<D>)}, smem);
+  if (e != cudaSuccess) return e;
   return launch_dep(attn_prefill_tc_kernel<D>, dim3(grid), dim3(kAttnThreads), smem, st, pdl, 1, qm, km, vm, p);
 }
 

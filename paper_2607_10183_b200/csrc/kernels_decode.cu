@@ -802,16 +802,18 @@ cudaError_t launch_attn_decode_fused(AttnDecodeParams p, int d, int pdl, cudaStr
   cfg.gridDim = dim3(splits, p.n_kv * hsplit);
   cfg.blockDim = dim3(p.group / hsplit * pc);
   cfg.dynamicSmemBytes = (size_t)pc * (d * 4 + 16);
-  static uint64_t attr_done = 0;
-  if (first_use_on_device(&attr_done)) {
-    cudaError_t e[4] = {
+  static std::atomic<uint64_t> attr_done;
+  const cudaError_t e = once_per_device(&attr_done, [] {
+    const cudaError_t e[4] = {
         cudaFuncSetAttribute(attn_decode_fused_kernel<128, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * (128 * 4 + 16)),
         cudaFuncSetAttribute(attn_decode_fused_kernel<128, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, 128 * (128 * 4 + 16)),
         cudaFuncSetAttribute(attn_decode_fused_kernel<64, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * (64 * 4 + 16)),
         cudaFuncSetAttribute(attn_decode_fused_kernel<64, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, 128 * (64 * 4 + 16))};
     for (cudaError_t x : e)
       if (x != cudaSuccess) return x;
-  }
+    return cudaSuccess;
+  });
+  if (e != cudaSuccess) return e;
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -1269,17 +1271,18 @@ cudaError_t launch_router_topk_norm(const __half* h, const __half* wr, int M, in
     // (chains of a multiple of eight rows: 2048 / E of them in each range)
     if (M >= kRouterManyTokens && !norm_gain && E == Epad && 2048 % E == 0 && H / kRouterCluster % (kRouterStageRows * R) == 0 && smem_tok(3) <= kMost) {
       const int stages = smem_tok(4) <= kMost ? 4 : 3;
-      const cudaError_t e = cudaFuncSetAttribute(router_topk_tokens_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_tok(stages));
+      static std::atomic<uint64_t> attr_done;
+      const cudaError_t e = smem_limit_once(&attr_done, {reinterpret_cast<const void*>(router_topk_tokens_kernel)}, kMost);
       if (e != cudaSuccess) return e;
       ++*n_launch;
       return launch_dep(router_topk_tokens_kernel, dim3((M + kRouterTok - 1) / kRouterTok), dim3(kRouterTokThreads), smem_tok(stages), st, pdl, 1,
                         h, wr, M, H, E, Epad, k, renorm, stages, ids, gates);
     }
-    if (smem_cl <= 160 * 1024) {
-      if (smem_cl > 48 * 1024) {  // (cheap; set on every call because the size depends on the shape)
-        cudaError_t e = cudaFuncSetAttribute(router_topk_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_cl);
-        if (e != cudaSuccess) return e;
-      }
+    constexpr size_t kMostCl = 160 * 1024;
+    if (smem_cl <= kMostCl) {
+      static std::atomic<uint64_t> attr_done;
+      const cudaError_t e = smem_limit_once(&attr_done, {reinterpret_cast<const void*>(router_topk_cluster_kernel)}, kMostCl);
+      if (e != cudaSuccess) return e;
       ++*n_launch;
       return launch_dep(router_topk_cluster_kernel, dim3(kRouterCluster, M), dim3(kRouterClThreads), smem_cl, st, pdl, kRouterCluster,
                         h, wr, H, E, Epad, k, renorm, ids, gates, norm_x, norm_x_f32, norm_gain, eps, const_cast<__half*>(h));
@@ -1291,7 +1294,8 @@ cudaError_t launch_router_topk_norm(const __half* h, const __half* wr, int M, in
   }
   const size_t smem = ((size_t)H + kRouterThreads + Epad) * sizeof(float);
   if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(router_topk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    static std::atomic<uint64_t> attr_done;
+    const cudaError_t e = smem_limit_once(&attr_done, {reinterpret_cast<const void*>(router_topk_kernel)}, 227 * 1024);
     if (e != cudaSuccess) return e;
   }
   ++*n_launch;

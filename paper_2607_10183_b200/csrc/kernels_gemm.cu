@@ -691,20 +691,13 @@ cudaError_t launch_gemm(const GemmParams& g, cudaStream_t st, uint64_t* n_launch
   p.grp_off = g.grp_off;
   p.grp_stride = g.grp_stride;
   for (int i = 0; i < 3; ++i) p.grp_tab[i] = g.grp_tab[i];
-  static uint64_t attr_done = 0;
-  if (first_use_on_device(&attr_done)) {
-    cudaError_t e1 = cudaFuncSetAttribute(gemm_q4_kernel<2, 256, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    cudaError_t e2 = cudaFuncSetAttribute(gemm_q4_kernel<1, 128, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    cudaError_t e3 = cudaFuncSetAttribute(gemm_q4_kernel<2, 256, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    cudaError_t e4 = cudaFuncSetAttribute(gemm_q4_kernel<1, 128, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    if (e1 != cudaSuccess) return e1;
-    if (e2 != cudaSuccess) return e2;
-    if (e3 != cudaSuccess) return e3;
-    if (e4 != cudaSuccess) return e4;
-  }
+  static std::atomic<uint64_t> attr_done;
+  cudaError_t e = smem_limit_once(&attr_done, {reinterpret_cast<const void*>(gemm_q4_kernel<2, 256, false>), reinterpret_cast<const void*>(gemm_q4_kernel<1, 128, false>),
+                                               reinterpret_cast<const void*>(gemm_q4_kernel<2, 256, true>), reinterpret_cast<const void*>(gemm_q4_kernel<1, 128, true>)},
+                                  200 * 1024);
+  if (e != cudaSuccess) return e;
   dim3 grid(tiles, tchunks, g.grp_off ? g.n_groups : p.splits);
   ++*n_launch;
-  cudaError_t e;
   if (wide) {
     using Cfg = TileCfg<2, 256>;
     p.stages = Cfg::kStages;

@@ -1082,14 +1082,10 @@ cudaError_t launch_gemm_pair(const GemmParams& g, int sm_count, cudaStream_t st,
     while (p.codes + p.stages <= kMaxCodes && fixed + p.xs * xs + (p.codes + p.stages) * cs <= kMost) p.codes += p.stages;
     smem = fixed + p.xs * xs + p.codes * cs;
   }
-  static uint64_t attr_done = 0;
-  if (first_use_on_device(&attr_done)) {
-    for (const void* k : {reinterpret_cast<const void*>(gemm_pair_kernel<kFmtQ4>), reinterpret_cast<const void*>(gemm_pair_kernel<kFmtMx>),
-                          reinterpret_cast<const void*>(gemm_pair_kernel<kFmtW16>)}) {
-      const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMost);
-      if (e != cudaSuccess) return e;
-    }
-  }
+  static std::atomic<uint64_t> attr_done;
+  const cudaError_t e = smem_limit_once(&attr_done, {reinterpret_cast<const void*>(gemm_pair_kernel<kFmtQ4>), reinterpret_cast<const void*>(gemm_pair_kernel<kFmtMx>),
+                                                     reinterpret_cast<const void*>(gemm_pair_kernel<kFmtW16>)}, kMost);
+  if (e != cudaSuccess) return e;
   ++*n_launch;
   auto run = [&](auto* kernel) { return launch_dep(kernel, dim3(2 * p.pairs), dim3(kPairThreads), smem, st, g.pdl, 2, xmap, maps, p); };
   return g.w16 ? run(gemm_pair_kernel<kFmtW16>) : g.mx ? run(gemm_pair_kernel<kFmtMx>) : run(gemm_pair_kernel<kFmtQ4>);

@@ -615,16 +615,11 @@ cudaError_t launch_gemv_mma(const GemvParams& g, cudaStream_t st, uint64_t* n_la
     p.ksplit = ks;
     const int ctas = (n_units + kRingWarps / ks - 1) / (kRingWarps / ks);
     const size_t smem = (size_t)kRingWarps * (sw ? 2 * kRingStagesSw : kRingStages) * kRingTile;
-    static uint64_t attr_done = 0;
-    if (first_use_on_device(&attr_done)) {
-      const int most = kRingWarps * std::max(kRingStages, 2 * kRingStagesSw) * kRingTile;
-      const void* kernels[4] = {reinterpret_cast<const void*>(gemv_mma_ring_kernel<false, false>), reinterpret_cast<const void*>(gemv_mma_ring_kernel<true, false>),
-                                reinterpret_cast<const void*>(gemv_mma_ring_kernel<false, true>), reinterpret_cast<const void*>(gemv_mma_ring_kernel<true, true>)};
-      for (const void* k : kernels) {
-        const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-        if (e != cudaSuccess) return e;
-      }
-    }
+    static std::atomic<uint64_t> attr_done;
+    const cudaError_t e = smem_limit_once(&attr_done, {reinterpret_cast<const void*>(gemv_mma_ring_kernel<false, false>), reinterpret_cast<const void*>(gemv_mma_ring_kernel<true, false>),
+                                                       reinterpret_cast<const void*>(gemv_mma_ring_kernel<false, true>), reinterpret_cast<const void*>(gemv_mma_ring_kernel<true, true>)},
+                                          kRingWarps * std::max(kRingStages, 2 * kRingStagesSw) * kRingTile);
+    if (e != cudaSuccess) return e;
     ++*n_launch;
     auto run = [&](auto* k) { return launch_dep(k, dim3(std::min(ctas, 2 * 148)), dim3(32 * kRingWarps), smem, st, g.pdl, 1, p); };
     if (g.mx) return sw ? run(gemv_mma_ring_kernel<true, true>) : run(gemv_mma_ring_kernel<true, false>);
@@ -672,16 +667,11 @@ cudaError_t launch_moe_gemv_mma(const MoeGemvParams& g, const MoeJobs* jobs, int
   none.n = 0;
   const size_t smem = (size_t)kRingWarps * (sw ? 2 * kRingStagesSw : kRingStages) * kRingTile;
   const long ctas = ((long)pairs * ((g.n_rows + 15) / 16) * ks + kRingWarps - 1) / kRingWarps;
-  static uint64_t attr_done = 0;
-  if (first_use_on_device(&attr_done)) {
-    const int most = kRingWarps * std::max(kRingStages, 2 * kRingStagesSw) * kRingTile;
-    const void* kernels[4] = {reinterpret_cast<const void*>(moe_mma_ring_kernel<false, false>), reinterpret_cast<const void*>(moe_mma_ring_kernel<true, false>),
-                              reinterpret_cast<const void*>(moe_mma_ring_kernel<false, true>), reinterpret_cast<const void*>(moe_mma_ring_kernel<true, true>)};
-    for (const void* k : kernels) {
-      const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-      if (e != cudaSuccess) return e;
-    }
-  }
+  static std::atomic<uint64_t> attr_done;
+  const cudaError_t e = smem_limit_once(&attr_done, {reinterpret_cast<const void*>(moe_mma_ring_kernel<false, false>), reinterpret_cast<const void*>(moe_mma_ring_kernel<true, false>),
+                                                     reinterpret_cast<const void*>(moe_mma_ring_kernel<false, true>), reinterpret_cast<const void*>(moe_mma_ring_kernel<true, true>)},
+                                        kRingWarps * std::max(kRingStages, 2 * kRingStagesSw) * kRingTile);
+  if (e != cudaSuccess) return e;
   ++*n_launch;
   auto run = [&](auto* k) {
     return launch_dep(k, dim3((unsigned)std::min<long>(ctas, 2L * sm_count)), dim3(32 * kRingWarps), smem, st, pdl, 1, p, jobs ? *jobs : none);

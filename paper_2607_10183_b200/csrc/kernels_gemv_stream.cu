@@ -116,12 +116,10 @@ cudaError_t launch_gemv_stream(const GemvParams& g, int* status, int sm_count, c
       default: kern = sw ? gemv_stream_kernel<8, true, false> : gemv_stream_kernel<8, false, false>; break;
     }
   }
-  static uint64_t attr_done[20] = {};
+  static std::atomic<uint64_t> attr_done[20];
   const int ki = ((shrt ? 4 : parts == 1 ? 0 : parts == 2 ? 1 : parts == 4 ? 2 : 3) * 2 + (sw ? 1 : 0)) * 2 + (g.mx ? 1 : 0);
-  if (first_use_on_device(&attr_done[ki])) {
-    cudaError_t e = set_stream_kernel_attributes(reinterpret_cast<const void*>(kern));
-    if (e != cudaSuccess) return e;
-  }
+  const cudaError_t attr_e = once_per_device(&attr_done[ki], [&] { return set_stream_kernel_attributes(reinterpret_cast<const void*>(kern)); });
+  if (attr_e != cudaSuccess) return attr_e;
   if (smem > kMaxDynSmem || p.n_stages < producers) return cudaErrorInvalidValue;
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(grid);
@@ -200,12 +198,10 @@ cudaError_t launch_moe_gemv_stream(const MoeGemvParams& g, const MoeJobs* jobs, 
       default: kern = sw ? gemv_stream_moe_kernel<8, true, false> : gemv_stream_moe_kernel<8, false, false>; break;
     }
   }
-  static uint64_t attr_done[20] = {};
+  static std::atomic<uint64_t> attr_done[20];
   const int ki = ((shrt ? 4 : parts == 1 ? 0 : parts == 2 ? 1 : parts == 4 ? 2 : 3) * 2 + (sw ? 1 : 0)) * 2 + (g.mx ? 1 : 0);
-  if (first_use_on_device(&attr_done[ki])) {
-    cudaError_t e = set_stream_kernel_attributes(reinterpret_cast<const void*>(kern));
-    if (e != cudaSuccess) return e;
-  }
+  const cudaError_t attr_e = once_per_device(&attr_done[ki], [&] { return set_stream_kernel_attributes(reinterpret_cast<const void*>(kern)); });
+  if (attr_e != cudaSuccess) return attr_e;
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(per_job, n_jobs);
   cfg.blockDim = dim3(shrt ? kThreadsShort : kThreads);
@@ -261,11 +257,9 @@ __global__ void __launch_bounds__(kProbeWarps * 32) hbm_read_probe_kernel(const 
 
 cudaError_t launch_hbm_read_probe(const uint8_t* src, uint64_t bytes, int* status, int sm_count, cudaStream_t st) {
   const size_t smem = (size_t)kProbeWarps * kProbeDepth * kProbeChunk;
-  static uint64_t attr_done = 0;
-  if (first_use_on_device(&attr_done)) {
-    cudaError_t e = cudaFuncSetAttribute(hbm_read_probe_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
+  static std::atomic<uint64_t> attr_done;
+  const cudaError_t e = smem_limit_once(&attr_done, {reinterpret_cast<const void*>(hbm_read_probe_kernel)}, smem);
+  if (e != cudaSuccess) return e;
   hbm_read_probe_kernel<<<sm_count, kProbeWarps * 32, smem, st>>>(src, bytes / kProbeChunk, status);
   return cudaGetLastError();
 }

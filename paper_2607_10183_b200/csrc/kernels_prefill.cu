@@ -275,15 +275,10 @@ cudaError_t launch_attn_prefill(const __half* q_rot16, const __half* kc, const _
   dim3 grid((T + kFaQ - 1) / kFaQ, n_q);
   const float scale = 1.0f / sqrtf((float)d);
   const size_t smem = (size_t)(kFaQ + 4 * kFaK) * (d + 8) * sizeof(__half);
-  static uint64_t attr_done = 0;
-  if (first_use_on_device(&attr_done)) {
-    cudaError_t e1 = cudaFuncSetAttribute(attn_prefill_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)((kFaQ + 4 * kFaK) * (128 + 8) * sizeof(__half)));
-    cudaError_t e2 = cudaFuncSetAttribute(attn_prefill_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)((kFaQ + 4 * kFaK) * (64 + 8) * sizeof(__half)));
-    if (e1 != cudaSuccess) return e1;
-    if (e2 != cudaSuccess) return e2;
-  }
+  static std::atomic<uint64_t> attr_done;
+  const cudaError_t e = smem_limit_once(&attr_done, {reinterpret_cast<const void*>(attn_prefill_kernel<128>), reinterpret_cast<const void*>(attn_prefill_kernel<64>)},
+                                        (kFaQ + 4 * kFaK) * (128 + 8) * sizeof(__half));
+  if (e != cudaSuccess) return e;
   ++*n_launch;
   if (d == 128)
     return launch_dep(attn_prefill_kernel<128>, grid, dim3(128), smem, st, pdl, 1, q_rot16, kc, vc, a16, T, n_q, n_q / n_kv, cap, pos0,
@@ -444,11 +439,9 @@ __global__ void __launch_bounds__(32, 1) host_gather_kernel(const CopyChunk* __r
 
 cudaError_t launch_host_gather(const CopyChunk* list, int n, int* status, int sm_count, cudaStream_t st, uint64_t* n_launch, int pdl) {
   if (n <= 0) return cudaSuccess;
-  static uint64_t attr_done = 0;
-  if (first_use_on_device(&attr_done)) {
-    cudaError_t e = cudaFuncSetAttribute(host_gather_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kCopyStages * kCopyChunk);
-    if (e != cudaSuccess) return e;
-  }
+  static std::atomic<uint64_t> attr_done;
+  const cudaError_t e = smem_limit_once(&attr_done, {reinterpret_cast<const void*>(host_gather_kernel)}, kCopyStages * kCopyChunk);
+  if (e != cudaSuccess) return e;
   ++*n_launch;
   return launch_dep(host_gather_kernel, dim3(std::min(n, sm_count)), dim3(32), (size_t)kCopyStages * kCopyChunk, st, pdl, 1, list, n, status);
 }

@@ -1160,3 +1160,40 @@ def test_bounded_wait_expiry_is_reported_and_leaves_other_contexts_usable(B, tor
     ctx2.sync()
     H.assert_close(y2.cpu().numpy(), want, what="gemv on a fresh context after the expiry")
     ctx2.close()
+
+
+@pytest.mark.parametrize("M,E,sizes", [(128, 128, (1024, 3072)), (3, 1024, (10240, 16384))])
+def test_two_threads_route_with_layers_of_different_sizes(B, torch, M, E, sizes):
+    """A kernel's shared-memory limit belongs to the device, not to a call: a thread whose router asks for little must not lower it
+    under the launch of a thread whose router asks for much.  Two contexts of their own streams, many calls of each."""
+    import threading
+    made, failed = [], []
+    for Hd in sizes:
+        ctx = make_ctx(B, Hd * E * 2 + MB)
+        rng = np.random.default_rng(Hd)
+        rid = ctx.register_f16((rng.standard_normal((Hd, E)) * 0.02).astype(np.float16))
+        ctx.set_placement([])
+        h = H.to_dev(rng.standard_normal((M, Hd)).astype(np.float16))
+        outs = [torch.empty((M, 4), dtype=torch.int32, device="cuda"), torch.empty((M, 4), dtype=torch.float32, device="cuda")]
+        made.append((ctx, rid, h, outs))
+    torch.cuda.synchronize()
+
+    def calls(ctx, rid, h, outs):
+        try:
+            for _ in range(3000):
+                ctx.route_topk(rid, h, M, 4, *outs)
+            ctx.sync()
+        except B.AtsError as e:
+            failed.append(e)
+    threads = [threading.Thread(target=calls, args=m) for m in made]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not failed, failed[0]
+    for ctx, rid, h, outs in made:
+        ids = outs[0].clone()
+        ctx.route_topk(rid, h, M, 4, *outs)
+        ctx.sync()
+        assert torch.equal(ids, outs[0])
+        ctx.close()
