@@ -331,7 +331,7 @@ static int32_t launch_gemm_any(ats_ctx* ctx, GemmParams p) {
   __half* act = p.act;
   p.counters = reinterpret_cast<int*>(ctx->ws) + 64;  // (the attention's: zero between launches, and launches follow one another)
   const bool pairs = !(ctx->cfg.flags & ATS_FLAG_NO_GEMM_PAIR);
-  if (pairs && gemm_pair_eligible(p)) {
+  if (pairs && gemm_pair_eligible(p, ctx->sm_count)) {
     e = launch_gemm_pair(p, ctx->sm_count, ctx->cs, &ctx->stats.kernel_launches, &err);
     act = nullptr;
   } else {
@@ -353,7 +353,7 @@ static int32_t run_gemm_group(ats_ctx* ctx, Operand* ops, int n, GemmParams p) {
     probe.counters = reinterpret_cast<int*>(ctx->ws) + 64;
     probe.n_seg = n;
     for (int i = 0; i < n; ++i) probe.seg[i] = GemvSeg{nullptr, (int)ops[i].t->d.n_out};
-    together = !(ctx->cfg.flags & ATS_FLAG_NO_GEMM_PAIR) && gemm_pair_eligible(probe);
+    together = !(ctx->cfg.flags & ATS_FLAG_NO_GEMM_PAIR) && gemm_pair_eligible(probe, ctx->sm_count);
   }
   if (together) {
     ATS_TRY(acquire_ops(ctx, ops, n));
@@ -467,7 +467,13 @@ static LayerWs layout_prefill(const ats_layer_desc& L, uint32_t T, uint8_t* base
   b.take(kWsReserved);
   const uint64_t H = L.hidden, qd = (uint64_t)L.n_q_heads * L.head_dim, kvd = (uint64_t)L.n_kv_heads * L.head_dim;
   uint64_t scratch = 0;
-  auto gemm_want = [&](int n, int k) { return std::max(gemm_scratch_bytes((int)T, n, k), gemm_pair_scratch_bytes((int)T, n, k)); };
+  auto gemm_want = [&](std::initializer_list<uint64_t> rows, uint64_t k, bool act) {
+    int n[3] = {0, 0, 0}, n_seg = 0, total = 0;
+    for (uint64_t r : rows) total += n[n_seg++] = (int)r;
+    uint64_t want = gemm_scratch_bytes((int)T, total, (int)k);
+    for (bool w16 : {false, true}) want = std::max(want, gemm_pair_scratch_bytes(n, n_seg, act, (int)T, (int)k, w16));
+    scratch = std::max(scratch, want);
+  };
   if (L.wq >= 0) {
     w.h16 = (__half*)b.take(T * H * 2);
     w.qkv16 = (__half*)b.take(T * (qd + 2 * kvd) * 2);
@@ -475,8 +481,8 @@ static LayerWs layout_prefill(const ats_layer_desc& L, uint32_t T, uint8_t* base
     w.a16 = (__half*)b.take(T * qd * 2);
     w.o16 = (__half*)b.take(T * H * 2);
     w.x1_16 = (__half*)b.take(T * H * 2);
-    scratch = std::max(scratch, gemm_want((int)(qd + 2 * kvd), (int)H));
-    scratch = std::max(scratch, gemm_want((int)H, (int)qd));
+    gemm_want({qd, kvd, kvd}, H, false);
+    gemm_want({H}, qd, false);
   }
   w.h2_16 = (__half*)b.take(T * H * 2);
   if (L.n_experts) {
@@ -495,8 +501,8 @@ static LayerWs layout_prefill(const ats_layer_desc& L, uint32_t T, uint8_t* base
     w.gu16 = (__half*)b.take((uint64_t)T * 2 * L.ffn * 2);
     w.act16 = (__half*)b.take((uint64_t)T * L.ffn * 2);
     w.d16 = (__half*)b.take(T * H * 2);
-    scratch = std::max(scratch, gemm_want((int)(2 * L.ffn), (int)H));
-    scratch = std::max(scratch, gemm_want((int)H, (int)L.ffn));
+    gemm_want({L.ffn, L.ffn}, H, true);
+    gemm_want({H}, L.ffn, false);
   }
   w.gemm_scratch = b.take(scratch);
   w.gemm_scratch_bytes = scratch;

@@ -615,6 +615,13 @@ uint64_t gemm_scratch_bytes(int T, int n_total, int K) {
   return pl.splits > 1 ? (uint64_t)pl.splits * T * n_total * 4 + 256 : 256;
 }
 
+int gemm_chain(const int* rows, int n_seg, int T, int K) {
+  int n_total = 0;
+  for (int i = 0; i < n_seg; ++i) n_total += rows[i];
+  const int total_ksteps = (K + BK - 1) / BK, splits = choose_plan(rows, n_seg, T, n_total, total_ksteps, 148, ~0ull).splits;
+  return (total_ksteps + splits - 1) / splits * BK;
+}
+
 cudaError_t launch_gemm(const GemmParams& g, cudaStream_t st, uint64_t* n_launch, std::string* err) {
   EncodeTiledFn enc = encode_tiled_fn();
   if (!enc) {

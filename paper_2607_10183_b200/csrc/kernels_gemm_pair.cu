@@ -896,25 +896,33 @@ __global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid
 
 // ------------------------------------------------------------------------------------------------- host side
 // Units that one accumulator adds up at most.  The tensor core truncates each sum, and what a chain drops grows with its
-// length: of the fp16 results 0.5 % differ from the exact sum's rounding after 1024 k, 1.7 % after 4096, 2.7 % after 7168.  A
-// prompt of 512 through a layer of 4096 features has 5.1e-4 of its outputs more than 2e-3 off with q, k, v in chains of 2048 k at
-// most (the softmax multiplies their errors), 9.8e-4 with 4096.  Wide matrices (gate and up) make no difference up to 4096, where a part
-// costs the most: 104 us against 118 in parts of 2048.  From 1024 tokens on a chain is the stretch.
-int units_at_once(int n_ft, int T, int K) { return T >= 1024 ? (K + kUnitK - 1) / kUnitK : (n_ft > 32 ? 4096 : 1536) / kUnitK; }
+// length: of the fp16 results 0.5 % differ from the exact sum's rounding after 1024 k, 1.7 % after 4096, 5 % after 14336.  So no
+// chain is longer than the single-CTA kernel's for the same product (fp16: for each matrix by itself, as that kernel takes them), except
+// that 1536 k are always allowed.
+int units_at_once(const int* rows, int n_seg, int T, int K, bool w16) {
+  int chain = K;
+  for (int i = 0; w16 && i < n_seg; ++i) chain = std::min(chain, gemm_chain(rows + i, 1, T, K));
+  if (!w16) chain = gemm_chain(rows, n_seg, T, K);
+  return (std::max(1536, chain) + kUnitK - 1) / kUnitK;
+}
+// Feature tiles of a segment (fused SwiGLU: a tile is 128 gate and 128 up rows, all counted with the gate).
+int feature_tiles(const int* rows, int seg, bool act) {
+  return act ? (seg ? 0 : (rows[0] + kFeat - 1) / kFeat) : (rows[seg] + 2 * kFeat - 1) / (2 * kFeat);
+}
 
 struct PairPlan {
-  int nt, n_tt, pairs, n_whole, split_pairs, slots2, own;
+  int nt, n_tt, pairs, n_whole, split_pairs, slots2, own, max_units;
   uint64_t scratch;
 };
 // Cost in SM cycles of the ways to divide the work (see the kernel's comment).  A unit costs its MMAs, the expansion of its weights
 // or their way from memory, whichever is longest; a tile its epilogue; a split tile the parts' way through L2; a stretch that is
-// added up in several parts theirs, unless the MMAs go on meanwhile in the other accumulator.
-PairPlan pair_plan(const int* ft_of_seg, int n_seg, int T, int K, bool w16, int max_pairs, uint64_t scratch_bytes) {
+// added up in several parts theirs, unless the MMAs go on meanwhile in the other accumulator.  pairs = 0: the scratch holds none.
+PairPlan pair_plan(const int* rows, int n_seg, bool act, int T, int K, bool w16, int max_pairs, uint64_t scratch_bytes) {
   PairPlan best{};
   double best_cost = 1e300;
   int n_ft = 0;
-  for (int i = 0; i < n_seg; ++i) n_ft += ft_of_seg[i];
-  const int units = (K + kUnitK - 1) / kUnitK, max_units = units_at_once(n_ft, T, K);
+  for (int i = 0; i < n_seg; ++i) n_ft += feature_tiles(rows, i, act);
+  const int units = (K + kUnitK - 1) / kUnitK, max_units = units_at_once(rows, n_seg, T, K, w16);
   int last = 0;
   for (int most : {256, 192, 128}) {
     const int n_tt = (T + most - 1) / most;
@@ -931,11 +939,11 @@ PairPlan pair_plan(const int* ft_of_seg, int n_seg, int T, int K, bool w16, int 
       const bool parts = std::max(len, waves || !slots ? (double)units : 0.0) > max_units;
       const int pairs = waves ? max_pairs : slots ? n : rem;
       const uint64_t need = ((uint64_t)n * slots + (parts ? pairs : 0)) * slot;
-      if (need > scratch_bytes && (slots || nt > 128)) return;  // (whole tiles of one token tile do without, in one part)
+      if (need > scratch_bytes) return;
       cost += waves * (stretch(units) + tile);
       if (cost >= best_cost) return;
       best_cost = cost;
-      best = PairPlan{nt, n_tt, pairs, slots ? tiles - rem : tiles, n, slots == 2, parts && need <= scratch_bytes, need > scratch_bytes ? 0 : need};
+      best = PairPlan{nt, n_tt, pairs, slots ? tiles - rem : tiles, n, slots == 2, parts, max_units, need};
     };
     take(rem ? stretch(units) + tile : 0.0, units, 0, 0);
     auto red = [&](double con) { return 5000.0 + (con - 1) * nt * 32.0; };
@@ -950,14 +958,19 @@ PairPlan pair_plan(const int* ft_of_seg, int n_seg, int T, int K, bool w16, int 
 
 int pairs_of_device(int sm_count) { return std::min(sm_count / 2, kAttnMaxCounters / 2); }
 
-}  // namespace
-
-uint64_t gemm_pair_scratch_bytes(int T, int n_total, int K) {
-  const int ft = (n_total + 2 * kFeat - 1) / (2 * kFeat);
-  return std::max(pair_plan(&ft, 1, T, K, false, 74, ~0ull).scratch, pair_plan(&ft, 1, T, K, true, 74, ~0ull).scratch) + 256;
+PairPlan plan_of(const GemmParams& g, int sm_count) {
+  int rows[3] = {0, 0, 0};
+  for (int i = 0; i < g.n_seg; ++i) rows[i] = g.seg[i].n_rows;
+  return pair_plan(rows, g.n_seg, g.act != nullptr, g.T, g.K, g.w16, pairs_of_device(sm_count), g.scratch ? g.scratch_bytes : 0);
 }
 
-bool gemm_pair_eligible(const GemmParams& g) {
+}  // namespace
+
+uint64_t gemm_pair_scratch_bytes(const int* rows, int n_seg, bool act, int T, int K, bool w16) {
+  return pair_plan(rows, n_seg, act, T, K, w16, 74, ~0ull).scratch;
+}
+
+bool gemm_pair_eligible(const GemmParams& g, int sm_count) {
   if ((g.w16 && g.grp_off) || g.n_seg < 1 || g.n_seg > 3 || !g.counters || g.K % (g.w16 ? 8 : 32) || g.ldx % 8) return false;
   if (reinterpret_cast<uintptr_t>(g.x) & 15) return false;
   if ((g.res != nullptr) != (g.y2 != nullptr)) return false;
@@ -968,8 +981,8 @@ bool gemm_pair_eligible(const GemmParams& g) {
   if (g.act && (g.n_seg != 2 || g.seg[0].n_rows != g.seg[1].n_rows || g.seg[0].n_rows % 8 || g.ldact % 8 || g.ldy % 8 || g.res ||
                 ((reinterpret_cast<uintptr_t>(g.act) | reinterpret_cast<uintptr_t>(g.y)) & 15)))
     return false;
-  if (g.grp_off && ((g.n_seg != 1 && !g.act) || g.grp_stride % 16 || g.res)) return false;
-  return true;
+  if (g.grp_off) return (g.n_seg == 1 || g.act) && g.grp_stride % 16 == 0 && !g.res;
+  return plan_of(g, sm_count).pairs > 0;
 }
 
 cudaError_t launch_gemm_pair(const GemmParams& g, int sm_count, cudaStream_t st, uint64_t* n_launch, std::string* err) {
@@ -980,12 +993,11 @@ cudaError_t launch_gemm_pair(const GemmParams& g, int sm_count, cudaStream_t st,
   }
   PairParams p{};
   p.n_seg = g.n_seg;
-  int ft_of_seg[3] = {0, 0, 0}, n_ft = 0, col = 0;
+  int rows[3] = {0, 0, 0}, n_ft = 0, col = 0;
   for (int i = 0; i < g.n_seg; ++i) {
-    const int ft = g.act ? (i ? 0 : (g.seg[0].n_rows + kFeat - 1) / kFeat) : (g.seg[i].n_rows + 2 * kFeat - 1) / (2 * kFeat);
-    p.seg[i] = PairSeg{g.seg[i].base, g.seg[i].n_rows, n_ft, col};
-    ft_of_seg[i] = ft;
-    n_ft += ft;
+    rows[i] = g.seg[i].n_rows;
+    p.seg[i] = PairSeg{g.seg[i].base, rows[i], n_ft, col};
+    n_ft += feature_tiles(rows, i, g.act != nullptr);
     col += g.seg[i].n_rows;
   }
   p.K = g.K;
@@ -993,7 +1005,7 @@ cudaError_t launch_gemm_pair(const GemmParams& g, int sm_count, cudaStream_t st,
   p.units = (g.K + kUnitK - 1) / kUnitK;
   p.ksteps = (g.K + 63) / 64;
   const int max_pairs = pairs_of_device(sm_count);
-  bool own = false;
+  p.max_units = p.units;
   if (g.grp_off) {
     if (g.n_groups <= 0 || g.grp_max_rows <= 0) return cudaErrorInvalidValue;
     p.n_tt = (g.grp_max_rows + 255) / 256;
@@ -1003,7 +1015,8 @@ cudaError_t launch_gemm_pair(const GemmParams& g, int sm_count, cudaStream_t st,
     p.pairs = (int)std::min<long long>((long long)p.n_ft * p.n_tt, max_pairs);
     p.n_whole = p.n_ft * p.n_tt;
   } else {
-    const PairPlan pl = pair_plan(ft_of_seg, g.n_seg, g.T, g.K, g.w16, max_pairs, g.scratch ? g.scratch_bytes : 0);
+    const PairPlan pl = plan_of(g, sm_count);
+    if (!pl.pairs) return cudaErrorInvalidValue;
     p.nt = pl.nt;
     p.n_tt = pl.n_tt;
     p.n_ft = n_ft;
@@ -1011,7 +1024,7 @@ cudaError_t launch_gemm_pair(const GemmParams& g, int sm_count, cudaStream_t st,
     p.n_whole = pl.n_whole;
     p.split_pairs = pl.split_pairs;
     p.slots2 = pl.slots2;
-    own = pl.own;
+    if (pl.own) p.max_units = pl.max_units;
   }
   p.sc16 = !g.w16 && g.K % 256 == 0;
   p.y = g.y;
@@ -1023,7 +1036,6 @@ cudaError_t launch_gemm_pair(const GemmParams& g, int sm_count, cudaStream_t st,
   p.partial = (float*)g.scratch;
   p.slot_tok = std::min(p.nt, g.T);
   p.own = p.partial + (size_t)(p.split_pairs * (p.slots2 ? 2 : 1)) * 2 * kFeat * p.slot_tok;
-  p.max_units = own ? units_at_once(n_ft, g.T, g.K) : p.units;
   p.counters = g.counters;
   p.status = g.status;
   p.grp_off = g.grp_off;
