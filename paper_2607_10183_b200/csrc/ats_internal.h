@@ -386,9 +386,10 @@ struct GemmParams {
 bool gemm_pair_eligible(const GemmParams& p, int sm_count);
 uint64_t gemm_pair_scratch_bytes(const int* rows, int n_seg, bool act, int T, int K, bool w16);
 cudaError_t launch_gemm_pair(const GemmParams& p, int sm_count, cudaStream_t st, uint64_t* n_launch, std::string* err);
-// the single-CTA kernel: scratch of its plan, and the k that the plan adds up in one accumulator
+// the single-CTA kernel: scratch of its plan, the k that the plan adds up in one accumulator, its time
 uint64_t gemm_scratch_bytes(int T, int n_total, int K);
 int gemm_chain(const int* rows, int n_seg, int T, int K);
+double gemm_us(const int* rows, int n_seg, int T, int K, bool w16);
 cudaError_t launch_gemm(const GemmParams& p, cudaStream_t st, uint64_t* n_launch, std::string* err);
 // fixed split-K scratch inside the library's device image (no allocation): capacity, and its address on the current device
 uint64_t gemm_static_scratch_capacity();

@@ -622,6 +622,23 @@ int gemm_chain(const int* rows, int n_seg, int T, int K) {
   return (total_ksteps + splits - 1) / splits * BK;
 }
 
+// Time in us of the plan with all the scratch it wants, for the choice between this kernel and the pairs of CTAs: waves of k-steps, and
+// the partial sums and their launch.  Fitted like the pairs' (6 % rms off for the 4-bit formats, 8 % for fp16).
+double gemm_us(const int* rows, int n_seg, int T, int K, bool w16) {
+  int n = 0;
+  for (int i = 0; i < n_seg; ++i) n += rows[i];
+  const int total_ksteps = (K + BK - 1) / BK;
+  const GemmPlan pl = choose_plan(rows, n_seg, T, n, total_ksteps, 148, ~0ull);
+  const int tt = pl.wide ? 256 : 128, per = (total_ksteps + pl.splits - 1) / pl.splits;
+  int tiles = 0;
+  for (int i = 0; i < n_seg; ++i) tiles += (rows[i] + pl.bf - 1) / pl.bf;
+  const int waves = (tiles * ((T + tt - 1) / tt) * pl.splits + 147) / 148;
+  const double kstep = (w16 ? 0.270 + 0.0021 * (pl.wide ? pl.bf : 224) : 0.503 + 0.00143 * (pl.wide ? pl.bf : 208));
+  double us = waves * (per * kstep + (w16 ? 4.0 : 3.6));
+  if (pl.splits > 1) us += (w16 ? 3.8 : 2.6) + (w16 ? 0.22 : 0.227) * (pl.splits + 1) * 4e-6 * T * n;
+  return w16 ? std::max(us, std::max(1.9e-9 * T, 0.4e-6) * n * K) : us;  // (at most 1050 TFLOP/s and 5 TB/s)
+}
+
 cudaError_t launch_gemm(const GemmParams& g, cudaStream_t st, uint64_t* n_launch, std::string* err) {
   EncodeTiledFn enc = encode_tiled_fn();
   if (!enc) {

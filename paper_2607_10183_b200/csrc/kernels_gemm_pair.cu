@@ -898,10 +898,11 @@ __global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid
 // Units that one accumulator adds up at most.  The tensor core truncates each sum, and what a chain drops grows with its
 // length: of the fp16 results 0.5 % differ from the exact sum's rounding after 1024 k, 1.7 % after 4096, 5 % after 14336.  So no
 // chain is longer than the single-CTA kernel's for the same product (fp16: for each matrix by itself, as that kernel takes them), except
-// that 1536 k are always allowed.
+// that 1536 k are always allowed, and fp16 matrices of enough large tiles (112 CTAs of 256 features x 256 tokens) are added up in one.
 int units_at_once(const int* rows, int n_seg, int T, int K, bool w16) {
   int chain = K;
-  for (int i = 0; w16 && i < n_seg; ++i) chain = std::min(chain, gemm_chain(rows + i, 1, T, K));
+  for (int i = 0; w16 && i < n_seg; ++i)
+    if (T < 384 || (rows[i] + 255) / 256 * ((T + 511) / 512) < 56) chain = std::min(chain, gemm_chain(rows + i, 1, T, K));
   if (!w16) chain = gemm_chain(rows, n_seg, T, K);
   return (std::max(1536, chain) + kUnitK - 1) / kUnitK;
 }
@@ -912,17 +913,23 @@ int feature_tiles(const int* rows, int seg, bool act) {
 
 struct PairPlan {
   int nt, n_tt, pairs, n_whole, split_pairs, slots2, own, max_units;
+  double us;
   uint64_t scratch;
 };
-// Cost in SM cycles of the ways to divide the work (see the kernel's comment).  A unit costs its MMAs, the expansion of its weights
-// or their way from memory, whichever is longest; a tile its epilogue; a split tile the parts' way through L2; a stretch that is
-// added up in several parts theirs, unless the MMAs go on meanwhile in the other accumulator.  pairs = 0: the scratch holds none.
+// Time in us of the ways to divide the work (see the kernel's comment).  A unit costs its MMAs, the expansion of its weights
+// or their way from memory, whichever is longest; a tile its epilogue; a stretch that is added up in several parts their way out and
+// back, less where the MMAs go on meanwhile in the other accumulator; a split tile the parts' way through L2, which the last to arrive
+// waits for in batches of tokens (shorter ones where there are several others).  The figures are fitted to about 800 launches, 16 shapes
+// of 1 to 160 MB, 9 to 2048 tokens, back to back on new weights: 7 % rms off for the 4-bit formats, 10 % for fp16.  pairs = 0: the
+// scratch holds none.
 PairPlan pair_plan(const int* rows, int n_seg, bool act, int T, int K, bool w16, int max_pairs, uint64_t scratch_bytes) {
   PairPlan best{};
-  double best_cost = 1e300;
+  best.us = 1e300;
   int n_ft = 0;
   for (int i = 0; i < n_seg; ++i) n_ft += feature_tiles(rows, i, act);
   const int units = (K + kUnitK - 1) / kUnitK, max_units = units_at_once(rows, n_seg, T, K, w16);
+  double weights_mb = 0;
+  for (int i = 0; i < n_seg; ++i) weights_mb += 2e-6 * rows[i] * K;
   int last = 0;
   for (int most : {256, 192, 128}) {
     const int n_tt = (T + most - 1) / most;
@@ -930,28 +937,29 @@ PairPlan pair_plan(const int* rows, int n_seg, bool act, int T, int K, bool w16,
     last = n_tt;
     const int nt = ((T + n_tt - 1) / n_tt + 31) / 32 * 32;
     const uint64_t slot = 2ull * kFeat * std::min(nt, T) * 4;
-    const double unit = std::max(w16 ? 1400.0 : 825.0 + 1.25 * nt, 6.65 * nt), tile = w16 ? 500.0 : 12.0 * nt;
-    const double flush = w16 || nt <= 128 ? 1500.0 : 100.0 * (nt - 110);
-    auto stretch = [&](double len) { return len * unit + (std::ceil(len / max_units) - 1) * flush; };
+    const double unit = w16 ? std::max(0.729, 0.186 + 0.0027 * nt) : std::max(0.391, 0.174 + 0.0020 * nt);
+    const double launch = w16 ? 5.0 : 4.2, tile = w16 ? 0.0 : 0.012 * nt, flush = w16 ? 1.1 : nt <= 128 ? 2.6 : 4.6;
+    const int tok = std::min(nt, T), batches = tok <= 16 ? 1 : (tok + 63) / 64 * 2;  // (16 tokens a batch and warp, two warps side by side)
+    auto stretch = [&](double len) { return len * unit + (std::ceil(len / max_units) - 1) * flush + tile; };
+    auto sum = [&](double con) { return (w16 ? 1.0 : 1.3) + batches * (w16 ? (con > 2 ? 2.7 : 1.6) : (con > 2 ? 2.5 : 1.3)); };
     // whole tiles in waves of one per pair; the rest, `rem`, whole in a wave of its own or divided over n pairs, `len` units each
     const int tiles = n_ft * n_tt, waves = tiles / max_pairs, rem = tiles % max_pairs;
-    auto take = [&](double cost, double len, int n, int slots) {
+    auto take = [&](double us, double len, int n, int slots) {
       const bool parts = std::max(len, waves || !slots ? (double)units : 0.0) > max_units;
       const int pairs = waves ? max_pairs : slots ? n : rem;
       const uint64_t need = ((uint64_t)n * slots + (parts ? pairs : 0)) * slot;
       if (need > scratch_bytes) return;
-      cost += waves * (stretch(units) + tile);
-      if (cost >= best_cost) return;
-      best_cost = cost;
-      best = PairPlan{nt, n_tt, pairs, slots ? tiles - rem : tiles, n, slots == 2, parts, max_units, need};
+      us += launch + waves * stretch(units);
+      if (w16) us = std::max(us, weights_mb / 4.5);
+      if (us >= best.us) return;
+      best = PairPlan{nt, n_tt, pairs, slots ? tiles - rem : tiles, n, slots == 2, parts, max_units, us, need};
     };
-    take(rem ? stretch(units) + tile : 0.0, units, 0, 0);
-    auto red = [&](double con) { return 5000.0 + (con - 1) * nt * 32.0; };
+    take(rem ? stretch(units) : 0.0, units, 0, 0);
     for (int s = 2; s <= kMaxParts && s <= units && rem && rem * s <= max_pairs; ++s)
-      if (units % s == 0 || units > 4 * s) take(stretch((units + s - 1) / s) + red(s), (units + s - 1) / s, rem * s, 1);
+      if (units % s == 0 || units > 4 * s) take(stretch((units + s - 1) / s) + sum(s), (units + s - 1) / s, rem * s, 1);
     const double per = (double)rem * units / max_pairs;
     if (per >= 1 && units <= per * (kMaxParts - 2))  // (a tile meets at most units / per + 2 ranges)
-      take(stretch(std::ceil(per)) + tile + 4000.0 + red(std::ceil(units / per) + 1), std::ceil(per), max_pairs, 2);
+      take(stretch(std::ceil(per)) + sum(std::ceil(units / per) + 1) + 3.1, std::ceil(per), max_pairs, 2);
   }
   return best;
 }
@@ -982,7 +990,22 @@ bool gemm_pair_eligible(const GemmParams& g, int sm_count) {
                 ((reinterpret_cast<uintptr_t>(g.act) | reinterpret_cast<uintptr_t>(g.y)) & 15)))
     return false;
   if (g.grp_off) return (g.n_seg == 1 || g.act) && g.grp_stride % 16 == 0 && !g.res;
-  return plan_of(g, sm_count).pairs > 0;
+  // The pairs win where there are tiles for all of them; a tile that has to be split waits for its parts, and the single-CTA kernel, with
+  // smaller tiles and the sum as a launch of its own, is the faster one (4096 x 4096: 128 tokens 22.1 us against 19.5, 512 tokens 23.8
+  // against 27.5; 1024 x 8192, 100 tokens: 26.4 against 17.8; fp16 4096 x 14336: 256 tokens 65 against 42).  It takes fp16 matrices one by
+  // one, SwiGLU is a launch of its own beside it, and rows of y that are not 16-byte aligned it stores by the element (3333 x 9984, 300
+  // tokens: 53 against 85).
+  const PairPlan pl = plan_of(g, sm_count);
+  if (g.ldy % 8 || (reinterpret_cast<uintptr_t>(g.y) & 15)) return pl.pairs > 0;
+  double single = 0;
+  for (int i = 0; g.w16 && i < g.n_seg; ++i) single += gemm_us(&g.seg[i].n_rows, 1, g.T, g.K, true);
+  if (!g.w16) {
+    int rows[3] = {0, 0, 0};
+    for (int i = 0; i < g.n_seg; ++i) rows[i] = g.seg[i].n_rows;
+    single = gemm_us(rows, g.n_seg, g.T, g.K, false);
+  }
+  if (g.act) single += 2.0 + 6e-6 / 4 * g.T * g.seg[0].n_rows;
+  return pl.pairs > 0 && pl.us <= single;
 }
 
 cudaError_t launch_gemm_pair(const GemmParams& g, int sm_count, cudaStream_t st, uint64_t* n_launch, std::string* err) {

@@ -119,3 +119,30 @@ def test_gemm_with_the_least_workspace_keeps_the_chains_short():
     differ = (y != (x.double() @ w.t()).half()).double().mean().item()
     print(f"q4 {N}x{K} T={T}, workspace {ws}: {differ:.3%}")
     assert ws > 1024 and differ <= 0.0065 * limit / 1000
+
+
+# Which kernel takes a product: the pairs where they are the faster ones, else the single-CTA kernel (few tiles: it splits K and adds the
+# parts up in a launch of its own), whose results those are then bit for bit.
+@pytest.mark.parametrize("fmt,N,K,T,pairs", [("w16", 4096, 4096, 256, False), ("w16", 1024, 8192, 1000, False), ("w16", 640, 5120, 128, False),
+                                             ("q4", 1024, 8192, 100, False), ("q4", 640, 5120, 128, False), ("mxfp4", 640, 5120, 512, False),
+                                             ("q4", 6144, 2048, 33, True), ("w16", 8192, 2048, 128, True), ("q4", 333, 4096, 100, True)])
+def test_few_tiles_go_to_the_single_cta_kernel(fmt, N, K, T, pairs):
+    import torch
+    from paper_2607_10183_b200 import binding as B
+    x = H.to_dev(W.activations(95, 0, (T, K)))
+    weights = (W.w16_matrix(95, 0, W.ROLE_UP, N, K),) if fmt == "w16" else (W.q4_packed if fmt == "q4" else W.mxfp4_packed)(95, 0, W.ROLE_UP, N, K)
+    ws = 64 * T * N + 2 * MB
+    outs, launches = [], []
+    for flags in (0, B.ATS_FLAG_NO_GEMM_PAIR):
+        ctx = B.Context(ws + 2 * N * K + 2 * MB, workspace_bytes=ws, flags=flags)
+        tid = (ctx.register_w16 if fmt == "w16" else ctx.register_q4)(*weights)
+        ctx.set_placement([(tid, -1, B.ATS_GPU)])
+        y = torch.empty((T, N), dtype=torch.float16, device="cuda")
+        ctx.linear(tid, x, y, T)
+        ctx.sync()
+        launches.append(ctx.stats().kernel_launches)
+        outs.append(y.cpu().numpy().view(np.uint16))
+        ctx.close()
+    assert launches[0] == (1 if pairs else launches[1])
+    if not pairs:
+        assert np.array_equal(outs[0], outs[1])
