@@ -161,16 +161,20 @@ int32_t ats_get_placement(const ats_ctx* ctx, int32_t id, int32_t expert, uint8_
 
 /* The per-tensor operator: y[m][n] = sum_k w[n][k] x[m][k], fp32 accumulation, fp16 output.
  * x DEVICE fp16 row-major [M][k_in]; y DEVICE fp16 row-major [M][n_out].  M <= 8 runs the memory-bound GEMV with exact
- * weights (scale * code in fp32): one or two rows on the streaming kernel (integer dot products on the CUDA cores), three
- * to eight rows on mma.sync tensor-core instructions, odd shapes on a generic kernel; M > 8 runs the tensor-core GEMM
- * (weights rounded once to fp16 operands).
- * Activations inside the single-row streaming kernel (also used by ats_layer_decode, ats_lm_head and the single-token MoE
- * stages): every block of 32 fp16 activations is re-expressed as 16-bit block fixed point, xi = rn(x * 2^sh) with
+ * weights (scale * code in fp32): one row of a 4-bit format on the streaming kernel (integer codes: integer dot products on the CUDA
+ * cores; microscaling floats: mma.sync tensor-core instructions), two (k_in a multiple of 256) or three to eight rows on mma.sync,
+ * other shapes on generic kernels; M > 8 runs a tensor-core GEMM (weights rounded once to fp16 operands).
+ * M > 8 needs the workspace bytes that the text of ATS_ERR_NOMEM names (partial sums of one of the two GEMM kernels).  The result is a
+ * function of the shapes and the operands, except that some products have a faster plan that takes more than that (at most 60 MB): it
+ * runs wherever the workspace holds it.  Both results are within the tolerance of the operator.
+ * Activations inside the single-row streaming kernel for integer codes (also used by ats_layer_decode, ats_lm_head and the single-token
+ * MoE stages): every block of 32 fp16 activations is re-expressed as 16-bit block fixed point, xi = rn(x * 2^sh) with
  * |xi| <= 32752, i.e. each element is rounded within 2^-17 of its block's largest magnitude (fp16 itself resolves that
  * maximum to 2^-11); block dot products are then exact integers and blocks are summed in fp32.  The perturbation of an
  * output is bounded by 2^-17 * sum over blocks of (block maximum * sum of |w| in the block), about 1e-5 of its scale for
  * the workloads here.  A block that holds an Inf or a NaN activation contributes NaN (as the plain definition would give
- * Inf or NaN), so a non-finite input never turns into a finite output.
+ * Inf or NaN), so a non-finite input never turns into a finite output.  All other kernels take the fp16 activations as they are
+ * (an Inf gives what the plain definition gives: Inf or NaN).
  * If the tensor is placed on the host it is streamed through the ring for this call. */
 int32_t ats_linear(ats_ctx* ctx, int32_t id, const void* x /*DEVICE*/, void* y /*DEVICE*/, uint32_t M);
 
@@ -196,16 +200,17 @@ int32_t ats_set_tensor_value(ats_ctx* ctx, int32_t id, int64_t value, int64_t sw
  * has given all device memory to another allocator.  ats_linear needs scratch for its split-K partial sums when
  * M > 8 and takes it from the workspace the caller allocated; this entry point takes it instead from a fixed array of
  * ATS_STATIC_SCRATCH_BYTES that is part of the library's device image, so that it calls no cudaMalloc / cudaFree /
- * allocating routine of any library.  Same arguments as ats_linear and the same kernels, so the same result (bit for bit
- * whenever both pick the same split-K plan, which holds unless the 8 MiB here admit a plan ats_linear's workspace did
- * not: k_in >= 8192 with M >= 1024; within the tolerance of the operator otherwise), with these differences:
+ * allocating routine of any library.  Same arguments as ats_linear, the same kernels and the same choice of a plan from the
+ * bytes at hand, so the result of an ats_linear whose context has workspace_bytes = 1024 + ATS_STATIC_SCRATCH_BYTES, bit for
+ * bit (M <= 8: of any).  Another workspace gives the same bits as long as the product's faster plan, if it has one, fits both or
+ * neither, and a result within the tolerance of the operator otherwise.  The differences:
  *  - dense ATS_FMT_Q4B32 and ATS_FMT_MXFP4 tensors only (ATS_FMT_W16: ATS_ERR_INVALID);
  *  - the context still needs the first kilobyte of a workspace (workspace_bytes >= 1024, set at ats_init): that is
  *    where the attention counters and, on systems without mapped pinned memory, the status word live.  Nothing else of
  *    the workspace is touched;
  *  - the tensor must be GPU-placed (streaming would need the ring) -> ATS_ERR_STATE otherwise;
- *  - if the split-K plan ats_linear would pick with unlimited workspace needs more than ATS_STATIC_SCRATCH_BYTES for its
- *    partial sums, the call fails with ATS_ERR_NOMEM and the text says how much was needed (no smaller plan is tried);
+ *  - where ats_linear asks for more workspace than ATS_STATIC_SCRATCH_BYTES (partial sums of the single-CTA kernel's plan), the
+ *    call fails with ATS_ERR_NOMEM and the text says how much was needed;
  *  - every GPU that loads the library holds the array from load to exit; all calls (all contexts, all streams of a
  *    process) share it, and nothing in it has to start at zero: each call fully writes the partials it later reads.
  *    Two calls that overlap on the GPU (different streams) would overwrite each other's partials: keep them on one stream;

@@ -682,7 +682,10 @@ cudaError_t launch_gemm(const GemmParams& g, cudaStream_t st, uint64_t* n_launch
   int seg_rows[3] = {0, 0, 0};
   for (int i = 0; i < g.n_seg; ++i) seg_rows[i] = g.seg[i].n_rows;
   const int total_ksteps = (g.K + BK - 1) / BK;
-  GemmPlan pl = choose_plan(seg_rows, g.n_seg, g.T, g.ldy, total_ksteps, sm_count, g.scratch ? g.scratch_bytes : 0);
+  // one matrix: the plan is a function of the shapes (with more scratch than it asks for, one in 600 shapes would get another one)
+  uint64_t scratch_bytes = g.scratch ? g.scratch_bytes : 0;
+  if (g.n_seg == 1) scratch_bytes = std::min(scratch_bytes, gemm_scratch_bytes(g.T, n_total, g.K));
+  GemmPlan pl = choose_plan(seg_rows, g.n_seg, g.T, g.ldy, total_ksteps, sm_count, scratch_bytes);
   if (g.grp_off) {
     // per-expert row counts are small next to the tile: 128-token tiles unless an expert holds several of them
     if (g.res || g.n_groups <= 0 || g.grp_max_rows <= 0) return cudaErrorInvalidValue;

@@ -966,10 +966,15 @@ PairPlan pair_plan(const int* rows, int n_seg, bool act, int T, int K, bool w16,
 
 int pairs_of_device(int sm_count) { return std::min(sm_count / 2, kAttnMaxCounters / 2); }
 
+// The plan of a launch depends on its shapes, and on the scratch in one point only: the best plan where the scratch holds it, else
+// the best one that the scratch of the single-CTA kernel's plan holds, which every caller has (there may be none).
 PairPlan plan_of(const GemmParams& g, int sm_count) {
-  int rows[3] = {0, 0, 0};
-  for (int i = 0; i < g.n_seg; ++i) rows[i] = g.seg[i].n_rows;
-  return pair_plan(rows, g.n_seg, g.act != nullptr, g.T, g.K, g.w16, pairs_of_device(sm_count), g.scratch ? g.scratch_bytes : 0);
+  int rows[3] = {0, 0, 0}, n = 0;
+  for (int i = 0; i < g.n_seg; ++i) n += rows[i] = g.seg[i].n_rows;
+  auto plan = [&](uint64_t bytes) { return pair_plan(rows, g.n_seg, g.act != nullptr, g.T, g.K, g.w16, pairs_of_device(sm_count), bytes); };
+  const uint64_t have = g.scratch ? g.scratch_bytes : 0;
+  const PairPlan best = plan(~0ull);
+  return best.scratch <= have ? best : plan(std::min(have, gemm_scratch_bytes(g.T, n, g.K)));
 }
 
 }  // namespace

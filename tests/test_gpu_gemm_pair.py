@@ -146,3 +146,34 @@ def test_few_tiles_go_to_the_single_cta_kernel(fmt, N, K, T, pairs):
     assert launches[0] == (1 if pairs else launches[1])
     if not pairs:
         assert np.array_equal(outs[0], outs[1])
+
+
+# 75 tiles for 74 pairs (the one that is left is split into two, three or four where there is scratch for it) and the same as one wave
+# and a half; 4-bit and fp16.
+@pytest.mark.parametrize("fmt,N,K,T", [("q4", 19200, 4096, 40), ("q4", 28672, 1024, 40), ("mxfp4", 14336, 2048, 300), ("w16", 19200, 2048, 40)])
+def test_the_workspace_chooses_between_two_plans_only(fmt, N, K, T):
+    import torch
+    from paper_2607_10183_b200 import binding as B
+    x = H.to_dev(W.activations(96, 0, (T, K)))
+    weights = (W.w16_matrix(96, 0, W.ROLE_UP, N, K),) if fmt == "w16" else (W.q4_packed if fmt == "q4" else W.mxfp4_packed)(96, 0, W.ROLE_UP, N, K)
+    results, static = [], None
+    at_8mib = 1024 + (8 << 20)
+    for ws in [1024 + 256 + (i << 16) for i in range(0, 6)] + [MB, 2 * MB, 4 * MB, 6 * MB, at_8mib, 12 * MB, 24 * MB, 48 * MB, 96 * MB]:
+        ctx = B.Context(ws + 2 * N * K + 2 * MB, workspace_bytes=ws)
+        tid = (ctx.register_w16 if fmt == "w16" else ctx.register_q4)(*weights)
+        ctx.set_placement([(tid, -1, B.ATS_GPU)])
+        y = torch.empty((T, N), dtype=torch.float16, device="cuda")
+        try:
+            ctx.linear(tid, x, y, T)
+            ctx.sync()
+            results.append(y)
+            if ws == at_8mib and fmt != "w16":
+                static = torch.empty_like(y)
+                ctx.linear_static_scratch(tid, x, static, T)
+                ctx.sync()
+                assert torch.equal(static, y)
+        except B.AtsError as e:
+            assert e.value == B.ATS_ERR_NOMEM and not results  # more is never refused after less was taken
+        ctx.close()
+    changes = [i for i in range(1, len(results)) if not torch.equal(results[i - 1], results[i])]
+    assert len(results) >= 9 and len(changes) <= 1, changes
