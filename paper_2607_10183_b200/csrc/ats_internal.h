@@ -381,10 +381,8 @@ struct GemmParams {
   int ldact;
   int* counters;  // kAttnMaxCounters ints, zero between launches (launch_gemm_pair: arrival counts of split tiles)
 };
-// GEMMs on pairs of CTAs (kernels_gemm_pair.cu): launches they take, the scratch of a launch's best plan (they take some with less), and
-// their launcher
+// GEMMs on pairs of CTAs (kernels_gemm_pair.cu): launches they take (operands, scratch, and faster there), and their launcher
 bool gemm_pair_eligible(const GemmParams& p, int sm_count);
-uint64_t gemm_pair_scratch_bytes(const int* rows, int n_seg, bool act, int T, int K, bool w16);
 cudaError_t launch_gemm_pair(const GemmParams& p, int sm_count, cudaStream_t st, uint64_t* n_launch, std::string* err);
 // the single-CTA kernel: scratch of its plan, the k that the plan adds up in one accumulator, its time
 uint64_t gemm_scratch_bytes(int T, int n_total, int K);

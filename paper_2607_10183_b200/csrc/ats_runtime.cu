@@ -402,6 +402,10 @@ struct Bump {
   }
 };
 
+struct GemmScratch {
+  uint8_t* p = nullptr;
+  uint64_t bytes = 0;
+};
 struct LayerWs {
   // decode
   __half* h16 = nullptr;
@@ -422,8 +426,7 @@ struct LayerWs {
   __half* x1_16 = nullptr;
   __half* gu16 = nullptr;
   __half* d16 = nullptr;
-  void* gemm_scratch = nullptr;
-  uint64_t gemm_scratch_bytes = 0;
+  GemmScratch qkv_scratch, o_scratch, gu_scratch, d_scratch;  // prefill: partial sums of each GEMM
   // MoE prefill: rows in expert order
   __half* xs16 = nullptr;
   int* order = nullptr;
@@ -461,28 +464,29 @@ static LayerWs layout_decode(const ats_layer_desc& L, uint32_t M, uint8_t* base,
   return w;
 }
 
+// Workspace of a prefill call.  Behind the buffers lie the partial sums that the single-CTA kernel's plans ask for.  A GEMM may use the
+// buffers that are written after it as well (they follow one another in the order of their use): the pairs' plans want more than that tail
+// (2048 tokens of a 4096-wide layer: up to 39 MB), and it comes out of what is there.
 static LayerWs layout_prefill(const ats_layer_desc& L, uint32_t T, uint8_t* base, uint64_t cap) {
   LayerWs w;
   Bump b(base, cap);
   b.take(kWsReserved);
   const uint64_t H = L.hidden, qd = (uint64_t)L.n_q_heads * L.head_dim, kvd = (uint64_t)L.n_kv_heads * L.head_dim;
-  uint64_t scratch = 0;
-  auto gemm_want = [&](std::initializer_list<uint64_t> rows, uint64_t k, bool act) {
-    int n[3] = {0, 0, 0}, n_seg = 0, total = 0;
-    for (uint64_t r : rows) total += n[n_seg++] = (int)r;
-    uint64_t want = gemm_scratch_bytes((int)T, total, (int)k);
-    for (bool w16 : {false, true}) want = std::max(want, gemm_pair_scratch_bytes(n, n_seg, act, (int)T, (int)k, w16));
-    scratch = std::max(scratch, want);
-  };
+  struct Product {
+    uint64_t rows, k, from;  // from: first byte that is free while it runs
+    GemmScratch* out;
+  } products[4];
+  int n_products = 0;
+  auto product = [&](uint64_t rows, uint64_t k, GemmScratch* out) { products[n_products++] = Product{rows, k, b.off, out}; };
   if (L.wq >= 0) {
     w.h16 = (__half*)b.take(T * H * 2);
     w.qkv16 = (__half*)b.take(T * (qd + 2 * kvd) * 2);
+    product(qd + 2 * kvd, H, &w.qkv_scratch);
     w.qrot16 = (__half*)b.take(T * qd * 2);
     w.a16 = (__half*)b.take(T * qd * 2);
     w.o16 = (__half*)b.take(T * H * 2);
     w.x1_16 = (__half*)b.take(T * H * 2);
-    gemm_want({qd, kvd, kvd}, H, false);
-    gemm_want({H}, qd, false);
+    product(H, qd, &w.o_scratch);
   }
   w.h2_16 = (__half*)b.take(T * H * 2);
   if (L.n_experts) {
@@ -500,12 +504,19 @@ static LayerWs layout_prefill(const ats_layer_desc& L, uint32_t T, uint8_t* base
   } else {
     w.gu16 = (__half*)b.take((uint64_t)T * 2 * L.ffn * 2);
     w.act16 = (__half*)b.take((uint64_t)T * L.ffn * 2);
+    product(2 * (uint64_t)L.ffn, H, &w.gu_scratch);
     w.d16 = (__half*)b.take(T * H * 2);
-    gemm_want({L.ffn, L.ffn}, H, true);
-    gemm_want({H}, L.ffn, false);
+    product(H, L.ffn, &w.d_scratch);
   }
-  w.gemm_scratch = b.take(scratch);
-  w.gemm_scratch_bytes = scratch;
+  const uint64_t end = align_up(b.off);
+  uint64_t tail = 0;
+  for (int i = 0; i < n_products; ++i)
+    tail = std::max(tail, gemm_scratch_bytes((int)T, (int)products[i].rows, (int)products[i].k));
+  b.take(tail);
+  for (int i = 0; i < n_products; ++i) {
+    const uint64_t from = align_up(products[i].from);
+    *products[i].out = GemmScratch{base ? base + from : nullptr, end + tail - from};
+  }
   w.total = align_up(b.off);
   w.ok = b.ok;
   return w;
@@ -1688,9 +1699,11 @@ int32_t ats_layer_prefill(ats_ctx* ctx, const ats_layer_desc* L, const void* x_i
   const int pdl = (ctx->cfg.flags & ATS_FLAG_NO_PDL) ? 0 : 1;
   GemmParams g{};
   g.T = (int)T;
-  g.scratch = w.gemm_scratch;
-  g.scratch_bytes = w.gemm_scratch_bytes;
   g.pdl = pdl;
+  auto scratch = [&](const GemmScratch& sc) {
+    g.scratch = sc.p;
+    g.scratch_bytes = sc.bytes;
+  };
   const __half* resid = (const __half*)x_in;
   if (attn) {
     ATS_CUDA(launch_rmsnorm(x_in, 0, (const __half*)ctx->tensors[L->attn_norm].f16_dev, w.h16, (int)T, H, L->rms_eps, ctx->cs, nl, pdl));
@@ -1698,6 +1711,7 @@ int32_t ats_layer_prefill(ats_ctx* ctx, const ats_layer_desc* L, const void* x_i
     g.ldx = H;
     g.y = w.qkv16;
     g.ldy = qd + 2 * kvd;
+    scratch(w.qkv_scratch);
     ATS_TRY(run_gemm_group(ctx, qkv, 3, g));
     ATS_CUDA(launch_rope_append_prefill(w.qkv16, qd + 2 * kvd, w.qrot16, (__half*)k_cache, (__half*)v_cache, (int)T, nq, nkv, d,
                                         (int)L->kv_capacity, (int)pos0, L->rope_theta, ctx->cs, nl, pdl));
@@ -1713,6 +1727,7 @@ int32_t ats_layer_prefill(ats_ctx* ctx, const ats_layer_desc* L, const void* x_i
     g.ldy = H;
     g.res = (const __half*)x_in;  // x1 = rn16(x + o) in the GEMM's own epilogue (or its split-K reduction)
     g.y2 = w.x1_16;
+    scratch(w.o_scratch);
     ATS_TRY(run_gemm_group(ctx, &wo, 1, g));
     g.res = nullptr;
     g.y2 = nullptr;
@@ -1833,6 +1848,7 @@ int32_t ats_layer_prefill(ats_ctx* ctx, const ats_layer_desc* L, const void* x_i
   g.ldy = 2 * (int)L->ffn;
   g.act = w.act16;
   g.ldact = (int)L->ffn;
+  scratch(w.gu_scratch);
   ATS_TRY(run_gemm_group(ctx, gu, 2, g));
   g.act = nullptr;
   g.x = w.act16;
@@ -1841,6 +1857,7 @@ int32_t ats_layer_prefill(ats_ctx* ctx, const ats_layer_desc* L, const void* x_i
   g.ldy = H;
   g.res = resid;  // y = rn16(x1 + d)
   g.y2 = (__half*)x_out;
+  scratch(w.d_scratch);
   ATS_TRY(run_gemm_group(ctx, &wd, 1, g));
   return ATS_OK;
 }

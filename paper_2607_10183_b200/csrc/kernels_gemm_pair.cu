@@ -979,10 +979,6 @@ PairPlan plan_of(const GemmParams& g, int sm_count) {
 
 }  // namespace
 
-uint64_t gemm_pair_scratch_bytes(const int* rows, int n_seg, bool act, int T, int K, bool w16) {
-  return pair_plan(rows, n_seg, act, T, K, w16, 74, ~0ull).scratch;
-}
-
 bool gemm_pair_eligible(const GemmParams& g, int sm_count) {
   if ((g.w16 && g.grp_off) || g.n_seg < 1 || g.n_seg > 3 || !g.counters || g.K % (g.w16 ? 8 : 32) || g.ldx % 8) return false;
   if (reinterpret_cast<uintptr_t>(g.x) & 15) return false;

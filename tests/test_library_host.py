@@ -191,3 +191,13 @@ def test_reschedule_gate_matches_oracle():
             assert B.host_transfer_latency(rb, start, b, *ref) == O.dynamic_transfer(list(b), *ref)[0]
         replans += did
     assert 2 <= replans <= 12  # the burst's start, its end and the slower link each trigger one; the rate limit holds the rest back
+
+
+def test_prefill_workspace_is_the_buffers_and_the_single_cta_kernels_partial_sums():
+    """2048 tokens of a 4096-wide layer: no plan of the single-CTA kernel splits K there (256 bytes of scratch), so a caller reserves the
+    buffers of one call, each padded to 256 bytes, and the staging rows of the host-driven decode step."""
+    B = _binding()
+    Hd, nq, nkv, d, F, T = 4096, 32, 8, 128, 14336, 2048
+    desc = B.layer_desc(hidden=Hd, ffn=F, n_q_heads=nq, n_kv_heads=nkv, head_dim=d, wq=0, kv_capacity=4096)
+    rows = [Hd, (nq + 2 * nkv) * d, nq * d, nq * d, Hd, Hd, Hd, 2 * F, F, Hd]  # h, q|k|v, q_rot, a, o, x1, h2, gate|up, act, d
+    assert B.workspace_bytes(desc, T) == 1024 + 2 * T * sum(rows) + 256 + 2 * (32 * Hd * 2) + 256
