@@ -382,9 +382,10 @@ __device__ __forceinline__ bool stream_consume(const StreamParams& p, const int 
   const int wg = warp % kGroupWarps;          // warp within the group
   const int tg = tid % (kGroupWarps * 32);    // thread within the group
   const int part = wg % PARTS, rsub = wg / PARTS;
-  // (microscaling: parts of whole groups of eight blocks; there are K / 256 of them)
+  // (microscaling: parts of whole groups of eight blocks; there are K / 256 of them, so the last parts may be empty.  Integer codes need no
+  // clamp, and with one the expert kernels take two to four more registers: eight rows through 2048 x 768 experts 44.3 -> 44.6 us)
   const int pblk = MX ? ((nblk + PARTS - 1) / PARTS + 7) / 8 * 8 : (nblk + PARTS - 1) / PARTS;
-  const int b0 = min(nblk, part * pblk), b1 = min(nblk, b0 + pblk);
+  const int b0 = MX ? min(nblk, part * pblk) : part * pblk, b1 = min(nblk, b0 + pblk);
   uint32_t xr[J][16];       // integer codes: this lane's blocks; microscaling: [4 j + i] = its run of block group i
   float xm[J], xc[J];
   constexpr int NG = 4 * J;  // microscaling: groups of eight blocks of the part
