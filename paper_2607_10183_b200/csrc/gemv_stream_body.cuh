@@ -11,7 +11,8 @@
 // up to two quantization blocks (32 k each) of a k-part of the row and keeps the activation for them in registers for the
 // whole kernel, so a weight byte is read once from shared memory and an activation never again.
 //
-// Arithmetic: the activation block is re-expressed once per CTA as 16-bit block fixed point, x_k ~ xi_k * 2^-sh with
+// Arithmetic of the integer codes (microscaling floats: fp16 products on mma.sync, see mx_run; the activations stay fp16 and an Inf or a
+// NaN gives what the plain definition gives): the activation block is re-expressed once per CTA as 16-bit block fixed point, x_k ~ xi_k * 2^-sh with
 // sh chosen from the block's largest exponent (exact for every element within 2^-4 of the block maximum, rounded at
 // 2^-16 of it otherwise: 32 times finer than fp16 resolves the maximum itself).  Pairs of xi meet pairs of masked 4-bit
 // codes in dp2a: block dot products are exact integers; one fp32 multiply-add per block applies the scale, and blocks

@@ -1,5 +1,7 @@
 // Dequantize-fused prefill GEMM on the 5th-generation tensor cores (sm_100a): Y[T][N] = X[T][K] * W^T, fp16 operands,
-// fp32 accumulation in tensor memory, fp16 output.
+// fp32 accumulation in tensor memory, fp16 output.  It takes the products whose tiles are too few for the pairs of CTAs
+// (gemm_pair_eligible compares the times of both plans), experts whose slices are found through address tables, operands that the pairs do
+// not take, and everything under ATS_FLAG_NO_GEMM_PAIR.
 //
 // One CTA computes a tile of 256 tokens x 256 output features (or 128 x 128) over a K range (split-K when the tiles do
 // not fill the GPU).  The activation tile is the MMA A operand (M = 128 tokens per instruction, two token blocks share

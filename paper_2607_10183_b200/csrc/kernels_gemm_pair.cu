@@ -23,8 +23,10 @@
 // the scratch: every contributor but the last to arrive leaves its part there; the last adds the parts in ascending k order (so
 // the result does not depend on who that is) and writes the tile.  Nobody waits for anybody.
 //
-// What bounds it: 4-bit, up to about 128 tokens, the expansion (about 900 cycles per unit and CTA: 3500 warp instructions at
-// close to one per cycle and scheduler); fp16 there the weights' way from memory; beyond that the MMAs and the power limit.
+// What bounds it: 4-bit, up to about 128 tokens, the expansion (a unit takes 0.39 us in launches with many of them); fp16 there the weights'
+// way from memory; with tiles for all pairs the MMAs and the power limit; with few tiles the launch (4 to 5 us) and the sum of split
+// tiles (up to 10 us with 128 tokens), which is why such products go to the single-CTA kernel (gemm_pair_eligible).  72 registers a thread
+// are all that 896 threads leave: the compiler spills 172 to 208 bytes, in the epilogue's sums.
 // Back to back on new weights, before -> now (before: weights as a shared-memory operand, 256-token tiles, with reduction,
 // residual and SwiGLU launches):
 //   77 tokens MXFP4: 28672 x 4096 with SwiGLU 66 -> 36 us, 6144 x 4096 25 -> 21, 4096 x 14336 41 -> 33
