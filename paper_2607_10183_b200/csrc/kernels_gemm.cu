@@ -638,7 +638,7 @@ double gemm_us(const int* rows, int n_seg, int T, int K, bool w16) {
   const double kstep = (w16 ? 0.270 + 0.0021 * (pl.wide ? pl.bf : 224) : 0.503 + 0.00143 * (pl.wide ? pl.bf : 208));
   double us = waves * (per * kstep + (w16 ? 4.0 : 3.6));
   if (pl.splits > 1) us += (w16 ? 3.8 : 2.6) + (w16 ? 0.22 : 0.227) * (pl.splits + 1) * 4e-6 * T * n;
-  return w16 ? std::max(us, std::max(1.9e-9 * T, 0.4e-6) * n * K) : us;  // (at most 1050 TFLOP/s and 5 TB/s)
+  return w16 ? std::max(us, std::max(2.08e-9 * T, 0.4e-6) * n * K) : us;  // (at most 960 TFLOP/s and 5 TB/s)
 }
 
 cudaError_t launch_gemm(const GemmParams& g, cudaStream_t st, uint64_t* n_launch, std::string* err) {

@@ -318,8 +318,10 @@ __global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid
   uint8_t* code_s = x_s + (size_t)NX * (FMT == kFmtW16 ? step_bytes : 2 * xbytes);   // [NC][128 rows][64 bytes], 16-byte pieces swizzled by row pair
   uint8_t* scale_s = code_s + (size_t)NC * kCodeBytes;
   uint8_t* out_s = scale_s + (size_t)NC * kScaleBytes;  // [nt][kStagePitch]
-  // two accumulators that take turns: of 128 columns beside the weights, of 256 where those are not in tensor memory
-  const bool two = FMT == kFmtW16 || p.nt <= 128;
+  // two accumulators that take turns: of 128 columns beside the weights, of 256 where those are not in tensor memory; a tile of 512
+  // tokens (fp16 weights) is all 512 columns
+  const bool wide = FMT == kFmtW16 && p.nt > 256;
+  const bool two = FMT == kFmtW16 ? !wide : p.nt <= 128;
   constexpr uint32_t kAcc = FMT == kFmtW16 ? 256 : 128;
   const int sc_pitch = p.sc16 ? 16 : 12;
 
@@ -456,7 +458,9 @@ __global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid
             ++n;
             const uint32_t dst = x0 + (uint32_t)(s * step_bytes), dw = dst + (uint32_t)xbytes;
             if (rank == 0) expect_tx_one(one, &xfull[s], (uint32_t)(2 * step_bytes));
-            tma_pair_2d(one, dst, &xmap, ks * 64, row, &xfull[s]);
+            // (wide: tokens 128 rank .. of each half of the tile, so that either half is one operand of the pair)
+            tma_pair_2d(one, dst, &xmap, ks * 64, wide ? row - (int)rank * 128 : row, &xfull[s]);
+            if (wide) tma_pair_2d(one, dst + (uint32_t)(xbytes / 2), &xmap, ks * 64, row - (int)rank * 128 + 256, &xfull[s]);
             tma_pair_3d(one, dw, &wmap.codes[sa], ks * 64, wa, &xfull[s]);
             tma_pair_3d(one, dw + kW16Bytes / 2, &wmap.codes[sb], ks * 64, wb, &xfull[s]);
             if (++s == NX) s = 0, par ^= 1u;
@@ -481,7 +485,7 @@ __global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid
       // ------------------------------------------------------------ MMA issue (leader)
       if (rank == 0) {
         const uint32_t one = elect_one();
-        const uint32_t idesc = umma_idesc_f16(2 * kFeat, p.nt);
+        const uint32_t idesc = umma_idesc_f16(2 * kFeat, wide ? 256 : p.nt);
         const uint64_t xd = umma_desc_sw128(smem_u32(x_s));
         Walk mine(p, pair);
         int s = 0, sx = 0, seg = 0;  // places in the rings, accumulator segments so far
@@ -519,13 +523,18 @@ __global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid
 #pragma unroll
                 for (int kk = 0; kk < 4; ++kk)
                   umma_ss_pair(one, d, ad + (uint64_t)(2 * kk), bd + (uint64_t)(2 * kk), idesc, kk > 0 ? 1u : accumulate);
+                if (wide) {
+#pragma unroll
+                  for (int kk = 0; kk < 4; ++kk)
+                    umma_ss_pair(one, d + 256u, ad + (uint64_t)(2 * kk), bd + (uint64_t)((xbytes >> 5) + 2 * kk), idesc, kk > 0 ? 1u : accumulate);
+                }
                 accumulate = 1;
                 umma_commit_both(one, &xempty[sx]);
                 sx = sxn, parx = parxn;
               }
               if (!ok) break;
               if (--left == 0) {
-                umma_commit_both(one, &acc_full[seg & 1]);
+                umma_commit_both(one, &acc_full[two ? seg & 1 : 0]);
                 ++seg;
               }
               continue;
@@ -933,14 +942,19 @@ PairPlan pair_plan(const int* rows, int n_seg, bool act, int T, int K, bool w16,
   double weights_mb = 0;
   for (int i = 0; i < n_seg; ++i) weights_mb += 2e-6 * rows[i] * K;
   int last = 0;
-  for (int most : {256, 192, 128}) {
+  for (int most : {512, 256, 192, 128}) {
     const int n_tt = (T + most - 1) / most;
-    if (n_tt == last) continue;
-    last = n_tt;
-    const int nt = ((T + n_tt - 1) / n_tt + 31) / 32 * 32;
+    if (most == 512 ? !w16 || T <= 256 || n_ft * n_tt > max_pairs : n_tt == last) continue;
+    last = most == 512 ? 0 : n_tt;
+    const int nt = most == 512 ? 512 : ((T + n_tt - 1) / n_tt + 31) / 32 * 32;
     const uint64_t slot = 2ull * kFeat * std::min(nt, T) * 4;
-    const double unit = w16 ? std::max(0.729, 0.186 + 0.0027 * nt) : std::max(0.391, 0.174 + 0.0020 * nt);
-    const double launch = w16 ? 5.0 : 4.2, tile = w16 ? 0.0 : 0.012 * nt, flush = w16 ? 1.1 : nt <= 128 ? 2.6 : 4.6;
+    // (fp16 tiles of 512 tokens: the weights serve two operands, but nothing runs under the epilogue and the ring is four steps deep.  Where
+    // they make one wave they are the faster ones: 4096 x 14336 over 2048 tokens 204 -> 186 us, 14336 x 4096 over 512 67 -> 55; in several
+    // waves they are not: 28672 x 4096 over 3000 tokens 527 -> 649.  fp16 weights that several token tiles share come out of L2 for all but
+    // one)
+    const double unit = w16 ? std::max(n_tt > 1 ? 0.55 : 0.729, nt == 512 ? 1.55 : 0.40 + 0.00165 * nt) : std::max(0.391, 0.174 + 0.0020 * nt);
+    const double launch = w16 ? 5.0 : 4.2, tile = w16 ? (nt == 512 ? 6.0 : 0.0) : 0.012 * nt;
+    const double flush = w16 ? 1.1 : nt <= 128 ? 2.6 : 4.6;
     const int tok = std::min(nt, T), batches = tok <= 16 ? 1 : (tok + 63) / 64 * 2;  // (16 tokens a batch and warp, two warps side by side)
     auto stretch = [&](double len) { return len * unit + (std::ceil(len / max_units) - 1) * flush + tile; };
     auto sum = [&](double con) { return (w16 ? 1.0 : 1.3) + batches * (w16 ? (con > 2 ? 2.7 : 1.6) : (con > 2 ? 2.5 : 1.3)); };
@@ -950,7 +964,7 @@ PairPlan pair_plan(const int* rows, int n_seg, bool act, int T, int K, bool w16,
       const bool parts = std::max(len, waves || !slots ? (double)units : 0.0) > max_units;
       const int pairs = waves ? max_pairs : slots ? n : rem;
       const uint64_t need = ((uint64_t)n * slots + (parts ? pairs : 0)) * slot;
-      if (need > scratch_bytes) return;
+      if (need > scratch_bytes || (nt == 512 && need)) return;  // (tiles of 512 tokens: whole ones in one part)
       us += launch + waves * stretch(units);
       if (w16) us = std::max(us, weights_mb / 4.5);
       if (us >= best.us) return;
@@ -1008,6 +1022,7 @@ bool gemm_pair_eligible(const GemmParams& g, int sm_count) {
     single = gemm_us(rows, g.n_seg, g.T, g.K, false);
   }
   if (g.act) single += 2.0 + 6e-6 / 4 * g.T * g.seg[0].n_rows;
+  if (g.w16 && pl.n_whole > pl.pairs) single *= 1.06;  // (the fit is that far off there: 14336 x 4096 over 700 tokens 83 us on the pairs, 97)
   return pl.pairs > 0 && pl.us <= single;
 }
 
@@ -1068,7 +1083,7 @@ cudaError_t launch_gemm_pair(const GemmParams& g, int sm_count, cudaStream_t st,
   p.grp_stride = g.grp_stride;
   CUtensorMap xmap;
   const cuuint64_t dims[2] = {(cuuint64_t)g.K, (cuuint64_t)g.T}, strides[1] = {(cuuint64_t)g.ldx * 2};
-  const cuuint32_t box[2] = {64, (cuuint32_t)(p.nt / 2)}, es[2] = {1, 1};
+  const cuuint32_t box[2] = {64, (cuuint32_t)(p.nt > 256 ? p.nt / 4 : p.nt / 2)}, es[2] = {1, 1};
   if (enc(&xmap, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, const_cast<__half*>(g.x), dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
           CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS) {
     if (err) *err = "cuTensorMapEncodeTiled failed for the activation tile";

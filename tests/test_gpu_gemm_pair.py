@@ -177,3 +177,33 @@ def test_the_workspace_chooses_between_two_plans_only(fmt, N, K, T):
         ctx.close()
     changes = [i for i in range(1, len(results)) if not torch.equal(results[i - 1], results[i])]
     assert len(results) >= 9 and len(changes) <= 1, changes
+
+
+# fp16 weights in tiles of 512 tokens (both accumulators at once): ragged last tiles of tokens and features, full ones, one tile
+# of tokens
+@pytest.mark.parametrize("N,K,T", [(4001, 8200, 1800), (9001, 4104, 1000), (4096, 8192, 2048), (15001, 4104, 450)])
+def test_gemm_w16_tiles_of_512_tokens_match_oracle(N, K, T):
+    import torch
+    from paper_2607_10183_b200 import binding as B
+    w = W.w16_matrix(97, 0, W.ROLE_UP, N, K)
+    x = W.activations(97, 0, (T, K))
+    ws = 64 * MB
+    ctx = B.Context(ws + 2 * N * K + 2 * MB, workspace_bytes=ws)
+    tid = ctx.register_w16(w)
+    ctx.set_placement([(tid, -1, B.ATS_GPU)])
+    xd = H.to_dev(x)
+    outs = []
+    for _ in range(2):
+        y = torch.full((T + 1, N), 7.0, dtype=torch.float16, device="cuda")
+        ctx.linear(tid, xd, y, T)
+        ctx.sync()
+        outs.append(y.cpu().numpy())
+    ctx.close()
+    edges = np.r_[0, 127, 128, 255, 256, 383, 384, 511, 512, T - 1, np.arange(0, T, 211)]
+    rows = np.unique(edges[edges < T])
+    H.assert_close(outs[0][rows], O.linear_w16(x[rows], w, round_out=True), what=f"w16 {N}x{K} T={T}")
+    got, want = torch.from_numpy(outs[0][:T]).cuda().double(), xd.double() @ torch.from_numpy(w).cuda().double().t()  # all rows, in 64 bits
+    assert (got - want).abs().max() <= 2e-3 * want.abs().max()
+    assert ((got - want).norm() / want.norm()).item() <= 3e-4  # rounding to fp16's 11 bits alone is 2.1e-4 rms
+    assert np.all(outs[0][T] == 7.0)
+    assert np.array_equal(outs[0].view(np.uint16), outs[1].view(np.uint16))
