@@ -1,7 +1,8 @@
 // GEMM of prompts on pairs of CTAs (sm_100a, tcgen05 cta_group::2): Y[T][N] = X[T][K] W^T for the two 4-bit block formats and for
 // fp16 matrices; fp16 operands (4-bit: w = rn16(scale * code), one rounding), fp32 accumulation.
 //
-// The weights are the A operand (M = 256 features, 128 per CTA), the tokens are the instruction's N (32..256, chosen from T).
+// The weights are the A operand (M = 256 features, 128 per CTA), the tokens are the instruction's N (32..256, chosen from T; fp16 weights
+// also tiles of 512 tokens, two instructions).
 // 4-bit weights are expanded into tensor memory: a thread of the sixteen dequantization warps turns 32-weight blocks of one
 // feature (its lane) into sixteen columns each; nothing is stored to shared memory, no swizzle, no proxy fence.  (With the
 // weights as a shared-memory operand a 64-k step of 256 features took about 1700 cycles, whatever the number of tokens, for the
@@ -27,11 +28,10 @@
 // way from memory; with tiles for all pairs the MMAs and the power limit; with few tiles the launch (4 to 5 us) and the sum of split
 // tiles (up to 10 us with 128 tokens), which is why such products go to the single-CTA kernel (gemm_pair_eligible).  72 registers a thread
 // are all that 896 threads leave: the compiler spills 172 to 208 bytes, in the epilogue's sums.
-// Back to back on new weights, before -> now (before: weights as a shared-memory operand, 256-token tiles, with reduction,
-// residual and SwiGLU launches):
-//   77 tokens MXFP4: 28672 x 4096 with SwiGLU 66 -> 36 us, 6144 x 4096 25 -> 21, 4096 x 14336 41 -> 33
+// Back to back on new weights, single-CTA kernel (with reduction, residual and SwiGLU launches) -> pairs:
+//   77 tokens MXFP4: 28672 x 4096 with SwiGLU 66 -> 36 us, 4096 x 14336 41 -> 33
 //   512 tokens Q4: gate and up 143 -> 103-107 us, 4096 x 14336 78 -> 69;  2048 tokens: gate and up 462 -> 351 (1372 TFLOP/s)
-//   2048 tokens fp16: q, k, v 152 -> 78 us, o 66 -> 59, gate and up 451 -> 346 (1390 TFLOP/s), 4096 x 14336 189 -> 196
+//   2048 tokens fp16: q, k, v 152 -> 78 us, o 66 -> 59, gate and up 451 -> 346 (1390 TFLOP/s)
 //
 // Roles per CTA: warp 0 = activation loads (fp16: and weights), warp 1 = tensor-memory allocation and (leader) MMA issue, warps 2, 3
 // = code and scale loads, warps 4..11 = epilogue, warps 12..27 = dequantization: four groups of four.  Every mbarrier wait is
