@@ -21,12 +21,12 @@
 // read the same weights and tokens from L2 at the same time (contiguous ranges of tiles per pair instead: 2048 tokens, fp16 gate
 // and up 447 us against 346, 4096 x 14336 254 against 196).  The units of the tiles that are left for the last wave form one line
 // of work that is cut into equal contiguous ranges.  A tile that falls into several of them is summed through fp32 partials in
-// the scratch: every contributor but the last to arrive leaves its part there; the last adds the parts in ascending k order (so
-// the result does not depend on who that is) and writes the tile.  Nobody waits for anybody.
+// the scratch: every contributor leaves its part there, 32 tokens at a time; the last one to do so for these tokens adds the parts in
+// ascending k order (so the result does not depend on who that is) and writes them.  Nobody waits for anybody.
 //
 // What bounds it: 4-bit, up to about 128 tokens, the expansion (a unit takes 0.39 us in launches with many of them); fp16 there the weights'
-// way from memory; with tiles for all pairs the MMAs and the power limit; with few tiles the launch (4 to 5 us) and the sum of split
-// tiles (up to 10 us with 128 tokens), which is why such products go to the single-CTA kernel (gemm_pair_eligible).  72 registers a thread
+// way from memory; with tiles for all pairs the MMAs and the power limit; with few tiles the launch (4 to 5 us) and what every tile pays
+// for its sums, which is why such products go to the single-CTA kernel (gemm_pair_eligible).  72 registers a thread
 // are all that 896 threads leave: the compiler spills 172 to 208 bytes, in the epilogue's sums.
 // Back to back on new weights, single-CTA kernel (with reduction, residual and SwiGLU launches) -> pairs:
 //   77 tokens MXFP4: 28672 x 4096 with SwiGLU 66 -> 36 us, 4096 x 14336 41 -> 33
@@ -210,19 +210,6 @@ __device__ __forceinline__ bool wait_warp(uint64_t* bar, uint32_t parity) {
 // A test whose result is looked at later: its latency (about 200 cycles here) passes under other work.
 __device__ __forceinline__ bool peek(uint64_t* bar, uint32_t parity) { return mbar_test_wait(bar, parity); }
 
-__device__ __forceinline__ void tmem_ld_x16(uint32_t taddr, uint32_t* v) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]), "=r"(v[9]),
-        "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
-      : "r"(taddr)
-      : "memory");
-}
-__device__ __forceinline__ void tmem_ld_wait_x16(uint32_t* v) {
-  asm volatile("tcgen05.wait::ld.sync.aligned;"
-               : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]), "+r"(v[6]), "+r"(v[7]), "+r"(v[8]), "+r"(v[9]),
-                 "+r"(v[10]), "+r"(v[11]), "+r"(v[12]), "+r"(v[13]), "+r"(v[14]), "+r"(v[15])::"memory");
-}
 template <int N>
 struct Int {
   static constexpr int value = N;
@@ -307,7 +294,7 @@ __global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   __shared__ uint64_t afull[kMaxA], aempty[kMaxA], xfull[kMaxX], xempty[kMaxX], cfull[kMaxCodes], cempty[kMaxCodes], acc_full[2], d_empty[2];
   __shared__ uint32_t tmem_s;
-  __shared__ int last_s;
+  __shared__ int last_s[2][4];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t rank = cta_rank();
   const int pair = blockIdx.x >> 1;
@@ -691,8 +678,9 @@ __global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid
       };
       for (int g = 0; g < n_part; ++g, ++seg) {
         const int b = two ? seg & 1 : 0, use = two ? seg >> 1 : seg;
-        const bool got = wait_warp(&acc_full[b], use & 1);
-        ok = g + 1 == n_part || !got ? epi_all(got) : got;  // (the eight warps give up together: they share barriers)
+        bool got = true;  // (one warp polls, the others sleep at the barrier: polls take issue slots from the expansion)
+        if (warp == 4) got = wait_warp(&acc_full[b], use & 1);
+        ok = epi_all(got);
         if (!ok) break;
         tc_fence_after();
         col = d_col + kAcc * b;
@@ -714,159 +702,61 @@ __global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid
       if (!ok) break;
       const int last_b = two ? seg & 1 : 0;
       ++seg;
-      const bool split = st.u0 > 0 || st.u1 < p.units;
-      bool write = true;
-      // contributors of a split tile: the pairs whose ranges meet it.  Pair q holds units n q / P .. n (q + 1) / P - 1, so
-      // unit u lies with q = ((u + 1) P - 1) / n.
-      int first = pair, n_con = 1;
-      auto part_of = [&](int q) {  // this CTA's half of what pair q leaves of the tile
-        // (the first contributor begins the tile, the others come upon it at the start of their range)
-        return p.partial + ((size_t)(p.slots2 && q == first ? p.split_pairs + q : q) * 2 + rank) * kFeat * p.slot_tok;
+      auto stage = [&](const float* v, auto n_tok, int row) {  // this thread's feature of n_tok tokens
+        __half* o = reinterpret_cast<__half*>(out_s + (size_t)row * kStagePitch) + feat;
+#pragma unroll
+        for (int i = 0; i < decltype(n_tok)::value; ++i) o[i * (kStagePitch / 2)] = __float2half_rn(v[i]);
       };
-      if (split) {
-        const long long n_units = (long long)(p.n_ft * p.n_tt - p.n_whole) * p.units, lo = (long long)(st.tile - p.n_whole) * p.units;
-        first = (int)(((lo + 1) * p.split_pairs - 1) / n_units);
-        n_con = (int)(((lo + p.units) * p.split_pairs - 1) / n_units) - first + 1;
-        int* cnt = p.counters + 2 * first + rank;
-        if (tid == 0) {
-          int v;
-          asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(cnt) : "memory");
-          last_s = v == n_con - 1;
-        }
-        epi_sync();
-        write = last_s != 0;
-        if (!write) {
-          float* dst = part_of(pair) + feat;
-#pragma unroll 1
-          for (int c0 = 32 * half; c0 < ntok; c0 += 64) {
-            float v[32];
-            tmem_ld_x32(col + c0, reinterpret_cast<uint32_t*>(v));
-            tmem_ld_wait_x32(reinterpret_cast<uint32_t*>(v));
-            if (n_part > 1) add_own(v, c0, Int<32>{});
-#pragma unroll
-            for (int i = 0; i < 32; ++i)
-              if (c0 + i < ntok) __stcg(dst + (size_t)(c0 + i) * kFeat, v[i]);
-          }
-          epi_sync();  // every part is written (and last_s read) before the arrival that releases them
-          if (tid == 0) {
-            int prev;
-            asm volatile("atom.add.acq_rel.gpu.global.s32 %0, [%1], 1;" : "=r"(prev) : "l"(cnt) : "memory");
-            last_s = prev == n_con - 1;
-          }
-          epi_sync();
-          write = last_s != 0;  // all the others arrived in the meantime
-        }
-        epi_sync();
-        if (write && tid == 0) *cnt = 0;  // ready for the next launch
-      }
-      const int me = pair - first;
-      // the other contributors' parts (NO of them at most) come in batches of NT tokens and are added in the order of the pairs
-      auto add_parts = [&](auto tokens, auto others, int c0, float (&v)[16]) {
-        constexpr int NT = decltype(tokens)::value, NO = decltype(others)::value;
-#pragma unroll
-        for (int h = 0; h < 16; h += NT) {
-          float w[NO][NT];
-#pragma unroll
-          for (int c = 0; c < NO; ++c) {
-            const float* src = part_of(first + (c + 1 < n_con ? c + (c >= me) : 0)) + (size_t)(c0 + h) * kFeat + feat;
-#pragma unroll
-            for (int i = 0; i < NT; ++i) w[c][i] = c + 1 < n_con && c0 + h + i < ntok ? __ldcg(src + i * kFeat) : 0.f;
-          }
-#pragma unroll
-          for (int i = 0; i < NT; ++i) {
-            float acc = 0.f;
-#pragma unroll
-            for (int c = 0; c <= NO; ++c) {
-              if (c == me) acc += v[h + i];
-              if (c < NO) acc += w[c][i];
-            }
-            v[h + i] = acc;
-          }
-        }
-      };
-      for (int h0 = 0; h0 < ntok; h0 += p.stage_tok) {  // as many tokens at a time as the staging holds
-      const int h1 = min(h0 + p.stage_tok, ntok);
-      auto stage16 = [&](const float* v, int c0) {
-        __half* o = reinterpret_cast<__half*>(out_s + (size_t)(c0 - h0) * kStagePitch) + feat;
-#pragma unroll
-        for (int i = 0; i < 16; ++i) o[i * (kStagePitch / 2)] = __float2half_rn(v[i]);
-      };
-      if (write) {
-#pragma unroll 1
-        for (int c0 = h0 + 32 * half; c0 < h1; c0 += 64) {
-          if (!split) {
-            float v[32];
-            tmem_ld_x32(col + c0, reinterpret_cast<uint32_t*>(v));
-            tmem_ld_wait_x32(reinterpret_cast<uint32_t*>(v));
-            if (n_part > 1) add_own(v, c0, Int<32>{});
-            stage16(v, c0);
-            stage16(v + 16, c0 + 16);
-          } else {
-#pragma unroll 1
-            for (int h = c0; h < min(c0 + 32, h1); h += 16) {
-              float v[16];
-              tmem_ld_x16(col + h, reinterpret_cast<uint32_t*>(v));
-              tmem_ld_wait_x16(reinterpret_cast<uint32_t*>(v));
-              if (n_part > 1) add_own(v, h, Int<16>{});
-              if (n_con == 2) add_parts(Int<16>{}, Int<1>{}, h, v);
-              else add_parts(Int<8>{}, Int<kMaxParts - 1>{}, h, v);
-              stage16(v, h);
-            }
-          }
-        }
-      }
-      if (h1 == ntok) {
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) arrive_leader(&d_empty[last_b]);  // the accumulator may be overwritten
-      }
-      if (!write) continue;
-      epi_sync();
-      const size_t trow = (size_t)tl.rowoff + tl.t0;
-      if (p.act) {
-        const int F = p.seg[0].n_rows, f0 = tl.row0 + (int)rank * 64;
-        const int c = (tid & 7) * 8;
-        const int live = F - f0 - c;  // F is a multiple of 8: a run of eight is live or not
-        if (live > 0) {
+      // The staged tokens h0 .. h1-1 (rows row0 ..) to memory, by N threads.
+      auto write_out = [&](auto n_thr, int id, int h0, int h1, int row0) {
+        constexpr int N = decltype(n_thr)::value;
+        const uint8_t* rows = out_s + (size_t)row0 * kStagePitch;
+        const size_t trow = (size_t)tl.rowoff + tl.t0;
+        if (p.act) {
+          const int F = p.seg[0].n_rows, f0 = tl.row0 + (int)rank * 64;
+          const int c = (id & 7) * 8;
+          const int live = F - f0 - c;  // F is a multiple of 8: a run of eight is live or not
+          if (live > 0) {
 #pragma unroll 2
-          for (int t = h0 + (tid >> 3); t < h1; t += 32) {
-            const uint4 g4 = *reinterpret_cast<const uint4*>(out_s + (size_t)(t - h0) * kStagePitch + c * 2);
-            const uint4 u4 = *reinterpret_cast<const uint4*>(out_s + (size_t)(t - h0) * kStagePitch + 128 + c * 2);
-            const uint32_t gw[4] = {g4.x, g4.y, g4.z, g4.w}, uw[4] = {u4.x, u4.y, u4.z, u4.w};
-            uint32_t a[4];
+            for (int t = h0 + (id >> 3); t < h1; t += N / 8) {
+              const uint4 g4 = *reinterpret_cast<const uint4*>(rows + (size_t)(t - h0) * kStagePitch + c * 2);
+              const uint4 u4 = *reinterpret_cast<const uint4*>(rows + (size_t)(t - h0) * kStagePitch + 128 + c * 2);
+              const uint32_t gw[4] = {g4.x, g4.y, g4.z, g4.w}, uw[4] = {u4.x, u4.y, u4.z, u4.w};
+              uint32_t a[4];
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-              const float2 g = __half22float2(as_h2(gw[q])), u = __half22float2(as_h2(uw[q]));
-              a[q] = as_u32(__floats2half2_rn(silu_times(g.x, u.x), silu_times(g.y, u.y)));
-            }
-            *reinterpret_cast<uint4*>(p.act + (trow + t) * p.ldact + f0 + c) = make_uint4(a[0], a[1], a[2], a[3]);
-            if (p.y) {
-              *reinterpret_cast<uint4*>(p.y + (trow + t) * p.ldy + f0 + c) = g4;
-              *reinterpret_cast<uint4*>(p.y + (trow + t) * p.ldy + F + f0 + c) = u4;
+              for (int q = 0; q < 4; ++q) {
+                const float2 g = __half22float2(as_h2(gw[q])), u = __half22float2(as_h2(uw[q]));
+                a[q] = as_u32(__floats2half2_rn(silu_times(g.x, u.x), silu_times(g.y, u.y)));
+              }
+              *reinterpret_cast<uint4*>(p.act + (trow + t) * p.ldact + f0 + c) = make_uint4(a[0], a[1], a[2], a[3]);
+              if (p.y) {
+                *reinterpret_cast<uint4*>(p.y + (trow + t) * p.ldy + f0 + c) = g4;
+                *reinterpret_cast<uint4*>(p.y + (trow + t) * p.ldy + F + f0 + c) = u4;
+              }
             }
           }
+          return;
         }
-      } else {
         const int r0 = tl.row0 + (int)rank * kFeat;
         const int live = min(kFeat, p.seg[tl.sg].n_rows - r0);
         const int colbase = p.seg[tl.sg].col0 + r0;
         const bool vec = (p.ldy % 8 == 0) && (colbase % 8 == 0) &&
                          (((reinterpret_cast<uintptr_t>(p.y) | reinterpret_cast<uintptr_t>(p.res) | reinterpret_cast<uintptr_t>(p.y2)) & 15) == 0);
-        const int c = (tid & 15) * 8;
+        const int c = (id & 15) * 8;
         if (vec && c + 8 <= live) {
-          for (int tb = h0 + (tid >> 4); tb < h1; tb += 64) {
+          for (int tb = h0 + (id >> 4); tb < h1; tb += N / 4) {
             // four tokens at a time, their residuals requested before anything is stored
             uint4 r4[4];
             if (p.res) {
 #pragma unroll
               for (int q = 0; q < 4; ++q)
-                if (tb + 16 * q < h1) r4[q] = __ldg(reinterpret_cast<const uint4*>(p.res + (trow + tb + 16 * q) * p.ldy + colbase + c));
+                if (tb + N / 16 * q < h1) r4[q] = __ldg(reinterpret_cast<const uint4*>(p.res + (trow + tb + N / 16 * q) * p.ldy + colbase + c));
             }
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
-              const int t = tb + 16 * q;
+              const int t = tb + N / 16 * q;
               if (t >= h1) break;
-              const uint4 o4 = *reinterpret_cast<const uint4*>(out_s + (size_t)(t - h0) * kStagePitch + c * 2);
+              const uint4 o4 = *reinterpret_cast<const uint4*>(rows + (size_t)(t - h0) * kStagePitch + c * 2);
               const size_t off = (trow + t) * p.ldy + colbase + c;
               *reinterpret_cast<uint4*>(p.y + off) = o4;
               if (p.res) {
@@ -882,8 +772,8 @@ __global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid
             }
           }
         } else if (c < live) {
-          for (int t = h0 + (tid >> 4); t < h1; t += 16) {
-            const __half* o = reinterpret_cast<const __half*>(out_s + (size_t)(t - h0) * kStagePitch) + c;
+          for (int t = h0 + (id >> 4); t < h1; t += N / 16) {
+            const __half* o = reinterpret_cast<const __half*>(rows + (size_t)(t - h0) * kStagePitch) + c;
             const size_t off = (trow + t) * p.ldy + colbase + c;
             for (int q = 0; q < min(8, live - c); ++q) {
               p.y[off + q] = o[q];
@@ -891,9 +781,106 @@ __global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid
             }
           }
         }
+      };
+      if (st.u0 == 0 && st.u1 == p.units) {  // a whole tile, as many tokens at a time as the staging holds
+        for (int h0 = 0; h0 < ntok; h0 += p.stage_tok) {
+          const int h1 = min(h0 + p.stage_tok, ntok);
+#pragma unroll 1
+          for (int c0 = h0 + 32 * half; c0 < h1; c0 += 64) {
+            float v[32];
+            tmem_ld_x32(col + c0, reinterpret_cast<uint32_t*>(v));
+            tmem_ld_wait_x32(reinterpret_cast<uint32_t*>(v));
+            if (n_part > 1) add_own(v, c0, Int<32>{});
+            stage(v, Int<32>{}, c0 - h0);
+          }
+          if (h1 == ntok) {
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) arrive_leader(&d_empty[last_b]);  // the accumulator may be overwritten
+          }
+          epi_sync();
+          write_out(Int<256>{}, tid, h0, h1, 0);
+          epi_sync();  // the staging may be filled again
+        }
+        continue;
       }
-      epi_sync();  // the staging may be filled again
+      // ---- A split tile.  Its contributors are the pairs whose ranges meet it: pair q holds units n q / P .. n (q + 1) / P - 1, so unit u
+      // lies with q = ((u + 1) P - 1) / n.  Each leaves its part in the scratch, 32 tokens at a time, and counts itself in for these
+      // tokens; the last one to do so adds their parts up in ascending k order and writes them.  The contributors, which finish at
+      // about the same time, begin with different tokens, so that each is the last for some of them (4-bit, 4096 x 14336 in four parts: 77
+      // tokens 28.6 -> 25.1 us, 256 tokens in two parts 46.9 -> 40.2, against one contributor that sums the whole tile).  The warps of even
+      // and odd runs of tokens go their own ways.
+      const long long n_units = (long long)(p.n_ft * p.n_tt - p.n_whole) * p.units, lo = (long long)(st.tile - p.n_whole) * p.units;
+      const int first = (int)(((lo + 1) * p.split_pairs - 1) / n_units);
+      const int n_con = (int)(((lo + p.units) * p.split_pairs - 1) / n_units) - first + 1;
+      auto part_of = [&](int q) {  // this CTA's half of what pair q leaves of the tile
+        // (the first contributor begins the tile, the others come upon it at the start of their range)
+        return p.partial + ((size_t)(p.slots2 && q == first ? p.split_pairs + q : q) * 2 + rank) * kFeat * p.slot_tok + feat;
+      };
+      auto half_sync = [&] { asm volatile("bar.sync %0, 128;" ::"r"(3 + half) : "memory"); };
+      unsigned* cnt = reinterpret_cast<unsigned*>(p.counters) + 2 * first + rank;  // four bits for every 32 tokens
+      const int n_run = ((ntok + 31) / 32 - half + 1) / 2;  // runs of this half
+      const int turn = (pair - first) * n_run / n_con;
+      {
+        float* dst = part_of(pair);
+        uint32_t prev = 0;
+        int mine_j = -1;
+#pragma unroll 1
+        for (int i = 0; i < n_run; ++i) {
+          const int j = turn + i < n_run ? turn + i : turn + i - n_run, c0 = 64 * j + 32 * half;
+          float v[32];
+          tmem_ld_x32(col + c0, reinterpret_cast<uint32_t*>(v));
+          tmem_ld_wait_x32(reinterpret_cast<uint32_t*>(v));
+          if (n_part > 1) add_own(v, c0, Int<32>{});
+#pragma unroll
+          for (int t = 0; t < 32; ++t)
+            if (c0 + t < ntok) __stcg(dst + (size_t)(c0 + t) * kFeat, v[t]);
+          half_sync();  // the run's words are written: one thread releases them (another warp's each time: nobody waits for the count)
+          if (quarter == i && lane == 0) {
+            mine_j = j;
+            asm volatile("atom.add.release.gpu.global.u32 %0, [%1], %2;" : "=r"(prev) : "l"(cnt), "r"(1u << (4 * (2 * j + half))) : "memory");
+          }
+        }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) arrive_leader(&d_empty[last_b]);  // the accumulator may be overwritten
+        if (mine_j >= 0) {
+          const int at = 4 * (2 * mine_j + half);
+          const bool last = ((prev >> at) & 15u) == (uint32_t)(n_con - 1);
+          asm volatile("fence.acq_rel.gpu;" ::: "memory");
+          if (last) atomicSub(cnt, (uint32_t)n_con << at);  // ready for the next launch
+          last_s[half][mine_j] = last;
+        }
+        half_sync();
       }
+#pragma unroll 1
+      for (int j = 0; j < n_run; ++j) {
+        if (!last_s[half][j]) continue;
+        const int c0 = 64 * j + 32 * half, c1 = min(c0 + 32, ntok), row = 32 * half;
+#pragma unroll 1
+        for (int h = c0; h < c1; h += 16) {
+          float v[16];
+#pragma unroll
+          for (int i = 0; i < 16; ++i) v[i] = 0.f;
+#pragma unroll 1
+          for (int q = 0; q < n_con; q += 2) {  // two parts' words on their way at a time
+            const float *s0 = part_of(first + q) + (size_t)h * kFeat, *s1 = part_of(first + min(q + 1, n_con - 1)) + (size_t)h * kFeat;
+            float w0[16], w1[16];
+#pragma unroll
+            for (int i = 0; i < 16; ++i) {
+              w0[i] = h + i < ntok ? __ldcg(s0 + i * kFeat) : 0.f;
+              w1[i] = h + i < ntok && q + 1 < n_con ? __ldcg(s1 + i * kFeat) : 0.f;
+            }
+#pragma unroll
+            for (int i = 0; i < 16; ++i) v[i] = (v[i] + w0[i]) + w1[i];
+          }
+          stage(v, Int<16>{}, row + h - c0);
+        }
+        half_sync();
+        write_out(Int<128>{}, tid & 127, c0, c1, row);
+        half_sync();  // the staging may be filled again
+      }
+      epi_sync();
     }
   }
   __syncwarp();
@@ -946,7 +933,7 @@ PairPlan pair_plan(const int* rows, int n_seg, bool act, int T, int K, bool w16,
     const int n_tt = (T + most - 1) / most;
     if (most == 512 ? !w16 || T <= 256 || n_ft * n_tt > max_pairs : n_tt == last) continue;
     last = most == 512 ? 0 : n_tt;
-    const int nt = most == 512 ? 512 : ((T + n_tt - 1) / n_tt + 31) / 32 * 32;
+    const int nt = most == 512 ? 512 : ((T + n_tt - 1) / n_tt + 15) / 16 * 16;
     const uint64_t slot = 2ull * kFeat * std::min(nt, T) * 4;
     // (fp16 tiles of 512 tokens: the weights serve two operands, but nothing runs under the epilogue and the ring is four steps deep.  Where
     // they make one wave they are the faster ones: 4096 x 14336 over 2048 tokens 204 -> 186 us, 14336 x 4096 over 512 67 -> 55; in several
@@ -957,7 +944,7 @@ PairPlan pair_plan(const int* rows, int n_seg, bool act, int T, int K, bool w16,
     const double flush = w16 ? 1.1 : nt <= 128 ? 2.6 : 4.6;
     const int tok = std::min(nt, T), batches = tok <= 16 ? 1 : (tok + 63) / 64 * 2;  // (16 tokens a batch and warp, two warps side by side)
     auto stretch = [&](double len) { return len * unit + (std::ceil(len / max_units) - 1) * flush + tile; };
-    auto sum = [&](double con) { return (w16 ? 1.0 : 1.3) + batches * (w16 ? (con > 2 ? 2.7 : 1.6) : (con > 2 ? 2.5 : 1.3)); };
+    auto sum = [&](double con) { return w16 ? 1.0 + batches * (con > 2 ? 2.7 : 1.6) : 1.0 + 0.25 * batches + 0.3 * con; };
     // whole tiles in waves of one per pair; the rest, `rem`, whole in a wave of its own or divided over n pairs, `len` units each
     const int tiles = n_ft * n_tt, waves = tiles / max_pairs, rem = tiles % max_pairs;
     auto take = [&](double us, double len, int n, int slots) {
@@ -1050,7 +1037,7 @@ cudaError_t launch_gemm_pair(const GemmParams& g, int sm_count, cudaStream_t st,
   if (g.grp_off) {
     if (g.n_groups <= 0 || g.grp_max_rows <= 0) return cudaErrorInvalidValue;
     p.n_tt = (g.grp_max_rows + 255) / 256;
-    p.nt = ((g.grp_max_rows + p.n_tt - 1) / p.n_tt + 31) / 32 * 32;
+    p.nt = ((g.grp_max_rows + p.n_tt - 1) / p.n_tt + 15) / 16 * 16;
     p.ft_per = n_ft;
     p.n_ft = n_ft * g.n_groups;
     p.pairs = (int)std::min<long long>((long long)p.n_ft * p.n_tt, max_pairs);
@@ -1127,8 +1114,8 @@ cudaError_t launch_gemm_pair(const GemmParams& g, int sm_count, cudaStream_t st,
     p.xs = (int)std::min<size_t>(kMaxX, (kMost - fixed) / step);
     smem = fixed + p.xs * step;
   } else {  // three activation stages and a code ring twice as deep as the weight stages, then more activations
-    p.stage_tok = p.nt;
-    const size_t fixed = 1024 + (size_t)p.nt * kStagePitch, xs = (size_t)p.nt * 128, cs = kCodeBytes + kScaleBytes;
+    p.stage_tok = (p.nt + 31) / 32 * 32;
+    const size_t fixed = 1024 + (size_t)p.stage_tok * kStagePitch, xs = (size_t)p.nt * 128, cs = kCodeBytes + kScaleBytes;
     p.stages = fixed + 3 * xs + 8 * cs <= kMost ? 4 : 3;
     p.codes = 2 * p.stages;
     p.xs = (int)std::min<size_t>(kMaxX, (kMost - fixed - p.codes * cs) / xs);

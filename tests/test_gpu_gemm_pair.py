@@ -40,6 +40,33 @@ def test_gemm_edges_match_oracle(fmt, N, K, T):
     assert np.array_equal(outs[0].view(np.uint16), outs[1].view(np.uint16))
 
 
+# Split tiles are summed 32 tokens at a time by whichever contributor comes last for them: token counts around the runs of 32 and the two
+# halves of the epilogue, two to four contributors, one and two accumulators.
+@pytest.mark.parametrize("N,K", [(2816, 4096), (4096, 6016)])
+@pytest.mark.parametrize("T", [31, 33, 64, 65, 97, 130, 225, 256])
+def test_split_tiles_match_oracle_in_every_run_of_tokens(N, K, T):
+    import torch
+    from paper_2607_10183_b200 import binding as B
+    packed, scales = W.q4_packed(96, 0, W.ROLE_UP, N, K)
+    x = W.activations(96, 0, (T, K))
+    ws = 8 * T * N * 4 + 2 * MB
+    ctx = B.Context(ws + W.q4_bytes(N, K) + 2 * MB, workspace_bytes=ws)
+    tid = ctx.register_q4(packed, scales)
+    ctx.set_placement([(tid, -1, B.ATS_GPU)])
+    xd = H.to_dev(x)
+    outs = []
+    for _ in range(3):  # whoever is last adds in the same order
+        y = torch.full((T + 1, N), 7.0, dtype=torch.float16, device="cuda")
+        ctx.linear(tid, xd, y, T)
+        ctx.sync()
+        outs.append(y.cpu().numpy().view(np.uint16))
+    ctx.close()
+    rows = np.unique(np.r_[np.arange(0, T, 32), np.arange(31, T, 32), T - 1])
+    H.assert_close(outs[0].view(np.float16)[rows], O.linear(x[rows], packed, scales, O.WEIGHT_F16, round_out=True), what=f"{N}x{K} T={T}")
+    assert np.all(outs[0].view(np.float16)[T] == 7.0)
+    assert np.array_equal(outs[0], outs[1]) and np.array_equal(outs[0], outs[2])
+
+
 # fp16 weights: K around the 64-k step and the 128-k unit (multiples of 8), the same edges of N and T, tiles of up to 256 tokens in
 # two accumulators, in several parts and with several contributors, and more tiles than pairs with a remainder
 @pytest.mark.parametrize("N,K,T", [(1, 8, 9), (127, 56, 31), (129, 72, 33), (255, 136, 255), (257, 200, 256), (256, 256, 257), (300, 1000, 513),
