@@ -102,10 +102,13 @@ __device__ __forceinline__ uint32_t cta_rank() {
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
   return r;
 }
+__device__ __forceinline__ void pair_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void pair_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 __device__ __forceinline__ void pair_sync() {
-  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  pair_arrive();
+  pair_wait();
 }
+__device__ __forceinline__ void prefetch_map(const CUtensorMap* map) { asm volatile("prefetch.tensormap [%0];" ::"l"(map) : "memory"); }
 // arrival on the leader's copy of a barrier (from either CTA)
 __device__ __forceinline__ void arrive_leader(uint64_t* own) {
   uint32_t a;
@@ -312,6 +315,13 @@ __global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid
   constexpr uint32_t kAcc = FMT == kFmtW16 ? 256 : 128;
   const int sc_pitch = p.sc16 ? 16 : 12;
 
+  if (warp == 4 && lane == 0) {
+    prefetch_map(&xmap);
+    for (int i = 0; i < p.n_seg; ++i) {
+      prefetch_map(&wmap.codes[i]);
+      if (p.sc16) prefetch_map(&wmap.scales[i]);
+    }
+  }
   if (threadIdx.x == 0) {
     for (int s = 0; s < S; ++s) {
       mbar_init(&afull[s], 8);      // (leader) four dequantization warps of each CTA
@@ -400,23 +410,24 @@ __global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid
       if (++ld_cs == NC) ld_cs = 0, ld_par ^= 1u;
     }
   };
-  if (FMT != kFmtW16 && (warp == 2 || warp == 3)) {
-    asm volatile("bar.sync 2, 64;" ::: "memory");  // the barriers are initialised
-    __syncwarp();
-    if (p.grp_off) asm volatile("griddepcontrol.wait;" ::: "memory");
-    load_units(min(4, NC));
-  }
+  // The weights do not depend on the preceding kernel; the activations (and the grouped form's row offsets) do.  What the
+  // epilogue touches is ordered behind the activation loads.  Whoever has something to wait for or to request does so between its arrival
+  // and its wait for the other CTA (with the first requests ahead of the arrival the CTAs met 1.5 us later, and the activations were
+  // requested another 2 us after that).
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_s)), "r"(512u) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
   }
+  if (FMT != kFmtW16 && (warp == 2 || warp == 3)) asm volatile("bar.sync 2, 64;" ::: "memory");  // the loaders' barriers are initialised
   tc_fence_before();
-  pair_sync();
+  __syncwarp();
+  pair_arrive();
+  if (warp == 0 || p.grp_off) asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (FMT != kFmtW16 && (warp == 2 || warp == 3)) load_units(min(4, NC));
+  __syncwarp();
+  pair_wait();
   tc_fence_after();
   const uint32_t tmem = tmem_s;
-  // The weights do not depend on the preceding kernel; the activations (and the grouped form's row offsets) do.  What the
-  // epilogue touches is ordered behind the activation loads.
-  if (warp == 0 || p.grp_off) asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
   // 72 registers a thread at launch; the epilogue's sums need more: 56 + 4 x 64 + 2 x 96 = 7 x 72
