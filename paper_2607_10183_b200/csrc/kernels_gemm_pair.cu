@@ -77,6 +77,7 @@ struct PairParams {
   int n_whole;        // tiles that a pair has to itself; the units of the others are divided over ...
   int split_pairs;    // ... this many pairs
   int stages, codes, xs;  // depths of the rings: weights in tensor memory, codes (a multiple of it), activations
+  int xu;             // units of activations that a place in their ring holds
   int sc16;           // scale rows are 16-byte aligned
   __half* y;
   int ldy;
@@ -172,6 +173,23 @@ __device__ __forceinline__ void cp_async4z(uint32_t dst, const void* src, bool l
 __device__ __forceinline__ void cp_async_arrive(uint64_t* bar) {
   asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
+// (32-bit shared addresses: the pointers into the aligned dynamic array would make generic accesses)
+__device__ __forceinline__ uint4 lds128(uint32_t a) {
+  uint4 v;
+  asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a));
+  return v;
+}
+__device__ __forceinline__ uint2 lds64(uint32_t a) {
+  uint2 v;
+  asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(a));
+  return v;
+}
+__device__ __forceinline__ uint32_t lds32(uint32_t a) {
+  uint32_t v;
+  asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a));
+  return v;
+}
+__device__ __forceinline__ void sts16(uint32_t a, __half v) { asm volatile("st.shared.u16 [%0], %1;" ::"r"(a), "h"(__half_as_ushort(v)) : "memory"); }
 __device__ __forceinline__ __half2 as_h2(uint32_t v) {
   __half2 h;
   *reinterpret_cast<uint32_t*>(&h) = v;
@@ -228,13 +246,13 @@ struct Stretch {
 struct Walk {
   int tile, step, n_whole;  // whole tiles: pair, pair + pairs, ... (neighbours in L2 run at the same time)
   int units;
-  long long at, end;        // the pair's range of the last tiles' units, counted from tile n_whole on
+  unsigned at, end;         // the pair's range of the last tiles' units, counted from tile n_whole on
   __device__ __forceinline__ Walk(const PairParams& p, int pair) {
     units = p.units;
     tile = pair;
     step = p.pairs;
     n_whole = p.n_whole;
-    const long long n = (long long)(p.n_ft * p.n_tt - n_whole) * units;
+    const unsigned n = (unsigned)(p.n_ft * p.n_tt - n_whole) * units;  // (below 74 tiles of 128k units, see gemm_pair_eligible)
     at = pair < p.split_pairs ? n * pair / p.split_pairs : 0;
     end = pair < p.split_pairs ? n * (pair + 1) / p.split_pairs : 0;
   }
@@ -247,10 +265,10 @@ struct Walk {
       return true;
     }
     if (at >= end) return false;
-    const int t = (int)(at / units);
+    const int t = (int)(at / (unsigned)units);
     s.tile = n_whole + t;
-    s.u0 = (int)(at - (long long)t * units);
-    s.u1 = (int)min((long long)units, s.u0 + (end - at));
+    s.u0 = (int)at - t * units;
+    s.u1 = min(units, s.u0 + (int)(end - at));
     at += s.u1 - s.u0;
     return true;
   }
@@ -303,9 +321,9 @@ __global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid
   const int pair = blockIdx.x >> 1;
   const int S = p.stages, NC = p.codes, NX = p.xs;
   const int xbytes = p.nt / 2 * 128;                 // this CTA's activation bytes of a 64-k step
-  uint8_t* x_s = smem;                               // [NX][2][nt / 2 rows][128 bytes], swizzled
+  uint8_t* x_s = smem;                               // [NX][2 xu][nt / 2 rows][128 bytes], swizzled
   const int step_bytes = xbytes + kW16Bytes;         // (fp16 weights: [NX] of a step's activations and weights, nothing else)
-  uint8_t* code_s = x_s + (size_t)NX * (FMT == kFmtW16 ? step_bytes : 2 * xbytes);   // [NC][128 rows][64 bytes], 16-byte pieces swizzled by row pair
+  uint8_t* code_s = x_s + (size_t)NX * (FMT == kFmtW16 ? step_bytes : p.xu * 2 * xbytes);   // [NC][128 rows][64 bytes], 16-byte pieces swizzled by row pair
   uint8_t* scale_s = code_s + (size_t)NC * kCodeBytes;
   uint8_t* out_s = scale_s + (size_t)NC * kScaleBytes;  // [nt][kStagePitch]
   // two accumulators that take turns: of 128 columns beside the weights, of 256 where those are not in tensor memory; a tile of 512
@@ -465,17 +483,16 @@ __global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid
           }
           continue;
         }
-        for (int u = u0; u < u1; ++u) {
+        for (int u = u0; u < u1; u += p.xu) {
           if (n >= NX && !wait_warp(&xempty[s], par)) {
             ok = false;
             break;
           }
           ++n;
-          const bool two = 2 * u + 1 < p.ksteps;
-          const uint32_t dst = x0 + (uint32_t)(s * 2 * xbytes);
-          if (rank == 0) expect_tx_one(one, &xfull[s], (uint32_t)((two ? 4 : 2) * xbytes));
-          tma_pair_2d(one, dst, &xmap, u * 128, row, &xfull[s]);
-          if (two) tma_pair_2d(one, dst + (uint32_t)xbytes, &xmap, u * 128 + 64, row, &xfull[s]);
+          const int n_ks = min(2 * min(u + p.xu, u1), p.ksteps) - 2 * u;
+          const uint32_t dst = x0 + (uint32_t)(s * p.xu * 2 * xbytes);
+          if (rank == 0) expect_tx_one(one, &xfull[s], (uint32_t)(n_ks * 2 * xbytes));
+          for (int j = 0; j < n_ks; ++j) tma_pair_2d(one, dst + (uint32_t)(j * xbytes), &xmap, u * 128 + j * 64, row, &xfull[s]);
           if (++s == NX) s = 0, par ^= 1u;
         }
       }
@@ -486,7 +503,7 @@ __global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid
         const uint32_t idesc = umma_idesc_f16(2 * kFeat, wide ? 256 : p.nt);
         const uint64_t xd = umma_desc_sw128(smem_u32(x_s));
         Walk mine(p, pair);
-        int s = 0, sx = 0, seg = 0;  // places in the rings, accumulator segments so far
+        int s = 0, sx = 0, xi = 0, seg = 0;  // places in the rings, unit of the activations' place, accumulator segments so far
         uint32_t par = 0, parx = 0;
         bool ready = false, readyx = false;
         while (uniform(ok && mine.next(st))) {
@@ -537,17 +554,21 @@ __global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid
               }
               continue;
             }
-            if ((!__all_sync(0xffffffffu, ready) && !wait_warp(&afull[s], par)) ||
-                (!__all_sync(0xffffffffu, readyx) && !wait_warp(&xfull[sx], parx))) {
+            if (!__all_sync(0xffffffffu, ready) && !wait_warp(&afull[s], par)) {
+              ok = false;
+              break;
+            }
+            if (xi == 0 && !__all_sync(0xffffffffu, readyx) && !wait_warp(&xfull[sx], parx)) {
               ok = false;
               break;
             }
             tc_fence_after();
             const int sn = s + 1 == S ? 0 : s + 1, sxn = sx + 1 == NX ? 0 : sx + 1;
             const uint32_t parn = s + 1 == S ? par ^ 1u : par, parxn = sx + 1 == NX ? parx ^ 1u : parx;
+            const bool xlast = xi + 1 == p.xu || u + 1 == u1;  // the place in the activations' ring is done with
             ready = peek(&afull[sn], parn);
-            readyx = peek(&xfull[sxn], parxn);
-            const uint64_t bd = xd + (uint64_t)((uint32_t)sx * 2u * (uint32_t)(xbytes >> 4));
+            if (xlast) readyx = peek(&xfull[sxn], parxn);
+            const uint64_t bd = xd + (uint64_t)((uint32_t)(sx * p.xu + xi) * 2u * (uint32_t)(xbytes >> 4));
             const uint32_t at = kColA + 64u * s;  // (all 512 columns are this CTA's: the allocation starts at 0)
 #pragma unroll
             for (int kk = 0; kk < 4; ++kk) umma_ts_pair(one, d, at + 8u * kk, bd + (uint64_t)(2 * kk), idesc, kk > 0 ? 1u : accumulate);
@@ -558,13 +579,14 @@ __global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid
             }
             accumulate = 1;
             umma_commit_both(one, &aempty[s]);
-            umma_commit_both(one, &xempty[sx]);
+            if (xlast) umma_commit_both(one, &xempty[sx]);
             if (--left == 0) {
               umma_commit_both(one, &acc_full[two ? seg & 1 : 0]);
               ++seg;
             }
             s = sn, par = parn;
-            sx = sxn, parx = parxn;
+            xi = xlast ? 0 : xi + 1;
+            if (xlast) sx = sxn, parx = parxn;
           }
         }
       }
@@ -584,8 +606,7 @@ __global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid
     const int row = quarter * 32 + lane;
     const int nblk = p.K / 32;
     const uint32_t a_col = tmem + ((uint32_t)(quarter * 32) << 16) + kColA + 64u * grp;
-    const uint8_t* code_row = code_s + row * 64;
-    const uint8_t* scale_row = scale_s + row * sc_pitch;
+    const uint32_t code_row = smem_u32(code_s) + (uint32_t)(row * 64), scale_row = smem_u32(scale_s) + (uint32_t)(row * sc_pitch);
     const uint32_t swz = (uint32_t)((row >> 1) & 3) << 4;
     Walk mine(p, pair);
     int skip = grp;               // units until this group's next
@@ -603,14 +624,12 @@ __global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid
           break;
         }
         const bool free_seen = peek(&aempty[grp], apar);
-        const uint8_t* cr = code_row + (uint32_t)(cs * kCodeBytes);
-        const uint8_t* sr = scale_row + (uint32_t)(cs * kScaleBytes);
+        const uint32_t cr = code_row + (uint32_t)(cs * kCodeBytes), sr = scale_row + (uint32_t)(cs * kScaleBytes);
         uint2 sw;  // four scales
         if (p.sc16) {
-          sw = *reinterpret_cast<const uint2*>(sr + (u & 1) * 8);
+          sw = lds64(sr + (uint32_t)(u & 1) * 8);
         } else {
-          const uint32_t w0 = *reinterpret_cast<const uint32_t*>(sr), w1 = *reinterpret_cast<const uint32_t*>(sr + 4),
-                         w2 = *reinterpret_cast<const uint32_t*>(sr + 8);
+          const uint32_t w0 = lds32(sr), w1 = lds32(sr + 4), w2 = lds32(sr + 8);
           sw = odd ? make_uint2(__byte_perm(w0, w1, 0x5432), __byte_perm(w1, w2, 0x5432)) : make_uint2(w0, w1);
           const int left = nblk - u * 4;  // blocks that exist; what follows belongs to the next row
           if (left < 4) sw.y &= left < 3 ? 0u : 0x0000FFFFu;
@@ -622,7 +641,7 @@ __global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid
           const uint32_t pairs = c ? sw.y : sw.x;
 #pragma unroll
           for (int b = 0; b < 2; ++b) {
-            const uint4 q = *reinterpret_cast<const uint4*>(cr + (((uint32_t)(2 * c + b) << 4) ^ swz));
+            const uint4 q = lds128(cr + (((uint32_t)(2 * c + b) << 4) ^ swz));
             const __half2 sc = as_h2(__byte_perm(pairs, 0, b ? 0x3232 : 0x1010));
             expand_word<FMT == kFmtMx>(q.x, sc, o + 16 * b);
             expand_word<FMT == kFmtMx>(q.y, sc, o + 16 * b + 4);
@@ -659,7 +678,7 @@ __global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid
     const int half = (warp - 4) >> 2;        // two warps per quarter: even and odd runs of 32 tokens
     const int tid = threadIdx.x - 128;       // 0..255
     const int feat = quarter * 32 + lane;    // this thread's feature of the CTA's 128
-    const uint32_t d_col = tmem + ((uint32_t)(quarter * 32) << 16);
+    const uint32_t d_col = tmem + ((uint32_t)(quarter * 32) << 16), out_u = smem_u32(out_s);
     auto epi_sync = [] { asm volatile("bar.sync 1, 256;" ::: "memory"); };
     auto epi_all = [](bool v) {
       uint32_t r;
@@ -714,14 +733,14 @@ __global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid
       const int last_b = two ? seg & 1 : 0;
       ++seg;
       auto stage = [&](const float* v, auto n_tok, int row) {  // this thread's feature of n_tok tokens
-        __half* o = reinterpret_cast<__half*>(out_s + (size_t)row * kStagePitch) + feat;
+        const uint32_t o = out_u + (uint32_t)(row * kStagePitch + 2 * feat);
 #pragma unroll
-        for (int i = 0; i < decltype(n_tok)::value; ++i) o[i * (kStagePitch / 2)] = __float2half_rn(v[i]);
+        for (int i = 0; i < decltype(n_tok)::value; ++i) sts16(o + (uint32_t)(i * kStagePitch), __float2half_rn(v[i]));
       };
       // The staged tokens h0 .. h1-1 (rows row0 ..) to memory, by N threads.
       auto write_out = [&](auto n_thr, int id, int h0, int h1, int row0) {
         constexpr int N = decltype(n_thr)::value;
-        const uint8_t* rows = out_s + (size_t)row0 * kStagePitch;
+        const uint32_t rows = out_u + (uint32_t)(row0 * kStagePitch);
         const size_t trow = (size_t)tl.rowoff + tl.t0;
         if (p.act) {
           const int F = p.seg[0].n_rows, f0 = tl.row0 + (int)rank * 64;
@@ -730,8 +749,8 @@ __global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid
           if (live > 0) {
 #pragma unroll 2
             for (int t = h0 + (id >> 3); t < h1; t += N / 8) {
-              const uint4 g4 = *reinterpret_cast<const uint4*>(rows + (size_t)(t - h0) * kStagePitch + c * 2);
-              const uint4 u4 = *reinterpret_cast<const uint4*>(rows + (size_t)(t - h0) * kStagePitch + 128 + c * 2);
+              const uint4 g4 = lds128(rows + (uint32_t)((t - h0) * kStagePitch + c * 2));
+              const uint4 u4 = lds128(rows + (uint32_t)((t - h0) * kStagePitch + 128 + c * 2));
               const uint32_t gw[4] = {g4.x, g4.y, g4.z, g4.w}, uw[4] = {u4.x, u4.y, u4.z, u4.w};
               uint32_t a[4];
 #pragma unroll
@@ -767,7 +786,7 @@ __global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid
             for (int q = 0; q < 4; ++q) {
               const int t = tb + N / 16 * q;
               if (t >= h1) break;
-              const uint4 o4 = *reinterpret_cast<const uint4*>(rows + (size_t)(t - h0) * kStagePitch + c * 2);
+              const uint4 o4 = lds128(rows + (uint32_t)((t - h0) * kStagePitch + c * 2));
               const size_t off = (trow + t) * p.ldy + colbase + c;
               *reinterpret_cast<uint4*>(p.y + off) = o4;
               if (p.res) {
@@ -784,7 +803,7 @@ __global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid
           }
         } else if (c < live) {
           for (int t = h0 + (id >> 4); t < h1; t += N / 16) {
-            const __half* o = reinterpret_cast<const __half*>(rows + (size_t)(t - h0) * kStagePitch) + c;
+            const __half* o = reinterpret_cast<const __half*>(out_s + (size_t)(row0 + t - h0) * kStagePitch) + c;
             const size_t off = (trow + t) * p.ldy + colbase + c;
             for (int q = 0; q < min(8, live - c); ++q) {
               p.y[off + q] = o[q];
@@ -821,7 +840,7 @@ __global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid
       // about the same time, begin with different tokens, so that each is the last for some of them (4-bit, 4096 x 14336 in four parts: 77
       // tokens 28.6 -> 25.1 us, 256 tokens in two parts 46.9 -> 40.2, against one contributor that sums the whole tile).  The warps of even
       // and odd runs of tokens go their own ways.
-      const long long n_units = (long long)(p.n_ft * p.n_tt - p.n_whole) * p.units, lo = (long long)(st.tile - p.n_whole) * p.units;
+      const unsigned n_units = (unsigned)(p.n_ft * p.n_tt - p.n_whole) * p.units, lo = (unsigned)(st.tile - p.n_whole) * p.units;
       const int first = (int)(((lo + 1) * p.split_pairs - 1) / n_units);
       const int n_con = (int)(((lo + p.units) * p.split_pairs - 1) / n_units) - first + 1;
       auto part_of = [&](int q) {  // this CTA's half of what pair q leaves of the tile
@@ -994,7 +1013,7 @@ PairPlan plan_of(const GemmParams& g, int sm_count) {
 }  // namespace
 
 bool gemm_pair_eligible(const GemmParams& g, int sm_count) {
-  if ((g.w16 && g.grp_off) || g.n_seg < 1 || g.n_seg > 3 || !g.counters || g.K % (g.w16 ? 8 : 32) || g.ldx % 8) return false;
+  if ((g.w16 && g.grp_off) || g.n_seg < 1 || g.n_seg > 3 || !g.counters || g.K % (g.w16 ? 8 : 32) || g.K > (1 << 24) || g.ldx % 8) return false;
   if (reinterpret_cast<uintptr_t>(g.x) & 15) return false;
   if ((g.res != nullptr) != (g.y2 != nullptr)) return false;
   for (int i = 0; i < g.n_seg; ++i) {
@@ -1126,7 +1145,9 @@ cudaError_t launch_gemm_pair(const GemmParams& g, int sm_count, cudaStream_t st,
     smem = fixed + p.xs * step;
   } else {  // three activation stages and a code ring twice as deep as the weight stages, then more activations
     p.stage_tok = (p.nt + 31) / 32 * 32;
-    const size_t fixed = 1024 + (size_t)p.stage_tok * kStagePitch, xs = (size_t)p.nt * 128, cs = kCodeBytes + kScaleBytes;
+    const size_t fixed = 1024 + (size_t)p.stage_tok * kStagePitch, cs = kCodeBytes + kScaleBytes;
+    p.xu = p.nt <= 128 ? 2 : 1;
+    const size_t xs = (size_t)p.nt * 128 * p.xu;
     p.stages = fixed + 3 * xs + 8 * cs <= kMost ? 4 : 3;
     p.codes = 2 * p.stages;
     p.xs = (int)std::min<size_t>(kMaxX, (kMost - fixed - p.codes * cs) / xs);
