@@ -729,6 +729,20 @@ static int32_t fetch_ids(ats_ctx* ctx, const int32_t* ids_dev, int P, int E) {
   return ATS_OK;
 }
 
+// Wait until the device has written `seq` to the completion word: a bounded poll (about two seconds), then the stream itself decides.
+static int32_t wait_done(ats_ctx* ctx, int seq) {
+  const auto t0 = std::chrono::steady_clock::now();
+  uint32_t spins = 0;
+  while (*ctx->done_host != seq) {
+    if ((++spins & 0xFFFFu) == 0) {
+      if (cudaStreamQuery(ctx->cs) != cudaErrorNotReady) break;  // finished (or failed) without the word: settle below
+      if (std::chrono::steady_clock::now() - t0 > std::chrono::seconds(2)) break;
+    }
+  }
+  if (*ctx->done_host != seq) ATS_CUDA(cudaStreamSynchronize(ctx->cs));
+  return ATS_OK;
+}
+
 // Plan the streamed slices of an MoE stage set: for each selected expert (ascending) the host-placed gate and up
 // slices, then the host-placed down slices (only selected experts move, Section 4.2.2).
 static void plan_moe(ats_ctx* ctx, const int32_t* ids_host, int P, const int* tensor_ids, int n_first, int n_total) {
@@ -1613,16 +1627,7 @@ int32_t ats_layer_decode_host(ats_ctx* ctx, const ats_layer_desc* L, const void*
     // system-wide fence in every CTA, was measured and is slower: 57.8 against 54.9 us per step.)
     const int seq = ++ctx->done_seq;
     ATS_CUDA(launch_signal_done(ctx->done_dev, seq, (ctx->cfg.flags & ATS_FLAG_NO_PDL) ? 0 : 1, ctx->cs, &ctx->stats.kernel_launches));
-    // bounded poll (about two seconds), then the stream itself decides
-    const auto t0 = std::chrono::steady_clock::now();
-    uint32_t spins = 0;
-    while (*ctx->done_host != seq) {
-      if ((++spins & 0xFFFFu) == 0) {
-        if (cudaStreamQuery(ctx->cs) != cudaErrorNotReady) break;  // finished (or failed) without the word: settle below
-        if (std::chrono::steady_clock::now() - t0 > std::chrono::seconds(2)) break;
-      }
-    }
-    if (*ctx->done_host != seq) ATS_CUDA(cudaStreamSynchronize(ctx->cs));
+    ATS_TRY(wait_done(ctx, seq));
   } else {
     if (!fast) ATS_CUDA(cudaMemcpyAsync(x_out, xout_dev, row_bytes, cudaMemcpyDeviceToHost, ctx->cs));
     ATS_CUDA(cudaStreamSynchronize(ctx->cs));
@@ -1736,23 +1741,35 @@ int32_t ats_layer_prefill(ats_ctx* ctx, const ats_layer_desc* L, const void* x_i
   ATS_CUDA(launch_rmsnorm(resid, 0, (const __half*)ctx->tensors[L->ffn_norm].f16_dev, w.h2_16, (int)T, H, L->rms_eps, ctx->cs, nl, pdl));
   if (moe) {
     // Routed FFN over T tokens: every (token, slot) pair becomes a row; rows are sorted by expert so that each expert's
-    // rows are one contiguous block of a grouped GEMM (one launch for all experts).  The sort runs on the host from the
-    // routing ids (one synchronisation per call); expert slices are read where they are: resident copies, or the pinned
-    // host store through its device mapping for host-placed experts (every slice is read once per 128 of its rows).
+    // rows are one contiguous block of a grouped GEMM (one launch for all experts).  With all experts resident the sort runs on the
+    // device and the call waits for the router only when everything is queued.  Host-placed experts: the host has to know which
+    // of them are wanted, so it sorts, from the routing ids; their slices are read through the device mapping of the pinned store
+    // (every slice once per 128 of its rows).
     const int k = (int)L->top_k, E = (int)L->n_experts, P = (int)T * k, F = (int)L->ffn;
+    const Tensor &tg = ctx->tensors[L->w_gate], &tu = ctx->tensors[L->w_up], &td = ctx->tensors[L->w_down];
+    const bool on_device = tg.contiguous_dev && tu.contiguous_dev && td.contiguous_dev && ctx->done_dev && !(ctx->cfg.flags & ATS_FLAG_NO_GEMM_PAIR);
+    if (on_device) {  // (a wait for the router cannot be captured)
+      cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+      ATS_CUDA(cudaStreamIsCapturing(ctx->cs, &capturing));
+      if (capturing != cudaStreamCaptureStatusNone) ATS_CUDA(cudaErrorStreamCaptureUnsupported);
+    }
     ATS_CUDA(launch_router_topk(w.h2_16, (const __half*)ctx->tensors[L->router].f16_dev, (int)T, H, E, k,
                                 (L->flags & ATS_LAYER_NO_TOPK_RENORM) ? 0 : 1, w.ids, w.gates, ctx->cs, nl, pdl));
-    ATS_TRY(fetch_ids(ctx, w.ids, P, E));
     // the sort's arrays, laid out as the workspace has them, so that one copy takes all three
     int32_t* order_h = ctx->ids_host + kMaxPairs;              // sorted position -> pair
     int32_t* pos_h = order_h + (w.pos - w.order);              // pair -> sorted position
     int32_t* off_h = order_h + (w.grp_off - w.order);          // expert -> first sorted position; [E] = P
-    int max_rows = 0;
-    if (ats_host_group_pairs(ctx->ids_host, (uint32_t)P, (uint32_t)E, order_h, pos_h, off_h, &max_rows) != ATS_OK)
-      return fail(ctx, ATS_ERR_INVALID, "routing ids out of range");
-    ATS_CUDA(cudaMemcpyAsync(w.order, order_h, (size_t)(off_h + E + 1 - order_h) * 4, cudaMemcpyHostToDevice, ctx->cs));
+    int max_rows = 0, seq = 0;
+    if (on_device) {
+      seq = ++ctx->done_seq;
+      ATS_CUDA(launch_moe_group(w.ids, P, E, w.order, w.pos, w.grp_off, ctx->dev_status, ctx->done_dev, seq, ctx->cs, nl, pdl));
+    } else {
+      ATS_TRY(fetch_ids(ctx, w.ids, P, E));
+      if (ats_host_group_pairs(ctx->ids_host, (uint32_t)P, (uint32_t)E, order_h, pos_h, off_h, &max_rows) != ATS_OK)
+        return fail(ctx, ATS_ERR_INVALID, "routing ids out of range");
+      ATS_CUDA(cudaMemcpyAsync(w.order, order_h, (size_t)(off_h + E + 1 - order_h) * 4, cudaMemcpyHostToDevice, ctx->cs));
+    }
     ATS_CUDA(launch_moe_gather_rows(w.h2_16, w.order, k, w.xs16, P, H, ctx->cs, nl, pdl));
-    const Tensor &tg = ctx->tensors[L->w_gate], &tu = ctx->tensors[L->w_up], &td = ctx->tensors[L->w_down];
     auto slice0 = [](const Tensor& t) -> const uint8_t* { return t.contiguous_dev ? t.slices[0].dev : nullptr; };
     // Host-placed experts that some token selected: one SM-driven gather brings their slices into what the workspace has
     // left beyond this layer's buffers, and per-call address tables point the GEMMs there.  Without that room (or
@@ -1840,7 +1857,10 @@ int32_t ats_layer_prefill(ats_ctx* ctx, const ats_layer_desc* L, const void* x_i
     m.ldy = H;
     ATS_TRY(launch_gemm_any(ctx, m));
     ATS_CUDA(launch_moe_combine_sorted(resid, w.gates, w.d16, w.pos, (__half*)x_out, (int)T, k, H, ctx->cs, nl, pdl));
-    return ATS_OK;
+    if (!on_device) return ATS_OK;
+    ATS_TRY(wait_done(ctx, seq));
+    ctx->stats.host_syncs++;
+    return check_status(ctx);
   }
   g.x = w.h2_16;
   g.ldx = H;

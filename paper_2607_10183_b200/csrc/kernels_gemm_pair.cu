@@ -38,6 +38,8 @@
 // bounded; on expiry the CTA raises the status word, skips the rest, and every thread still reaches the closing cluster barrier.
 #include <cuda.h>
 
+#include <cmath>
+
 #include "ats_internal.h"
 #include "sm100_umma.cuh"
 
@@ -94,7 +96,7 @@ struct PairParams {
   int* counters;      // [2 * pairs], zero between launches
   int* status;
   const int* grp_off;  // grouped form: row offsets per expert
-  int ft_per;          // ... feature tiles per expert
+  int ft_per, n_groups, list_at;  // ... feature tiles per expert, experts, place of the list of blocks in shared memory
   unsigned long long grp_stride;
 };
 
@@ -247,12 +249,12 @@ struct Walk {
   int tile, step, n_whole;  // whole tiles: pair, pair + pairs, ... (neighbours in L2 run at the same time)
   int units;
   unsigned at, end;         // the pair's range of the last tiles' units, counted from tile n_whole on
-  __device__ __forceinline__ Walk(const PairParams& p, int pair) {
+  __device__ __forceinline__ Walk(const PairParams& p, int pair, int whole) {
     units = p.units;
     tile = pair;
     step = p.pairs;
-    n_whole = p.n_whole;
-    const unsigned n = (unsigned)(p.n_ft * p.n_tt - n_whole) * units;  // (below 74 tiles of 128k units, see gemm_pair_eligible)
+    n_whole = whole;
+    const unsigned n = p.grp_off ? 0u : (unsigned)(p.n_ft * p.n_tt - whole) * units;  // (below 74 tiles of 128k units, see gemm_pair_eligible)
     at = pair < p.split_pairs ? n * pair / p.split_pairs : 0;
     end = pair < p.split_pairs ? n * (pair + 1) / p.split_pairs : 0;
   }
@@ -276,25 +278,26 @@ struct Walk {
 // Which rows, tokens and expert a tile stands for.
 struct Tile {
   int sg, row0;        // segment, first feature row of the PAIR within it (SwiGLU: first feature of the 128)
-  int t0, T, rowoff;   // first token, tokens of the (expert's) matrix, its first row
+  int t0, T, rowoff;   // first token, tokens of the matrix (of the block of an expert's rows), its first row
   int expert;
-  bool empty;
 };
-__device__ __forceinline__ Tile tile_of(const PairParams& p, int tile) {
+// Grouped form: the experts' rows in blocks of at most nt, in shared memory: {expert | rows << 10, first row}.
+__device__ __forceinline__ Tile tile_of(const PairParams& p, int tile, const int2* blocks) {
   Tile r;
-  int ft = tile / p.n_tt;
-  const int tt = tile - ft * p.n_tt;
-  r.expert = 0;
-  r.T = p.T;
-  r.rowoff = 0;
-  if (p.grp_off) {  // feature tiles of one expert after another
-    r.expert = ft / p.ft_per;
-    ft -= r.expert * p.ft_per;
-    r.rowoff = p.grp_off[r.expert];
-    r.T = p.grp_off[r.expert + 1] - r.rowoff;
+  int ft = tile / (p.grp_off ? p.ft_per : p.n_tt);
+  if (p.grp_off) {  // feature tiles of one block after another
+    const int2 b = blocks[ft];
+    ft = tile - ft * p.ft_per;
+    r.expert = b.x & 1023;
+    r.t0 = 0;
+    r.T = b.x >> 10;
+    r.rowoff = b.y;
+  } else {
+    r.expert = 0;
+    r.t0 = (tile - ft * p.n_tt) * p.nt;
+    r.T = p.T;
+    r.rowoff = 0;
   }
-  r.t0 = tt * p.nt;
-  r.empty = r.t0 >= r.T;
   r.sg = 0;
   if (p.act) {
     r.row0 = ft * kFeat;
@@ -315,7 +318,7 @@ __global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   __shared__ uint64_t afull[kMaxA], aempty[kMaxA], xfull[kMaxX], xempty[kMaxX], cfull[kMaxCodes], cempty[kMaxCodes], acc_full[2], d_empty[2];
   __shared__ uint32_t tmem_s;
-  __shared__ int last_s[2][4];
+  __shared__ int last_s[2][4], n_blocks_s;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t rank = cta_rank();
   const int pair = blockIdx.x >> 1;
@@ -362,11 +365,48 @@ __global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid
     }
     mbar_fence_init();
   }
+  // The weights do not depend on the preceding kernel; the activations (and the grouped form's row offsets) do.  What the
+  // epilogue touches is ordered behind the activation loads.  Whoever has something to wait for or to request does so between its arrival
+  // and its wait for the other CTA (with the first requests ahead of the arrival the CTAs met 1.5 us later, and the activations were
+  // requested another 2 us after that).
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_s)), "r"(512u) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+  }
+  if (FMT != kFmtW16 && (warp == 2 || warp == 3)) asm volatile("bar.sync 2, 64;" ::: "memory");  // the loaders' barriers are initialised
+  tc_fence_before();
+  __syncwarp();
+  pair_arrive();
+  if (warp == 0 || p.grp_off) asm volatile("griddepcontrol.wait;" ::: "memory");
+  // Grouped form: every CTA lists the blocks of rows for itself from the experts' offsets.
+  int2* const blocks = reinterpret_cast<int2*>(smem + p.list_at);
+  int n_whole = p.n_whole;
+  if (p.grp_off) {
+    if (warp == 4) {
+      const int per = (p.n_groups + 31) / 32, e0 = min(lane * per, p.n_groups), e1 = min(e0 + per, p.n_groups);
+      int n = 0, incl;
+      for (int e = e0; e < e1; ++e) n += (p.grp_off[e + 1] - p.grp_off[e] + p.nt - 1) / p.nt;
+      incl = n;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += v;
+      }
+      int at = incl - n;
+      for (int e = e0; e < e1; ++e) {
+        const int hi = p.grp_off[e + 1];
+        for (int r = p.grp_off[e]; r < hi; r += p.nt) blocks[at++] = make_int2(e | min(p.nt, hi - r) << 10, r);
+      }
+      if (lane == 31) n_blocks_s = incl;
+    }
+    __syncthreads();
+    n_whole = n_blocks_s * p.ft_per;
+  }
   // ---- code loads (warp 2) and scale loads (warp 3; both where the scales' rows are not 16-byte aligned).  Weights depend on nothing:
   // the first units are requested before the CTAs of the pair meet, the rest by the loaders' own branch below.
   bool ok = true;
   Stretch st;
-  Walk ld_walk(p, pair);
+  Walk ld_walk(p, pair, n_whole);
   int ld_n = 0, ld_u = 0, ld_end = 0, ld_cs = 0;   // units requested; next and last unit of the current stretch; ring place
   int ld_first = 0, ld_e = 0, ld_sa = 0, ld_sb = 0;
   uint32_t ld_par = 1;
@@ -376,8 +416,7 @@ __global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid
     while (ld_n < upto) {
       if (ld_u == ld_end) {
         if (!uniform(ld_walk.next(st))) return;
-        const Tile tl = tile_of(p, st.tile);
-        if (uniform(tl.empty)) continue;
+        const Tile tl = tile_of(p, st.tile, blocks);
         ld_u = uniform(st.u0);
         ld_end = uniform(st.u1);
         ld_e = uniform(tl.expert);
@@ -428,19 +467,6 @@ __global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid
       if (++ld_cs == NC) ld_cs = 0, ld_par ^= 1u;
     }
   };
-  // The weights do not depend on the preceding kernel; the activations (and the grouped form's row offsets) do.  What the
-  // epilogue touches is ordered behind the activation loads.  Whoever has something to wait for or to request does so between its arrival
-  // and its wait for the other CTA (with the first requests ahead of the arrival the CTAs met 1.5 us later, and the activations were
-  // requested another 2 us after that).
-  if (warp == 1) {
-    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_s)), "r"(512u) : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
-  }
-  if (FMT != kFmtW16 && (warp == 2 || warp == 3)) asm volatile("bar.sync 2, 64;" ::: "memory");  // the loaders' barriers are initialised
-  tc_fence_before();
-  __syncwarp();
-  pair_arrive();
-  if (warp == 0 || p.grp_off) asm volatile("griddepcontrol.wait;" ::: "memory");
   if (FMT != kFmtW16 && (warp == 2 || warp == 3)) load_units(min(4, NC));
   __syncwarp();
   pair_wait();
@@ -454,13 +480,13 @@ __global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid
     if (warp == 0) {
       // ------------------------------------------------------------ activations
       const uint32_t one = elect_one();
-      Walk mine(p, pair);
+      Walk mine(p, pair, n_whole);
       const uint32_t x0 = smem_u32(x_s);
       int s = 0, n = 0;
       uint32_t par = 1;
       while (uniform(ok && mine.next(st))) {
-        const Tile tl = tile_of(p, st.tile);
-        const int u0 = uniform(st.u0), u1 = uniform(tl.empty ? 0 : st.u1);
+        const Tile tl = tile_of(p, st.tile, blocks);
+        const int u0 = uniform(st.u0), u1 = uniform(st.u1);
         const int row = uniform(tl.rowoff + tl.t0 + (int)rank * (p.nt / 2));
         if constexpr (FMT == kFmtW16) {
           const int sa = p.act ? 0 : uniform(tl.sg), sb = p.act ? 1 : sa;
@@ -502,16 +528,15 @@ __global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid
         const uint32_t one = elect_one();
         const uint32_t idesc = umma_idesc_f16(2 * kFeat, wide ? 256 : p.nt);
         const uint64_t xd = umma_desc_sw128(smem_u32(x_s));
-        Walk mine(p, pair);
+        Walk mine(p, pair, n_whole);
         int s = 0, sx = 0, xi = 0, seg = 0;  // places in the rings, unit of the activations' place, accumulator segments so far
         uint32_t par = 0, parx = 0;
         bool ready = false, readyx = false;
         while (uniform(ok && mine.next(st))) {
-          const Tile tl = tile_of(p, st.tile);
-          const int u0 = uniform(st.u0), u1 = uniform(tl.empty ? 0 : st.u1);
+          const Tile tl = tile_of(p, st.tile, blocks);
+          const int u0 = uniform(st.u0), u1 = uniform(st.u1);
           int left = 0;  // units until the accumulator is handed over
           uint32_t d = 0, accumulate = 0;
-          if (u1 == 0) continue;
           const int part = seg_units(p, u1 - u0);
           for (int u = u0; u < u1; ++u) {
             if (left == 0) {
@@ -608,13 +633,12 @@ __global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid
     const uint32_t a_col = tmem + ((uint32_t)(quarter * 32) << 16) + kColA + 64u * grp;
     const uint32_t code_row = smem_u32(code_s) + (uint32_t)(row * 64), scale_row = smem_u32(scale_s) + (uint32_t)(row * sc_pitch);
     const uint32_t swz = (uint32_t)((row >> 1) & 3) << 4;
-    Walk mine(p, pair);
+    Walk mine(p, pair, n_whole);
     int skip = grp;               // units until this group's next
     int cs = grp;                 // its place in the code ring
     uint32_t cpar = 0, apar = 1;  // (the first wait for an empty stage passes at once)
     while (FMT != kFmtW16 && ok && grp < S && mine.next(st)) {
-      const Tile tl = tile_of(p, st.tile);
-      if (tl.empty) continue;
+      const Tile tl = tile_of(p, st.tile, blocks);
       const int first = p.act ? tl.row0 + (int)rank * 64 + (row & 63) : tl.row0 + (int)rank * kFeat + row;
       const int odd = p.sc16 ? 0 : (int)(((long long)first * nblk) & 1);  // units start at even offsets: the row decides
       int u = st.u0 + skip;
@@ -688,11 +712,10 @@ __global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid
                    : "memory");
       return r != 0;
     };
-    Walk mine(p, pair);
+    Walk mine(p, pair, n_whole);
     int seg = 0;
     while (ok && mine.next(st)) {
-      const Tile tl = tile_of(p, st.tile);
-      if (tl.empty) continue;
+      const Tile tl = tile_of(p, st.tile, blocks);
       const int ntok = min(p.nt, tl.T - tl.t0);
       // ---- all parts but the last of the stretch: added up in this thread's own words of the scratch
       const int n = st.u1 - st.u0, part = seg_units(p, n), n_part = (n + part - 1) / part;
@@ -1029,15 +1052,18 @@ bool gemm_pair_eligible(const GemmParams& g, int sm_count) {
   // against 27.5; 1024 x 8192, 100 tokens: 26.4 against 17.8; fp16 4096 x 14336: 256 tokens 65 against 42).  It takes fp16 matrices one by
   // one, SwiGLU is a launch of its own beside it, and rows of y that are not 16-byte aligned it stores by the element (3333 x 9984, 300
   // tokens: 53 against 85).
+  int rows[3] = {0, 0, 0};
+  for (int i = 0; i < g.n_seg; ++i) rows[i] = g.seg[i].n_rows;
   const PairPlan pl = plan_of(g, sm_count);
   if (g.ldy % 8 || (reinterpret_cast<uintptr_t>(g.y) & 15)) return pl.pairs > 0;
+  int n_ft = 0;
+  for (int i = 0; i < g.n_seg; ++i) n_ft += feature_tiles(rows, i, g.act != nullptr);
+  // (up to 1024 features over more than 64 tokens there is nothing in it: 1024 x 8192, 77 tokens 17.2 us either way, 128 tokens 18.7 on the
+  // pairs and 17.7, 512 tokens 22.1 and 23.3; over 16 tokens 13.0 and 16.7)
+  if (!g.w16 && n_ft <= 4 && g.T > 64) return false;
   double single = 0;
   for (int i = 0; g.w16 && i < g.n_seg; ++i) single += gemm_us(&g.seg[i].n_rows, 1, g.T, g.K, true);
-  if (!g.w16) {
-    int rows[3] = {0, 0, 0};
-    for (int i = 0; i < g.n_seg; ++i) rows[i] = g.seg[i].n_rows;
-    single = gemm_us(rows, g.n_seg, g.T, g.K, false);
-  }
+  if (!g.w16) single = gemm_us(rows, g.n_seg, g.T, g.K, false);
   if (g.act) single += 2.0 + 6e-6 / 4 * g.T * g.seg[0].n_rows;
   if (g.w16 && pl.n_whole > pl.pairs) single *= 1.06;  // (the fit is that far off there: 14336 x 4096 over 700 tokens 83 us on the pairs, 97)
   return pl.pairs > 0 && pl.us <= single;
@@ -1064,14 +1090,19 @@ cudaError_t launch_gemm_pair(const GemmParams& g, int sm_count, cudaStream_t st,
   p.ksteps = (g.K + 63) / 64;
   const int max_pairs = pairs_of_device(sm_count);
   p.max_units = p.units;
+  int max_blocks = 0;
   if (g.grp_off) {
-    if (g.n_groups <= 0 || g.grp_max_rows <= 0) return cudaErrorInvalidValue;
-    p.n_tt = (g.grp_max_rows + 255) / 256;
-    p.nt = ((g.grp_max_rows + p.n_tt - 1) / p.n_tt + 15) / 16 * 16;
+    if (g.n_groups <= 0 || g.n_groups > 1024 || g.T <= 0) return cudaErrorInvalidValue;
+    // The rows of an expert are known on the device only: blocks as high as an expert's rows are expected to be at most where the pairs
+    // spread evenly (mean + 3 standard deviations), in equal parts of at most 256.  An expert with more takes more blocks.
+    const double mean = (double)g.T / g.n_groups, most = mean + 3 * std::sqrt(mean);
+    const int parts = (int)std::ceil(most / 256);
+    p.nt = std::min(256, ((int)std::ceil(most / parts) + 15) / 16 * 16);
+    p.n_groups = g.n_groups;
+    max_blocks = std::min(g.n_groups, g.T) + g.T / p.nt;
     p.ft_per = n_ft;
-    p.n_ft = n_ft * g.n_groups;
-    p.pairs = (int)std::min<long long>((long long)p.n_ft * p.n_tt, max_pairs);
-    p.n_whole = p.n_ft * p.n_tt;
+    p.n_tt = 1;
+    p.pairs = (int)std::min<long long>((long long)n_ft * max_blocks, max_pairs);
   } else {
     const PairPlan pl = plan_of(g, sm_count);
     if (!pl.pairs) return cudaErrorInvalidValue;
@@ -1145,7 +1176,7 @@ cudaError_t launch_gemm_pair(const GemmParams& g, int sm_count, cudaStream_t st,
     smem = fixed + p.xs * step;
   } else {  // three activation stages and a code ring twice as deep as the weight stages, then more activations
     p.stage_tok = (p.nt + 31) / 32 * 32;
-    const size_t fixed = 1024 + (size_t)p.stage_tok * kStagePitch, cs = kCodeBytes + kScaleBytes;
+    const size_t fixed = 1024 + (size_t)p.stage_tok * kStagePitch + (size_t)max_blocks * sizeof(int2), cs = kCodeBytes + kScaleBytes;
     p.xu = p.nt <= 128 ? 2 : 1;
     const size_t xs = (size_t)p.nt * 128 * p.xu;
     p.stages = fixed + 3 * xs + 8 * cs <= kMost ? 4 : 3;
@@ -1153,6 +1184,7 @@ cudaError_t launch_gemm_pair(const GemmParams& g, int sm_count, cudaStream_t st,
     p.xs = (int)std::min<size_t>(kMaxX, (kMost - fixed - p.codes * cs) / xs);
     while (p.codes + p.stages <= kMaxCodes && fixed + p.xs * xs + (p.codes + p.stages) * cs <= kMost) p.codes += p.stages;
     smem = fixed + p.xs * xs + p.codes * cs;
+    p.list_at = (int)(smem - 1024 - (size_t)max_blocks * sizeof(int2));
   }
   static std::atomic<uint64_t> attr_done;
   const cudaError_t e = smem_limit_once(&attr_done, {reinterpret_cast<const void*>(gemm_pair_kernel<kFmtQ4>), reinterpret_cast<const void*>(gemm_pair_kernel<kFmtMx>),

@@ -490,3 +490,36 @@ def test_linear_gemm_4bit_as_cta_pair_matches_oracle(B, torch, fmt, N, K, T):
     H.assert_close(outs[0][rows], want, what=f"{fmt} pair gemm, sampled tokens")
     H.assert_close(outs[1][rows], want, what=f"{fmt} single-CTA gemm, sampled tokens")
     H.assert_close(outs[0], outs[1].astype(np.float64), what="pair against single-CTA kernel")
+
+
+@pytest.mark.parametrize("E,k,T,skew", [(16, 4, 1, 0.0), (24, 2, 333, 0.0), (24, 2, 700, 4.0), (8, 1, 520, 0.0), (40, 3, 129, 8.0)])
+def test_moe_prefill_sorted_on_the_device_has_the_bits_of_the_host_sort(B, torch, E, k, T, skew):
+    """All experts resident: the pairs are sorted on the device and the experts' rows cut into blocks whose height is chosen
+    before the routing is known.  ``skew`` makes one expert take most tokens (many blocks), with 24 and 40 experts some take none.
+    The host sorts under ATS_FLAG_NO_GEMM_PAIR, for the single-CTA kernel; one chain per sum in both."""
+    Hd, F = 256, 96
+    rng = np.random.default_rng(7)
+    router = (rng.standard_normal((Hd, E)) * 0.02).astype(np.float16)
+    x = (rng.standard_normal((T, Hd)) + 0.5).astype(np.float16)
+    router[:, 3] += np.float16(skew * 0.01)
+    gain = np.ones(Hd, np.float16)
+    mats = [(rng.integers(0, 256, (E, n, kk // 2), dtype=np.uint8), np.abs(rng.standard_normal((E, n, kk // 32)) * 0.02).astype(np.float16))
+            for n, kk in ((F, Hd), (F, Hd), (Hd, F))]
+    outs = []
+    for flags in (0, B.ATS_FLAG_NO_GEMM_PAIR):
+        probe = B.layer_desc(hidden=Hd, ffn=F, n_experts=E, top_k=k, w_gate=0, w_up=0, w_down=0)
+        ws = B.workspace_bytes(probe, T)
+        ctx = B.Context(ws + 3 * E * (F * Hd) + 4 * MB, workspace_bytes=ws, flags=flags)
+        ids = dict(ffn_norm=ctx.register_f16(gain), router=ctx.register_f16(router))
+        ids.update(zip(("w_gate", "w_up", "w_down"), (ctx.register_q4(*m) for m in mats)))
+        ctx.set_placement([(ids[n], e, B.ATS_GPU) for n in ("w_gate", "w_up", "w_down") for e in range(E)])
+        desc = B.layer_desc(hidden=Hd, ffn=F, n_experts=E, top_k=k, **ids)
+        y = torch.empty((T, Hd), dtype=torch.float16, device="cuda")
+        for _ in range(2):
+            ctx.layer_prefill(desc, H.to_dev(x), y, None, None, 0, T)
+        ctx.sync()
+        assert ctx.stats().host_syncs == 2
+        outs.append(y.cpu().numpy())
+        ctx.close()
+    assert np.all(np.isfinite(outs[0].astype(np.float64)))
+    assert np.array_equal(outs[0].view(np.uint16), outs[1].view(np.uint16))
