@@ -335,25 +335,34 @@ __global__ void __launch_bounds__(kGroupThreads) moe_group_kernel(const int32_t*
   asm volatile("griddepcontrol.wait;" ::: "memory");  // the ids come from the router
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int per = (P + kGroupThreads - 1) / kGroupThreads * 32, lo = min(w * per, P), hi = min(lo + per, P);
-  for (int p0 = lo; p0 < hi; p0 += 32) {
-    const int p = p0 + lane;
-    int e = p < hi ? ids[p] : -1;
-    if (p < hi && (unsigned)e >= (unsigned)E) {  // an id that names no expert: expert 0 stands in and the status word says so
-      raise_status(status, 7);
-      e = 0;
-    }
+  // (a warp's first kKept votes of 32 pairs stay in registers from one pass to the next)
+  constexpr int kKept = 4;
+  int id[kKept], place[kKept];
+  auto vote = [&](int e) {  // the pair's place among the warp's pairs of its expert
     const unsigned same = __match_any_sync(0xFFFFFFFFu, e);
     const int rank = __popc(same & ((1u << lane) - 1u)), before = e < 0 ? 0 : cnt[e];
     __syncwarp();
     if (e >= 0 && rank == 0) cnt[e] = before + __popc(same);
     __syncwarp();
-    if (e >= 0) pos[p] = before + rank;  // (within the warp's part; this thread adds the rest below)
+    return before + rank;
+  };
+  auto checked = [&](int e) {  // an id that names no expert: expert 0 stands in and the status word says so
+    if ((unsigned)e < (unsigned)E) return e;
+    raise_status(status, 7);
+    return 0;
+  };
+#pragma unroll
+  for (int i = 0; i < kKept; ++i) id[i] = lo + 32 * i + lane < hi ? ids[lo + 32 * i + lane] : -1;
+#pragma unroll
+  for (int i = 0; i < kKept; ++i) {
+    if (lo + 32 * i + lane < hi) id[i] = checked(id[i]);
+    if (lo + 32 * i < hi) place[i] = vote(id[i]);
+  }
+  for (int p0 = lo + 32 * kKept; p0 < hi; p0 += 32) {
+    const int p = p0 + lane, at = vote(p < hi ? checked(ids[p]) : -1);
+    if (p < hi) pos[p] = at;  // (this thread adds the rest below)
   }
   __syncthreads();
-  if (done && threadIdx.x == 0) {
-    *reinterpret_cast<volatile int*>(done) = seq;
-    __threadfence_system();
-  }
   const int e = threadIdx.x;
   int total = 0;
   if (e < E) {
@@ -373,7 +382,8 @@ __global__ void __launch_bounds__(kGroupThreads) moe_group_kernel(const int32_t*
   if (lane == 31) sum_s[w] = incl;
   __syncthreads();
   int first = incl - total;
-  for (int i = 0; i < w; ++i) first += sum_s[i];
+#pragma unroll
+  for (int i = 0; i < 32; ++i) first += i < w ? sum_s[i] : 0;
   if (e < E) {
     off[e] = first;
     if (e == E - 1) off[E] = P;
@@ -381,13 +391,22 @@ __global__ void __launch_bounds__(kGroupThreads) moe_group_kernel(const int32_t*
     for (int i = 0; i < 32; ++i) cnt_s[i * E + e] += first;
   }
   __syncthreads();
-  for (int p = lo + lane; p < hi; p += 32) {
-    int q = ids[p];
-    if ((unsigned)q >= (unsigned)E) q = 0;
-    const int r = pos[p] + cnt[q];
+#pragma unroll
+  for (int i = 0; i < kKept; ++i) {
+    const int p = lo + 32 * i + lane;
+    if (p < hi) {
+      const int r = place[i] + cnt[id[i]];
+      pos[p] = r;
+      order[r] = p;
+    }
+  }
+  for (int p = lo + 32 * kKept + lane; p < hi; p += 32) {
+    const int q = ids[p], r = pos[p] + cnt[(unsigned)q < (unsigned)E ? q : 0];
     pos[p] = r;
     order[r] = p;
   }
+  // (at the end, and without a fence: one that waits for the host's memory held the whole sort up)
+  if (done && threadIdx.x == 0) *reinterpret_cast<volatile int*>(done) = seq;
 }
 
 cudaError_t launch_moe_group(const int32_t* ids, int P, int E, int* order, int* pos, int* off, int* status, int* done, int seq, cudaStream_t st,
