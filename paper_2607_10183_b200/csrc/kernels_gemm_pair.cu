@@ -969,10 +969,10 @@ struct PairPlan {
 };
 // Time in us of the ways to divide the work (see the kernel's comment).  A unit costs its MMAs, the expansion of its weights
 // or their way from memory, whichever is longest; a tile its epilogue; a stretch that is added up in several parts their way out and
-// back, less where the MMAs go on meanwhile in the other accumulator; a split tile the parts' way through L2, which the last to arrive
-// waits for in batches of tokens (shorter ones where there are several others).  The figures are fitted to about 800 launches, 16 shapes
-// of 1 to 160 MB, 9 to 2048 tokens, back to back on new weights: 7 % rms off for the 4-bit formats, 10 % for fp16.  pairs = 0: the
-// scratch holds none.
+// back, less where the MMAs go on meanwhile in the other accumulator; a split tile the parts' way through L2.  The figures are fitted
+// to launches back to back on new weights: the 4-bit formats' to 330, 14 shapes of 6 to 66 MB, 12 to 1000 tokens, in the ways that come
+// within a third of the best (6 % rms off; many waves run 8 % slower, at the power limit), fp16's to about 400 with the sums of split tiles
+// as they were when one contributor made them (10 %).  pairs = 0: the scratch holds none.
 PairPlan pair_plan(const int* rows, int n_seg, bool act, int T, int K, bool w16, int max_pairs, uint64_t scratch_bytes) {
   PairPlan best{};
   best.us = 1e300;
@@ -992,12 +992,12 @@ PairPlan pair_plan(const int* rows, int n_seg, bool act, int T, int K, bool w16,
     // they make one wave they are the faster ones: 4096 x 14336 over 2048 tokens 204 -> 186 us, 14336 x 4096 over 512 67 -> 55; in several
     // waves they are not: 28672 x 4096 over 3000 tokens 527 -> 649.  fp16 weights that several token tiles share come out of L2 for all but
     // one)
-    const double unit = w16 ? std::max(n_tt > 1 ? 0.55 : 0.729, nt == 512 ? 1.55 : 0.40 + 0.00165 * nt) : std::max(0.391, 0.174 + 0.0020 * nt);
-    const double launch = w16 ? 5.0 : 4.2, tile = w16 ? (nt == 512 ? 6.0 : 0.0) : 0.012 * nt;
-    const double flush = w16 ? 1.1 : nt <= 128 ? 2.6 : 4.6;
+    const double unit = w16 ? std::max(n_tt > 1 ? 0.55 : 0.729, nt == 512 ? 1.55 : 0.40 + 0.00165 * nt) : std::max(0.416, 0.155 + 0.0020 * nt) * (n_ft * n_tt >= 4 * max_pairs ? 1.08 : 1.0);
+    const double launch = w16 ? 5.0 : 4.9, tile = w16 ? (nt == 512 ? 6.0 : 0.0) : 0.0077 * nt;
+    const double flush = w16 ? 1.1 : std::max(0.3, 0.0284 * nt - 1.56);
     const int tok = std::min(nt, T), batches = tok <= 16 ? 1 : (tok + 63) / 64 * 2;  // (16 tokens a batch and warp, two warps side by side)
     auto stretch = [&](double len) { return len * unit + (std::ceil(len / max_units) - 1) * flush + tile; };
-    auto sum = [&](double con) { return w16 ? 1.0 + batches * (con > 2 ? 2.7 : 1.6) : 1.0 + 0.25 * batches + 0.3 * con; };
+    auto sum = [&](double con) { return w16 ? 1.0 + batches * (con > 2 ? 2.7 : 1.6) : 2.2 + 0.0284 * tok + 0.1 * con; };
     // whole tiles in waves of one per pair; the rest, `rem`, whole in a wave of its own or divided over n pairs, `len` units each
     const int tiles = n_ft * n_tt, waves = tiles / max_pairs, rem = tiles % max_pairs;
     auto take = [&](double us, double len, int n, int slots) {
@@ -1015,7 +1015,7 @@ PairPlan pair_plan(const int* rows, int n_seg, bool act, int T, int K, bool w16,
       if (units % s == 0 || units > 4 * s) take(stretch((units + s - 1) / s) + sum(s), (units + s - 1) / s, rem * s, 1);
     const double per = (double)rem * units / max_pairs;
     if (per >= 1 && units <= per * (kMaxParts - 2))  // (a tile meets at most units / per + 2 ranges)
-      take(stretch(std::ceil(per)) + sum(std::ceil(units / per) + 1) + 3.1, std::ceil(per), max_pairs, 2);
+      take(stretch(std::ceil(per)) + sum(std::ceil(units / per) + 1) + (w16 ? 3.1 : 6.2), std::ceil(per), max_pairs, 2);
   }
   return best;
 }
