@@ -309,7 +309,9 @@ __device__ __forceinline__ Tile tile_of(const PairParams& p, int tile, const int
 }
 
 // Units that go into an accumulator before it is handed over: a stretch in equal parts of p.max_units at most.
-__device__ __forceinline__ int seg_units(const PairParams& p, int n) { return (n + (n - 1) / p.max_units) / ((n + p.max_units - 1) / p.max_units); }
+__device__ __forceinline__ int seg_units(const PairParams& p, int n) {
+  return n <= p.max_units ? n : (n + (n - 1) / p.max_units) / ((n + p.max_units - 1) / p.max_units);
+}
 
 template <int FMT>
 __global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ PairMaps wmap,
@@ -533,7 +535,6 @@ __global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid
         uint32_t par = 0, parx = 0;
         bool ready = false, readyx = false;
         while (uniform(ok && mine.next(st))) {
-          const Tile tl = tile_of(p, st.tile, blocks);
           const int u0 = uniform(st.u0), u1 = uniform(st.u1);
           int left = 0;  // units until the accumulator is handed over
           uint32_t d = 0, accumulate = 0;
@@ -638,9 +639,11 @@ __global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid
     int cs = grp;                 // its place in the code ring
     uint32_t cpar = 0, apar = 1;  // (the first wait for an empty stage passes at once)
     while (FMT != kFmtW16 && ok && grp < S && mine.next(st)) {
-      const Tile tl = tile_of(p, st.tile, blocks);
-      const int first = p.act ? tl.row0 + (int)rank * 64 + (row & 63) : tl.row0 + (int)rank * kFeat + row;
-      const int odd = p.sc16 ? 0 : (int)(((long long)first * nblk) & 1);  // units start at even offsets: the row decides
+      int odd = 0;
+      if (!p.sc16) {  // units start at even offsets: the row decides
+        const Tile tl = tile_of(p, st.tile, blocks);
+        odd = ((p.act ? tl.row0 + (int)rank * 64 + (row & 63) : tl.row0 + (int)rank * kFeat + row) & nblk) & 1;
+      }
       int u = st.u0 + skip;
       for (; u < st.u1; u += S) {
         if (!wait_warp(&cfull[cs], cpar)) {
@@ -718,7 +721,7 @@ __global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid
       const Tile tl = tile_of(p, st.tile, blocks);
       const int ntok = min(p.nt, tl.T - tl.t0);
       // ---- all parts but the last of the stretch: added up in this thread's own words of the scratch
-      const int n = st.u1 - st.u0, part = seg_units(p, n), n_part = (n + part - 1) / part;
+      const int n = st.u1 - st.u0, part = seg_units(p, n), n_part = part == n ? 1 : (n + part - 1) / part;
       uint32_t col = 0;
       float* own = p.own + (size_t)blockIdx.x * kFeat * p.slot_tok + feat;
       auto add_own = [&](float* v, int c0, auto n_tok) {  // (all loads before the first addition)
