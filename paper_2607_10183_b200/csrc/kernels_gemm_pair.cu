@@ -379,7 +379,7 @@ __global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid
   tc_fence_before();
   __syncwarp();
   pair_arrive();
-  if (warp == 0 || p.grp_off) asm volatile("griddepcontrol.wait;" ::: "memory");
+  if ((warp == 0 && FMT != kFmtW16) || p.grp_off) asm volatile("griddepcontrol.wait;" ::: "memory");
   // Grouped form: every CTA lists the blocks of rows for itself from the experts' offsets.
   int2* const blocks = reinterpret_cast<int2*>(smem + p.list_at);
   int n_whole = p.n_whole;
@@ -494,19 +494,29 @@ __global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid
           const int sa = p.act ? 0 : uniform(tl.sg), sb = p.act ? 1 : sa;
           const int wa = uniform(tl.row0 + (int)rank * (p.act ? 64 : kFeat)), wb = p.act ? wa : wa + 64;
           const int k1 = min(2 * u1, p.ksteps);
+          auto weights = [&](int ks, int place) {
+            const uint32_t dw = x0 + (uint32_t)(place * step_bytes + xbytes);
+            if (rank == 0) expect_tx_one(one, &xfull[place], (uint32_t)(2 * step_bytes));
+            tma_pair_3d(one, dw, &wmap.codes[sa], ks * 64, wa, &xfull[place]);
+            tma_pair_3d(one, dw + kW16Bytes / 2, &wmap.codes[sb], ks * 64, wb, &xfull[place]);
+          };
+          // The weights of the first steps do not wait for the preceding kernel, their activations do (18944 x 1024, 32 tokens 11.9 -> 10.6 us).
+          const int ahead = n == 0 ? min(NX, k1 - 2 * u0) : 0;
+          if (n == 0) {
+            for (int i = 0; i < ahead; ++i) weights(2 * u0 + i, i);
+            asm volatile("griddepcontrol.wait;" ::: "memory");
+          }
           for (int ks = 2 * u0; ks < k1; ++ks) {
             if (n >= NX && !wait_warp(&xempty[s], par)) {
               ok = false;
               break;
             }
             ++n;
-            const uint32_t dst = x0 + (uint32_t)(s * step_bytes), dw = dst + (uint32_t)xbytes;
-            if (rank == 0) expect_tx_one(one, &xfull[s], (uint32_t)(2 * step_bytes));
+            if (ks - 2 * u0 >= ahead) weights(ks, s);
+            const uint32_t dst = x0 + (uint32_t)(s * step_bytes);
             // (wide: tokens 128 rank .. of each half of the tile, so that either half is one operand of the pair)
             tma_pair_2d(one, dst, &xmap, ks * 64, wide ? row - (int)rank * 128 : row, &xfull[s]);
             if (wide) tma_pair_2d(one, dst + (uint32_t)(xbytes / 2), &xmap, ks * 64, row - (int)rank * 128 + 256, &xfull[s]);
-            tma_pair_3d(one, dw, &wmap.codes[sa], ks * 64, wa, &xfull[s]);
-            tma_pair_3d(one, dw + kW16Bytes / 2, &wmap.codes[sb], ks * 64, wb, &xfull[s]);
             if (++s == NX) s = 0, par ^= 1u;
           }
           continue;
