@@ -1,8 +1,8 @@
 // GEMM of prompts on pairs of CTAs (sm_100a, tcgen05 cta_group::2): Y[T][N] = X[T][K] W^T for the two 4-bit block formats and for
 // fp16 matrices; fp16 operands (4-bit: w = rn16(scale * code), one rounding), fp32 accumulation.
 //
-// The weights are the A operand (M = 256 features, 128 per CTA), the tokens are the instruction's N (32..256, chosen from T; fp16 weights
-// also tiles of 512 tokens, two instructions).
+// The weights are the A operand (M = 256 features, 128 per CTA), the tokens are the instruction's N (multiples of 16 up to 256, chosen from T; fp16
+// weights also tiles of 512 tokens, two instructions).
 // 4-bit weights are expanded into tensor memory: a thread of the sixteen dequantization warps turns 32-weight blocks of one
 // feature (its lane) into sixteen columns each; nothing is stored to shared memory, no swizzle, no proxy fence.  (With the
 // weights as a shared-memory operand a 64-k step of 256 features took about 1700 cycles, whatever the number of tokens, for the
@@ -24,13 +24,16 @@
 // the scratch: every contributor leaves its part there, 32 tokens at a time; the last one to do so for these tokens adds the parts in
 // ascending k order (so the result does not depend on who that is) and writes them.  Nobody waits for anybody.
 //
-// What bounds it: 4-bit, up to about 128 tokens, the expansion (a unit takes 0.39 us in launches with many of them); fp16 there the weights'
-// way from memory; with tiles for all pairs the MMAs and the power limit; with few tiles the launch (4 to 5 us) and what every tile pays
-// for its sums, which is why such products go to the single-CTA kernel (gemm_pair_eligible).  72 registers a thread
-// are all that 896 threads leave: the compiler spills 172 to 208 bytes, in the epilogue's sums.
+// What bounds it: 4-bit, up to about 128 tokens, the MMA warp's chain: its eight MMAs and its commits take 430 cycles to issue among the
+// expanding warps of its scheduler, whatever the number of tokens (alone: 200), and a wait that is not known to be over when it begins costs
+// 200 more; a unit takes 0.42 to 0.47 us, of which the MMAs of 80 tokens are 0.16 and the expansion alone would be 0.16 (HBM 0.21).  That
+// is why the barriers are tested ahead and why activations come two units at a time.  fp16 there the weights' way from memory; with
+// tiles for all pairs the MMAs and the power limit; with few tiles the launch (5 us and more: entry, the pair's meeting, first loads, output)
+// and the sum of split tiles.  72 registers a thread are all that 896 threads leave: the compiler spills 84 to 128 bytes, in the
+// epilogue's sums.
 // Back to back on new weights, single-CTA kernel (with reduction, residual and SwiGLU launches) -> pairs:
-//   77 tokens MXFP4: 28672 x 4096 with SwiGLU 66 -> 36 us, 4096 x 14336 41 -> 33
-//   512 tokens Q4: gate and up 143 -> 103-107 us, 4096 x 14336 78 -> 69;  2048 tokens: gate and up 462 -> 351 (1372 TFLOP/s)
+//   77 tokens MXFP4: 28672 x 4096 with SwiGLU 66 -> 35 us, 4096 x 14336 41 -> 25
+//   512 tokens Q4: gate and up 143 -> 91 us, 4096 x 14336 78 -> 60;  2048 tokens: gate and up 462 -> 328 to 351 (1372 TFLOP/s)
 //   2048 tokens fp16: q, k, v 152 -> 78 us, o 66 -> 59, gate and up 451 -> 346 (1390 TFLOP/s)
 //
 // Roles per CTA: warp 0 = activation loads (fp16: and weights), warp 1 = tensor-memory allocation and (leader) MMA issue, warps 2, 3
@@ -1060,9 +1063,9 @@ bool gemm_pair_eligible(const GemmParams& g, int sm_count) {
                 ((reinterpret_cast<uintptr_t>(g.act) | reinterpret_cast<uintptr_t>(g.y)) & 15)))
     return false;
   if (g.grp_off) return (g.n_seg == 1 || g.act) && g.grp_stride % 16 == 0 && !g.res;
-  // The pairs win where there are tiles for all of them; a tile that has to be split waits for its parts, and the single-CTA kernel, with
-  // smaller tiles and the sum as a launch of its own, is the faster one (4096 x 4096: 128 tokens 22.1 us against 19.5, 512 tokens 23.8
-  // against 27.5; 1024 x 8192, 100 tokens: 26.4 against 17.8; fp16 4096 x 14336: 256 tokens 65 against 42).  It takes fp16 matrices one by
+  // The pairs win where there are tiles for most of them (4-bit 4096 x 4096: 128 tokens 15.7 us against 18.2, 512 tokens 23.5 against 27.7);
+  // where tiles have to be split the single-CTA kernel, with smaller tiles, eight splits and the sum as a launch of its own, can be the
+  // faster one (4-bit 4096 x 14336, 256 tokens: 40.3 against 38.7; fp16: 43 against 41.5).  It takes fp16 matrices one by
   // one, SwiGLU is a launch of its own beside it, and rows of y that are not 16-byte aligned it stores by the element (3333 x 9984, 300
   // tokens: 53 against 85).
   int rows[3] = {0, 0, 0};
