@@ -964,14 +964,15 @@ __global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid
 // ------------------------------------------------------------------------------------------------- host side
 // Units that one accumulator adds up at most.  The tensor core truncates each sum, and what a chain drops grows with its
 // length: of the fp16 results 0.5 % differ from the exact sum's rounding after 1024 k, 1.7 % after 4096, 5 % after 14336.  So no
-// chain is longer than the single-CTA kernel's for the same product (fp16: for each matrix by itself, as that kernel takes them), except
-// that 1536 k are always allowed, and fp16 matrices of enough large tiles (112 CTAs of 256 features x 256 tokens) are added up in one.
-int units_at_once(const int* rows, int n_seg, int T, int K, bool w16) {
+// chain is longer (by more than part of a unit) than the single-CTA kernel's for the same product (fp16: for each matrix by itself, as that
+// kernel takes them), except that 1536 k are allowed where plan_of says so (`longer`), and fp16 matrices of enough large tiles (112 CTAs of 256 features x 256
+// tokens) are added up in one.
+int units_at_once(const int* rows, int n_seg, int T, int K, bool w16, bool longer) {
   int chain = K;
   for (int i = 0; w16 && i < n_seg; ++i)
     if (T < 384 || (rows[i] + 255) / 256 * ((T + 511) / 512) < 56) chain = std::min(chain, gemm_chain(rows + i, 1, T, K));
   if (!w16) chain = gemm_chain(rows, n_seg, T, K);
-  return (std::max(1536, chain) + kUnitK - 1) / kUnitK;
+  return ((longer ? std::max(1536, chain) : chain) + kUnitK - 1) / kUnitK;
 }
 // Feature tiles of a segment (fused SwiGLU: a tile is 128 gate and 128 up rows, all counted with the gate).
 int feature_tiles(const int* rows, int seg, bool act) {
@@ -989,12 +990,12 @@ struct PairPlan {
 // to launches back to back on new weights: the 4-bit formats' to 330, 14 shapes of 6 to 66 MB, 12 to 1000 tokens, in the ways that come
 // within a third of the best (6 % rms off; many waves run 8 % slower, at the power limit), fp16's to about 400 with the sums of split tiles
 // as they were when one contributor made them (10 %).  pairs = 0: the scratch holds none.
-PairPlan pair_plan(const int* rows, int n_seg, bool act, int T, int K, bool w16, int max_pairs, uint64_t scratch_bytes) {
+PairPlan pair_plan(const int* rows, int n_seg, bool act, int T, int K, bool w16, bool longer, int max_pairs, uint64_t scratch_bytes) {
   PairPlan best{};
   best.us = 1e300;
   int n_ft = 0;
   for (int i = 0; i < n_seg; ++i) n_ft += feature_tiles(rows, i, act);
-  const int units = (K + kUnitK - 1) / kUnitK, max_units = units_at_once(rows, n_seg, T, K, w16);
+  const int units = (K + kUnitK - 1) / kUnitK, max_units = units_at_once(rows, n_seg, T, K, w16, longer);
   double weights_mb = 0;
   for (int i = 0; i < n_seg; ++i) weights_mb += 2e-6 * rows[i] * K;
   int last = 0;
@@ -1038,15 +1039,39 @@ PairPlan pair_plan(const int* rows, int n_seg, bool act, int T, int K, bool w16,
 
 int pairs_of_device(int sm_count) { return std::min(sm_count / 2, kAttnMaxCounters / 2); }
 
+// 16-byte rows of y: others the single-CTA kernel stores by the element, so that it is no match for the pairs.
+bool rows_aligned(const GemmParams& g) { return g.ldy % 8 == 0 && (reinterpret_cast<uintptr_t>(g.y) & 15) == 0; }
+
+// Time of the product on the single-CTA kernel, which takes fp16 matrices one by one and has SwiGLU as a launch of its own beside it.
+double single_cta_us(const GemmParams& g) {
+  int rows[3] = {0, 0, 0};
+  double us = 0;
+  for (int i = 0; i < g.n_seg; ++i) rows[i] = g.seg[i].n_rows;
+  for (int i = 0; g.w16 && i < g.n_seg; ++i) us += gemm_us(rows + i, 1, g.T, g.K, true);
+  if (!g.w16) us = gemm_us(rows, g.n_seg, g.T, g.K, false);
+  if (g.act) us += 2.0 + 6e-6 / 4 * g.T * rows[0];
+  return us;
+}
+
 // The plan of a launch depends on its shapes, and on the scratch in one point only: the best plan where the scratch holds it, else
 // the best one that the scratch of the single-CTA kernel's plan holds, which every caller has (there may be none).
-PairPlan plan_of(const GemmParams& g, int sm_count) {
-  int rows[3] = {0, 0, 0}, n = 0;
+// `single`: time of the single-CTA kernel.  Chains of 1536 k are for products that the pairs take in clearly less: where both kernels are
+// about equally fast, the one that drops more has nothing to offer.  The more contributors a tile has, the fewer the tiles and the shorter
+// the single-CTA kernel's own chains (6144 x 4096, 77 tokens: three contributors would sum 1408 k in one accumulator against its 704).
+PairPlan plan_of(const GemmParams& g, int sm_count, double single) {
+  int rows[3] = {0, 0, 0}, n = 0, n_ft = 0;
   for (int i = 0; i < g.n_seg; ++i) n += rows[i] = g.seg[i].n_rows;
-  auto plan = [&](uint64_t bytes) { return pair_plan(rows, g.n_seg, g.act != nullptr, g.T, g.K, g.w16, pairs_of_device(sm_count), bytes); };
+  for (int i = 0; i < g.n_seg; ++i) n_ft += feature_tiles(rows, i, g.act != nullptr);
   const uint64_t have = g.scratch ? g.scratch_bytes : 0;
-  const PairPlan best = plan(~0ull);
-  return best.scratch <= have ? best : plan(std::min(have, gemm_scratch_bytes(g.T, n, g.K)));
+  auto plan = [&](bool longer) {
+    auto within = [&](uint64_t bytes) { return pair_plan(rows, g.n_seg, g.act != nullptr, g.T, g.K, g.w16, longer, pairs_of_device(sm_count), bytes); };
+    const PairPlan best = within(~0ull);
+    return best.scratch <= have ? best : within(std::min(have, gemm_scratch_bytes(g.T, n, g.K)));
+  };
+  const PairPlan pl = plan(true);
+  const int split = n_ft * pl.n_tt - pl.n_whole;  // tiles that several pairs share
+  const double most = pl.split_pairs == 0 ? 0.96 : pl.split_pairs <= 2 * split ? 0.93 : 0.75;
+  return rows_aligned(g) && pl.us > most * single ? plan(false) : pl;
 }
 
 }  // namespace
@@ -1068,19 +1093,15 @@ bool gemm_pair_eligible(const GemmParams& g, int sm_count) {
   // faster one (4-bit 4096 x 14336, 256 tokens: 40.3 against 38.7; fp16: 43 against 41.5).  It takes fp16 matrices one by
   // one, SwiGLU is a launch of its own beside it, and rows of y that are not 16-byte aligned it stores by the element (3333 x 9984, 300
   // tokens: 53 against 85).
-  int rows[3] = {0, 0, 0};
+  double single = single_cta_us(g);
+  const PairPlan pl = plan_of(g, sm_count, single);
+  if (!rows_aligned(g)) return pl.pairs > 0;
+  int rows[3] = {0, 0, 0}, n_ft = 0;
   for (int i = 0; i < g.n_seg; ++i) rows[i] = g.seg[i].n_rows;
-  const PairPlan pl = plan_of(g, sm_count);
-  if (g.ldy % 8 || (reinterpret_cast<uintptr_t>(g.y) & 15)) return pl.pairs > 0;
-  int n_ft = 0;
   for (int i = 0; i < g.n_seg; ++i) n_ft += feature_tiles(rows, i, g.act != nullptr);
   // (up to 1024 features over more than 64 tokens there is nothing in it: 1024 x 8192, 77 tokens 17.2 us either way, 128 tokens 18.7 on the
   // pairs and 17.7, 512 tokens 22.1 and 23.3; over 16 tokens 13.0 and 16.7)
   if (!g.w16 && n_ft <= 4 && g.T > 64) return false;
-  double single = 0;
-  for (int i = 0; g.w16 && i < g.n_seg; ++i) single += gemm_us(&g.seg[i].n_rows, 1, g.T, g.K, true);
-  if (!g.w16) single = gemm_us(rows, g.n_seg, g.T, g.K, false);
-  if (g.act) single += 2.0 + 6e-6 / 4 * g.T * g.seg[0].n_rows;
   if (g.w16 && pl.n_whole > pl.pairs) single *= 1.06;  // (the fit is that far off there: 14336 x 4096 over 700 tokens 83 us on the pairs, 97)
   return pl.pairs > 0 && pl.us <= single;
 }
@@ -1120,7 +1141,7 @@ cudaError_t launch_gemm_pair(const GemmParams& g, int sm_count, cudaStream_t st,
     p.n_tt = 1;
     p.pairs = (int)std::min<long long>((long long)n_ft * max_blocks, max_pairs);
   } else {
-    const PairPlan pl = plan_of(g, sm_count);
+    const PairPlan pl = plan_of(g, sm_count, single_cta_us(g));
     if (!pl.pairs) return cudaErrorInvalidValue;
     p.nt = pl.nt;
     p.n_tt = pl.n_tt;

@@ -123,6 +123,15 @@ def test_gemm_chains_are_no_longer_than_the_single_cta_kernels(fmt, N, K, T, lim
     assert differ <= 0.0065 * limit / 1000
 
 
+# Products of few tiles that both kernels take in about the same time: there is no reason to add up longer chains than the single-CTA
+# kernel, whose splits are shorter than 1536 k (`limit`; chains twice as long gave 0.58 to 0.76 % with q4 codes where 0.30 to 0.43 are
+# measured with these).  The last two are taken in clearly less time, with the 1536 k.
+@pytest.mark.parametrize("fmt,N,K,T,limit", [("q4", 6144, 4096, 77, 768), ("q4", 4096, 4096, 77, 512), ("q4", 5632, 4608, 79, 768), ("q4", 4096, 3072, 144, 512),
+                                             ("q4", 2560, 4096, 183, 512), ("w16", 3072, 2048, 131, 512), ("q4", 4096, 4096, 512, 1536), ("q4", 9472, 2304, 82, 1536)])
+def test_gemm_chains_of_products_that_both_kernels_take_as_fast(fmt, N, K, T, limit):
+    test_gemm_chains_are_no_longer_than_the_single_cta_kernels(fmt, N, K, T, limit)
+
+
 def test_gemm_with_the_least_workspace_keeps_the_chains_short():
     import re
     import torch
