@@ -1096,12 +1096,6 @@ bool gemm_pair_eligible(const GemmParams& g, int sm_count) {
   double single = single_cta_us(g);
   const PairPlan pl = plan_of(g, sm_count, single);
   if (!rows_aligned(g)) return pl.pairs > 0;
-  int rows[3] = {0, 0, 0}, n_ft = 0;
-  for (int i = 0; i < g.n_seg; ++i) rows[i] = g.seg[i].n_rows;
-  for (int i = 0; i < g.n_seg; ++i) n_ft += feature_tiles(rows, i, g.act != nullptr);
-  // (up to 1024 features over more than 64 tokens there is nothing in it: 1024 x 8192, 77 tokens 17.2 us either way, 128 tokens 18.7 on the
-  // pairs and 17.7, 512 tokens 22.1 and 23.3; over 16 tokens 13.0 and 16.7)
-  if (!g.w16 && n_ft <= 4 && g.T > 64) return false;
   if (g.w16 && pl.n_whole > pl.pairs) single *= 1.06;  // (the fit is that far off there: 14336 x 4096 over 700 tokens 83 us on the pairs, 97)
   return pl.pairs > 0 && pl.us <= single;
 }

@@ -184,6 +184,12 @@ def test_few_tiles_go_to_the_single_cta_kernel(fmt, N, K, T, pairs):
         assert np.array_equal(outs[0], outs[1])
 
 
+# Few features over many tokens are as many tiles as many features over few (1024 x 2048, 2048 tokens: 13.7 us on the pairs, 26.4).
+@pytest.mark.parametrize("fmt,N,K,T", [("q4", 512, 2048, 2048), ("mxfp4", 1024, 3072, 2048), ("q4", 1024, 4096, 2048)])
+def test_few_features_over_many_tokens_go_to_the_pairs(fmt, N, K, T):
+    test_few_tiles_go_to_the_single_cta_kernel(fmt, N, K, T, True)
+
+
 # 75 tiles for 74 pairs (the one that is left is split into two, three or four where there is scratch for it) and the same as one wave
 # and a half; 4-bit and fp16.
 @pytest.mark.parametrize("fmt,N,K,T", [("q4", 19200, 4096, 40), ("q4", 28672, 1024, 40), ("mxfp4", 14336, 2048, 300), ("w16", 19200, 2048, 40)])
