@@ -1036,8 +1036,9 @@ struct PairPlan {
 // or their way from memory, whichever is longest; a tile its epilogue; a stretch that is added up in several parts their way out and
 // back, less where the MMAs go on meanwhile in the other accumulator; a split tile the parts' way through L2.  The figures are fitted
 // to launches back to back on new weights: the 4-bit formats' to 330, 14 shapes of 6 to 66 MB, 12 to 1000 tokens, in the ways that come
-// within a third of the best (6 % rms off; many waves run 8 % slower, at the power limit), fp16's to about 400 with the sums of split tiles
-// as they were when one contributor made them (10 %).  pairs = 0: the scratch holds none.
+// within a third of the best (6 % rms off; many waves run 8 % slower, at the power limit; later 8 products whose contributors have several parts,
+// 6144 x 4096 over 160 tokens among them, taken at 21.4 us for 24.2, where the single-CTA kernel needs 22.5), fp16's to about 400 with the sums
+// of split tiles as they were when one contributor made them (10 %).  pairs = 0: the scratch holds none.
 PairPlan pair_plan(const int* rows, int n_seg, bool act, int T, int K, bool w16, bool longer, int max_pairs, uint64_t scratch_bytes) {
   PairPlan best{};
   best.us = 1e300;
@@ -1061,7 +1062,13 @@ PairPlan pair_plan(const int* rows, int n_seg, bool act, int T, int K, bool w16,
     const double launch = w16 ? 5.0 : 4.9, tile = w16 ? (nt == 512 ? 6.0 : 0.0) : 0.0077 * nt;
     const double flush = w16 ? 1.1 : std::max(0.3, 0.0284 * nt - 1.56);
     const int tok = std::min(nt, T), batches = tok <= 16 ? 1 : (tok + 63) / 64 * 2;  // (16 tokens a batch and warp, two warps side by side)
-    auto stretch = [&](double len) { return len * unit + (std::ceil(len / max_units) - 1) * flush + tile; };
+    // (slots: of a split tile.  Its contributors' parts come back from the scratch in the way of the sum, where they do not meet in tensor
+    // memory; those that do cost less than `flush`, which is not counted on: near the line the single-CTA kernel keeps what it had)
+    auto stretch = [&](double len, int slots) {
+      const double parts = std::ceil(len / max_units);
+      const bool back = slots == 1 && parts > 1 && !w16 && (parts > 2 || nt > 128);
+      return len * unit + (parts - 1) * flush + (back ? 0.012 * std::max(0, nt - 24) : 0.0) + tile;
+    };
     auto sum = [&](double con) { return w16 ? 1.0 + batches * (con > 2 ? 2.7 : 1.6) : 2.2 + 0.0284 * tok + 0.1 * con; };
     // whole tiles in waves of one per pair; the rest, `rem`, whole in a wave of its own or divided over n pairs, `len` units each
     const int tiles = n_ft * n_tt, waves = tiles / max_pairs, rem = tiles % max_pairs;
@@ -1070,17 +1077,17 @@ PairPlan pair_plan(const int* rows, int n_seg, bool act, int T, int K, bool w16,
       const int pairs = waves ? max_pairs : slots ? n : rem;
       const uint64_t need = ((uint64_t)n * slots + (parts ? pairs : 0)) * slot;
       if (need > scratch_bytes || (nt == 512 && need)) return;  // (tiles of 512 tokens: whole ones in one part)
-      us += launch + waves * stretch(units);
+      us += launch + waves * stretch(units, 0);
       if (w16) us = std::max(us, weights_mb / 4.5);
       if (us >= best.us) return;
       best = PairPlan{nt, n_tt, pairs, slots ? tiles - rem : tiles, n, slots == 2, parts, max_units, us, need};
     };
-    take(rem ? stretch(units) : 0.0, units, 0, 0);
+    take(rem ? stretch(units, 0) : 0.0, units, 0, 0);
     for (int s = 2; s <= kMaxParts && s <= units && rem && rem * s <= max_pairs; ++s)
-      if (units % s == 0 || units > 4 * s) take(stretch((units + s - 1) / s) + sum(s), (units + s - 1) / s, rem * s, 1);
+      if (units % s == 0 || units > 4 * s) take(stretch((units + s - 1) / s, 1) + sum(s), (units + s - 1) / s, rem * s, 1);
     const double per = (double)rem * units / max_pairs;
     if (per >= 1 && units <= per * (kMaxParts - 2))  // (a tile meets at most units / per + 2 ranges)
-      take(stretch(std::ceil(per)) + sum(std::ceil(units / per) + 1) + (w16 ? 3.1 : 6.2), std::ceil(per), max_pairs, 2);
+      take(stretch(std::ceil(per), 2) + sum(std::ceil(units / per) + 1) + (w16 ? 3.1 : 6.2), std::ceil(per), max_pairs, 2);
   }
   return best;
 }
