@@ -297,17 +297,18 @@ struct Tile {
   int t0, T, rowoff;   // first token, tokens of the matrix (of the block of an expert's rows), its first row
   int expert;
 };
-// Grouped form: the experts' rows in blocks of at most nt, in shared memory: {expert | rows << 10, first row}.
-__device__ __forceinline__ Tile tile_of(const PairParams& p, int tile, const int2* blocks) {
+// Grouped form: the experts' rows in blocks of at most nt, in shared memory: expert | first row << 10.  The blocks follow one another, so the
+// next one's first row ends it (behind the last: all rows).
+__device__ __forceinline__ Tile tile_of(const PairParams& p, int tile, const uint32_t* blocks) {
   Tile r;
   int ft = tile / (p.grp_off ? p.ft_per : p.n_tt);
   if (p.grp_off) {  // feature tiles of one block after another
-    const int2 b = blocks[ft];
+    const uint32_t b = blocks[ft], e = blocks[ft + 1];
     ft = tile - ft * p.ft_per;
-    r.expert = b.x & 1023;
+    r.expert = (int)(b & 1023u);
     r.t0 = 0;
-    r.T = b.x >> 10;
-    r.rowoff = b.y;
+    r.rowoff = (int)(b >> 10);
+    r.T = (int)(e >> 10) - r.rowoff;
   } else {
     r.expert = 0;
     r.t0 = (tile - ft * p.n_tt) * p.nt;
@@ -397,7 +398,7 @@ __global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid
   pair_arrive();
   if ((warp == 0 && FMT != kFmtW16) || p.grp_off) asm volatile("griddepcontrol.wait;" ::: "memory");
   // Grouped form: every CTA lists the blocks of rows for itself from the experts' offsets.
-  int2* const blocks = reinterpret_cast<int2*>(smem + p.list_at);
+  uint32_t* const blocks = reinterpret_cast<uint32_t*>(smem + p.list_at);
   int n_whole = p.n_whole;
   if (p.grp_off) {
     if (warp == 4) {
@@ -413,9 +414,12 @@ __global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid
       int at = incl - n;
       for (int e = e0; e < e1; ++e) {
         const int hi = p.grp_off[e + 1];
-        for (int r = p.grp_off[e]; r < hi; r += p.nt) blocks[at++] = make_int2(e | min(p.nt, hi - r) << 10, r);
+        for (int r = p.grp_off[e]; r < hi; r += p.nt) blocks[at++] = (uint32_t)(e | r << 10);
       }
-      if (lane == 31) n_blocks_s = incl;
+      if (lane == 31) {
+        blocks[incl] = (uint32_t)p.T << 10;
+        n_blocks_s = incl;
+      }
     }
     __syncthreads();
     n_whole = n_blocks_s * p.ft_per;
@@ -1176,9 +1180,9 @@ cudaError_t launch_gemm_pair(const GemmParams& g, int sm_count, cudaStream_t st,
   p.ksteps = (g.K + 63) / 64;
   const int max_pairs = pairs_of_device(sm_count);
   p.max_units = p.units;
-  int max_blocks = 0;
+  int max_blocks = 0;  // of an expert's rows, at most
   if (g.grp_off) {
-    if (g.n_groups <= 0 || g.n_groups > 1024 || g.T <= 0) return cudaErrorInvalidValue;
+    if (g.n_groups <= 0 || g.n_groups > 1024 || g.T <= 0 || g.T >= 1 << 22) return cudaErrorInvalidValue;
     // The rows of an expert are known on the device only: blocks as high as an expert's rows are expected to be at most where the pairs
     // spread evenly (mean + 3 standard deviations), in equal parts of at most 256.  An expert with more takes more blocks.
     const double mean = (double)g.T / g.n_groups, most = mean + 3 * std::sqrt(mean);
@@ -1262,15 +1266,18 @@ cudaError_t launch_gemm_pair(const GemmParams& g, int sm_count, cudaStream_t st,
     smem = fixed + p.xs * step;
   } else {  // three activation stages and a code ring twice as deep as the weight stages, then more activations
     p.stage_tok = (p.nt + 31) / 32 * 32;
-    const size_t fixed = 1024 + (size_t)p.stage_tok * kStagePitch + (size_t)max_blocks * sizeof(int2), cs = kCodeBytes + kScaleBytes;
     p.xu = p.nt <= 128 ? 2 : 1;
-    const size_t xs = (size_t)p.nt * 128 * p.xu;
+    const size_t xs = (size_t)p.nt * 128 * p.xu, cs = kCodeBytes + kScaleBytes, list = g.grp_off ? (size_t)(max_blocks + 1) * sizeof(uint32_t) : 0;
+    // (beside three places for 256 rows there is room for a list of 255 blocks; more of them: the staging in two halves.  8 experts, 32768 rows:
+    // a list of 8 bytes a block had left two places, 829 -> 807 us for the layer)
+    if (1024 + (size_t)p.stage_tok * kStagePitch + list + 3 * xs + 6 * cs > kMost) p.stage_tok = 128;
+    const size_t fixed = 1024 + (size_t)p.stage_tok * kStagePitch + list;
     p.stages = fixed + 3 * xs + 8 * cs <= kMost ? 4 : 3;
     p.codes = 2 * p.stages;
     p.xs = (int)std::min<size_t>(kMaxX, (kMost - fixed - p.codes * cs) / xs);
     while (p.codes + p.stages <= kMaxCodes && fixed + p.xs * xs + (p.codes + p.stages) * cs <= kMost) p.codes += p.stages;
     smem = fixed + p.xs * xs + p.codes * cs;
-    p.list_at = (int)(smem - 1024 - (size_t)max_blocks * sizeof(int2));
+    p.list_at = (int)(smem - 1024 - list);
   }
   static std::atomic<uint64_t> attr_done;
   const cudaError_t e = smem_limit_once(&attr_done, {reinterpret_cast<const void*>(gemm_pair_kernel<kFmtQ4>), reinterpret_cast<const void*>(gemm_pair_kernel<kFmtMx>),
