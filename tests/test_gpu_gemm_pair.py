@@ -13,7 +13,8 @@ MB = 1 << 20
 # K: one 32-wide block, a 64-k step and its neighbours, a 128-k unit and its neighbours, an odd number of blocks per row (scales
 # read from 4-byte boundaries); N around one CTA's 128 and the pair's 256 features; T around 32, the tiles of 128 and 256 and
 # their multiples; long reductions of few tiles (a tile summed by two to four CTA pairs, each in several parts, with one
-# accumulator and with two) and many tiles (ranges that begin and end inside tiles).
+# accumulator and with two) and many tiles (whole ones; ranges that begin and end inside tiles are in
+# test_tiles_of_several_contributors_match_oracle).
 @pytest.mark.parametrize("fmt", ["q4", "mxfp4"])
 @pytest.mark.parametrize("N,K,T", [(1, 32, 9), (127, 64, 31), (129, 96, 33), (255, 160, 255), (257, 224, 256), (256, 256, 257), (300, 288, 513),
                                    (128, 16384, 10), (200, 4128, 65), (513, 2080, 300), (9600, 512, 12), (6001, 1056, 270), (8192, 1024, 600)])
@@ -65,6 +66,67 @@ def test_split_tiles_match_oracle_in_every_run_of_tokens(N, K, T):
     H.assert_close(outs[0].view(np.float16)[rows], O.linear(x[rows], packed, scales, O.WEIGHT_F16, round_out=True), what=f"{N}x{K} T={T}")
     assert np.all(outs[0].view(np.float16)[T] == 7.0)
     assert np.array_equal(outs[0], outs[1]) and np.array_equal(outs[0], outs[2])
+
+
+# The same for MXFP4 and fp16, with 16-byte rows and without, one accumulator and two, several parts to a contributor, and for ranges that
+# are not cut at equal fractions of a tile, so that a pair leaves parts of two (the last four).
+@pytest.mark.parametrize("fmt,N,K,T", [("mxfp4", 4096, 6016, 65), ("mxfp4", 4096, 2560, 225), ("q4", 4096, 2560, 256), ("q4", 2812, 4096, 225), ("mxfp4", 6144, 8192, 160),
+                                       ("w16", 2812, 4096, 97), ("w16", 2812, 4096, 225), ("w16", 9472, 2560, 64),
+                                       ("q4", 9728, 6144, 33), ("mxfp4", 9728, 6144, 33), ("q4", 1280, 10752, 2048), ("w16", 11494, 3904, 24)])
+def test_tiles_of_several_contributors_match_oracle(fmt, N, K, T):
+    import torch
+    from paper_2607_10183_b200 import binding as B
+    weights = (W.w16_matrix(98, 0, W.ROLE_UP, N, K),) if fmt == "w16" else (W.q4_packed if fmt == "q4" else W.mxfp4_packed)(98, 0, W.ROLE_UP, N, K)
+    x = W.activations(98, 0, (T, K))
+    ws = 16 * T * N * 4 + 2 * MB
+    ctx = B.Context(ws + 2 * N * K + 2 * MB, workspace_bytes=ws)
+    tid = (ctx.register_w16 if fmt == "w16" else ctx.register_q4)(*weights)
+    ctx.set_placement([(tid, -1, B.ATS_GPU)])
+    xd = H.to_dev(x)
+    outs = []
+    for _ in range(3):
+        y = torch.full((T + 1, N), 7.0, dtype=torch.float16, device="cuda")
+        ctx.linear(tid, xd, y, T)
+        ctx.sync()
+        outs.append(y.cpu().numpy().view(np.uint16))
+    assert ctx.stats().kernel_launches == 3  # (the sum needs no launch of its own: this is the kernel on pairs)
+    ctx.close()
+    w = torch.from_numpy(weights[0] if fmt == "w16" else O.dequantize(*weights, O.WEIGHT_F16).astype(np.float32)).cuda().double()
+    want = (xd.double() @ w.t()).cpu().numpy()  # all rows, in 64 bits
+    H.assert_close(outs[0].view(np.float16)[:T], want, what=f"{fmt} {N}x{K} T={T}")
+    assert np.all(outs[0].view(np.float16)[T] == 7.0)
+    assert np.array_equal(outs[0], outs[1]) and np.array_equal(outs[0], outs[2])
+
+
+# The residual of a down projection whose tiles have several contributors: y = rn16(x + d), bit for bit, with the d that is stored beside it.
+@pytest.mark.parametrize("fmt", ["q4", "mxfp4"])
+@pytest.mark.parametrize("T", [65, 97])
+def test_residual_in_a_tile_of_several_contributors(fmt, T):
+    import torch
+    from paper_2607_10183_b200 import binding as B
+    Hd, F = 4096, 6016
+    packed = W.q4_packed if fmt == "q4" else W.mxfp4_packed
+    mats = [packed(99, 0, role, n, k) for role, n, k in ((W.ROLE_GATE, F, Hd), (W.ROLE_UP, F, Hd), (W.ROLE_DOWN, Hd, F))]
+    x = W.activations(99, 0, (T, Hd))
+    ws = B.workspace_bytes(B.layer_desc(hidden=Hd, ffn=F, w_gate=0, w_up=0, w_down=0), T)
+    ctx = B.Context(ws + 3 * Hd * F + 4 * MB, workspace_bytes=ws)
+    ids = dict(ffn_norm=ctx.register_f16(W.norm_gain(99, 0, W.ROLE_FFN_NORM, Hd)))
+    ids.update(zip(("w_gate", "w_up", "w_down"), (ctx.register_q4(*m) for m in mats)))
+    ctx.set_placement([(ids[n], -1, B.ATS_GPU) for n in ("w_gate", "w_up", "w_down")])
+    desc = B.layer_desc(hidden=Hd, ffn=F, **ids)
+    y = torch.empty((T, Hd), dtype=torch.float16, device="cuda")
+    outs = []
+    for _ in range(2):
+        ctx.layer_prefill(desc, H.to_dev(x), y, None, None, 0, T)
+        ctx.sync()
+        outs.append(y.cpu().numpy())
+    assert ctx.stats().kernel_launches == 2 * 3  # norm, gate and up, down
+    act, d = ctx.debug_prefill_buffer(desc, T, 8), ctx.debug_prefill_buffer(desc, T, 9)
+    ctx.close()
+    w = torch.from_numpy(O.dequantize(*mats[2], O.WEIGHT_F16).astype(np.float32)).cuda().double()
+    H.assert_close(d, (torch.from_numpy(act.copy()).cuda().double() @ w.t()).cpu().numpy(), what=f"{fmt} down T={T}")
+    assert np.array_equal(outs[0].view(np.uint16), (x.astype(np.float32) + d.astype(np.float32)).astype(np.float16).view(np.uint16))
+    assert np.array_equal(outs[0].view(np.uint16), outs[1].view(np.uint16))
 
 
 # fp16 weights: K around the 64-k step and the 128-k unit (multiples of 8), the same edges of N and T, tiles of up to 256 tokens in
@@ -191,8 +253,9 @@ def test_few_features_over_many_tokens_go_to_the_pairs(fmt, N, K, T):
 
 
 # 75 tiles for 74 pairs (the one that is left is split into two, three or four where there is scratch for it) and the same as one wave
-# and a half; 4-bit and fp16.
-@pytest.mark.parametrize("fmt,N,K,T", [("q4", 19200, 4096, 40), ("q4", 28672, 1024, 40), ("mxfp4", 14336, 2048, 300), ("w16", 19200, 2048, 40)])
+# and a half (whose plans want no scratch: there is nothing to choose between); a remainder of two tiles whose parts are sums themselves; 4-bit
+# and fp16.
+@pytest.mark.parametrize("fmt,N,K,T", [("q4", 19200, 4096, 40), ("q4", 28672, 1024, 40), ("mxfp4", 14336, 2048, 300), ("w16", 19200, 2048, 40), ("mxfp4", 19456, 4096, 33)])
 def test_the_workspace_chooses_between_two_plans_only(fmt, N, K, T):
     import torch
     from paper_2607_10183_b200 import binding as B
