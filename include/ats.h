@@ -284,7 +284,10 @@ int32_t ats_unregister_host_buffer(ats_ctx* ctx, void* ptr /*HOST*/);
 /* Prefill: T tokens of one sequence at cache positions pos0 .. pos0+T-1 (pos0+T <= kv_capacity); projections run as
  * dequantize-fused tensor-core GEMMs.  Same buffers as decode with M = T.
  * Layers with routed experts (the MoE prefill of Section 5's workloads): every (token, slot) pair becomes a row, rows
- * are sorted by expert on the host from the routing ids (one synchronisation per call; T * top_k <= 65536) and each
+ * are sorted by expert (T * top_k <= 65536), on the device where every expert is resident: the call then waits for the
+ * router at its end, when everything is queued, and reports an error of a kernel up to there; else on the host from the
+ * routing ids, for which the call waits before the experts' work is queued (one synchronisation per call either way;
+ * ATS_FLAG_NO_GEMM_PAIR takes the latter for resident experts too; neither can be captured into a graph).  Each
  * projection is ONE grouped GEMM launch in which every expert multiplies its own block of rows with its own slice;
  * y = rn16(x1 + sum_j gate_j d_j) with the expert outputs d_j rounded to fp16 as every GEMM output of the prefill
  * contract is.  Host-placed experts that some token selected are brought into the part of the workspace that lies beyond

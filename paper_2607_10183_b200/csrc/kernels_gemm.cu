@@ -690,7 +690,7 @@ cudaError_t launch_gemm(const GemmParams& g, cudaStream_t st, uint64_t* n_launch
   GemmPlan pl = choose_plan(seg_rows, g.n_seg, g.T, g.ldy, total_ksteps, sm_count, scratch_bytes);
   if (g.grp_off) {
     // per-expert row counts are small next to the tile: 128-token tiles unless an expert holds several of them
-    if (g.res || g.n_groups <= 0 || g.grp_max_rows <= 0) return cudaErrorInvalidValue;
+    if (g.res || g.n_groups <= 0 || g.grp_max_rows <= 0) return cudaErrorInvalidValue;  // (no max: sorted on the device, for the pairs only)
     pl = GemmPlan{g.grp_max_rows > 256, 1, g.grp_max_rows > 256 ? 256 : 128};
   }
   const bool wide = pl.wide;

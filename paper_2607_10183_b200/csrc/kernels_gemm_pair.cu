@@ -15,7 +15,8 @@
 // to 16-byte stores (optionally + residual, or SwiGLU of 64 gate and 64 up features per CTA).  Two accumulators take turns where
 // tensor memory has room (fp16 weights; tiles of at most 128 tokens), so that the epilogue of one runs under the MMAs of the next.
 // The tensor core truncates what it adds to an accumulator, so long chains drift: where units_at_once says so, a stretch is
-// added up in parts, rounding, in words of the scratch that belong to the thread that reads them back.
+// added up in parts, rounding, in words of the scratch that belong to the thread that reads them back (two parts of a split tile: in an
+// accumulator each, where there are two).
 //
 // Work division: the (feature tile, token tile) tiles go to the pairs (one CTA per SM, persistent) in waves of neighbours, which
 // read the same weights and tokens from L2 at the same time (contiguous ranges of tiles per pair instead: 2048 tokens, fp16 gate
@@ -29,7 +30,7 @@
 // 200 more; a unit takes 0.42 to 0.47 us, of which the MMAs of 80 tokens are 0.16 and the expansion alone would be 0.16 (HBM 0.21).  That
 // is why the barriers are tested ahead and why activations come two units at a time.  fp16 there the weights' way from memory; with
 // tiles for all pairs the MMAs and the power limit; with few tiles the launch (5 us and more: entry, the pair's meeting, first loads, output)
-// and the sum of split tiles.  72 registers a thread are all that 896 threads leave: the compiler spills 84 to 128 bytes, in the
+// and the sum of split tiles.  72 registers a thread are all that 896 threads leave: the compiler spills 104 to 112 bytes, in the
 // epilogue's sums.
 // Back to back on new weights, single-CTA kernel (with reduction, residual and SwiGLU launches) -> pairs:
 //   77 tokens MXFP4: 28672 x 4096 with SwiGLU 66 -> 35 us, 4096 x 14336 41 -> 25

@@ -346,7 +346,7 @@ __global__ void __launch_bounds__(kGroupThreads) moe_group_kernel(const int32_t*
     __syncwarp();
     return before + rank;
   };
-  auto checked = [&](int e) {  // an id that names no expert: expert 0 stands in and the status word says so
+  auto checked = [&](int e) {  // an id that names no expert (the router writes none): expert 0 stands in and the status word says so
     if ((unsigned)e < (unsigned)E) return e;
     raise_status(status, 7);
     return 0;
@@ -423,7 +423,7 @@ cudaError_t launch_moe_group(const int32_t* ids, int P, int E, int* order, int* 
 // 16 bytes per thread.
 __global__ void moe_gather_rows_kernel(const __half* __restrict__ h, const int* __restrict__ order, int k, __half* __restrict__ xs,
                                        uint64_t n8, int H) {
-  asm volatile("griddepcontrol.wait;" ::: "memory");  // h comes from the preceding kernel, order from a preceding copy
+  asm volatile("griddepcontrol.wait;" ::: "memory");  // h and order come from preceding kernels (or order from a copy)
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int per_row = H / 8;
   for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n8; i += (uint64_t)gridDim.x * blockDim.x) {
