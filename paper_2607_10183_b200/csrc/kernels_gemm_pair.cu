@@ -1122,16 +1122,16 @@ PairPlan plan_of(const GemmParams& g, int sm_count, double single) {
   int rows[3] = {0, 0, 0}, n = 0, n_ft = 0;
   for (int i = 0; i < g.n_seg; ++i) n += rows[i] = g.seg[i].n_rows;
   for (int i = 0; i < g.n_seg; ++i) n_ft += feature_tiles(rows, i, g.act != nullptr);
-  const uint64_t have = g.scratch ? g.scratch_bytes : 0;
-  auto plan = [&](bool longer) {
-    auto within = [&](uint64_t bytes) { return pair_plan(rows, g.n_seg, g.act != nullptr, g.T, g.K, g.w16, longer, pairs_of_device(sm_count), bytes); };
-    const PairPlan best = within(~0ull);
-    return best.scratch <= have ? best : within(std::min(have, gemm_scratch_bytes(g.T, n, g.K)));
+  auto plan = [&](bool longer, uint64_t bytes) {
+    return pair_plan(rows, g.n_seg, g.act != nullptr, g.T, g.K, g.w16, longer, pairs_of_device(sm_count), bytes);
   };
-  const PairPlan pl = plan(true);
-  const int split = n_ft * pl.n_tt - pl.n_whole;  // tiles that several pairs share
-  const double most = pl.split_pairs == 0 ? 0.96 : pl.split_pairs <= 2 * split ? 0.93 : 0.75;
-  return rows_aligned(g) && pl.us > most * single ? plan(false) : pl;
+  PairPlan best = plan(true, ~0ull);
+  const int split = n_ft * best.n_tt - best.n_whole;  // tiles that several pairs share
+  const double most = best.split_pairs == 0 ? 0.96 : best.split_pairs <= 2 * split ? 0.93 : 0.75;
+  const bool longer = !rows_aligned(g) || best.us <= most * single;
+  if (!longer) best = plan(false, ~0ull);
+  const uint64_t have = g.scratch ? g.scratch_bytes : 0;
+  return best.scratch <= have ? best : plan(longer, std::min(have, gemm_scratch_bytes(g.T, n, g.K)));
 }
 
 }  // namespace
