@@ -383,9 +383,15 @@ struct GemmParams {
   int ldact;
   int* counters;  // kAttnMaxCounters ints, zero between launches (launch_gemm_pair: arrival counts of split tiles)
 };
-// GEMMs on pairs of CTAs (kernels_gemm_pair.cu): launches they take (operands, scratch, and faster there), and their launcher
-bool gemm_pair_eligible(const GemmParams& p, int sm_count);
-cudaError_t launch_gemm_pair(const GemmParams& p, int sm_count, cudaStream_t st, uint64_t* n_launch, std::string* err);
+// GEMMs on pairs of CTAs (kernels_gemm_pair.cu): launches they take (operands, scratch, and faster there), how they divide the work (of a launch
+// that is not grouped), and their launcher
+struct GemmPairPlan {
+  int nt, n_tt, pairs, n_whole, split_pairs, slots2, own, max_units;
+  double us;
+  uint64_t scratch;
+};
+bool gemm_pair_eligible(const GemmParams& p, int sm_count, GemmPairPlan* plan);
+cudaError_t launch_gemm_pair(const GemmParams& p, const GemmPairPlan& plan, int sm_count, cudaStream_t st, uint64_t* n_launch, std::string* err);
 // the single-CTA kernel: scratch of its plan, the k that the plan adds up in one accumulator, its time
 uint64_t gemm_scratch_bytes(int T, int n_total, int K);
 int gemm_chain(const int* rows, int n_seg, int T, int K);

@@ -331,8 +331,9 @@ static int32_t launch_gemm_any(ats_ctx* ctx, GemmParams p) {
   __half* act = p.act;
   p.counters = reinterpret_cast<int*>(ctx->ws) + 64;  // (the attention's: zero between launches, and launches follow one another)
   const bool pairs = !(ctx->cfg.flags & ATS_FLAG_NO_GEMM_PAIR);
-  if (pairs && gemm_pair_eligible(p, ctx->sm_count)) {
-    e = launch_gemm_pair(p, ctx->sm_count, ctx->cs, &ctx->stats.kernel_launches, &err);
+  GemmPairPlan plan{};
+  if (pairs && gemm_pair_eligible(p, ctx->sm_count, &plan)) {
+    e = launch_gemm_pair(p, plan, ctx->sm_count, ctx->cs, &ctx->stats.kernel_launches, &err);
     act = nullptr;
   } else {
     e = launch_gemm(p, ctx->cs, &ctx->stats.kernel_launches, &err);
@@ -353,7 +354,8 @@ static int32_t run_gemm_group(ats_ctx* ctx, Operand* ops, int n, GemmParams p) {
     probe.counters = reinterpret_cast<int*>(ctx->ws) + 64;
     probe.n_seg = n;
     for (int i = 0; i < n; ++i) probe.seg[i] = GemvSeg{nullptr, (int)ops[i].t->d.n_out};
-    together = !(ctx->cfg.flags & ATS_FLAG_NO_GEMM_PAIR) && gemm_pair_eligible(probe, ctx->sm_count);
+    GemmPairPlan plan{};
+    together = !(ctx->cfg.flags & ATS_FLAG_NO_GEMM_PAIR) && gemm_pair_eligible(probe, ctx->sm_count, &plan);
   }
   if (together) {
     ATS_TRY(acquire_ops(ctx, ops, n));

@@ -1032,11 +1032,6 @@ int feature_tiles(const int* rows, int seg, bool act) {
   return act ? (seg ? 0 : (rows[0] + kFeat - 1) / kFeat) : (rows[seg] + 2 * kFeat - 1) / (2 * kFeat);
 }
 
-struct PairPlan {
-  int nt, n_tt, pairs, n_whole, split_pairs, slots2, own, max_units;
-  double us;
-  uint64_t scratch;
-};
 // Time in us of the ways to divide the work (see the kernel's comment).  A unit costs its MMAs, the expansion of its weights
 // or their way from memory, whichever is longest; a tile its epilogue; a stretch that is added up in several parts their way out and
 // back, less where the MMAs go on meanwhile in the other accumulator; a split tile the parts' way through L2.  The figures are fitted
@@ -1044,8 +1039,8 @@ struct PairPlan {
 // within a third of the best (6 % rms off; many waves run 8 % slower, at the power limit; later 8 products whose contributors have several parts,
 // 6144 x 4096 over 160 tokens among them, taken at 21.4 us for 24.2, where the single-CTA kernel needs 22.5), fp16's to about 400 with the sums
 // of split tiles as they were when one contributor made them (10 %).  pairs = 0: the scratch holds none.
-PairPlan pair_plan(const int* rows, int n_seg, bool act, int T, int K, bool w16, bool longer, int max_pairs, uint64_t scratch_bytes) {
-  PairPlan best{};
+GemmPairPlan pair_plan(const int* rows, int n_seg, bool act, int T, int K, bool w16, bool longer, int max_pairs, uint64_t scratch_bytes) {
+  GemmPairPlan best{};
   best.us = 1e300;
   int n_ft = 0;
   for (int i = 0; i < n_seg; ++i) n_ft += feature_tiles(rows, i, act);
@@ -1085,7 +1080,7 @@ PairPlan pair_plan(const int* rows, int n_seg, bool act, int T, int K, bool w16,
       us += launch + waves * stretch(units, 0);
       if (w16) us = std::max(us, weights_mb / 4.5);
       if (us >= best.us) return;
-      best = PairPlan{nt, n_tt, pairs, slots ? tiles - rem : tiles, n, slots == 2, parts, max_units, us, need};
+      best = GemmPairPlan{nt, n_tt, pairs, slots ? tiles - rem : tiles, n, slots == 2, parts, max_units, us, need};
     };
     take(rem ? stretch(units, 0) : 0.0, units, 0, 0);
     for (int s = 2; s <= kMaxParts && s <= units && rem && rem * s <= max_pairs; ++s)
@@ -1118,14 +1113,14 @@ double single_cta_us(const GemmParams& g) {
 // `single`: time of the single-CTA kernel.  Chains of 1536 k are for products that the pairs take in clearly less: where both kernels are
 // about equally fast, the one that drops more has nothing to offer.  The more contributors a tile has, the fewer the tiles and the shorter
 // the single-CTA kernel's own chains (6144 x 4096, 77 tokens: three contributors would sum 1408 k in one accumulator against its 704).
-PairPlan plan_of(const GemmParams& g, int sm_count, double single) {
+GemmPairPlan plan_of(const GemmParams& g, int sm_count, double single) {
   int rows[3] = {0, 0, 0}, n = 0, n_ft = 0;
   for (int i = 0; i < g.n_seg; ++i) n += rows[i] = g.seg[i].n_rows;
   for (int i = 0; i < g.n_seg; ++i) n_ft += feature_tiles(rows, i, g.act != nullptr);
   auto plan = [&](bool longer, uint64_t bytes) {
     return pair_plan(rows, g.n_seg, g.act != nullptr, g.T, g.K, g.w16, longer, pairs_of_device(sm_count), bytes);
   };
-  PairPlan best = plan(true, ~0ull);
+  GemmPairPlan best = plan(true, ~0ull);
   const int split = n_ft * best.n_tt - best.n_whole;  // tiles that several pairs share
   const double most = best.split_pairs == 0 ? 0.96 : best.split_pairs <= 2 * split ? 0.93 : 0.75;
   const bool longer = !rows_aligned(g) || best.us <= most * single;
@@ -1136,7 +1131,7 @@ PairPlan plan_of(const GemmParams& g, int sm_count, double single) {
 
 }  // namespace
 
-bool gemm_pair_eligible(const GemmParams& g, int sm_count) {
+bool gemm_pair_eligible(const GemmParams& g, int sm_count, GemmPairPlan* plan) {
   if ((g.w16 && g.grp_off) || g.n_seg < 1 || g.n_seg > 3 || !g.counters || g.K % (g.w16 ? 8 : 32) || g.K > (1 << 24) || g.ldx % 8) return false;
   if (reinterpret_cast<uintptr_t>(g.x) & 15) return false;
   if ((g.res != nullptr) != (g.y2 != nullptr)) return false;
@@ -1154,13 +1149,13 @@ bool gemm_pair_eligible(const GemmParams& g, int sm_count) {
   // one, SwiGLU is a launch of its own beside it, and rows of y that are not 16-byte aligned it stores by the element (3333 x 9984, 300
   // tokens: 53 against 85).
   double single = single_cta_us(g);
-  const PairPlan pl = plan_of(g, sm_count, single);
+  const GemmPairPlan pl = *plan = plan_of(g, sm_count, single);
   if (!rows_aligned(g)) return pl.pairs > 0;
   if (g.w16 && pl.n_whole > pl.pairs) single *= 1.06;  // (the fit is that far off there: 14336 x 4096 over 700 tokens 83 us on the pairs, 97)
   return pl.pairs > 0 && pl.us <= single;
 }
 
-cudaError_t launch_gemm_pair(const GemmParams& g, int sm_count, cudaStream_t st, uint64_t* n_launch, std::string* err) {
+cudaError_t launch_gemm_pair(const GemmParams& g, const GemmPairPlan& pl, int sm_count, cudaStream_t st, uint64_t* n_launch, std::string* err) {
   TensorMapEncodeFn enc = tensor_map_encode();
   if (!enc) {
     if (err) *err = "cuTensorMapEncodeTiled is not available from the driver";
@@ -1201,7 +1196,6 @@ cudaError_t launch_gemm_pair(const GemmParams& g, int sm_count, cudaStream_t st,
     p.n_tt = 1;
     p.pairs = (int)std::min<long long>((long long)n_ft * max_blocks, max_pairs);
   } else {
-    const PairPlan pl = plan_of(g, sm_count, single_cta_us(g));
     if (!pl.pairs) return cudaErrorInvalidValue;
     p.nt = pl.nt;
     p.n_tt = pl.n_tt;
