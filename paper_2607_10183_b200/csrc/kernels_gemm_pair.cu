@@ -25,15 +25,17 @@
 // the scratch: every contributor leaves its part there, 32 tokens at a time; the last one to do so for these tokens adds the parts in
 // ascending k order (so the result does not depend on who that is) and writes them.  Nobody waits for anybody.
 //
-// What bounds it: 4-bit, up to about 128 tokens, the MMA warp's chain: its eight MMAs and its commits take 430 cycles to issue among the
-// expanding warps of its scheduler, whatever the number of tokens (alone: 200), and a wait that is not known to be over when it begins costs
-// 200 more; a unit takes 0.42 to 0.47 us, of which the MMAs of 80 tokens are 0.16 and the expansion alone would be 0.16 (HBM 0.21).  That
-// is why the barriers are tested ahead and why activations come two units at a time.  fp16 there the weights' way from memory; with
-// tiles for all pairs the MMAs and the power limit; with few tiles the launch (5 us and more: entry, the pair's meeting, first loads, output)
-// and the sum of split tiles.  72 registers a thread are all that 896 threads leave: the compiler spills 104 to 112 bytes, in the
-// epilogue's sums.
+// What bounds it: 4-bit, up to about 128 tokens, the MMA warp's chain among the expanding warps of its scheduler; a wait that is not known
+// to be over when it begins costs 200 cycles: that is why the barriers are tested ahead and why activations come two units at a time.  A
+// unit takes 0.32 to 0.39 us, of which the MMAs of 80 tokens are 0.16 and the expansion alone would be 0.16 (HBM 0.21).  The roles branch on a
+// warp number that the compiler knows to be the same for the warp, and nothing in the MMA warp's loop looks as if lanes could differ: else
+// every operand of every MMA is moved to a uniform register by itself, and eight MMAs and two commits take 180 cycles to issue where they
+// take 80 (430 among the expanding warps; a unit 0.42 to 0.48 us; 77 tokens MXFP4, 28672 x 4096 31.5 -> 27.7 us, 512 tokens Q4, 4096 x 14336
+// 59.2 -> 54.9).  fp16 there the weights' way from memory; with tiles for all pairs the MMAs and the power limit; with few tiles the launch
+// (5 us and more: entry, the pair's meeting, first loads, output) and the sum of split tiles.  72 registers a thread are all that 896 threads
+// leave: the compiler spills 96 to 104 bytes, in the epilogue's sums.
 // Back to back on new weights, single-CTA kernel (with reduction, residual and SwiGLU launches) -> pairs:
-//   77 tokens MXFP4: 28672 x 4096 with SwiGLU 66 -> 35 us, 4096 x 14336 41 -> 25
+//   77 tokens MXFP4: 28672 x 4096 with SwiGLU 66 -> 32 us, 4096 x 14336 41 -> 24
 //   512 tokens Q4: gate and up 143 -> 91 us, 4096 x 14336 78 -> 60;  2048 tokens: gate and up 462 -> 328 to 351 (1372 TFLOP/s)
 //   2048 tokens fp16: q, k, v 152 -> 78 us, o 66 -> 59, gate and up 451 -> 346 (1390 TFLOP/s)
 //
@@ -44,8 +46,7 @@
 
 #include <cmath>
 
-#include "ats_internal.h"
-#include "sm100_umma.cuh"
+#include "gemm_tiles.cuh"
 
 namespace ats {
 
@@ -66,30 +67,15 @@ constexpr int kMaxParts = 4;               // contributors of a split tile at mo
 constexpr uint32_t kColA = 256;            // tensor-memory columns: accumulator 0..255, weight stages from 256 on
 constexpr uint32_t kClearPeer = 0xFEFFFFFFu;
 
-struct PairSeg {
-  const uint8_t* base;
-  int n_rows;
-  int tile0;  // first feature tile of the segment
-  int col0;   // first output column of the segment
-};
-struct PairParams {
-  PairSeg seg[3];
-  int n_seg;
-  int K, T;
-  int n_ft, n_tt;     // feature tiles, token tiles
-  int nt;             // tokens per tile
-  int units, ksteps;  // per tile: 128-k units, 64-k steps
-  int pairs;
-  int n_whole;        // tiles that a pair has to itself; the units of the others are divided over ...
-  int split_pairs;    // ... this many pairs
+struct PairParams : TileWork {  // (workers: pairs; units: 128 k)
+  int ksteps;             // 64-k steps per tile
   int stages, codes, xs;  // depths of the rings: weights in tensor memory, codes (a multiple of it), activations
   int xu;             // units of activations that a place in their ring holds
   int sc16;           // scale rows are 16-byte aligned
-  __half* y;
+  __half* y;          // (SwiGLU: may be null)
   int ldy;
   const __half* res;  // optional: y2 = rn16(res + y)
   __half* y2;
-  __half* act;        // optional: SwiGLU of segments 0 (gate) and 1 (up); y may then be null
   int ldact;
   float* partial;     // slots of 2 * 128 features x slot_tok tokens
   int slot_tok;
@@ -99,8 +85,6 @@ struct PairParams {
   int max_units;      // units that one accumulator adds up at most
   int* counters;      // [2 * pairs], zero between launches
   int* status;
-  const int* grp_off;  // grouped form: row offsets per expert
-  int ft_per, n_groups, list_at;  // ... feature tiles per expert, experts, place of the list of blocks in shared memory
   unsigned long long grp_stride;
 };
 
@@ -115,14 +99,12 @@ __device__ __forceinline__ void pair_sync() {
   pair_arrive();
   pair_wait();
 }
-__device__ __forceinline__ void prefetch_map(const CUtensorMap* map) { asm volatile("prefetch.tensormap [%0];" ::"l"(map) : "memory"); }
 // arrival on the leader's copy of a barrier (from either CTA)
 __device__ __forceinline__ void arrive_leader(uint64_t* own) {
   uint32_t a;
   asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(a) : "r"(smem_u32(own)));
   asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(a) : "memory");
 }
-// Loads are issued like MMAs: by all lanes of a warp, in flow that is the same for the warp, with the instruction left to one.
 __device__ __forceinline__ void tma_pair_2d(uint32_t one, uint32_t dst, const CUtensorMap* map, int x, int y, uint64_t* own_bar) {
   asm volatile(
       "{\n.reg .pred q;\nsetp.ne.b32 q, %5, 0;\n@q cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes "
@@ -137,20 +119,6 @@ __device__ __forceinline__ void tma_pair_3d(uint32_t one, uint32_t dst, const CU
       "l"(map), "r"(x), "r"(y), "r"(0), "r"(smem_u32(own_bar) & kClearPeer), "r"(one)
       : "memory");
 }
-__device__ __forceinline__ void tma_3d_one(uint32_t one, uint32_t dst, const CUtensorMap* map, int x, int y, int z, uint64_t* bar) {
-  asm volatile(
-      "{\n.reg .pred q;\nsetp.ne.b32 q, %6, 0;\n@q cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, "
-      "{%2, %3, %4}], [%5];\n}" ::"r"(dst),
-      "l"(map), "r"(x), "r"(y), "r"(z), "r"(smem_u32(bar)), "r"(one)
-      : "memory");
-}
-__device__ __forceinline__ void expect_tx_one(uint32_t one, uint64_t* bar, uint32_t bytes) {
-  asm volatile("{\n.reg .pred q;\nsetp.ne.b32 q, %2, 0;\n@q mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n}" ::"r"(smem_u32(bar)),
-               "r"(bytes), "r"(one)
-               : "memory");
-}
-// The value of any lane (all hold the same) as one the compiler knows to be the same for the warp.
-__device__ __forceinline__ int uniform(int v) { return (int)__reduce_max_sync(0xffffffffu, (unsigned)v); }
 __device__ __forceinline__ void umma_ts_pair(uint32_t one, uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
   asm volatile(
       "{\n.reg .pred p, q;\nsetp.ne.b32 p, %4, 0;\nsetp.ne.b32 q, %5, 0;\n@q tcgen05.mma.cta_group::2.kind::f16 [%0], [%1], %2, %3, p;\n}" ::"r"(
@@ -179,77 +147,6 @@ __device__ __forceinline__ void cp_async4z(uint32_t dst, const void* src, bool l
 __device__ __forceinline__ void cp_async_arrive(uint64_t* bar) {
   asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
-// (32-bit shared addresses: the pointers into the aligned dynamic array would make generic accesses)
-__device__ __forceinline__ uint4 lds128(uint32_t a) {
-  uint4 v;
-  asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a));
-  return v;
-}
-__device__ __forceinline__ uint2 lds64(uint32_t a) {
-  uint2 v;
-  asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(a));
-  return v;
-}
-__device__ __forceinline__ uint32_t lds32(uint32_t a) {
-  uint32_t v;
-  asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a));
-  return v;
-}
-__device__ __forceinline__ void sts16(uint32_t a, __half v) { asm volatile("st.shared.u16 [%0], %1;" ::"r"(a), "h"(__half_as_ushort(v)) : "memory"); }
-__device__ __forceinline__ __half2 as_h2(uint32_t v) {
-  __half2 h;
-  *reinterpret_cast<uint32_t*>(&h) = v;
-  return h;
-}
-__device__ __forceinline__ uint32_t as_u32(__half2 h) { return *reinterpret_cast<uint32_t*>(&h); }
-// (v & mask) | or_bits in one instruction (left to itself the compiler takes eight logic operations per word, not five)
-__device__ __forceinline__ uint32_t and_or(uint32_t v, uint32_t mask, uint32_t or_bits) {
-  uint32_t d;
-  asm("lop3.b32 %0, %1, %2, %3, 0xEA;" : "=r"(d) : "r"(v), "r"(mask), "r"(or_bits));
-  return d;
-}
-// One code word (8 codes, internal nibble order) times the block scale -> 8 fp16 weights, k ascending.
-template <bool MX>
-__device__ __forceinline__ void expand_word(uint32_t w, __half2 s2, uint32_t* o) {
-  if (MX) {
-    // byte j of a word: codes (0, 2), (4, 6), (1, 3), (5, 7); half of the instructions of shifts and masks (77 tokens, 28672 x
-    // 4096: 41.1 -> 37.2 us)
-    uint32_t c[4];
-    cvt_e2m1x8(w, c);
-    o[0] = as_u32(__hmul2(as_h2(__byte_perm(c[0], c[2], 0x5410)), s2));
-    o[1] = as_u32(__hmul2(as_h2(__byte_perm(c[0], c[2], 0x7632)), s2));
-    o[2] = as_u32(__hmul2(as_h2(__byte_perm(c[1], c[3], 0x5410)), s2));
-    o[3] = as_u32(__hmul2(as_h2(__byte_perm(c[1], c[3], 0x7632)), s2));
-  } else {
-    const uint32_t kMagic = 0x64006400u, w8 = w >> 8;
-    const __half2 k1032 = as_h2(0x64086408u), k16th = as_h2(0x2C002C00u), kM72 = as_h2(0xD480D480u);
-    o[0] = as_u32(__hmul2(__hsub2(as_h2(and_or(w, 0x000F000Fu, kMagic)), k1032), s2));
-    o[1] = as_u32(__hmul2(__hfma2(as_h2(and_or(w, 0x00F000F0u, kMagic)), k16th, kM72), s2));
-    o[2] = as_u32(__hmul2(__hsub2(as_h2(and_or(w8, 0x000F000Fu, kMagic)), k1032), s2));
-    o[3] = as_u32(__hmul2(__hfma2(as_h2(and_or(w8, 0x00F000F0u, kMagic)), k16th, kM72), s2));
-  }
-}
-// A warp waits with all its lanes; try_wait lets the hardware park it, so that the many waiting warps leave the issue slots
-// and the barrier unit to those that work (polling with test_wait cost 3 to 20 %).
-__device__ __forceinline__ bool wait_warp(uint64_t* bar, uint32_t parity) {
-  return __all_sync(0xffffffffu, mbar_wait_suspending(bar, parity));
-}
-// A test whose result is looked at later: its latency (about 200 cycles here) passes under other work.
-__device__ __forceinline__ bool peek(uint64_t* bar, uint32_t parity) { return mbar_test_wait(bar, parity); }
-
-__device__ __forceinline__ void tmem_ld_x16(uint32_t taddr, uint32_t* v) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]), "=r"(v[9]),
-        "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
-      : "r"(taddr)
-      : "memory");
-}
-__device__ __forceinline__ void tmem_ld_wait_x16(uint32_t* v) {
-  asm volatile("tcgen05.wait::ld.sync.aligned;"
-               : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]), "+r"(v[6]), "+r"(v[7]), "+r"(v[8]), "+r"(v[9]),
-                 "+r"(v[10]), "+r"(v[11]), "+r"(v[12]), "+r"(v[13]), "+r"(v[14]), "+r"(v[15])::"memory");
-}
 template <int N>
 struct Int {
   static constexpr int value = N;
@@ -257,75 +154,6 @@ struct Int {
 struct PairMaps {
   CUtensorMap codes[3], scales[3];  // of the segments (scales: where their rows are 16-byte aligned)
 };
-// One stretch of a pair's work: units u0 .. u1-1 of a tile.
-struct Stretch {
-  int tile, u0, u1;
-};
-// Walks a pair's stretches; the same sequence in every role of both CTAs.
-struct Walk {
-  int tile, step, n_whole;  // whole tiles: pair, pair + pairs, ... (neighbours in L2 run at the same time)
-  int units;
-  unsigned at, end;         // the pair's range of the last tiles' units, counted from tile n_whole on
-  __device__ __forceinline__ Walk(const PairParams& p, int pair, int whole) {
-    units = p.units;
-    tile = pair;
-    step = p.pairs;
-    n_whole = whole;
-    const unsigned n = p.grp_off ? 0u : (unsigned)(p.n_ft * p.n_tt - whole) * units;  // (below 74 tiles of 128k units, see gemm_pair_eligible)
-    at = pair < p.split_pairs ? n * pair / p.split_pairs : 0;
-    end = pair < p.split_pairs ? n * (pair + 1) / p.split_pairs : 0;
-  }
-  __device__ __forceinline__ bool next(Stretch& s) {
-    if (tile < n_whole) {
-      s.tile = tile;
-      s.u0 = 0;
-      s.u1 = units;
-      tile += step;
-      return true;
-    }
-    if (at >= end) return false;
-    const int t = (int)(at / (unsigned)units);
-    s.tile = n_whole + t;
-    s.u0 = (int)at - t * units;
-    s.u1 = min(units, s.u0 + (int)(end - at));
-    at += s.u1 - s.u0;
-    return true;
-  }
-};
-// Which rows, tokens and expert a tile stands for.
-struct Tile {
-  int sg, row0;        // segment, first feature row of the PAIR within it (SwiGLU: first feature of the 128)
-  int t0, T, rowoff;   // first token, tokens of the matrix (of the block of an expert's rows), its first row
-  int expert;
-};
-// Grouped form: the experts' rows in blocks of at most nt, in shared memory: expert | first row << 10.  The blocks follow one another, so the
-// next one's first row ends it (behind the last: all rows).
-__device__ __forceinline__ Tile tile_of(const PairParams& p, int tile, const uint32_t* blocks) {
-  Tile r;
-  int ft = tile / (p.grp_off ? p.ft_per : p.n_tt);
-  if (p.grp_off) {  // feature tiles of one block after another
-    const uint32_t b = blocks[ft], e = blocks[ft + 1];
-    ft = tile - ft * p.ft_per;
-    r.expert = (int)(b & 1023u);
-    r.t0 = 0;
-    r.rowoff = (int)(b >> 10);
-    r.T = (int)(e >> 10) - r.rowoff;
-  } else {
-    r.expert = 0;
-    r.t0 = (tile - ft * p.n_tt) * p.nt;
-    r.T = p.T;
-    r.rowoff = 0;
-  }
-  r.sg = 0;
-  if (p.act) {
-    r.row0 = ft * kFeat;
-  } else {
-    while (r.sg + 1 < p.n_seg && ft >= p.seg[r.sg + 1].tile0) ++r.sg;
-    r.row0 = (ft - p.seg[r.sg].tile0) * 2 * kFeat;
-  }
-  return r;
-}
-
 // Units that go into an accumulator before it is handed over: a stretch in equal parts of p.max_units at most.
 __device__ __forceinline__ int seg_units(const PairParams& p, int n) {
   return n <= p.max_units ? n : (n + (n - 1) / p.max_units) / ((n + p.max_units - 1) / p.max_units);
@@ -339,7 +167,7 @@ __global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid
   __shared__ uint64_t afull[kMaxA], aempty[kMaxA], xfull[kMaxX], xempty[kMaxX], cfull[kMaxCodes], cempty[kMaxCodes], acc_full[2], d_empty[2];
   __shared__ uint32_t tmem_s;
   __shared__ int last_s[2][4], n_blocks_s;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31, warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);  // (the same for the warp, and known to be)
   const uint32_t rank = cta_rank();
   const int pair = blockIdx.x >> 1;
   const int S = p.stages, NC = p.codes, NX = p.xs;
@@ -403,24 +231,8 @@ __global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid
   int n_whole = p.n_whole;
   if (p.grp_off) {
     if (warp == 4) {
-      const int per = (p.n_groups + 31) / 32, e0 = min(lane * per, p.n_groups), e1 = min(e0 + per, p.n_groups);
-      int n = 0, incl;
-      for (int e = e0; e < e1; ++e) n += (p.grp_off[e + 1] - p.grp_off[e] + p.nt - 1) / p.nt;
-      incl = n;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int v = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += v;
-      }
-      int at = incl - n;
-      for (int e = e0; e < e1; ++e) {
-        const int hi = p.grp_off[e + 1];
-        for (int r = p.grp_off[e]; r < hi; r += p.nt) blocks[at++] = (uint32_t)(e | r << 10);
-      }
-      if (lane == 31) {
-        blocks[incl] = (uint32_t)p.T << 10;
-        n_blocks_s = incl;
-      }
+      const int n = list_blocks(p, blocks, lane);
+      if (lane == 31) n_blocks_s = n;
     }
     __syncthreads();
     n_whole = n_blocks_s * p.ft_per;
@@ -575,7 +387,7 @@ __global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid
         int s = 0, sx = 0, xi = 0, seg = 0;  // places in the rings, unit of the activations' place, accumulator segments so far
         uint32_t par = 0, parx = 0;
         bool ready = false, readyx = false;
-        while (uniform(ok && mine.next(st))) {
+        while (uniform(mine.next(st))) {
           const int u0 = uniform(st.u0), u1 = uniform(st.u1);
           int left = 0;  // units until the accumulator is handed over
           uint32_t d = 0, accumulate = 0;
@@ -586,17 +398,11 @@ __global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid
               accumulate = 0;
               const int b = two ? seg & 1 : 0, use = two ? seg >> 1 : seg;
               d = kAcc * b;
-              if (use > 0 && !wait_warp(&d_empty[b], (use - 1) & 1)) {
-                ok = false;
-                break;
-              }
+              if (use > 0 && !wait_warp(&d_empty[b], (use - 1) & 1)) return false;
             }
             if constexpr (FMT == kFmtW16) {
-              for (int ks = 2 * u; ok && ks < min(2 * u + 2, p.ksteps); ++ks) {
-                if (!__all_sync(0xffffffffu, readyx) && !wait_warp(&xfull[sx], parx)) {
-                  ok = false;
-                  break;
-                }
+              for (int ks = 2 * u; ks < min(2 * u + 2, p.ksteps); ++ks) {
+                if (!__all_sync(0xffffffffu, readyx) && !wait_warp(&xfull[sx], parx)) return false;
                 tc_fence_after();
                 const int sxn = sx + 1 == NX ? 0 : sx + 1;
                 const uint32_t parxn = sx + 1 == NX ? parx ^ 1u : parx;
@@ -614,21 +420,14 @@ __global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid
                 umma_commit_both(one, &xempty[sx]);
                 sx = sxn, parx = parxn;
               }
-              if (!ok) break;
               if (--left == 0) {
                 umma_commit_both(one, &acc_full[two ? seg & 1 : 0]);
                 ++seg;
               }
               continue;
             }
-            if (!__all_sync(0xffffffffu, ready) && !wait_warp(&afull[s], par)) {
-              ok = false;
-              break;
-            }
-            if (xi == 0 && !__all_sync(0xffffffffu, readyx) && !wait_warp(&xfull[sx], parx)) {
-              ok = false;
-              break;
-            }
+            if (!__all_sync(0xffffffffu, ready) && !wait_warp(&afull[s], par)) return false;
+            if (xi == 0 && !__all_sync(0xffffffffu, readyx) && !wait_warp(&xfull[sx], parx)) return false;
             tc_fence_after();
             const int sn = s + 1 == S ? 0 : s + 1, sxn = sx + 1 == NX ? 0 : sx + 1;
             const uint32_t parn = s + 1 == S ? par ^ 1u : par, parxn = sx + 1 == NX ? parx ^ 1u : parx;
@@ -656,10 +455,11 @@ __global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid
             if (xlast) sx = sxn, parx = parxn;
           }
         }
+        return true;
       };
       if (rank == 0) {
-        if (FMT != kFmtW16 && p.xu == 2) issue(Int<2>{});
-        else issue(Int<1>{});
+        if (FMT != kFmtW16 && p.xu == 2) ok = issue(Int<2>{});
+        else ok = issue(Int<1>{});
       }
     } else {
       // ------------------------------------------------------------ code and scale loaders, continued
@@ -921,11 +721,11 @@ __global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid
       // tokens 28.6 -> 25.1 us, 256 tokens in two parts 46.9 -> 40.2, against one contributor that sums the whole tile).  The warps of even
       // and odd runs of tokens go their own ways.
       const unsigned n_units = (unsigned)(p.n_ft * p.n_tt - p.n_whole) * p.units, lo = (unsigned)(st.tile - p.n_whole) * p.units;
-      const int first = (int)(((lo + 1) * p.split_pairs - 1) / n_units);
-      const int n_con = (int)(((lo + p.units) * p.split_pairs - 1) / n_units) - first + 1;
+      const int first = (int)(((lo + 1) * p.split_workers - 1) / n_units);
+      const int n_con = (int)(((lo + p.units) * p.split_workers - 1) / n_units) - first + 1;
       auto part_of = [&](int q) {  // this CTA's half of what pair q leaves of the tile
         // (the first contributor begins the tile, the others come upon it at the start of their range)
-        return p.partial + ((size_t)(p.slots2 && q == first ? p.split_pairs + q : q) * 2 + rank) * kFeat * p.slot_tok + feat;
+        return p.partial + ((size_t)(p.slots2 && q == first ? p.split_workers + q : q) * 2 + rank) * kFeat * p.slot_tok + feat;
       };
       auto half_sync = [&] { asm volatile("bar.sync %0, 128;" ::"r"(3 + half) : "memory"); };
       unsigned* cnt = reinterpret_cast<unsigned*>(p.counters) + 2 * first + rank;  // four bits for every 32 tokens
@@ -1166,7 +966,7 @@ cudaError_t launch_gemm_pair(const GemmParams& g, const GemmPairPlan& pl, int sm
   int rows[3] = {0, 0, 0}, n_ft = 0, col = 0;
   for (int i = 0; i < g.n_seg; ++i) {
     rows[i] = g.seg[i].n_rows;
-    p.seg[i] = PairSeg{g.seg[i].base, rows[i], n_ft, col};
+    p.seg[i] = TileSeg{g.seg[i].base, rows[i], n_ft, col};
     n_ft += feature_tiles(rows, i, g.act != nullptr);
     col += g.seg[i].n_rows;
   }
@@ -1174,6 +974,7 @@ cudaError_t launch_gemm_pair(const GemmParams& g, const GemmPairPlan& pl, int sm
   p.T = g.T;
   p.units = (g.K + kUnitK - 1) / kUnitK;
   p.ksteps = (g.K + 63) / 64;
+  p.tile_rows = g.act ? kFeat : 2 * kFeat;
   const int max_pairs = pairs_of_device(sm_count);
   p.max_units = p.units;
   int max_blocks = 0;  // of an expert's rows, at most
@@ -1194,15 +995,15 @@ cudaError_t launch_gemm_pair(const GemmParams& g, const GemmPairPlan& pl, int sm
     max_blocks = std::min(g.n_groups, g.T) + g.T / p.nt;
     p.ft_per = n_ft;
     p.n_tt = 1;
-    p.pairs = (int)std::min<long long>((long long)n_ft * max_blocks, max_pairs);
+    p.workers = (int)std::min<long long>((long long)n_ft * max_blocks, max_pairs);
   } else {
     if (!pl.pairs) return cudaErrorInvalidValue;
     p.nt = pl.nt;
     p.n_tt = pl.n_tt;
     p.n_ft = n_ft;
-    p.pairs = pl.pairs;
+    p.workers = pl.pairs;
     p.n_whole = pl.n_whole;
-    p.split_pairs = pl.split_pairs;
+    p.split_workers = pl.split_pairs;
     p.slots2 = pl.slots2;
     if (pl.own) p.max_units = pl.max_units;
   }
@@ -1215,7 +1016,7 @@ cudaError_t launch_gemm_pair(const GemmParams& g, const GemmPairPlan& pl, int sm
   p.ldact = g.ldact;
   p.partial = (float*)g.scratch;
   p.slot_tok = std::min(p.nt, g.T);
-  p.own = p.partial + (size_t)(p.split_pairs * (p.slots2 ? 2 : 1)) * 2 * kFeat * p.slot_tok;
+  p.own = p.partial + (size_t)(p.split_workers * (p.slots2 ? 2 : 1)) * 2 * kFeat * p.slot_tok;
   p.counters = g.counters;
   p.status = g.status;
   p.grp_off = g.grp_off;
@@ -1285,7 +1086,7 @@ cudaError_t launch_gemm_pair(const GemmParams& g, const GemmPairPlan& pl, int sm
                                                      reinterpret_cast<const void*>(gemm_pair_kernel<kFmtW16>)}, kMost);
   if (e != cudaSuccess) return e;
   ++*n_launch;
-  auto run = [&](auto* kernel) { return launch_dep(kernel, dim3(2 * p.pairs), dim3(kPairThreads), smem, st, g.pdl, 2, xmap, maps, p); };
+  auto run = [&](auto* kernel) { return launch_dep(kernel, dim3(2 * p.workers), dim3(kPairThreads), smem, st, g.pdl, 2, xmap, maps, p); };
   return g.w16 ? run(gemm_pair_kernel<kFmtW16>) : g.mx ? run(gemm_pair_kernel<kFmtMx>) : run(gemm_pair_kernel<kFmtQ4>);
 }
 
