@@ -77,7 +77,7 @@ enum {
   ATS_FLAG_SKIP_SCALE_CHECK = 2u, /* do not scan scales for Inf/NaN at registration */
   ATS_FLAG_TIME_KERNELS = 4u,     /* bracket every GEMV / grouped GEMV / GEMM launch with CUDA events (see ats_stats.timed_*) */
   ATS_FLAG_NO_PDL = 8u,           /* launch every kernel fully serialized (no programmatic dependent launch overlap) */
-  ATS_FLAG_NO_GEMM_PAIR = 32u,    /* do not run large GEMMs as pairs of CTAs on two SMs (tcgen05 cta_group::2): the single-CTA kernel only */
+  ATS_FLAG_NO_GEMM_PAIR = 32u,    /* do not run large GEMMs as pairs of CTAs on two SMs (tcgen05 cta_group::2): the single-CTA kernels only */
   ATS_FLAG_MOE_RING_ONLY = 16u,   /* Decode-step MoE stages with host-placed experts always take the staging ring (ids to
                                      the host, one cudaMemcpyAsync per chunk of every selected host-placed slice on the
                                      transfer stream, counted in ats_stats.streamed_bytes / copies / host_syncs).

@@ -391,7 +391,20 @@ struct GemmPairPlan {
   uint64_t scratch;
 };
 bool gemm_pair_eligible(const GemmParams& p, int sm_count, GemmPairPlan* plan);
+// the one of these two kernels that would take the product with all the scratch it wants: its time, and the k that it adds up in one accumulator
+struct GemmOther {
+  double us;
+  int chain;
+};
+GemmOther gemm_other(const GemmParams& p, int sm_count);
 cudaError_t launch_gemm_pair(const GemmParams& p, const GemmPairPlan& plan, int sm_count, cudaStream_t st, uint64_t* n_launch, std::string* err);
+// GEMMs of few tokens, 4-bit formats, on single CTAs (kernels_gemm_few.cu)
+struct GemmFewPlan {
+  int mode, nt, n_tt, n_ft, parts, turns, max_units;
+  double us;
+};
+bool gemm_few_eligible(const GemmParams& p, int sm_count, GemmFewPlan* plan);
+cudaError_t launch_gemm_few(const GemmParams& p, const GemmFewPlan& plan, int sm_count, cudaStream_t st, uint64_t* n_launch, std::string* err);
 // the single-CTA kernel: scratch of its plan, the k that the plan adds up in one accumulator, its time
 uint64_t gemm_scratch_bytes(int T, int n_total, int K);
 int gemm_chain(const int* rows, int n_seg, int T, int K);

@@ -323,7 +323,8 @@ static int32_t run_gemv_group(ats_ctx* ctx, Operand* ops, int n, GemvParams p) {
   return ATS_OK;
 }
 
-// One GEMM launch: on pairs of CTAs, or the single-CTA kernel (slice address tables; ATS_FLAG_NO_GEMM_PAIR).  A SwiGLU that was
+// One GEMM launch: on the kernel for few tokens, on pairs of CTAs, or on the kernel of plain tiles (slice address tables).  Under
+// ATS_FLAG_NO_GEMM_PAIR nothing runs on pairs, and the grouped form (which the host has sorted then) on plain tiles.  A SwiGLU that was
 // asked for runs in the epilogue or as a launch of its own.
 static int32_t launch_gemm_any(ats_ctx* ctx, GemmParams p) {
   std::string err;
@@ -332,7 +333,11 @@ static int32_t launch_gemm_any(ats_ctx* ctx, GemmParams p) {
   p.counters = reinterpret_cast<int*>(ctx->ws) + 64;  // (the attention's: zero between launches, and launches follow one another)
   const bool pairs = !(ctx->cfg.flags & ATS_FLAG_NO_GEMM_PAIR);
   GemmPairPlan plan{};
-  if (pairs && gemm_pair_eligible(p, ctx->sm_count, &plan)) {
+  GemmFewPlan few{};
+  if ((pairs || !p.grp_off) && gemm_few_eligible(p, ctx->sm_count, &few)) {
+    e = launch_gemm_few(p, few, ctx->sm_count, ctx->cs, &ctx->stats.kernel_launches, &err);
+    act = nullptr;
+  } else if (pairs && gemm_pair_eligible(p, ctx->sm_count, &plan)) {
     e = launch_gemm_pair(p, plan, ctx->sm_count, ctx->cs, &ctx->stats.kernel_launches, &err);
     act = nullptr;
   } else {

@@ -83,7 +83,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
   __shared__ float factor_s[2][kQRows];  // what the row's O shrinks by
   __shared__ uint32_t tmem_s;
   __shared__ int fail_s;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31, warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);  // (the same for the warp, and known to be)
 
   // ---- which tiles
   const int per_tb = gridDim.x / p.n_tb;                // work items of a token block: head pairs or heads
@@ -148,7 +148,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
 #pragma unroll
         for (int kk = 0; kk < D / 16; ++kk) {
           const uint64_t off = (uint64_t)((kk / 4) * (kChunk >> 4) + (kk % 4) * 2);
-          umma_ss(one, tmem + 128u * x, qd + (uint64_t)(x * (kTileBytes >> 4)) + off, kd + off + (uint64_t)(slot * (kSlot >> 4)), idesc_s,
+          umma_ss(one, 128u * x, qd + (uint64_t)(x * (kTileBytes >> 4)) + off, kd + off + (uint64_t)(slot * (kSlot >> 4)), idesc_s,
                   kk > 0);
         }
         umma_commit_to(one, &s_full[x]);
@@ -156,7 +156,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1)
       auto issue_o = [&](int x, int slot, bool accumulate) {
 #pragma unroll
         for (int kk = 0; kk < kKeys / 16; ++kk)
-          umma_ts(one, tmem + kColO + 128u * x, tmem + 128u * x + 8u * kk, vd + (uint64_t)(slot * (kSlot >> 4) + kk * (2048 >> 4)), idesc_o,
+          umma_ts(one, kColO + 128u * x, 128u * x + 8u * kk, vd + (uint64_t)(slot * (kSlot >> 4) + kk * (2048 >> 4)), idesc_o,
                   accumulate || kk > 0);
       };
       bool ok = mbar_wait_all(&q_full, 0) && mbar_wait_all(&kv_full[0], 0);
