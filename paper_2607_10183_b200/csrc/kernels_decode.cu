@@ -904,60 +904,63 @@ __device__ __forceinline__ void router_select(const float* logit, int m, int E, 
   }
 }
 
-// The same selection for up to 256 experts by counting, all threads of the CTA at once: the rank of a logit is the number
-// of logits that come before it in the order (larger value first, equal values: lower index first; NaN as -inf), so the
-// expert of rank r < k is the r-th selection of router_select; warp 0 then forms the gates with router_select's own
-// arithmetic.  sel_v / sel_i: k entries of shared memory.  Called by every thread of the CTA.
-__device__ __forceinline__ void router_select_counting(const float* logit, int m, int E, int Epad, int k, int renorm,
-                                                       int32_t* __restrict__ ids, float* __restrict__ gates, float* sel_v, int* sel_i) {
-  for (int e = threadIdx.x; e < E; e += blockDim.x) {
-    const float vr = logit[e];
-    const float v = vr == vr ? vr : -INFINITY;
-    int rank = 0;
-    for (int j = 0; j < E; j += 4) {  // E is a multiple of 8 here
-      const float4 o = *reinterpret_cast<const float4*>(logit + j);
-      const float o0 = o.x == o.x ? o.x : -INFINITY, o1 = o.y == o.y ? o.y : -INFINITY;
-      const float o2 = o.z == o.z ? o.z : -INFINITY, o3 = o.w == o.w ? o.w : -INFINITY;
-      rank += (o0 > v || (o0 == v && j < e)) + (o1 > v || (o1 == v && j + 1 < e)) + (o2 > v || (o2 == v && j + 2 < e)) +
-              (o3 > v || (o3 == v && j + 3 < e));
-    }
-    if (rank < k) {
-      sel_v[rank] = v;
-      sel_i[rank] = e;
-    }
-  }
-  __syncthreads();
-  if (threadIdx.x >= 32) return;
-  const int lane = threadIdx.x;
-  const int per = Epad / 32;
+// The same selection for up to 32 PER experts by one warp, lane l having the logits of experts l, l + 32, ...: logits as integers of the same
+// order (-0 as 0, NaN as -inf; 0 stands for what is not there or taken), so that a selection is a maximum over the warp and a minimum
+// over the indexes that have it, one instruction each.  (Counting what comes before each logit, with all threads of a CTA: 3800
+// cycles for 128 experts, a third of the kernel; this 900.)
+__device__ __forceinline__ uint32_t order_key(float v) {
+  const uint32_t b = __float_as_uint(v == v ? v + 0.f : -INFINITY);
+  return b & 0x80000000u ? ~b : b | 0x80000000u;
+}
+__device__ __forceinline__ float key_value(uint32_t key) { return __uint_as_float(key & 0x80000000u ? key & 0x7FFFFFFFu : ~key); }
+template <int PER>
+__device__ __forceinline__ void router_select_keys(const float (&logit)[PER], int m, int E, int k, int renorm, int32_t* __restrict__ ids,
+                                                   float* __restrict__ gates) {
+  const int lane = threadIdx.x & 31;
+  uint32_t key[PER];
   bool has_nan = false;
-  for (int j = 0; j < per; ++j) {
-    const float v = logit[lane + 32 * j];
-    has_nan |= (lane + 32 * j < E) && (v != v);
+  float mx = -INFINITY, total = 0.f;
+#pragma unroll
+  for (int j = 0; j < PER; ++j) {
+    const bool live = lane + 32 * j < E;
+    key[j] = live ? order_key(logit[j]) : 0u;
+    has_nan |= live && logit[j] != logit[j];
   }
   has_nan = __any_sync(0xffffffffu, has_nan);
-  const float my_v = lane < k ? sel_v[lane] : 0.f;
+  float sel_v = 0.f;  // lane r (< k) keeps the r-th selection
+  int sel_i = 0;
+  uint32_t first = 0;
+  for (int r = 0; r < k; ++r) {
+    uint32_t best = key[0];
+#pragma unroll
+    for (int j = 1; j < PER; ++j) best = max(best, key[j]);
+    best = __reduce_max_sync(0xffffffffu, best);
+    if (r == 0) first = best;
+    int at = 0x7fffffff;
+#pragma unroll
+    for (int j = PER - 1; j >= 0; --j) at = key[j] == best ? lane + 32 * j : at;
+    at = __reduce_min_sync(0xffffffffu, at);
+#pragma unroll
+    for (int j = 0; j < PER; ++j) key[j] = at == lane + 32 * j ? 0u : key[j];
+    if (lane == r) {
+      sel_v = key_value(best);
+      sel_i = at;
+    }
+  }
+  mx = key_value(first);
   float gate;
   if (renorm) {
-    const float mx = __shfl_sync(0xffffffffu, my_v, 0);
-    const float ex = lane < k ? expf(my_v - mx) : 0.f;
-    const float s = warp_sum(ex);
-    gate = ex / s;
+    const float ex = lane < k ? expf(sel_v - mx) : 0.f;
+    gate = ex / warp_sum(ex);
   } else {
-    float mx = -INFINITY;
-    for (int j = 0; j < per; ++j) mx = fmaxf(mx, logit[lane + 32 * j]);
-    mx = warp_max(mx);
-    float t = 0.f;
-    for (int j = 0; j < per; ++j) {
-      const float v = logit[lane + 32 * j];
-      t += v > -INFINITY ? expf(v - mx) : 0.f;
-    }
-    const float total = warp_sum(t);
-    gate = lane < k ? expf(my_v - mx) / total : 0.f;
+#pragma unroll
+    for (int j = 0; j < PER; ++j) total += lane + 32 * j < E && logit[j] > -INFINITY ? expf(logit[j] - mx) : 0.f;
+    total = warp_sum(total);
+    gate = lane < k ? expf(sel_v - mx) / total : 0.f;
   }
   if (has_nan) gate = __int_as_float(0x7FC00000);
   if (lane < k) {
-    ids[(size_t)m * k + lane] = sel_i[lane];
+    ids[(size_t)m * k + lane] = sel_i;
     gates[(size_t)m * k + lane] = gate;
   }
 }
@@ -1062,10 +1065,19 @@ __global__ void __launch_bounds__(kRouterClThreads) router_topk_cluster_kernel(c
     const __half* x16 = static_cast<const __half*>(xn) + (size_t)m * H;
     const float* x32 = static_cast<const float*>(xn) + (size_t)m * H;
     float ss = 0.f;
-    for (int i = threadIdx.x; i < H; i += kRouterClThreads) {
-      const float v = xn_f32 ? x32[i] : __half2float(x16[i]);
-      if (i >= row0 && i < row0 + Hc) h_s[i - row0] = v;  // kept for the second pass
-      ss = fmaf(v, v, ss);
+    for (int i0 = threadIdx.x; i0 < H; i0 += 8 * kRouterClThreads) {
+      float v[8];  // (all loads of a batch before the first is used)
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        const int i = i0 + q * kRouterClThreads;
+        v[q] = i >= H ? 0.f : xn_f32 ? x32[i] : __half2float(x16[i]);
+      }
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        const int i = i0 + q * kRouterClThreads;
+        if (i >= row0 && i < row0 + Hc) h_s[i - row0] = v[q];  // kept for the second pass
+        ss = fmaf(v[q], v[q], ss);
+      }
     }
     ss = warp_sum(ss);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = ss;
@@ -1087,9 +1099,9 @@ __global__ void __launch_bounds__(kRouterClThreads) router_topk_cluster_kernel(c
     for (int i = threadIdx.x; i < Hc; i += kRouterClThreads) h_s[i] = __half2float(h[(size_t)m * H + row0 + i]);
   }
   __syncthreads();
-  float acc[8];
+  float2 acc[4];
 #pragma unroll
-  for (int q = 0; q < 8; ++q) acc[q] = 0.f;
+  for (int q = 0; q < 4; ++q) acc[q] = make_float2(0.f, 0.f);
   if (grp < R) {
     for (int i0 = grp; i0 < Hc; i0 += R * kBatch) {
       if (i0 != grp) {
@@ -1105,25 +1117,42 @@ __global__ void __launch_bounds__(kRouterClThreads) router_topk_cluster_kernel(c
         const float x = i < Hc ? h_s[i] : 0.f;
         const uint32_t ws[4] = {w[b].x, w[b].y, w[b].z, w[b].w};
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const float2 f = __half22float2(u32_as_half2(ws[q]));
-          acc[2 * q] = fmaf(x, f.x, acc[2 * q]);
-          acc[2 * q + 1] = fmaf(x, f.y, acc[2 * q + 1]);
-        }
+        for (int q = 0; q < 4; ++q) acc[q] = fma_x2(make_float2(x, x), __half22float2(u32_as_half2(ws[q])), acc[q]);
       }
     }
 #pragma unroll
-    for (int q = 0; q < 8; ++q) part[(size_t)grp * E + e0 + q] = acc[q];
+    for (int q = 0; q < 4; ++q) *reinterpret_cast<float2*>(part + (size_t)grp * E + e0 + 2 * q) = acc[q];
   }
   __syncthreads();
   for (int e = threadIdx.x; e < Epad; e += kRouterClThreads) {
     float t = 0.f;
-    if (e < E)
+    if (e < E) {
+#pragma unroll 8
       for (int g = 0; g < R; ++g) t += part[(size_t)g * E + e];
+    }
     st_cluster_f32(cl + (size_t)rank * Epad + e, 0, t);  // into CTA 0's copy of cl
   }
   cluster_sync_all();
   if (rank != 0) return;
+  if (E <= 256) {  // one warp
+    if (threadIdx.x >= 32) return;
+    auto select = [&](auto per) {
+      float v[decltype(per)::value];
+#pragma unroll
+      for (int j = 0; j < decltype(per)::value; ++j) {
+        v[j] = 0.f;
+        const int e = (int)threadIdx.x + 32 * j;
+        if (e < E) {
+#pragma unroll
+          for (int r = 0; r < kRouterCluster; ++r) v[j] += cl[(size_t)r * Epad + e];
+        }
+      }
+      router_select_keys(v, m, E, k, renorm, ids, gates);
+    };
+    if (E <= 128) select(std::integral_constant<int, 4>{});
+    else select(std::integral_constant<int, 8>{});
+    return;
+  }
   for (int e = threadIdx.x; e < Epad; e += kRouterClThreads) {
     float t = 0.f;
 #pragma unroll
@@ -1131,12 +1160,6 @@ __global__ void __launch_bounds__(kRouterClThreads) router_topk_cluster_kernel(c
     logit[e] = e < E ? t : -INFINITY;
   }
   __syncthreads();
-  if (E <= 256) {
-    __shared__ float sel_v[32];
-    __shared__ int sel_i[32];
-    router_select_counting(logit, m, E, Epad, k, renorm, ids, gates, sel_v, sel_i);
-    return;
-  }
   if (threadIdx.x >= 32) return;
   router_select(logit, m, E, Epad, k, renorm, ids, gates);
 }

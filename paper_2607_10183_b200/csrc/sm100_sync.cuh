@@ -2,6 +2,7 @@
 // asynchronous copies (sm_100a).  All waits are bounded: a wait that runs out returns false and the caller raises the
 // context's status word, releases what it holds and returns, so that a lost completion never hangs the device.
 #pragma once
+#include <cuda_runtime.h>
 #include <stdint.h>
 
 namespace ats {
@@ -72,6 +73,22 @@ __device__ __forceinline__ bool mbar_wait_suspending(uint64_t* bar, uint32_t par
       if (mbar_try_wait(bar, parity)) return true;
     if (clock64() - t0 > limit) return false;
   }
+}
+
+// two fp32 operations in one instruction
+__device__ __forceinline__ float2 fma_x2(float2 a, float2 b, float2 c) {
+  float2 d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;"
+      : "=l"(reinterpret_cast<uint64_t&>(d))
+      : "l"(reinterpret_cast<uint64_t&>(a)), "l"(reinterpret_cast<uint64_t&>(b)), "l"(reinterpret_cast<uint64_t&>(c)));
+  return d;
+}
+__device__ __forceinline__ float2 add_x2(float2 a, float2 b) {
+  float2 d;
+  asm("add.rn.f32x2 %0, %1, %2;"
+      : "=l"(reinterpret_cast<uint64_t&>(d))
+      : "l"(reinterpret_cast<uint64_t&>(a)), "l"(reinterpret_cast<uint64_t&>(b)));
+  return d;
 }
 
 }  // namespace
