@@ -6,6 +6,9 @@
 // two logic ops and one half2 op per pair, accumulates sum_k code*x in fp32 per block, and applies the block scale
 // once: y += scale * sum.  No tensor cores, no atomics; reductions run in a fixed order so results are reproducible
 // run to run and independent of where the weight bytes live (resident region or staging slot).
+#include <algorithm>
+#include <type_traits>
+
 #include "ats_internal.h"
 #include "sm100_sync.cuh"
 #include "attn_decode_body.cuh"
@@ -1164,112 +1167,118 @@ __global__ void __launch_bounds__(kRouterClThreads) router_topk_cluster_kernel(c
   router_select(logit, m, E, Epad, k, renorm, ids, gates);
 }
 
-// The same routing for many tokens: a CTA takes four tokens and streams the whole router matrix through shared memory (16-byte
-// asynchronous copies, stages of 32 KB), so that a weight is read from L2 and converted once for four tokens.  Thread (row
-// group, four experts) sums its chain of rows in each of the eight ranges, and the chains and ranges are added up in
-// router_topk_cluster_kernel's order, so a token's logits have the same bits whichever kernel ran.  Bound by instruction issue
-// (16 multiply-adds, 4 conversions and 2 shared-memory loads per row and thread).  512 tokens of 2048 through 128 experts: 71.7 ->
-// 24.8 us, 512 of 2048 through 256: 140 -> 39 us.
-constexpr int kRouterTok = 4;
-constexpr int kRouterTokThreads = 512;   // 4 experts each: E / 4 x (2048 / E) row groups
-constexpr int kRouterStageRows = 8;      // rows of a chain per stage
-constexpr int kRouterStageElems = kRouterStageRows * 2048;  // ... of all R = 2048 / E chains: contiguous rows of W_r
-// One wave of CTAs takes 23 us (128 experts of 2048) to 45 us (512 of 1024) whatever the tokens, the cluster kernel 14.5 and 31 us for 64
-// tokens, 22.9 and 48.5 us for 128.
-constexpr int kRouterManyTokens = 128;
+// The same routing for many tokens.  A cluster of 8 CTAs takes `tok` tokens; CTA r holds its range of W_r (an eighth of the rows) and the tokens' part of
+// it in shared memory, so that a weight is read from L2 once for all of them.  A thread sums four tokens x four experts over the whole range,
+// chain by chain in router_topk_cluster_kernel's order (rows g, g + R, ...; chains in ascending order), the ranges are added up by the CTA a
+// token belongs to, a warp per token: a token's logits have the same bits whichever kernel ran.  Bound by instruction issue (4 conversions, 8
+// paired multiply-adds, two shared-memory loads a row and thread), under 18 tokens by the chain of its latencies.  Back to back, a CTA with four
+// tokens and the whole matrix before -> now, us: 2048 x 128, 128 / 512 / 2048 tokens 22.0 / 22.1 / 84.6 -> 10.8 / 15.8 / 48.3; 2880 x 64 (a
+// cluster per token before), 512 / 2048 tokens 63 / 244 -> 20 / 41.
+constexpr int kRouterTokThreads = 256;
+// From here on (the cluster kernel takes 10.6 us for 64 tokens, 18.3 for 128; this one 10 to 13).
+constexpr int kRouterManyTokens = 96;
 
 __global__ void __launch_bounds__(kRouterTokThreads) router_topk_tokens_kernel(const __half* __restrict__ h, const __half* __restrict__ wr, int M,
-                                                                               int H, int E, int Epad, int k, int renorm, int stages,
+                                                                               int H, int E, int tok, int k, int renorm,
                                                                                int32_t* __restrict__ ids, float* __restrict__ gates) {
   extern __shared__ __align__(16) float smem[];
-  const int Hc = H / kRouterCluster, R = 2048 / E, per_range = Hc / R / kRouterStageRows, n_st = kRouterCluster * per_range;
-  __half* w_s = reinterpret_cast<__half*>(smem);                                   // [stages][8 R rows][E]
-  float4* h_s = reinterpret_cast<float4*>(w_s + (size_t)stages * kRouterStageElems);  // [H]: the row's element of the four tokens
-  float* part = reinterpret_cast<float*>(h_s + H);                                 // [R][kRouterTok][E]
-  float* logit = part + (size_t)2048 * kRouterTok;                                 // [kRouterTok][Epad]
-  const int tid = threadIdx.x, m0 = blockIdx.x * kRouterTok, live = min(kRouterTok, M - m0);
-  const int lanes = E / 4, grp = tid / lanes, e0 = (tid % lanes) * 4;
-  int ld_st = 0, ld_at = 0;  // next stage to load and its place in the ring
-  const __half* src = wr;
-  const uint32_t ring = (uint32_t)__cvta_generic_to_shared(w_s);
-  auto load = [&] {
-    if (ld_st < n_st) {
-      const uint32_t dst = ring + (uint32_t)(ld_at * kRouterStageElems * 2);
-#pragma unroll
-      for (int q = 0; q < kRouterStageElems / 8 / kRouterTokThreads; ++q) {
-        const int c = (tid + q * kRouterTokThreads) * 8;
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + 2u * c), "l"(src + c) : "memory");
-      }
-      src += kRouterStageElems;
-      ++ld_st;
-      if (++ld_at == stages) ld_at = 0;
-    }
-    asm volatile("cp.async.commit_group;" ::: "memory");
-  };
-  load();  // (the router matrix does not depend on the preceding kernel)
-  load();
-  if (stages == 4) load();
+  const int Hc = H / kRouterCluster, R = kRouterClThreads / (E / 8), own = tok / kRouterCluster;
+  const int pitch = Hc + 4;
+  float* x_s = smem;                                            // [tok][pitch]
+  float* cl = x_s + (size_t)pitch * tok;                        // [kRouterCluster][own][E]: the ranges' sums of this CTA's tokens
+  __half* w_s = reinterpret_cast<__half*>(cl + (size_t)tok * E);  // [Hc][E]
+  const int tid = threadIdx.x, m0 = (int)(blockIdx.x / kRouterCluster) * tok;
+  const uint32_t rank = cluster_ctarank();
+  const int row0 = (int)rank * Hc;
+  {  // (the router matrix does not depend on the preceding kernel)
+    const uint32_t dst = (uint32_t)__cvta_generic_to_shared(w_s);
+    const __half* src = wr + (size_t)row0 * E;
+    for (int c = tid * 8; c < Hc * E; c += kRouterTokThreads * 8)
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + 2u * c), "l"(src + c) : "memory");
+  }
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");  // (nobody writes into a CTA that has not begun)
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  for (int j = tid; j < kRouterTok * (H / 8); j += kRouterTokThreads) {
-    const int t = j & 3, i = (j >> 2) * 8;
-    const uint4 v = t < live ? *reinterpret_cast<const uint4*>(h + (size_t)(m0 + t) * H + i) : make_uint4(0, 0, 0, 0);
-    const uint32_t vs[4] = {v.x, v.y, v.z, v.w};
-    float* d = reinterpret_cast<float*>(h_s + i) + t;
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const float2 f = __half22float2(u32_as_half2(vs[q]));
-      d[8 * q] = f.x;
-      d[8 * q + 4] = f.y;
-    }
+  const int row8 = Hc / 8;
+#pragma unroll 4
+  for (int j = tid; j < tok * row8; j += kRouterTokThreads) {
+    const int t = j / row8, i = (j - t * row8) * 8;
+    const uint4 v = m0 + t < M ? *reinterpret_cast<const uint4*>(h + (size_t)(m0 + t) * H + row0 + i) : make_uint4(0, 0, 0, 0);
+    const float2 a = __half22float2(u32_as_half2(v.x)), b = __half22float2(u32_as_half2(v.y)), c = __half22float2(u32_as_half2(v.z)),
+                 d = __half22float2(u32_as_half2(v.w));
+    float4* dst = reinterpret_cast<float4*>(x_s + (size_t)t * pitch + i);
+    dst[0] = make_float4(a.x, a.y, b.x, b.y);
+    dst[1] = make_float4(c.x, c.y, d.x, d.y);
   }
-  for (int j = tid; j < kRouterTok * Epad; j += kRouterTokThreads) logit[j] = 0.f;
-  float acc[kRouterTok][4];
-  int at = 0, in_range = 0;  // place in the ring, stage of the range
-  const __half* w0 = w_s + (size_t)grp * E + e0;
-  const float4* xr = h_s + grp;
-  for (int st = 0; st < n_st; ++st) {
-    if (stages == 4) asm volatile("cp.async.wait_group 2;" ::: "memory");
-    else asm volatile("cp.async.wait_group 1;" ::: "memory");
-    __syncthreads();  // stage st is there, and everybody has read stage st - 1: its place is free
-    load();
-    if (in_range == 0) {
-#pragma unroll
-      for (int t = 0; t < kRouterTok; ++t)
-#pragma unroll
-        for (int q = 0; q < 4; ++q) acc[t][q] = 0.f;
-    }
-    const __half* w = w0 + at * kRouterStageElems;
-#pragma unroll
-    for (int b = 0; b < kRouterStageRows; ++b) {
-      const float4 x = xr[b * R];
-      const uint2 wv = *reinterpret_cast<const uint2*>(w + b * 2048);
-      const float2 wa = __half22float2(u32_as_half2(wv.x)), wb = __half22float2(u32_as_half2(wv.y));
-      const float xs[kRouterTok] = {x.x, x.y, x.z, x.w}, ws[4] = {wa.x, wa.y, wb.x, wb.y};
-#pragma unroll
-      for (int t = 0; t < kRouterTok; ++t)
-#pragma unroll
-        for (int q = 0; q < 4; ++q) acc[t][q] = fmaf(xs[t], ws[q], acc[t][q]);
-    }
-    xr += kRouterStageRows * R;
-    if (++at == stages) at = 0;
-    if (++in_range == per_range) {  // the range's chains are complete
-      in_range = 0;
-#pragma unroll
-      for (int t = 0; t < kRouterTok; ++t)
-        *reinterpret_cast<float4*>(part + ((size_t)grp * kRouterTok + t) * E + e0) = make_float4(acc[t][0], acc[t][1], acc[t][2], acc[t][3]);
-      __syncthreads();
-      for (int j = tid; j < kRouterTok * E; j += kRouterTokThreads) {
-        float v = 0.f;
-#pragma unroll 8
-        for (int g = 0; g < R; ++g) v += part[g * kRouterTok * E + j];
-        logit[j] += v;  // (E >= 32 is a power of two: E = Epad)
-      }
-    }
-  }
+  asm volatile("cp.async.wait_all;" ::: "memory");
   __syncthreads();
-  const int t = tid >> 5;  // one warp per token
-  if (t < live) router_select(logit + t * Epad, m0 + t, E, Epad, k, renorm, ids, gates);
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  const int lanes = E / 4, items = tok / 4 * lanes;
+  for (int it = tid; it < items; it += kRouterTokThreads) {
+    const int t0 = it / lanes * 4, e0 = it % lanes * 4;
+    float2 sum[4][2];
+#pragma unroll
+    for (int t = 0; t < 4; ++t) sum[t][0] = sum[t][1] = make_float2(0.f, 0.f);
+    const float* xr = x_s + (size_t)t0 * pitch;
+    for (int g = 0; g < R; g += 4) {  // four chains side by side: their rows follow one another (R and Hc are multiples of 4)
+      float2 acc[4][4][2];
+#pragma unroll
+      for (int c = 0; c < 4; ++c)
+#pragma unroll
+        for (int t = 0; t < 4; ++t) acc[c][t][0] = acc[c][t][1] = make_float2(0.f, 0.f);
+#pragma unroll 2
+      for (int i = g; i < Hc; i += R) {
+        float4 x[4];
+#pragma unroll
+        for (int t = 0; t < 4; ++t) x[t] = *reinterpret_cast<const float4*>(xr + (size_t)t * pitch + i);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          const uint2 w = *reinterpret_cast<const uint2*>(w_s + (size_t)(i + c) * E + e0);
+          const float2 wa = __half22float2(u32_as_half2(w.x)), wb = __half22float2(u32_as_half2(w.y));
+#pragma unroll
+          for (int t = 0; t < 4; ++t) {
+            const float xv = c == 0 ? x[t].x : c == 1 ? x[t].y : c == 2 ? x[t].z : x[t].w;
+            acc[c][t][0] = fma_x2(make_float2(xv, xv), wa, acc[c][t][0]);
+            acc[c][t][1] = fma_x2(make_float2(xv, xv), wb, acc[c][t][1]);
+          }
+        }
+      }
+#pragma unroll
+      for (int c = 0; c < 4; ++c)
+#pragma unroll
+        for (int t = 0; t < 4; ++t)
+#pragma unroll
+          for (int q = 0; q < 2; ++q) sum[t][q] = add_x2(sum[t][q], acc[c][t][q]);
+    }
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+      const int to = (t0 + t) / own, at = (t0 + t) % own;
+      uint32_t la = (uint32_t)__cvta_generic_to_shared(cl + ((size_t)rank * own + at) * E + e0), ra;
+      asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(la), "r"(to));
+      asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(ra), "f"(sum[t][0].x), "f"(sum[t][0].y), "f"(sum[t][1].x), "f"(sum[t][1].y)
+                   : "memory");
+    }
+  }
+  cluster_sync_all();
+  const int lane = tid & 31;
+  for (int at = tid >> 5; at < own; at += kRouterTokThreads / 32) {
+    const int m = m0 + (int)rank * own + at;
+    if (m >= M) return;
+    auto select = [&](auto per) {
+      float v[decltype(per)::value];
+#pragma unroll
+      for (int j = 0; j < decltype(per)::value; ++j) {
+        v[j] = 0.f;
+        if (lane + 32 * j < E) {
+#pragma unroll
+          for (int r = 0; r < kRouterCluster; ++r) v[j] += cl[((size_t)r * own + at) * E + lane + 32 * j];
+        }
+      }
+      router_select_keys(v, m, E, k, renorm, ids, gates);
+    };
+    if (E <= 128) select(std::integral_constant<int, 4>{});
+    else select(std::integral_constant<int, 8>{});
+  }
 }
 
 cudaError_t launch_router_topk(const __half* h, const __half* wr, int M, int H, int E, int k, int renorm, int32_t* ids,
@@ -1287,19 +1296,28 @@ cudaError_t launch_router_topk_norm(const __half* h, const __half* wr, int M, in
   if (E % 8 == 0 && H % (8 * kRouterCluster) == 0 && H <= 8 * kRouterClThreads * kRouterCluster && (((uintptr_t)wr | (uintptr_t)h) & 15) == 0) {
     const int L = E / 8, R = kRouterClThreads / L;
     const size_t smem_cl = ((size_t)H / kRouterCluster + (size_t)R * E + (size_t)(kRouterCluster + 1) * Epad) * sizeof(float);
-    auto smem_tok = [&](int stages) {
-      return (size_t)stages * kRouterStageElems * 2 + ((size_t)4 * H + 2048 * kRouterTok + (size_t)kRouterTok * Epad) * sizeof(float);
-    };
-    constexpr size_t kMost = 227 * 1024 - 2048;
-    // (chains of a multiple of eight rows: 2048 / E of them in each range)
-    if (M >= kRouterManyTokens && !norm_gain && E == Epad && 2048 % E == 0 && H / kRouterCluster % (kRouterStageRows * R) == 0 && smem_tok(3) <= kMost) {
-      const int stages = smem_tok(4) <= kMost ? 4 : 3;
-      static std::atomic<uint64_t> attr_done;
-      const cudaError_t e = smem_limit_once(&attr_done, {reinterpret_cast<const void*>(router_topk_tokens_kernel)}, kMost);
-      if (e != cudaSuccess) return e;
-      ++*n_launch;
-      return launch_dep(router_topk_tokens_kernel, dim3((M + kRouterTok - 1) / kRouterTok), dim3(kRouterTokThreads), smem_tok(stages), st, pdl, 1,
-                        h, wr, M, H, E, Epad, k, renorm, stages, ids, gates);
+    auto smem_tok = [&](int tok) { return (((size_t)H / kRouterCluster + 4) * tok + (size_t)tok * E) * sizeof(float) + (size_t)H / kRouterCluster * E * 2; };
+    constexpr size_t kMostTok = 227 * 1024 - 1024;
+    if (M >= kRouterManyTokens && !norm_gain && E <= 256 && R % 4 == 0) {
+      // Tokens to a cluster: a cluster takes 10 us or, from 18 tokens on (128 experts of 2048), 0.315 more a token; 15 run at a time, and another 17
+      // beside them, in half as much again, where two CTAs fit an SM.
+      int tok = 0;
+      double best = 1e30;
+      for (int t = 8; t <= 64; t += 8) {
+        if (smem_tok(t) > kMostTok) break;
+        const int c = (M + t - 1) / t;
+        const double us = std::max(10.0, 4.3 + 0.315 * t * ((double)H * E / (2048 * 128)));
+        const double all = us * (c <= 15 ? 1.0 : smem_tok(t) <= kMostTok / 2 ? 1.5 * ((c + 31) / 32) : (double)((c + 14) / 15));
+        if (all < best) best = all, tok = t;
+      }
+      if (tok) {
+        static std::atomic<uint64_t> attr_done;
+        const cudaError_t e = smem_limit_once(&attr_done, {reinterpret_cast<const void*>(router_topk_tokens_kernel)}, kMostTok);
+        if (e != cudaSuccess) return e;
+        ++*n_launch;
+        return launch_dep(router_topk_tokens_kernel, dim3((M + tok - 1) / tok * kRouterCluster), dim3(kRouterTokThreads), smem_tok(tok), st, pdl,
+                          kRouterCluster, h, wr, M, H, E, tok, k, renorm, ids, gates);
+      }
     }
     constexpr size_t kMostCl = 160 * 1024;
     if (smem_cl <= kMostCl) {

@@ -1,0 +1,37 @@
+"""The router for many tokens: the bits of the router for few, whatever the tokens of a cluster, the ranges and the chains."""
+import numpy as np
+import pytest
+
+from tests import helpers as H
+
+pytestmark = pytest.mark.gpu
+
+
+# One and several rounds of clusters, a last cluster with few tokens, chains of unequal length (2880 rows, 64 experts), one row to a chain (512 x 16),
+# more than 128 experts (a shorter block of tokens where shared memory is full); equal logits and a NaN among the tokens.
+@pytest.mark.parametrize("hidden,E,k,M", [(2048, 128, 8, 96), (2048, 128, 8, 513), (2880, 64, 4, 130), (512, 16, 2, 700), (1024, 32, 4, 2000), (1024, 256, 8, 250),
+                                          (3072, 256, 6, 97), (4096, 64, 4, 1100)])
+def test_router_of_many_tokens_has_the_bits_of_the_router_of_few(hidden, E, k, M):
+    import torch
+    from paper_2607_10183_b200 import binding as B
+    rng = np.random.default_rng(hidden + E + M)
+    wr = (rng.standard_normal((hidden, E)) * 0.02).astype(np.float16)
+    wr[:, 5] = wr[:, 3]  # equal logits: the lower index first
+    ctx = B.Context(4 * hidden * E + (8 << 20), workspace_bytes=1 << 20)
+    rid = ctx.register_f16(wr)
+    ctx.set_placement([])
+    h = H.to_dev(rng.standard_normal((M, hidden)).astype(np.float16))
+    h[M - 2, 7] = float("nan")
+
+    def route(lo, hi):
+        ids = torch.full((hi - lo, k), -1, dtype=torch.int32, device="cuda")
+        gates = torch.zeros((hi - lo, k), dtype=torch.float32, device="cuda")
+        ctx.route_topk(rid, h[lo:hi].contiguous(), hi - lo, k, ids, gates)
+        ctx.sync()
+        return ids, gates.view(torch.int32)
+
+    ids, gates = route(0, M)
+    parts = [route(lo, min(M, lo + 64)) for lo in range(0, M, 64)]
+    assert torch.equal(ids, torch.cat([p[0] for p in parts]))
+    assert torch.equal(gates, torch.cat([p[1] for p in parts]))
+    ctx.close()
