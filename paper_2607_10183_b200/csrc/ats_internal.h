@@ -329,8 +329,8 @@ bool attn_prefill_tc_eligible(const __half* q_rot16, const __half* kc, const __h
 cudaError_t launch_attn_prefill_tc(const __half* q_rot16, const __half* kc, const __half* vc, __half* a16, int T, int n_q, int n_kv, int d,
                                    int cap, int pos0, int* status, cudaStream_t st, uint64_t* n_launch, int pdl = 0);
 // MoE prefill helpers (kernels_prefill.cu): rows gathered in expert order, and the gated sum back in token order
-cudaError_t launch_moe_group(const int32_t* ids, int P, int E, int* order, int* pos, int* off, int* status, int* done, int seq, cudaStream_t st,
-                             uint64_t* n_launch, int pdl);
+cudaError_t launch_moe_sort_gather(const int32_t* ids, int P, int E, int k, int H, const __half* h, int* order, int* pos, int* off, __half* xs,
+                                   int* status, int* done, int seq, cudaStream_t st, uint64_t* n_launch, int pdl);
 cudaError_t launch_moe_gather_rows(const __half* h, const int* order, int k, __half* xs, int P, int H, cudaStream_t st,
                                    uint64_t* n_launch, int pdl = 0);
 cudaError_t launch_moe_combine_sorted(const __half* res, const float* gates, const __half* d, const int* pos, __half* y, int T, int k,

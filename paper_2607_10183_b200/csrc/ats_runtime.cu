@@ -1771,14 +1771,14 @@ int32_t ats_layer_prefill(ats_ctx* ctx, const ats_layer_desc* L, const void* x_i
     int max_rows = 0, seq = 0;
     if (on_device) {
       seq = ++ctx->done_seq;
-      ATS_CUDA(launch_moe_group(w.ids, P, E, w.order, w.pos, w.grp_off, ctx->dev_status, ctx->done_dev, seq, ctx->cs, nl, pdl));
+      ATS_CUDA(launch_moe_sort_gather(w.ids, P, E, k, H, w.h2_16, w.order, w.pos, w.grp_off, w.xs16, ctx->dev_status, ctx->done_dev, seq, ctx->cs, nl, pdl));
     } else {
       ATS_TRY(fetch_ids(ctx, w.ids, P, E));
       if (ats_host_group_pairs(ctx->ids_host, (uint32_t)P, (uint32_t)E, order_h, pos_h, off_h, &max_rows) != ATS_OK)
         return fail(ctx, ATS_ERR_INVALID, "routing ids out of range");
       ATS_CUDA(cudaMemcpyAsync(w.order, order_h, (size_t)(off_h + E + 1 - order_h) * 4, cudaMemcpyHostToDevice, ctx->cs));
+      ATS_CUDA(launch_moe_gather_rows(w.h2_16, w.order, k, w.xs16, P, H, ctx->cs, nl, pdl));
     }
-    ATS_CUDA(launch_moe_gather_rows(w.h2_16, w.order, k, w.xs16, P, H, ctx->cs, nl, pdl));
     auto slice0 = [](const Tensor& t) -> const uint8_t* { return t.contiguous_dev ? t.slices[0].dev : nullptr; };
     // Host-placed experts that some token selected: one SM-driven gather brings their slices into what the workspace has
     // left beyond this layer's buffers, and per-call address tables point the GEMMs there.  Without that room (or

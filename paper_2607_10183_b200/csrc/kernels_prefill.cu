@@ -317,106 +317,112 @@ cudaError_t launch_swiglu16(const __half* gu, int ld, int ffn, __half* act, int 
   return launch_dep(swiglu16_kernel, dim3(grid), dim3(256), 0, st, pdl, 1, gu, ld, ffn, act, n8);
 }
 
-// MoE prefill: the stable sort of the (token, slot) pairs by expert, on the device: order[r] = the pair at sorted position r, pos[p] =
-// the position of pair p, off[e] = the first position of expert e, off[E] = P: what ats_host_group_pairs makes of the same ids.
-// One CTA: a warp counts a contiguous part of the pairs by expert (pairs of one expert among 32 find each other with a vote and keep
-// their order), the warps' counts are added up per expert and over the experts, and a second pass places the pairs.  It is a chain of
-// latencies (ids, counts, sums, places).  The completion word tells the host that the router has run.  512 tokens through 8 of 128
-// experts each: the layer 226 us with the sort on the host (ids out, sort, arrays back: 38 us of it), 209 with this launch.
-constexpr int kGroupThreads = 1024;
-__global__ void __launch_bounds__(kGroupThreads) moe_group_kernel(const int32_t* __restrict__ ids, int P, int E, int* __restrict__ order,
-                                                                  int* __restrict__ pos, int* __restrict__ off, int* status, int* done, int seq) {
-  extern __shared__ int cnt_s[];  // [32][E]: pairs of expert e in warp w's part; later the position of the first of them
-  __shared__ int sum_s[32];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  int* cnt = cnt_s + w * E;
-  for (int i = threadIdx.x; i < 32 * E; i += kGroupThreads) cnt_s[i] = 0;
-  __syncthreads();
+// MoE prefill: the stable sort of the (token, slot) pairs by expert, on the device, and the rows in that order: order[r] = the pair at sorted
+// position r, pos[p] = the position of pair p, off[e] = the first position of expert e, off[E] = P: what ats_host_group_pairs makes of
+// the same ids; xs[r] = the row of order[r]'s token.
+// 1 << shift CTAs to an expert: each counts for itself the pairs of lower experts and, in the order of its threads' contiguous parts, of its own
+// (16 KB of ids for 4096 pairs), then places every 1 << shift-th of them and copies their rows.  The completion word tells the host that the
+// router has run.  Bound by latencies (ids twice, two sums over the CTA, rows) and the copies (4096 rows of 4 KB written: 2.6 us).  512
+// tokens through 8 of 128 experts: one CTA that sorts, then a launch that copies 9.8 + 4.9 us, this 11.2.
+constexpr int kSortThreads = 256, kSortList = 512;
+__global__ void __launch_bounds__(kSortThreads) moe_sort_gather_kernel(const int32_t* __restrict__ ids, int P, int E, int shift, int k, int H,
+                                                                       const __half* __restrict__ h, int* __restrict__ order, int* __restrict__ pos,
+                                                                       int* __restrict__ off, __half* __restrict__ xs, int* status, int* done, int seq) {
+  __shared__ int lower_s[kSortThreads / 32], own_s[kSortThreads / 32], list_s[kSortList];
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  const int e = blockIdx.x >> shift, s = blockIdx.x & ((1 << shift) - 1);
+  const int per = (P + kSortThreads * 4 - 1) / (kSortThreads * 4) * 4, lo = min(tid * per, P), hi = min(lo + per, P);
   asm volatile("griddepcontrol.wait;" ::: "memory");  // the ids come from the router
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  const int per = (P + kGroupThreads - 1) / kGroupThreads * 32, lo = min(w * per, P), hi = min(lo + per, P);
-  // (a warp's first kKept votes of 32 pairs stay in registers from one pass to the next)
-  constexpr int kKept = 4;
-  int id[kKept], place[kKept];
-  auto vote = [&](int e) {  // the pair's place among the warp's pairs of its expert
-    const unsigned same = __match_any_sync(0xFFFFFFFFu, e);
-    const int rank = __popc(same & ((1u << lane) - 1u)), before = e < 0 ? 0 : cnt[e];
-    __syncwarp();
-    if (e >= 0 && rank == 0) cnt[e] = before + __popc(same);
-    __syncwarp();
-    return before + rank;
-  };
-  auto checked = [&](int e) {  // an id that names no expert (the router writes none): expert 0 stands in and the status word says so
-    if ((unsigned)e < (unsigned)E) return e;
-    raise_status(status, 7);
-    return 0;
-  };
+  // (an id that names no expert, which the router does not write, counts as expert 0 and the status word says so)
+  int4 kept[4];  // the first 16 of this thread's ids, requested together
 #pragma unroll
-  for (int i = 0; i < kKept; ++i) id[i] = lo + 32 * i + lane < hi ? ids[lo + 32 * i + lane] : -1;
+  for (int q = 0; q < 4; ++q) {
+    const int p = lo + 4 * q;
+    kept[q] = p + 4 <= hi ? *reinterpret_cast<const int4*>(ids + p)
+                          : make_int4(p < hi ? ids[p] : -1, p + 1 < hi ? ids[p + 1] : -1, p + 2 < hi ? ids[p + 2] : -1, -1);
+  }
+  auto each = [&](auto f) {  // f(pair, id), pairs in ascending order
 #pragma unroll
-  for (int i = 0; i < kKept; ++i) {
-    if (lo + 32 * i + lane < hi) id[i] = checked(id[i]);
-    if (lo + 32 * i < hi) place[i] = vote(id[i]);
-  }
-  for (int p0 = lo + 32 * kKept; p0 < hi; p0 += 32) {
-    const int p = p0 + lane, at = vote(p < hi ? checked(ids[p]) : -1);
-    if (p < hi) pos[p] = at;  // (this thread adds the rest below)
-  }
-  __syncthreads();
-  const int e = threadIdx.x;
-  int total = 0;
-  if (e < E) {
-#pragma unroll 8
-    for (int i = 0; i < 32; ++i) {
-      const int c = cnt_s[i * E + e];
-      cnt_s[i * E + e] = total;
-      total += c;
+    for (int q = 0; q < 4; ++q) {
+      const int p = lo + 4 * q;
+      if (p < hi) f(p, kept[q].x);
+      if (p + 1 < hi) f(p + 1, kept[q].y);
+      if (p + 2 < hi) f(p + 2, kept[q].z);
+      if (p + 3 < hi) f(p + 3, kept[q].w);
     }
-  }
-  int incl = total;
+    for (int p = lo + 16; p < hi; p += 4) {
+      if (p + 4 <= hi) {
+        const int4 v = *reinterpret_cast<const int4*>(ids + p);
+        f(p, v.x), f(p + 1, v.y), f(p + 2, v.z), f(p + 3, v.w);
+      } else {
+        for (int q = p; q < hi; ++q) f(q, ids[q]);
+      }
+    }
+  };
+  int lower = 0, own = 0;
+  bool bad = false;
+  each([&](int, int id) {
+    bad |= (unsigned)id >= (unsigned)E;
+    id = (unsigned)id < (unsigned)E ? id : 0;
+    lower += id < e;
+    own += id == e;
+  });
+  if (bad && blockIdx.x == 0) raise_status(status, 7);
+  int incl = own;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
     const int v = __shfl_up_sync(0xFFFFFFFFu, incl, o);
     if (lane >= o) incl += v;
   }
-  if (lane == 31) sum_s[w] = incl;
+  lower = __reduce_add_sync(0xFFFFFFFFu, lower);
+  if (lane == 31) own_s[w] = incl;
+  if (lane == 0) lower_s[w] = lower;
   __syncthreads();
-  int first = incl - total;
+  int first = 0, at = incl - own, n = 0;
 #pragma unroll
-  for (int i = 0; i < 32; ++i) first += i < w ? sum_s[i] : 0;
-  if (e < E) {
+  for (int i = 0; i < kSortThreads / 32; ++i) {
+    first += lower_s[i];
+    at += i < w ? own_s[i] : 0;
+    n += own_s[i];
+  }
+  if (tid == 0 && s == 0) {
     off[e] = first;
     if (e == E - 1) off[E] = P;
-#pragma unroll 8
-    for (int i = 0; i < 32; ++i) cnt_s[i * E + e] += first;
+  }
+  if (own) {
+    each([&](int p, int id) {
+      if (((unsigned)id < (unsigned)E ? id : 0) != e) return;
+      const int m = at >> shift;
+      if ((at & ((1 << shift) - 1)) == s) {
+        order[first + at] = p;
+        pos[p] = first + at;
+        if (m < kSortList) list_s[m] = p / k;
+      }
+      ++at;
+    });
   }
   __syncthreads();
-#pragma unroll
-  for (int i = 0; i < kKept; ++i) {
-    const int p = lo + 32 * i + lane;
-    if (p < hi) {
-      const int r = place[i] + cnt[id[i]];
-      pos[p] = r;
-      order[r] = p;
+  const int rows = (n - s + (1 << shift) - 1) >> shift;  // (s < 1 << shift: at least 0)
+  for (int c = tid; c < H / 8; c += kSortThreads) {
+#pragma unroll 8
+    for (int m = 0; m < rows; ++m) {
+      const int r = first + s + (m << shift), t = m < kSortList ? list_s[m] : order[r] / k;
+      reinterpret_cast<uint4*>(xs + (size_t)r * H)[c] = __ldg(reinterpret_cast<const uint4*>(h + (size_t)t * H) + c);
     }
   }
-  for (int p = lo + 32 * kKept + lane; p < hi; p += 32) {
-    const int q = ids[p], r = pos[p] + cnt[(unsigned)q < (unsigned)E ? q : 0];
-    pos[p] = r;
-    order[r] = p;
-  }
-  // (at the end, and without a fence: one that waits for the host's memory held the whole sort up)
-  if (done && threadIdx.x == 0) *reinterpret_cast<volatile int*>(done) = seq;
+  // (without a fence: one that waits for the host's memory held the sort up)
+  if (done && blockIdx.x == 0 && tid == 0) *reinterpret_cast<volatile int*>(done) = seq;
 }
 
-cudaError_t launch_moe_group(const int32_t* ids, int P, int E, int* order, int* pos, int* off, int* status, int* done, int seq, cudaStream_t st,
-                             uint64_t* n_launch, int pdl) {
-  if (E < 1 || E > kGroupThreads || P < 1) return cudaErrorInvalidValue;
-  static std::atomic<uint64_t> attr_done;
-  const cudaError_t e = smem_limit_once(&attr_done, {reinterpret_cast<const void*>(moe_group_kernel)}, 32 * kGroupThreads * sizeof(int));
-  if (e != cudaSuccess) return e;
+cudaError_t launch_moe_sort_gather(const int32_t* ids, int P, int E, int k, int H, const __half* h, int* order, int* pos, int* off, __half* xs,
+                                   int* status, int* done, int seq, cudaStream_t st, uint64_t* n_launch, int pdl) {
+  if (E < 1 || P < 1) return cudaErrorInvalidValue;
+  int shift = 0;
+  while ((2 << shift) * E <= 4 * 148) ++shift;  // (one CTA to an SM 19.8 us, two 14.0, four 11.2, eight 12.9: copies in flight against ids read)
   ++*n_launch;
-  return launch_dep(moe_group_kernel, dim3(1), dim3(kGroupThreads), (size_t)32 * E * sizeof(int), st, pdl, 1, ids, P, E, order, pos, off, status, done, seq);
+  return launch_dep(moe_sort_gather_kernel, dim3(E << shift), dim3(kSortThreads), 0, st, pdl, 1, ids, P, E, shift, k, H, h, order, pos, off, xs, status,
+                    done, seq);
 }
 
 // MoE prefill: rows sorted by expert.  xs[r] = h[order[r] / k] (order[r] = the (token, slot) pair at sorted position r);
@@ -444,12 +450,11 @@ cudaError_t launch_moe_gather_rows(const __half* h, const int* order, int k, __h
 // y[t] = rn16(res[t] + sum_j gates[t][j] * d[pos[t k + j]]) with the sum in slot order, fp32; pos[p] = sorted position
 // of pair p.  8 columns per thread.
 __global__ void moe_combine_sorted_kernel(const __half* __restrict__ res, const float* __restrict__ gates, const __half* __restrict__ d,
-                                          const int* __restrict__ pos, __half* __restrict__ y, uint64_t n8, int k, int H) {
+                                          const int* __restrict__ pos, __half* __restrict__ y, int k, int H) {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  const int per_row = H / 8;
-  for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n8; i += (uint64_t)gridDim.x * blockDim.x) {
-    const uint64_t t = i / per_row, c = (i % per_row) * 8;
+  const uint64_t t = blockIdx.x;
+  for (int c = threadIdx.x * 8; c < H; c += blockDim.x * 8) {
     float acc[8];
     {
       const uint4 rv = *reinterpret_cast<const uint4*>(res + t * H + c);
@@ -461,6 +466,7 @@ __global__ void moe_combine_sorted_kernel(const __half* __restrict__ res, const 
         acc[2 * q + 1] = f.y;
       }
     }
+#pragma unroll 8
     for (int j = 0; j < k; ++j) {
       const float gj = gates[t * k + j];
       const uint4 dv = *reinterpret_cast<const uint4*>(d + (uint64_t)pos[t * k + j] * H + c);
@@ -484,10 +490,8 @@ __global__ void moe_combine_sorted_kernel(const __half* __restrict__ res, const 
 
 cudaError_t launch_moe_combine_sorted(const __half* res, const float* gates, const __half* d, const int* pos, __half* y, int T, int k,
                                       int H, cudaStream_t st, uint64_t* n_launch, int pdl) {
-  const uint64_t n8 = (uint64_t)T * H / 8;
-  const int grid = (int)std::min<uint64_t>((n8 + 255) / 256, 148 * 8);
   ++*n_launch;
-  return launch_dep(moe_combine_sorted_kernel, dim3(grid), dim3(256), 0, st, pdl, 1, res, gates, d, pos, y, n8, k, H);
+  return launch_dep(moe_combine_sorted_kernel, dim3(T), dim3(std::min(256, (H / 8 + 31) / 32 * 32)), 0, st, pdl, 1, res, gates, d, pos, y, k, H);
 }
 
 // ---------------------------------------------------------------------------------------------------------------
