@@ -1,5 +1,5 @@
-// GEMM of few tokens to a tile (at most 128) on single CTAs (sm_100a, tcgen05): Y[T][N] = X[T][K] W^T for the two 4-bit block formats, K a
-// multiple of 256; fp16 operands (w = rn16(scale * code), one rounding), fp32 accumulation.
+// GEMM of few tokens to a tile (at most 128) on single CTAs (sm_100a, tcgen05): Y[T][N] = X[T][K] W^T for the two 4-bit block formats;
+// fp16 operands (w = rn16(scale * code), one rounding), fp32 accumulation.
 //
 // As on the pairs of CTAs (kernels_gemm_pair.cu) the weights are the A operand, expanded straight into tensor memory (a thread has one
 // feature, its lane), and the tokens the instruction's N.  There the one MMA warp of a pair was the bottleneck up to 128 tokens and beyond:
@@ -23,6 +23,7 @@
 // gemm_q4_kernel) -> now, us:
 //   1024 x 1024, 16 tokens Q4       5.8 -> 3.3      4096 x 4096, 16 / 77 / 512 tokens MXFP4   10.8 / 13.9 / 21.5 -> 7.2 / 10.6 / 17.5
 //   14336 x 4096, 16 / 128 Q4       17.0 / 20.7 -> 11.3 / 15.3      4096 x 14336, 16 / 77 / 512 Q4   17.8 / 21.2 / 55.7 -> 14.2 / 18.0 / 50
+//   2880 x 2880, 16 / 300 Q4        10.2 / 17.9 -> 6.9 / 11.7       13600 x 4000, 16 / 77 MXFP4               21.7 / 24.8 -> 13.0 / 14.4
 //   28672 x 4096, 16 / 77 MXFP4     24.8 / 26.9 -> 17.4 / 20.3      2048 x 5632, 16 / 300 MXFP4   10.3 / 23.9 -> 7.0 / 15
 //
 // Roles per CTA: warp 0 = activation loads, warps 1 and 2 = MMA issue (and tensor-memory allocation), warp 3 = code and scale loads, warps 4..11 =
@@ -43,6 +44,10 @@ constexpr int kRows = 128;                  // features that one MMA takes: tens
 constexpr int kUnitK = 256;                 // k per unit of work: 128 bytes of codes and one 16-byte line of scales per row
 constexpr int kCodeBytes = kRows * 128;     // of 128 rows: 16 KB
 constexpr int kScaleBytes = kRows * 16;     // 2 KB
+// K no multiple of 256: a warp fetches the scales of its 32 rows for 128 k itself, three words of each from the 4-byte boundary at or below the
+// first, three steps ahead.  (From one warp, five words of each row for a unit: 0.93 us a unit where this takes 0.44; as a flag instead of a kernel of
+// its own it cost the other products 0.4 us of instruction fetch.)
+constexpr int kFeed = 4, kFeedBytes = 32 * 12;
 constexpr int kMaxCodes = 8, kMaxX = 12;    // ring depths at most
 constexpr int kStagePitch = 272;            // bytes per token of the output staging: 128 halves + 16
 constexpr int kStageTok = 16;               // tokens staged at a time
@@ -63,6 +68,7 @@ enum {
 
 struct FewParams : TileWork {  // (workers: CTAs; units: 256 k)
   int codes, xs;      // depths of the rings
+  unsigned long long grp_stride;
   __half* y;          // (SwiGLU: may be null)
   int ldy;
   const __half* res;  // optional: y2 = rn16(res + y)
@@ -126,7 +132,7 @@ __device__ __forceinline__ int part_units(const FewParams& p, int n) {
   return n <= p.max_units ? n : (n + (n - 1) / p.max_units) / ((n + p.max_units - 1) / p.max_units);
 }
 
-template <bool MX, int MODE, int SUMS>
+template <bool MX, int MODE, int SUMS, bool LINES>
 __global__ void __launch_bounds__(kFewThreads, 1) gemm_few_kernel(const __grid_constant__ FewMaps maps, const __grid_constant__ FewParams p) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -145,7 +151,7 @@ __global__ void __launch_bounds__(kFewThreads, 1) gemm_few_kernel(const __grid_c
   uint8_t* x_s = smem;
   uint8_t* code_s = x_s + (size_t)NX * xbytes;
   uint8_t* scale_s = code_s + (size_t)NC * kPlaceBytes;
-  uint8_t* out_s = scale_s + (size_t)NC * kSubs * kScaleBytes;
+  uint8_t* out_s = scale_s + (LINES ? NC * kSubs * kScaleBytes : 16 * kFeed * kFeedBytes);  // (LINES: K is a multiple of 256)
   uint8_t* recv_s = out_s + kStageBytes;              // sums from the other CTAs of the cluster
   // Several accumulators per half where tensor memory has room: two that take tiles in turn, or the steps of a CTA's one tile (shorter
   // chains).  Accumulator i of half s lies at s * pitch + i * 2 * pitch.
@@ -170,7 +176,7 @@ __global__ void __launch_bounds__(kFewThreads, 1) gemm_few_kernel(const __grid_c
   if (warp == 3 && lane == 0) {  // (the loader's own barriers: it starts before the others are ready)
     for (int i = 0; i < p.n_seg; ++i) {
       prefetch_map(&maps.codes[i]);
-      prefetch_map(&maps.scales[i]);
+      if (LINES) prefetch_map(&maps.scales[i]);
     }
     for (int s = 0; s < NC; ++s) {
       mbar_init(&cfull[s], 1);
@@ -226,12 +232,12 @@ __global__ void __launch_bounds__(kFewThreads, 1) gemm_few_kernel(const __grid_c
       uint64_t* bar = &cfull[ld_cs];
       const uint32_t dst = smem_u32(code_s) + (uint32_t)ld_cs * kPlaceBytes, sdst = smem_u32(scale_s) + (uint32_t)(ld_cs * kSubs * kScaleBytes);
       const int second = MODE == kSwiglu ? ld_first : ld_first + kRows;
-      expect_tx_one(one, bar, kPlaceBytes + (uint32_t)(kSubs * kScaleBytes));
-      // rows beyond the matrix read as zeros
+      expect_tx_one(one, bar, kPlaceBytes + (LINES ? (uint32_t)(kSubs * kScaleBytes) : 0u));
+      // rows beyond the matrix and k beyond its end read as zeros
       tma_3d_one(one, dst, &maps.codes[ld_sa], ld_u * 128, ld_first, ld_e, bar);
       if (kSubs == 2) tma_3d_one(one, dst + kCodeBytes, &maps.codes[ld_sb], ld_u * 128, second, ld_e, bar);
-      tma_3d_one(one, sdst, &maps.scales[ld_sa], ld_u * 8, ld_first, ld_e, bar);
-      if (kSubs == 2) tma_3d_one(one, sdst + kScaleBytes, &maps.scales[ld_sb], ld_u * 8, second, ld_e, bar);
+      if (LINES) tma_3d_one(one, sdst, &maps.scales[ld_sa], ld_u * 8, ld_first, ld_e, bar);
+      if (LINES && kSubs == 2) tma_3d_one(one, sdst + kScaleBytes, &maps.scales[ld_sb], ld_u * 8, second, ld_e, bar);
       ++ld_u;
       if (++ld_cs == NC) {
         ld_cs = 0;
@@ -266,7 +272,12 @@ __global__ void __launch_bounds__(kFewThreads, 1) gemm_few_kernel(const __grid_c
             break;
           }
           expect_tx_one(one, &xfull[s], (uint32_t)box * 4096u);
-          tma_3d_one(one, x0 + (uint32_t)s * xbytes, &maps.x[box - 1], 0, row, 2 * i, &xfull[s]);
+          if (LINES) {  // (both chunks in one box)
+            tma_3d_one(one, x0 + (uint32_t)s * xbytes, &maps.x[box - 1], 0, row, 2 * i, &xfull[s]);
+          } else {
+            tma_3d_one(one, x0 + (uint32_t)s * xbytes, &maps.x[box - 1], 128 * i, row, 0, &xfull[s]);
+            tma_3d_one(one, x0 + (uint32_t)s * xbytes + (uint32_t)box * 2048u, &maps.x[box - 1], 128 * i + 64, row, 0, &xfull[s]);
+          }
           if (++s == NX) s = 0, par ^= 1u;
         }
       }
@@ -340,21 +351,83 @@ __global__ void __launch_bounds__(kFewThreads, 1) gemm_few_kernel(const __grid_c
     const int kh = MODE == kDeep ? sub : h;  // which 128 k of a unit
     const uint32_t a_col = tmem + ((uint32_t)(quarter * 32) << 16) + kColA + 64u * slot;
     const uint32_t code_row = smem_u32(code_s) + (uint32_t)((MODE == kDeep ? 0 : sub * kCodeBytes) + row * 128);
-    const uint32_t scale_row = smem_u32(scale_s) + (uint32_t)((MODE == kDeep ? 0 : sub * kScaleBytes) + row * 16 + kh * 8);
+    const uint32_t scale_row = LINES ? smem_u32(scale_s) + (uint32_t)((MODE == kDeep ? 0 : sub * kScaleBytes) + row * 16 + kh * 8)
+                                     : smem_u32(scale_s) + (uint32_t)((warp - 12) * kFeed * kFeedBytes);
+    const int nblk = p.K / 32;
     const uint32_t swz = (uint32_t)(row & 7) << 4;
     constexpr int kStep = MODE == kDeep ? 2 : 1;  // (deep: the groups of a half take turns)
     int m = 0;  // units of this group so far
     auto expand = [&] {
       FewWalk mine(p, cluster, rank, n_tiles);
       int skip = MODE == kDeep ? h : 0, cs = skip;
+      // scales, three steps ahead: tile, next unit and its end, this lane's three words (row, word) = (l / 3, l % 3), l = lane + 32 j
+      FewWalk fd(p, cluster, rank, n_tiles);
+      const uint8_t* fd_base = nullptr;
+      uint32_t fd_at[3] = {0, 0, 0}, fd_hi = 0, fd_place = 0;
+      int fd_u = skip, fd_end = 0;
+      auto feed = [&] {
+        while (fd_u >= fd_end) {
+          int t;
+          if (!fd.next(&t)) {
+            fd_u = fd_end;
+            break;
+          }
+          const Tile tl = tile_of(p, t, blocks);
+          const TileSeg& sg = p.seg[MODE == kSwiglu ? sub : tl.sg];
+          fd_u = fd.u0 + fd_u - fd_end;
+          fd_end = fd.u1;
+          fd_base = sg.base + (unsigned long long)tl.expert * p.grp_stride + (size_t)sg.n_rows * (p.K / 2);
+          fd_hi = (uint32_t)sg.n_rows * nblk * 2;
+#pragma unroll
+          for (int j = 0; j < 3; ++j) {
+            const int l = lane + 32 * j, r = tl.row0 + (MODE == kWide ? sub * kRows : 0) + quarter * 32 + l / 3;
+            fd_at[j] = r < sg.n_rows ? (((uint32_t)r * nblk * 2) & ~3u) + kh * 8 + l % 3 * 4 : 0x80000000u;  // (at most 2 GB of scales, see the plan)
+          }
+        }
+        if (fd_u < fd_end) {
+#pragma unroll
+          for (int j = 0; j < 3; ++j) {
+            const uint32_t lo = fd_at[j] + (uint32_t)fd_u * 16;
+            const bool in = lo < fd_hi;
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(scale_row + fd_place * kFeedBytes + (uint32_t)(lane + 32 * j) * 4),
+                         "l"(fd_base + (in ? lo : 0)), "r"(in ? 4 : 0)
+                         : "memory");
+          }
+          fd_u += kStep;
+        }
+        fd_place = (fd_place + 1) & (kFeed - 1);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+      };
+      if (!LINES) {
+        feed();
+        feed();
+        feed();
+      }
       uint32_t cpar = 0, apar = 1;  // (the first wait for an empty slot passes at once)
       while (mine.next(&tile)) {
-        int u = mine.u0 + skip;
+        int u = mine.u0 + skip, odd = 0;
+        if (!LINES) {  // units begin at even scales: the row decides
+          const Tile tl = tile_of(p, tile, blocks);
+          odd = ((tl.row0 + (MODE == kWide ? sub * kRows : 0) + row) & nblk) & 1;
+        }
         for (; u < mine.u1; u += kStep) {
           if (!wait_warp(&cfull[cs], cpar)) return false;
           const bool free_seen = peek(&aempty[slot], apar);
           const uint32_t cr = code_row + (uint32_t)cs * kPlaceBytes;
-          const uint2 sw = lds64(scale_row + (uint32_t)(cs * kSubs * kScaleBytes));  // four scales
+          uint2 sw;  // four scales
+          if (LINES) {
+            sw = lds64(scale_row + (uint32_t)(cs * kSubs * kScaleBytes));
+          } else {
+            asm volatile("cp.async.wait_group 2;" ::: "memory");
+            __syncwarp();
+            const uint32_t sr = scale_row + (uint32_t)((m & (kFeed - 1)) * kFeedBytes + lane * 12);
+            const uint32_t w0 = lds32(sr), w1 = lds32(sr + 4), w2 = lds32(sr + 8);
+            sw = odd ? make_uint2(__byte_perm(w0, w1, 0x5432), __byte_perm(w1, w2, 0x5432)) : make_uint2(w0, w1);
+            const int left = nblk - (u * 8 + kh * 4);  // blocks that exist; what follows belongs to the next row
+            if (left < 4) sw.y &= left < 3 ? 0u : 0x0000FFFFu;
+            if (left < 2) sw.x &= left < 1 ? 0u : 0x0000FFFFu;
+            feed();  // (into the place that was read one step ago)
+          }
 #pragma unroll
           for (int c = 0; c < 2; ++c) {
             uint32_t o[32];
@@ -391,6 +464,7 @@ __global__ void __launch_bounds__(kFewThreads, 1) gemm_few_kernel(const __grid_c
       return true;
     };
     ok = expand();
+    if (!LINES) asm volatile("cp.async.wait_all;" ::: "memory");
     if (!ok) {  // whoever gives up goes on meeting the MMA warp, and does not come to the barrier before that has been there
       const int total = MODE == kDeep ? (total_units() - h + 1) / 2 : total_units();
       for (; m < total; ++m) asm volatile("bar.sync %0, 160;" ::"r"(1 + slot) : "memory");
@@ -696,10 +770,10 @@ struct FewRings {
   int codes, xs;
   size_t smem;
 };
-FewRings rings_of(int mode, int nt, int parts, size_t list) {
+FewRings rings_of(int mode, int nt, int parts, bool lines, size_t list) {
   const size_t own_runs = ((nt + kStageTok - 1) / kStageTok + parts - 1) / parts;
-  const size_t fixed = 1024 + kStageBytes + own_runs * (parts - 1) * (mode == kDeep ? 1 : 2) * kPartBytes + list;
-  const size_t xb = (size_t)nt * 256, cb = (size_t)(mode == kDeep ? 1 : 2) * (kCodeBytes + kScaleBytes);
+  const size_t fixed = 1024 + kStageBytes + own_runs * (parts - 1) * (mode == kDeep ? 1 : 2) * kPartBytes + list + (lines ? 0 : 16 * kFeed * kFeedBytes);
+  const size_t xb = (size_t)nt * 256, cb = (size_t)(mode == kDeep ? 1 : 2) * (kCodeBytes + (lines ? kScaleBytes : 0));
   const int step = mode == kDeep ? 2 : 1;
   auto fits = [&](int codes, int xs) { return fixed + xs * xb + codes * cb <= kMostSmem; };
   FewRings r{mode == kDeep ? 4 : 3, mode == kDeep ? 4 : 3, 0};
@@ -731,7 +805,7 @@ double few_us(const GemmParams& g, int rows, int mode, int nt, int n_tt, int act
 GemmFewPlan plan_of(const GemmParams& g, int sm_count, int limit) {
   GemmFewPlan best{};
   best.us = 1e300;
-  const int units = g.K / kUnitK;
+  const int units = (g.K + kUnitK - 1) / kUnitK;
   limit = std::max(limit, kUnitK);
   int n = 0;
   for (int i = 0; i < g.n_seg; ++i) n += g.seg[i].n_rows;
@@ -749,7 +823,7 @@ GemmFewPlan plan_of(const GemmParams& g, int sm_count, int limit) {
       for (int parts = 1; parts <= std::min(kMaxParts, units); ++parts) {
         // (clusters of more than two do not fill the machine: 33 of four, 26 of five, 22 of six at a time of 148 SMs)
         if (parts > 1 && tiles > (parts == 2 ? sm_count / 2 : (sm_count - 20) / parts)) break;
-        const FewRings r = rings_of(mode, nt, parts, 0);
+        const FewRings r = rings_of(mode, nt, parts, g.K % kUnitK == 0, 0);
         if (!r.smem || r.codes < (mode == kDeep ? 4 : 2)) continue;
         const int active = std::min(tiles * parts, sm_count), waves = (tiles * parts + sm_count - 1) / sm_count;
         const int per = (units + parts - 1) / parts, steps = mode == kDeep ? per : 2 * per;
@@ -778,12 +852,12 @@ GemmFewPlan plan_of(const GemmParams& g, int sm_count, int limit) {
 }  // namespace
 
 bool gemm_few_eligible(const GemmParams& g, int sm_count, GemmFewPlan* plan) {
-  if (g.w16 || g.n_seg < 1 || g.n_seg > 3 || g.K % kUnitK || g.K > (1 << 24) || g.ldx % 8) return false;
+  if (g.w16 || g.n_seg < 1 || g.n_seg > 3 || g.K % 32 || g.K > (1 << 24) || g.ldx % 8) return false;
   if (reinterpret_cast<uintptr_t>(g.x) & 15) return false;
   if ((g.res != nullptr) != (g.y2 != nullptr)) return false;
   for (int i = 0; i < g.n_seg; ++i) {
     if (reinterpret_cast<uintptr_t>(g.seg[i].base) & 15) return false;
-    if (g.grp_tab[i]) return false;
+    if (g.grp_tab[i] || (long long)g.seg[i].n_rows * (g.K / 16) >= 1ll << 31) return false;
   }
   if (g.act && (g.n_seg != 2 || g.seg[0].n_rows != g.seg[1].n_rows || g.seg[0].n_rows % 8 || g.ldact % 8 || g.ldy % 8 || g.res ||
                 ((reinterpret_cast<uintptr_t>(g.act) | reinterpret_cast<uintptr_t>(g.y)) & 15)))
@@ -814,7 +888,9 @@ cudaError_t launch_gemm_few(const GemmParams& g, const GemmFewPlan& pl, int sm_c
   }
   p.K = g.K;
   p.T = g.T;
-  p.units = g.K / kUnitK;
+  p.units = (g.K + kUnitK - 1) / kUnitK;
+  const bool lines = g.K % kUnitK == 0;
+  p.grp_stride = g.grp_stride;
   p.tile_rows = mode == kWide ? 2 * kRows : kRows;
   p.n_ft = n_ft;
   int max_blocks = 0;  // of an expert's rows, at most
@@ -851,12 +927,13 @@ cudaError_t launch_gemm_few(const GemmParams& g, const GemmFewPlan& pl, int sm_c
   p.grp_off = g.grp_off;
   FewMaps maps{};
   // activations as [64 k][tokens][chunks of 64 k]; boxes as high as tiles may be (grouped: any height)
-  const cuuint64_t xd[3] = {64, (cuuint64_t)g.T, (cuuint64_t)g.K / 64}, xs[2] = {(cuuint64_t)g.ldx * 2, 128};
+  // (K no multiple of 256: as [k][tokens], so that k beyond its end read as zeros, in boxes of 64 k)
+  const cuuint64_t xd[3] = {lines ? 64 : (cuuint64_t)g.K, (cuuint64_t)g.T, lines ? (cuuint64_t)g.K / 64 : 1}, xs[2] = {(cuuint64_t)g.ldx * 2, 128};
   const cuuint32_t one[3] = {1, 1, 1};
   const int last = ((g.T - (p.n_tt - 1) * p.nt) + 15) / 16;
   for (int h = 1; h <= p.nt / 16; ++h) {
     if (!g.grp_off && h != p.nt / 16 && h != last) continue;
-    const cuuint32_t xb[3] = {64, (cuuint32_t)(16 * h), 2};
+    const cuuint32_t xb[3] = {64, (cuuint32_t)(16 * h), lines ? 2u : 1u};
     if (enc(&maps.x[h - 1], CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3, const_cast<__half*>(g.x), xd, xs, xb, one, CU_TENSOR_MAP_INTERLEAVE_NONE,
             CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS) {
       if (err) *err = "cuTensorMapEncodeTiled failed for the activation tile";
@@ -876,16 +953,18 @@ cudaError_t launch_gemm_few(const GemmParams& g, const GemmFewPlan& pl, int sm_c
     // scales: [n_rows][K / 32] halves behind the codes, eight at a time
     const cuuint64_t sd[3] = {(cuuint64_t)g.K / 32, wd[1], groups}, ss[2] = {(cuuint64_t)g.K / 16, slice};
     const cuuint32_t sb[3] = {8, kRows, 1};
+    maps.scales[i] = maps.codes[0];
     if (enc(&maps.codes[i], CU_TENSOR_MAP_DATA_TYPE_UINT8, 3, const_cast<uint8_t*>(sg.base), wd, ws, wb, one, CU_TENSOR_MAP_INTERLEAVE_NONE,
             CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS ||
-        enc(&maps.scales[i], CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3, const_cast<uint8_t*>(sg.base) + (size_t)sg.n_rows * (g.K / 2), sd, ss, sb, one,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS) {
+        (lines && enc(&maps.scales[i], CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3, const_cast<uint8_t*>(sg.base) + (size_t)sg.n_rows * (g.K / 2), sd, ss, sb, one,
+                       CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                       CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)) {
       if (err) *err = "cuTensorMapEncodeTiled failed for the weights";
       return cudaErrorInvalidValue;
     }
   }
   const size_t list = g.grp_off ? (size_t)(max_blocks + 1) * sizeof(uint32_t) : 0;
-  const FewRings rings = rings_of(mode, p.nt, p.parts, list);
+  const FewRings rings = rings_of(mode, p.nt, p.parts, lines, list);
   if (!rings.smem) return cudaErrorInvalidValue;
   p.codes = rings.codes;
   p.xs = rings.xs;
@@ -894,9 +973,11 @@ cudaError_t launch_gemm_few(const GemmParams& g, const GemmFewPlan& pl, int sm_c
   ++*n_launch;
   const int how = p.parts > 1 || p.turns > 1 ? kShared : p.max_units < p.units ? kHanded : kPlain;
   auto run = [&](auto mode_of, auto how_of) {
-    auto kernel = g.mx ? gemm_few_kernel<true, decltype(mode_of)::value, decltype(how_of)::value> : gemm_few_kernel<false, decltype(mode_of)::value, decltype(how_of)::value>;
-    static std::atomic<uint64_t> attr_done[2];
-    const cudaError_t e = smem_limit_once(&attr_done[g.mx ? 1 : 0], {reinterpret_cast<const void*>(kernel)}, kMostSmem);
+    constexpr int kMode = decltype(mode_of)::value, kHow = decltype(how_of)::value;
+    auto kernel = g.mx ? lines ? gemm_few_kernel<true, kMode, kHow, true> : gemm_few_kernel<true, kMode, kHow, false>
+                       : lines ? gemm_few_kernel<false, kMode, kHow, true> : gemm_few_kernel<false, kMode, kHow, false>;
+    static std::atomic<uint64_t> attr_done[4];
+    const cudaError_t e = smem_limit_once(&attr_done[(g.mx ? 2 : 0) + lines], {reinterpret_cast<const void*>(kernel)}, kMostSmem);
     if (e != cudaSuccess) return e;
     return launch_dep(kernel, dim3(p.workers * p.parts), dim3(kFewThreads), smem, st, g.pdl, p.parts, maps, p);
   };

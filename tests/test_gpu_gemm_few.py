@@ -17,7 +17,10 @@ MB = 1 << 20
 @pytest.mark.parametrize("N,K,T", [(1, 256, 9), (127, 256, 16), (129, 512, 17), (255, 768, 48), (257, 1280, 64), (300, 1024, 65), (513, 256, 129), (1000, 1280, 33),
                                    (9600, 512, 12), (28672, 512, 77), (19200, 768, 128), (512, 512, 15), (4096, 4096, 16), (4095, 4096, 77), (704, 4096, 40),
                                    (2048, 5632, 31), (2048, 5632, 112), (1536, 8192, 100), (5120, 5120, 77), (6144, 4096, 77), (6141, 4096, 300), (6144, 4096, 512),
-                                   (4096, 14336, 77), (4096, 14336, 300)])
+                                   (4096, 14336, 77), (4096, 14336, 300),
+                                   # k that end within a unit, a chunk of 64 or half of one; rows of scales at 2, 4 and 8-byte boundaries
+                                   (1, 32, 9), (129, 96, 33), (300, 288, 65), (513, 2080, 100), (200, 4128, 70), (2048, 2880, 77), (2047, 2912, 16), (19200, 416, 60),
+                                   (5120, 2880, 300), (2880, 5664, 40), (2880, 1408, 500)])
 def test_gemm_of_few_tokens_matches_oracle(fmt, N, K, T):
     import torch
     from paper_2607_10183_b200 import binding as B
@@ -43,7 +46,7 @@ def test_gemm_of_few_tokens_matches_oracle(fmt, N, K, T):
 
 # Gate and up side by side with SwiGLU, and a down projection with the residual, in every way the sums go: whole tiles, clusters, several
 # accumulators.  act = rn16(silu(g) u) and y = rn16(x + d), bit for bit, with the g, u and d that are stored beside them.
-@pytest.mark.parametrize("fmt,Hd,F,T", [("q4", 4096, 4096, 16), ("mxfp4", 2048, 5632, 77), ("q4", 512, 256, 9), ("mxfp4", 1024, 2816, 100), ("q4", 5120, 1000, 40), ("q4", 2048, 12032, 130)])
+@pytest.mark.parametrize("fmt,Hd,F,T", [("q4", 4096, 4096, 16), ("mxfp4", 2048, 5632, 77), ("q4", 512, 256, 9), ("mxfp4", 1024, 2816, 100), ("q4", 5120, 1000, 40), ("q4", 2048, 12032, 130), ("mxfp4", 2880, 1440, 60), ("q4", 1536, 4128, 20)])
 def test_swiglu_and_residual_of_few_tokens(fmt, Hd, F, T):
     import torch
     from paper_2607_10183_b200 import binding as B
@@ -79,7 +82,7 @@ def test_swiglu_and_residual_of_few_tokens(fmt, Hd, F, T):
 # Routed experts, blocks of rows of every height, experts without rows, one expert with most of them: the bits of the kernel that the host
 # sorts for (one chain per sum in both).
 @pytest.mark.parametrize("fmt", ["q4", "mxfp4"])
-@pytest.mark.parametrize("E,k,T,F,skew", [(16, 4, 1, 256, 0.0), (24, 2, 333, 256, 0.0), (40, 3, 129, 512, 8.0), (64, 8, 500, 256, 0.0), (8, 2, 200, 768, 4.0)])
+@pytest.mark.parametrize("E,k,T,F,skew", [(16, 4, 1, 256, 0.0), (24, 2, 333, 256, 0.0), (40, 3, 129, 512, 8.0), (64, 8, 500, 256, 0.0), (8, 2, 200, 768, 4.0), (16, 4, 90, 1440, 0.0), (32, 2, 257, 96, 2.0)])
 def test_experts_of_few_rows_have_the_bits_of_the_host_sort(fmt, E, k, T, F, skew):
     import torch
     from paper_2607_10183_b200 import binding as B
