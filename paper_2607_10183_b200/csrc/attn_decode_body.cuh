@@ -124,7 +124,7 @@ __device__ __forceinline__ void attn_decode_compute(const AttnDecodeParams& p, c
   const int kvh = jy / p.hsplit;
   const int hbase = kvh * p.group + (jy % p.hsplit) * G;  // first of them
   const bool writer = jy % p.hsplit == 0;                 // one CTA per kv head appends to the caches
-  const int lane = tid & 31, warp = tid >> 5;
+  const int lane = tid & 31, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);  // (the same for the warp, and known to be: what follows from it needs one register a warp)
   const int g = warp / SUB, sub = warp % SUB;
   const int half = D / 2, n_ctx = p.pos + 1;
   const int qd = p.n_q * D, kvd = p.n_kv * D;

@@ -378,7 +378,7 @@ __device__ __forceinline__ bool stream_consume(const StreamParams& p, const int 
   const int n_stages = p.n_stages;
   const long long limit = p.wait_limit ? p.wait_limit : kWaitLimitCycles;
   const int tid = threadIdx.x;  // 0..511
-  const int lane = tid & 31, warp = tid >> 5;
+  const int lane = tid & 31, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);  // (the same for the warp, and known to be: what follows from it needs one register a warp)
   const int grp = warp / kGroupWarps;         // which of the two tile streams
   const int wg = warp % kGroupWarps;          // warp within the group
   const int tg = tid % (kGroupWarps * 32);    // thread within the group

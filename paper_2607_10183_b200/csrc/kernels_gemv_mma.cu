@@ -135,7 +135,7 @@ __global__ void __launch_bounds__(256) gemv_mma_kernel(const MmaGemvParams p) {
   constexpr int NT = SW ? 2 : 1;   // weight tiles per unit
   constexpr int NBK = SW ? 8 : 16;  // blocks in flight per thread and row
   __shared__ float red_s[8][NT][16][8];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31, w = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);  // (the same for the warp, and known to be)
   const int g = lane >> 2, t = lane & 3;
   const int K = p.K, nblk = K / 32, M = p.M;
   int n_rows = p.n_rows[0];  // rows side by side (SwiGLU: outputs)
@@ -322,7 +322,7 @@ __global__ void __launch_bounds__(32 * kRingWarps, 2) gemv_mma_ring_kernel(const
   constexpr int S = SW ? kRingStagesSw : kRingStages;
   extern __shared__ __align__(16) uint8_t ring[];
   __shared__ __align__(16) float red_s[2][kRingWarps][NT][16][8];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31, w = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);  // (the same for the warp, and known to be)
   const int g = lane >> 2, t = lane & 3;
   const int K = p.K, nblk = K / 32, M = p.M, n_step = K / 256;
   int n_rows = p.n_rows[0];
@@ -449,7 +449,7 @@ __global__ void __launch_bounds__(32 * kRingWarps, 2) moe_mma_ring_kernel(const 
   __shared__ unsigned long long key_s[kMoePairs];
   __shared__ uint8_t group_s[kMoePairs];               // of a group's first pair: the group
   __shared__ int warp_groups[kRingWarps];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;  // (known to be the same for the warp: 32 rows of 16 MXFP4 experts 55.7 -> 56.3 us)
   const int g = lane >> 2, t = lane & 3;
   asm volatile("griddepcontrol.wait;" ::: "memory");  // ids, activations and gathered weights come from the kernels before
   // ---- groups: thread q places pair q

@@ -132,7 +132,7 @@ __global__ void __launch_bounds__(128) attn_prefill_kernel(const __half* __restr
   __half* q_s = fa_smem;                          // [kFaQ][PITCH]
   __half* k_s = q_s + kFaQ * PITCH;               // [2][kFaK][PITCH]
   __half* v_s = k_s + 2 * kFaK * PITCH;           // [2][kFaK][PITCH]
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31, warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);  // (the same for the warp, and known to be)
   asm volatile("griddepcontrol.wait;" ::: "memory");  // inputs come from the preceding kernel
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int qb = blockIdx.x, hq = blockIdx.y, kvh = hq / group;
