@@ -319,8 +319,11 @@ cudaError_t launch_fill(void* p, uint64_t bytes, uint8_t v, cudaStream_t st, uin
 cudaError_t launch_signal_done(int* done_alias, int seq, int pdl, cudaStream_t st, uint64_t* n_launch);
 
 // prefill
+struct RopeFreq {
+  double inv[128];  // theta^(-2 i / d), i < d / 2 (0: no rotation)
+};
 cudaError_t launch_rope_append_prefill(const __half* qkv16, int ld, __half* q_rot16, __half* kc, __half* vc, int T,
-                                       int n_q, int n_kv, int d, int cap, int pos0, float theta, cudaStream_t st,
+                                       int n_q, int n_kv, int d, int cap, int pos0, const RopeFreq& freq, cudaStream_t st,
                                        uint64_t* n_launch, int pdl = 0);
 cudaError_t launch_attn_prefill(const __half* q_rot16, const __half* kc, const __half* vc, __half* a16, int T, int n_q,
                                 int n_kv, int d, int cap, int pos0, cudaStream_t st, uint64_t* n_launch, int pdl = 0);

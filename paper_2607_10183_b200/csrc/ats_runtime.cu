@@ -772,28 +772,30 @@ static const uint8_t* find_host_buffer(const ats_ctx* ctx, const void* p, uint64
   return nullptr;
 }
 
-// (cos, sin) of pos * theta^(-2i/d) for i < d/2, formed in fp64 on the host and rounded to fp32.  The inverse
-// frequencies are cached per (theta, d).
-static void rope_table(ats_ctx* ctx, float theta, int d, int pos, float* cs) {
-  const int half = d / 2;
-  if (theta == 0.f) {
-    for (int i = 0; i < half; ++i) {
-      cs[2 * i] = 1.f;
-      cs[2 * i + 1] = 0.f;
-    }
-    return;
-  }
+// theta^(-2i/d) for i < d/2 in fp64 (0: no rotation), kept per (theta, d).
+static const std::vector<double>& rope_inverse(ats_ctx* ctx, float theta, int d) {
   if (ctx->rope_theta != theta || ctx->rope_d != d) {
-    ctx->rope_inv.resize(half);
-    for (int i = 0; i < half; ++i) ctx->rope_inv[i] = pow((double)theta, -2.0 * (double)i / (double)d);
+    ctx->rope_inv.resize(d / 2);
+    for (int i = 0; i < d / 2; ++i) ctx->rope_inv[i] = theta == 0.f ? 0.0 : pow((double)theta, -2.0 * (double)i / (double)d);
     ctx->rope_theta = theta;
     ctx->rope_d = d;
   }
-  for (int i = 0; i < half; ++i) {
-    const double a = (double)pos * ctx->rope_inv[i];
+  return ctx->rope_inv;
+}
+// (cos, sin) of pos * theta^(-2i/d) for i < d/2, formed in fp64 on the host and rounded to fp32.
+static void rope_table(ats_ctx* ctx, float theta, int d, int pos, float* cs) {
+  const std::vector<double>& inv = rope_inverse(ctx, theta, d);
+  for (int i = 0; i < d / 2; ++i) {
+    const double a = (double)pos * inv[i];
     cs[2 * i] = (float)cos(a);
     cs[2 * i + 1] = (float)sin(a);
   }
+}
+static RopeFreq rope_freq(ats_ctx* ctx, float theta, int d) {
+  RopeFreq f{};
+  const std::vector<double>& inv = rope_inverse(ctx, theta, d);
+  std::copy_n(inv.begin(), std::min<size_t>(inv.size(), 128), f.inv);
+  return f;
 }
 
 }  // namespace ats
@@ -1726,7 +1728,7 @@ int32_t ats_layer_prefill(ats_ctx* ctx, const ats_layer_desc* L, const void* x_i
     scratch(w.qkv_scratch);
     ATS_TRY(run_gemm_group(ctx, qkv, 3, g));
     ATS_CUDA(launch_rope_append_prefill(w.qkv16, qd + 2 * kvd, w.qrot16, (__half*)k_cache, (__half*)v_cache, (int)T, nq, nkv, d,
-                                        (int)L->kv_capacity, (int)pos0, L->rope_theta, ctx->cs, nl, pdl));
+                                        (int)L->kv_capacity, (int)pos0, rope_freq(ctx, L->rope_theta, d), ctx->cs, nl, pdl));
     if (attn_prefill_tc_eligible(w.qrot16, (const __half*)k_cache, (const __half*)v_cache, w.a16, (int)T, d))
       ATS_CUDA(launch_attn_prefill_tc(w.qrot16, (const __half*)k_cache, (const __half*)v_cache, w.a16, (int)T, nq, nkv, d,
                                       (int)L->kv_capacity, (int)pos0, ctx->dev_status, ctx->cs, nl, pdl));

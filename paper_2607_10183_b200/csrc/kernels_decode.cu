@@ -642,21 +642,24 @@ __global__ void __launch_bounds__(256) rmsnorm_kernel(const TIn* __restrict__ x,
 __global__ void __launch_bounds__(256) rmsnorm16_vec_kernel(const __half* __restrict__ x, const __half* __restrict__ gain,
                                                             __half* __restrict__ out, int H, float eps) {
   __shared__ float red[8];
-  asm volatile("griddepcontrol.wait;" ::: "memory");  // inputs come from the preceding kernel
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int n8 = H / 8;
   const uint4* xr = reinterpret_cast<const uint4*>(x + (size_t)blockIdx.x * H);
   uint4 xv[4], gv[4];
   float ss = 0.f;
 #pragma unroll
+  for (int j = 0; j < 4; ++j) {  // (the gains are parameters)
+    const int c = threadIdx.x + 256 * j;
+    gv[j] = c < n8 ? __ldg(reinterpret_cast<const uint4*>(gain) + c) : make_uint4(0, 0, 0, 0);
+  }
+  asm volatile("griddepcontrol.wait;" ::: "memory");  // the row comes from the preceding kernel
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+#pragma unroll
   for (int j = 0; j < 4; ++j) {
     const int c = threadIdx.x + 256 * j;
-    xv[j] = make_uint4(0, 0, 0, 0);
-    gv[j] = make_uint4(0, 0, 0, 0);
-    if (c < n8) {
-      xv[j] = xr[c];
-      gv[j] = __ldg(reinterpret_cast<const uint4*>(gain) + c);
-    }
+    xv[j] = c < n8 ? xr[c] : make_uint4(0, 0, 0, 0);
+  }
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
     const uint32_t w[4] = {xv[j].x, xv[j].y, xv[j].z, xv[j].w};
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
