@@ -39,3 +39,11 @@ def test_prompt_attention_matches_oracle(T, pos0, nq, nkv, d, spare):
     ctx.close()
     want = np.stack([O.attention_one(q[i].reshape(nq, d), kg, vg, pos0 + i + 1).reshape(-1) for i in range(T)])
     H.assert_close(a, O.rn16(want), what="attention")
+
+
+# Contexts of six blocks and more, whose tiles take the even and the odd blocks: six, seven, eight and eleven of them, last blocks that the first
+# rows do not see, a second token block with one block more than the first.
+@pytest.mark.parametrize("T,pos0,nq,nkv,d", [(129, 639, 2, 1, 64), (130, 700, 3, 1, 128), (200, 701, 6, 2, 64), (130, 1151, 4, 2, 128), (260, 1020, 8, 1, 128)])
+@pytest.mark.parametrize("spare", [0, 70])
+def test_prompt_attention_over_even_and_odd_blocks(T, pos0, nq, nkv, d, spare):
+    test_prompt_attention_matches_oracle(T, pos0, nq, nkv, d, spare)
