@@ -1175,14 +1175,18 @@ __global__ void __launch_bounds__(kRouterClThreads) router_topk_cluster_kernel(c
 // it in shared memory, so that a weight is read from L2 once for all of them.  A thread sums four tokens x four experts over the whole range,
 // chain by chain in router_topk_cluster_kernel's order (rows g, g + R, ...; chains in ascending order), the ranges are added up by the CTA a
 // token belongs to, a warp per token: a token's logits have the same bits whichever kernel ran.  Bound by instruction issue (4 conversions, 8
-// paired multiply-adds, two shared-memory loads a row and thread), under 18 tokens by the chain of its latencies.  Back to back, a CTA with four
-// tokens and the whole matrix before -> now, us: 2048 x 128, 128 / 512 / 2048 tokens 22.0 / 22.1 / 84.6 -> 10.8 / 15.8 / 48.3; 2880 x 64 (a
-// cluster per token before), 512 / 2048 tokens 63 / 244 -> 20 / 41.
-constexpr int kRouterTokThreads = 256;
-// From here on (the cluster kernel takes 10.6 us for 64 tokens, 18.3 for 128; this one 10 to 13).
-constexpr int kRouterManyTokens = 96;
+// paired multiply-adds, two shared-memory loads a row and thread) where clusters fill the SMs in pairs.  Where every CTA has an SM to itself it is the
+// chain of a thread's latencies: two experts to a thread and 512 threads then (twice the threads; half as much again of issue where that is what
+// counts: 512 tokens through 128 experts 127.2 -> 138.8 us a layer, 2048 302 -> 330).  Back to back, a CTA with four tokens and the whole matrix
+// before -> four experts to a thread, us: 2048 x 128, 128 / 512 / 2048 tokens 22.0 / 22.1 / 84.6 -> 10.8 / 15.8 / 48.3; 2880 x 64 (a cluster per token
+// before), 512 / 2048 tokens 63 / 244 -> 20 / 41.  Layers, four experts -> two: 2048 x 128, 100 / 200 tokens 109.2 / 112.0 -> 103.0 / 107.8;
+// 2880 x 64, 128 / 512 tokens 112.3 / 127.9 -> 104.2 / 118.5; 1024 x 32, 300 tokens 39.7 -> 35.9.
+// From here on (a cluster per token before -> this, layers, us: 2048 x 128, 48 / 64 / 80 tokens 95.8 / 105.7 / 106.8 -> 94.6 / 102.4 / 101.6;
+// 2880 x 64 99.8 / 105.2 / 106.2 -> 100.3 / 103.1 / 103.3).
+constexpr int kRouterManyTokens = 56;
 
-__global__ void __launch_bounds__(kRouterTokThreads) router_topk_tokens_kernel(const __half* __restrict__ h, const __half* __restrict__ wr, int M,
+template <int EXPERTS, int THREADS>
+__global__ void __launch_bounds__(THREADS) router_topk_tokens_kernel(const __half* __restrict__ h, const __half* __restrict__ wr, int M,
                                                                                int H, int E, int tok, int k, int renorm,
                                                                                int32_t* __restrict__ ids, float* __restrict__ gates) {
   extern __shared__ __align__(16) float smem[];
@@ -1197,7 +1201,7 @@ __global__ void __launch_bounds__(kRouterTokThreads) router_topk_tokens_kernel(c
   {  // (the router matrix does not depend on the preceding kernel)
     const uint32_t dst = (uint32_t)__cvta_generic_to_shared(w_s);
     const __half* src = wr + (size_t)row0 * E;
-    for (int c = tid * 8; c < Hc * E; c += kRouterTokThreads * 8)
+    for (int c = tid * 8; c < Hc * E; c += THREADS * 8)
       asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + 2u * c), "l"(src + c) : "memory");
   }
   asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");  // (nobody writes into a CTA that has not begun)
@@ -1205,7 +1209,7 @@ __global__ void __launch_bounds__(kRouterTokThreads) router_topk_tokens_kernel(c
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int row8 = Hc / 8;
 #pragma unroll 4
-  for (int j = tid; j < tok * row8; j += kRouterTokThreads) {
+  for (int j = tid; j < tok * row8; j += THREADS) {
     const int t = j / row8, i = (j - t * row8) * 8;
     const uint4 v = m0 + t < M ? *reinterpret_cast<const uint4*>(h + (size_t)(m0 + t) * H + row0 + i) : make_uint4(0, 0, 0, 0);
     const float2 a = __half22float2(u32_as_half2(v.x)), b = __half22float2(u32_as_half2(v.y)), c = __half22float2(u32_as_half2(v.z)),
@@ -1217,19 +1221,23 @@ __global__ void __launch_bounds__(kRouterTokThreads) router_topk_tokens_kernel(c
   asm volatile("cp.async.wait_all;" ::: "memory");
   __syncthreads();
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-  const int lanes = E / 4, items = tok / 4 * lanes;
-  for (int it = tid; it < items; it += kRouterTokThreads) {
-    const int t0 = it / lanes * 4, e0 = it % lanes * 4;
-    float2 sum[4][2];
+  const int lanes = E / EXPERTS, items = tok / 4 * lanes;
+  for (int it = tid; it < items; it += THREADS) {
+    const int t0 = it / lanes * 4, e0 = it % lanes * EXPERTS;
+    float2 sum[4][EXPERTS / 2];
 #pragma unroll
-    for (int t = 0; t < 4; ++t) sum[t][0] = sum[t][1] = make_float2(0.f, 0.f);
+    for (int t = 0; t < 4; ++t)
+#pragma unroll
+      for (int q = 0; q < EXPERTS / 2; ++q) sum[t][q] = make_float2(0.f, 0.f);
     const float* xr = x_s + (size_t)t0 * pitch;
     for (int g = 0; g < R; g += 4) {  // four chains side by side: their rows follow one another (R and Hc are multiples of 4)
-      float2 acc[4][4][2];
+      float2 acc[4][4][EXPERTS / 2];
 #pragma unroll
       for (int c = 0; c < 4; ++c)
 #pragma unroll
-        for (int t = 0; t < 4; ++t) acc[c][t][0] = acc[c][t][1] = make_float2(0.f, 0.f);
+        for (int t = 0; t < 4; ++t)
+#pragma unroll
+          for (int q = 0; q < EXPERTS / 2; ++q) acc[c][t][q] = make_float2(0.f, 0.f);
 #pragma unroll 2
       for (int i = g; i < Hc; i += R) {
         float4 x[4];
@@ -1237,13 +1245,18 @@ __global__ void __launch_bounds__(kRouterTokThreads) router_topk_tokens_kernel(c
         for (int t = 0; t < 4; ++t) x[t] = *reinterpret_cast<const float4*>(xr + (size_t)t * pitch + i);
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
-          const uint2 w = *reinterpret_cast<const uint2*>(w_s + (size_t)(i + c) * E + e0);
-          const float2 wa = __half22float2(u32_as_half2(w.x)), wb = __half22float2(u32_as_half2(w.y));
+          float2 w[EXPERTS / 2];
+          if constexpr (EXPERTS == 4) {
+            const uint2 v = *reinterpret_cast<const uint2*>(w_s + (size_t)(i + c) * E + e0);
+            w[0] = __half22float2(u32_as_half2(v.x)), w[1] = __half22float2(u32_as_half2(v.y));
+          } else {
+            w[0] = __half22float2(*reinterpret_cast<const __half2*>(w_s + (size_t)(i + c) * E + e0));
+          }
 #pragma unroll
           for (int t = 0; t < 4; ++t) {
             const float xv = c == 0 ? x[t].x : c == 1 ? x[t].y : c == 2 ? x[t].z : x[t].w;
-            acc[c][t][0] = fma_x2(make_float2(xv, xv), wa, acc[c][t][0]);
-            acc[c][t][1] = fma_x2(make_float2(xv, xv), wb, acc[c][t][1]);
+#pragma unroll
+            for (int q = 0; q < EXPERTS / 2; ++q) acc[c][t][q] = fma_x2(make_float2(xv, xv), w[q], acc[c][t][q]);
           }
         }
       }
@@ -1252,20 +1265,23 @@ __global__ void __launch_bounds__(kRouterTokThreads) router_topk_tokens_kernel(c
 #pragma unroll
         for (int t = 0; t < 4; ++t)
 #pragma unroll
-          for (int q = 0; q < 2; ++q) sum[t][q] = add_x2(sum[t][q], acc[c][t][q]);
+          for (int q = 0; q < EXPERTS / 2; ++q) sum[t][q] = add_x2(sum[t][q], acc[c][t][q]);
     }
 #pragma unroll
     for (int t = 0; t < 4; ++t) {
       const int to = (t0 + t) / own, at = (t0 + t) % own;
       uint32_t la = (uint32_t)__cvta_generic_to_shared(cl + ((size_t)rank * own + at) * E + e0), ra;
       asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(la), "r"(to));
-      asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(ra), "f"(sum[t][0].x), "f"(sum[t][0].y), "f"(sum[t][1].x), "f"(sum[t][1].y)
-                   : "memory");
+      if constexpr (EXPERTS == 4)
+        asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(ra), "f"(sum[t][0].x), "f"(sum[t][0].y), "f"(sum[t][1].x), "f"(sum[t][1].y)
+                     : "memory");
+      else
+        asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(ra), "f"(sum[t][0].x), "f"(sum[t][0].y) : "memory");
     }
   }
   cluster_sync_all();
   const int lane = tid & 31;
-  for (int at = tid >> 5; at < own; at += kRouterTokThreads / 32) {
+  for (int at = tid >> 5; at < own; at += THREADS / 32) {
     const int m = m0 + (int)rank * own + at;
     if (m >= M) return;
     auto select = [&](auto per) {
@@ -1315,12 +1331,17 @@ cudaError_t launch_router_topk_norm(const __half* h, const __half* wr, int M, in
         if (all < best) best = all, tok = t;
       }
       if (tok) {
-        static std::atomic<uint64_t> attr_done;
-        const cudaError_t e = smem_limit_once(&attr_done, {reinterpret_cast<const void*>(router_topk_tokens_kernel)}, kMostTok);
-        if (e != cudaSuccess) return e;
-        ++*n_launch;
-        return launch_dep(router_topk_tokens_kernel, dim3((M + tok - 1) / tok * kRouterCluster), dim3(kRouterTokThreads), smem_tok(tok), st, pdl,
-                          kRouterCluster, h, wr, M, H, E, tok, k, renorm, ids, gates);
+        const int clusters = (M + tok - 1) / tok;  // (up to 15 run at once with an SM to each CTA)
+        auto run = [&](auto kernel, int threads) {
+          static std::atomic<uint64_t> attr_done;
+          const cudaError_t e = smem_limit_once(&attr_done, {reinterpret_cast<const void*>(router_topk_tokens_kernel<2, 512>),
+                                                             reinterpret_cast<const void*>(router_topk_tokens_kernel<4, 256>)}, kMostTok);
+          if (e != cudaSuccess) return e;
+          ++*n_launch;
+          return launch_dep(kernel, dim3(clusters * kRouterCluster), dim3(threads), smem_tok(tok), st, pdl, kRouterCluster, h, wr, M, H, E, tok, k,
+                            renorm, ids, gates);
+        };
+        return clusters <= 15 ? run(router_topk_tokens_kernel<2, 512>, 512) : run(router_topk_tokens_kernel<4, 256>, 256);
       }
     }
     constexpr size_t kMostCl = 160 * 1024;

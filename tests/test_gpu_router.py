@@ -10,7 +10,7 @@ pytestmark = pytest.mark.gpu
 # One and several rounds of clusters, a last cluster with few tokens, chains of unequal length (2880 rows, 64 experts), one row to a chain (512 x 16),
 # more than 128 experts (a shorter block of tokens where shared memory is full); equal logits and a NaN among the tokens.
 @pytest.mark.parametrize("hidden,E,k,M", [(2048, 128, 8, 96), (2048, 128, 8, 513), (2880, 64, 4, 130), (512, 16, 2, 700), (1024, 32, 4, 2000), (1024, 256, 8, 250),
-                                          (3072, 256, 6, 97), (4096, 64, 4, 1100)])
+                                          (3072, 256, 6, 97), (4096, 64, 4, 1100), (2048, 128, 8, 56), (2880, 64, 4, 121), (2048, 128, 8, 250)])
 def test_router_of_many_tokens_has_the_bits_of_the_router_of_few(hidden, E, k, M):
     import torch
     from paper_2607_10183_b200 import binding as B
@@ -31,7 +31,7 @@ def test_router_of_many_tokens_has_the_bits_of_the_router_of_few(hidden, E, k, M
         return ids, gates.view(torch.int32)
 
     ids, gates = route(0, M)
-    parts = [route(lo, min(M, lo + 64)) for lo in range(0, M, 64)]
+    parts = [route(lo, min(M, lo + 48)) for lo in range(0, M, 48)]
     assert torch.equal(ids, torch.cat([p[0] for p in parts]))
     assert torch.equal(gates, torch.cat([p[1] for p in parts]))
     ctx.close()
