@@ -333,7 +333,7 @@ cudaError_t launch_attn_prefill_tc(const __half* q_rot16, const __half* kc, cons
                                    int cap, int pos0, int* status, cudaStream_t st, uint64_t* n_launch, int pdl = 0);
 // MoE prefill helpers (kernels_prefill.cu): rows gathered in expert order, and the gated sum back in token order
 cudaError_t launch_moe_sort_gather(const int32_t* ids, int P, int E, int k, int H, const __half* h, int* order, int* pos, int* off, __half* xs,
-                                   int* status, int* done, int seq, cudaStream_t st, uint64_t* n_launch, int pdl);
+                                   int* status, int* done, int seq, int sm_count, cudaStream_t st, uint64_t* n_launch, int pdl);
 cudaError_t launch_moe_gather_rows(const __half* h, const int* order, int k, __half* xs, int P, int H, cudaStream_t st,
                                    uint64_t* n_launch, int pdl = 0);
 cudaError_t launch_moe_combine_sorted(const __half* res, const float* gates, const __half* d, const int* pos, __half* y, int T, int k,

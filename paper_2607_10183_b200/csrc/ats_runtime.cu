@@ -1773,7 +1773,7 @@ int32_t ats_layer_prefill(ats_ctx* ctx, const ats_layer_desc* L, const void* x_i
     int max_rows = 0, seq = 0;
     if (on_device) {
       seq = ++ctx->done_seq;
-      ATS_CUDA(launch_moe_sort_gather(w.ids, P, E, k, H, w.h2_16, w.order, w.pos, w.grp_off, w.xs16, ctx->dev_status, ctx->done_dev, seq, ctx->cs, nl, pdl));
+      ATS_CUDA(launch_moe_sort_gather(w.ids, P, E, k, H, w.h2_16, w.order, w.pos, w.grp_off, w.xs16, ctx->dev_status, ctx->done_dev, seq, ctx->sm_count, ctx->cs, nl, pdl));
     } else {
       ATS_TRY(fetch_ids(ctx, w.ids, P, E));
       if (ats_host_group_pairs(ctx->ids_host, (uint32_t)P, (uint32_t)E, order_h, pos_h, off_h, &max_rows) != ATS_OK)

@@ -318,18 +318,24 @@ cudaError_t launch_swiglu16(const __half* gu, int ld, int ffn, __half* act, int 
 // MoE prefill: the stable sort of the (token, slot) pairs by expert, on the device, and the rows in that order: order[r] = the pair at sorted
 // position r, pos[p] = the position of pair p, off[e] = the first position of expert e, off[E] = P: what ats_host_group_pairs makes of
 // the same ids; xs[r] = the row of order[r]'s token.
-// 1 << shift CTAs to an expert: each counts for itself the pairs of lower experts and, in the order of its threads' contiguous parts, of its own
-// (16 KB of ids for 4096 pairs), then places every 1 << shift-th of them and copies their rows.  The completion word tells the host that the
-// router has run.  Bound by latencies (ids twice, two sums over the CTA, rows) and the copies (4096 rows of 4 KB written: 2.6 us).  512
-// tokens through 8 of 128 experts: one CTA that sorts, then a launch that copies 9.8 + 4.9 us, this 11.2.
-constexpr int kSortThreads = 256, kSortList = 512;
-__global__ void __launch_bounds__(kSortThreads) moe_sort_gather_kernel(const int32_t* __restrict__ ids, int P, int E, int shift, int k, int H,
+// Every CTA counts the pairs for itself (16 KB of ids for 4096 pairs), finds those of its expert and run in the order of its threads' contiguous parts,
+// places them and copies their rows.  The completion word tells the host that the router has run.
+//   DEALT   an expert has as many CTAs as it has runs of `share` rows, so that none copies more than those however the tokens are routed
+//   else    an expert has 1 << shift CTAs, which need not know the other experts' counts: 0.6 to 1 us less
+// Bound by latencies (ids twice, a sum over the CTA, or two, rows) and the copies (4096 rows of 4 KB written: 2.6 us).
+constexpr int kSortThreads = 256, kSortShare = 512;
+template <bool DEALT>
+__global__ void __launch_bounds__(kSortThreads) moe_sort_gather_kernel(const int32_t* __restrict__ ids, int P, int E, int share, unsigned inv_share, int shift, int k, int H,
                                                                        const __half* __restrict__ h, int* __restrict__ order, int* __restrict__ pos,
                                                                        int* __restrict__ off, __half* __restrict__ xs, int* status, int* done, int seq) {
-  __shared__ int lower_s[kSortThreads / 32], own_s[kSortThreads / 32], list_s[kSortList];
+  __shared__ int count_s[DEALT ? 1024 : 1], sum_s[2][kSortThreads / 32], list_s[kSortShare], run_s[4];
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-  const int e = blockIdx.x >> shift, s = blockIdx.x & ((1 << shift) - 1);
   const int per = (P + kSortThreads * 4 - 1) / (kSortThreads * 4) * 4, lo = min(tid * per, P), hi = min(lo + per, P);
+  if (DEALT) {
+    for (int i = tid; i < E; i += kSortThreads) count_s[i] = 0;
+    if (tid == 0) run_s[0] = -1;
+    __syncthreads();
+  }
   asm volatile("griddepcontrol.wait;" ::: "memory");  // the ids come from the router
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   // (an id that names no expert, which the router does not write, counts as expert 0 and the status word says so)
@@ -358,69 +364,120 @@ __global__ void __launch_bounds__(kSortThreads) moe_sort_gather_kernel(const int
       }
     }
   };
-  int lower = 0, own = 0;
-  bool bad = false;
-  each([&](int, int id) {
-    bad |= (unsigned)id >= (unsigned)E;
-    id = (unsigned)id < (unsigned)E ? id : 0;
-    lower += id < e;
-    own += id == e;
-  });
-  if (bad && blockIdx.x == 0) raise_status(status, 7);
-  int incl = own;
+  auto before = [&](int v, int* sums) {  // the sum of the lanes' values before this one, the warp's to sums
+    int incl = v;
 #pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int v = __shfl_up_sync(0xFFFFFFFFu, incl, o);
-    if (lane >= o) incl += v;
+    for (int o = 1; o < 32; o <<= 1) {
+      const int u = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+      if (lane >= o) incl += u;
+    }
+    if (lane == 31) sums[w] = incl;
+    return incl - v;
+  };
+  bool bad = false;
+  int mine = (int)blockIdx.x >> shift, first = 0, from, to, own = 0, at;  // expert, its first position, the run's first row and end
+  if (DEALT) {
+    each([&](int, int id) {
+      bad |= (unsigned)id >= (unsigned)E;
+      atomicAdd(&count_s[(unsigned)id < (unsigned)E ? id : 0], 1);
+    });
+    __syncthreads();
+    // rows and runs of the experts before each, in one word (at most 65536 rows, below 2^15 runs)
+    auto runs_of = [&](int n) { return (int)__umulhi((unsigned)(n + share - 1), inv_share); };
+    const int each_e = (E + kSortThreads - 1) / kSortThreads, e0 = min(tid * each_e, E), e1 = min(e0 + each_e, E);
+    int both = 0;
+    for (int e = e0; e < e1; ++e) both += count_s[e] | runs_of(count_s[e]) << 17;
+    both = before(both, sum_s[0]);
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < kSortThreads / 32; ++i) both += i < w ? sum_s[0][i] : 0;
+    for (int e = e0; e < e1; ++e) {
+      const int n = count_s[e], s = (int)blockIdx.x - (both >> 17);
+      if (blockIdx.x == 0) off[e] = both & 0x1FFFF;
+      if (s >= 0 && s < runs_of(n)) {
+        run_s[0] = e;
+        run_s[1] = both & 0x1FFFF;
+        run_s[2] = s * share;
+        run_s[3] = min(n, (s + 1) * share);
+      }
+      both += n | runs_of(n) << 17;
+    }
+    __syncthreads();
+    mine = run_s[0], first = run_s[1], from = run_s[2], to = run_s[3];
+    if (mine >= 0) {
+      each([&](int, int id) { own += ((unsigned)id < (unsigned)E ? id : 0) == mine; });
+      at = before(own, sum_s[1]);
+    }
+  } else {
+    int lower = 0;
+    each([&](int, int id) {
+      bad |= (unsigned)id >= (unsigned)E;
+      id = (unsigned)id < (unsigned)E ? id : 0;
+      lower += id < mine;
+      own += id == mine;
+    });
+    at = before(own, sum_s[1]);
+    lower = __reduce_add_sync(0xFFFFFFFFu, lower);
+    if (lane == 0) sum_s[0][w] = lower;
   }
-  lower = __reduce_add_sync(0xFFFFFFFFu, lower);
-  if (lane == 31) own_s[w] = incl;
-  if (lane == 0) lower_s[w] = lower;
+  if (bad && blockIdx.x == 0) raise_status(status, 7);
+  if (mine < 0) return;  // (no run is left for this CTA; for CTA 0 there is one)
   __syncthreads();
-  int first = 0, at = incl - own, n = 0;
+  int n = 0;
 #pragma unroll
   for (int i = 0; i < kSortThreads / 32; ++i) {
-    first += lower_s[i];
-    at += i < w ? own_s[i] : 0;
-    n += own_s[i];
+    if (!DEALT) first += sum_s[0][i];
+    at += i < w ? sum_s[1][i] : 0;
+    n += sum_s[1][i];
   }
-  if (tid == 0 && s == 0) {
-    off[e] = first;
-    if (e == E - 1) off[E] = P;
+  if (!DEALT) {
+    const int s = (int)blockIdx.x & ((1 << shift) - 1);
+    from = n * s >> shift, to = n * (s + 1) >> shift;
+    if (tid == 0 && s == 0) off[mine] = first;
   }
-  if (own) {
+  if (blockIdx.x == 0 && tid == 0) off[E] = P;
+  if (own && at < to && at + own > from) {
     each([&](int p, int id) {
-      if (((unsigned)id < (unsigned)E ? id : 0) != e) return;
-      const int m = at >> shift;
-      if ((at & ((1 << shift) - 1)) == s) {
+      if (((unsigned)id < (unsigned)E ? id : 0) != mine) return;
+      if (at >= from && at < to) {
         order[first + at] = p;
         pos[p] = first + at;
-        if (m < kSortList) list_s[m] = p / k;
+        list_s[at - from] = p / k;
       }
       ++at;
     });
   }
   __syncthreads();
-  const int rows = (n - s + (1 << shift) - 1) >> shift;  // (s < 1 << shift: at least 0)
   for (int c = tid; c < H / 8; c += kSortThreads) {
 #pragma unroll 8
-    for (int m = 0; m < rows; ++m) {
-      const int r = first + s + (m << shift), t = m < kSortList ? list_s[m] : order[r] / k;
-      reinterpret_cast<uint4*>(xs + (size_t)r * H)[c] = __ldg(reinterpret_cast<const uint4*>(h + (size_t)t * H) + c);
-    }
+    for (int m = 0; m < to - from; ++m)
+      reinterpret_cast<uint4*>(xs + (size_t)(first + from + m) * H)[c] = __ldg(reinterpret_cast<const uint4*>(h + (size_t)list_s[m] * H) + c);
   }
   // (without a fence: one that waits for the host's memory held the sort up)
   if (done && blockIdx.x == 0 && tid == 0) *reinterpret_cast<volatile int*>(done) = seq;
 }
 
 cudaError_t launch_moe_sort_gather(const int32_t* ids, int P, int E, int k, int H, const __half* h, int* order, int* pos, int* off, __half* xs,
-                                   int* status, int* done, int seq, cudaStream_t st, uint64_t* n_launch, int pdl) {
-  if (E < 1 || P < 1) return cudaErrorInvalidValue;
-  int shift = 0;
-  while ((2 << shift) * E <= 4 * 148) ++shift;  // (one CTA to an SM 19.8 us, two 14.0, four 11.2, eight 12.9: copies in flight against ids read)
+                                   int* status, int* done, int seq, int sm_count, cudaStream_t st, uint64_t* n_launch, int pdl) {
+  if (E < 1 || E > 1024 || P < 1 || P > 65536) return cudaErrorInvalidValue;
   ++*n_launch;
-  return launch_dep(moe_sort_gather_kernel, dim3(E << shift), dim3(kSortThreads), 0, st, pdl, 1, ids, P, E, shift, k, H, h, order, pos, off, xs, status,
-                    done, seq);
+  // Four CTAs to an SM (with even routings one took 19.8 us, two 14.0, four 11.2, eight 12.9: copies in flight against ids read).
+  int shift = 0;
+  while ((2 << shift) * E <= 4 * sm_count) ++shift;
+  // An expert has at most a row of each token: where that is at most 16 to each of its 1 << shift CTAs there is nothing to deal.  (Layers, every token
+  // to other experts / all tokens to the same, us.  19 rows, 300 tokens through 4 of 32: fixed 126.4 / 129, dealt 127.1 / 125.5; 128 rows, 512 tokens through
+  // 8 of 128: 145 / 129, 143 / 101; 1024 rows, 4096 tokens: 588 / 884, 581 / 511.  1024 tokens through 8 of 1024 654 / 837, 658 / 585.)
+  if (P / k <= 16 << shift && k <= 32)
+    return launch_dep(moe_sort_gather_kernel<false>, dim3(E << shift), dim3(kSortThreads), 0, st, pdl, 1, ids, P, E, 0, 0u, shift, k, H, h, order, pos, off, xs,
+                      status, done, seq);
+  // A run that is not full can end each expert, so as many CTAs as there are experts (or rows) are on top of the P / share: many experts make it up to
+  // eight to an SM, all that run at once.
+  const int partial = std::min(E, P);
+  const int spare = std::max(std::min(std::max(4 * sm_count - partial, 2 * sm_count), 8 * sm_count - partial), std::max(sm_count, (P + kSortShare - 1) / kSortShare));
+  const int share = std::max(2, (P + spare - 1) / spare);
+  const unsigned inv_share = (unsigned)(((1ull << 32) + share - 1) / share);  // n / share = n * inv_share >> 32 while n * share < 2^32
+  return launch_dep(moe_sort_gather_kernel<true>, dim3(P / share + partial), dim3(kSortThreads), 0, st, pdl, 1, ids, P, E, share, inv_share, 0, k, H, h, order,
+                    pos, off, xs, status, done, seq);
 }
 
 // MoE prefill: rows sorted by expert.  xs[r] = h[order[r] / k] (order[r] = the (token, slot) pair at sorted position r);
