@@ -1181,8 +1181,8 @@ __global__ void __launch_bounds__(kRouterClThreads) router_topk_cluster_kernel(c
 // before -> four experts to a thread, us: 2048 x 128, 128 / 512 / 2048 tokens 22.0 / 22.1 / 84.6 -> 10.8 / 15.8 / 48.3; 2880 x 64 (a cluster per token
 // before), 512 / 2048 tokens 63 / 244 -> 20 / 41.  Layers, four experts -> two: 2048 x 128, 100 / 200 tokens 109.2 / 112.0 -> 103.0 / 107.8;
 // 2880 x 64, 128 / 512 tokens 112.3 / 127.9 -> 104.2 / 118.5; 1024 x 32, 300 tokens 39.7 -> 35.9.
-// From here on (a cluster per token before -> this, layers, us: 2048 x 128, 48 / 64 / 80 tokens 95.8 / 105.7 / 106.8 -> 94.6 / 102.4 / 101.6;
-// 2880 x 64 99.8 / 105.2 / 106.2 -> 100.3 / 103.1 / 103.3).
+// From here on the launcher compares the forms' times; below it a cluster per token takes no longer (layers, a cluster per token -> this, us: 2048 x 128,
+// 48 / 64 / 80 tokens 95.8 / 105.7 / 106.8 -> 94.6 / 102.4 / 101.6; 2880 x 64 99.8 / 105.2 / 106.2 -> 100.3 / 103.1 / 103.3).
 constexpr int kRouterManyTokens = 56;
 
 template <int EXPERTS, int THREADS>
@@ -1301,6 +1301,111 @@ __global__ void __launch_bounds__(THREADS) router_topk_tokens_kernel(const __hal
   }
 }
 
+// And for many tokens of a matrix whose eighth does not fit an SM's shared memory beside them, or leaves room for too few: a CTA takes four tokens and
+// streams the whole matrix through shared memory (16-byte asynchronous copies, stages of 32 KB), so that a weight is read from L2 and converted once
+// for four tokens.  Thread (row group, four experts) sums its chain of rows in each of the eight ranges, and the chains and ranges are added up in
+// router_topk_cluster_kernel's order: the same bits again.  Bound by instruction issue (16 multiply-adds, 4 conversions and 2 shared-memory loads
+// per row and thread).  A cluster per token -> this, us: 2048 x 512, 200 / 512 / 2048 tokens 93 / 213 / 799 -> 69 / 70 / 266; 1024 x 1024
+// 115 / 257 / 951 -> 80 / 80 / 311; 4096 x 256 69 / 162 / 619 -> 63 / 64 / 242; clusters of tokens -> this: 4096 x 128, 512 tokens 48 -> 37.
+constexpr int kRouterStreamTok = 4;
+constexpr int kRouterStreamThreads = 512;  // 4 experts each: E / 4 x (2048 / E) row groups
+constexpr int kRouterStageRows = 8;        // rows of a chain per stage
+constexpr int kRouterStageElems = kRouterStageRows * 2048;  // ... of all R = 2048 / E chains: contiguous rows of W_r
+
+__global__ void __launch_bounds__(kRouterStreamThreads) router_topk_stream_kernel(const __half* __restrict__ h, const __half* __restrict__ wr, int M,
+                                                                                  int H, int E, int Epad, int k, int renorm, int stages,
+                                                                                  int32_t* __restrict__ ids, float* __restrict__ gates) {
+  extern __shared__ __align__(16) float smem[];
+  const int Hc = H / kRouterCluster, R = 2048 / E, per_range = Hc / R / kRouterStageRows, n_st = kRouterCluster * per_range;
+  __half* w_s = reinterpret_cast<__half*>(smem);                                   // [stages][8 R rows][E]
+  float4* h_s = reinterpret_cast<float4*>(w_s + (size_t)stages * kRouterStageElems);  // [H]: the row's element of the four tokens
+  float* part = reinterpret_cast<float*>(h_s + H);                                 // [R][kRouterStreamTok][E]
+  float* logit = part + (size_t)2048 * kRouterStreamTok;                                 // [kRouterStreamTok][Epad]
+  const int tid = threadIdx.x, m0 = blockIdx.x * kRouterStreamTok, live = min(kRouterStreamTok, M - m0);
+  const int lanes = E / 4, grp = tid / lanes, e0 = (tid % lanes) * 4;
+  int ld_st = 0, ld_at = 0;  // next stage to load and its place in the ring
+  const __half* src = wr;
+  const uint32_t ring = (uint32_t)__cvta_generic_to_shared(w_s);
+  auto load = [&] {
+    if (ld_st < n_st) {
+      const uint32_t dst = ring + (uint32_t)(ld_at * kRouterStageElems * 2);
+#pragma unroll
+      for (int q = 0; q < kRouterStageElems / 8 / kRouterStreamThreads; ++q) {
+        const int c = (tid + q * kRouterStreamThreads) * 8;
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + 2u * c), "l"(src + c) : "memory");
+      }
+      src += kRouterStageElems;
+      ++ld_st;
+      if (++ld_at == stages) ld_at = 0;
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  load();  // (the router matrix does not depend on the preceding kernel)
+  load();
+  if (stages == 4) load();
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  for (int j = tid; j < kRouterStreamTok * (H / 8); j += kRouterStreamThreads) {
+    const int t = j & 3, i = (j >> 2) * 8;
+    const uint4 v = t < live ? *reinterpret_cast<const uint4*>(h + (size_t)(m0 + t) * H + i) : make_uint4(0, 0, 0, 0);
+    const uint32_t vs[4] = {v.x, v.y, v.z, v.w};
+    float* d = reinterpret_cast<float*>(h_s + i) + t;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const float2 f = __half22float2(u32_as_half2(vs[q]));
+      d[8 * q] = f.x;
+      d[8 * q + 4] = f.y;
+    }
+  }
+  for (int j = tid; j < kRouterStreamTok * Epad; j += kRouterStreamThreads) logit[j] = 0.f;
+  float acc[kRouterStreamTok][4];
+  int at = 0, in_range = 0;  // place in the ring, stage of the range
+  const __half* w0 = w_s + (size_t)grp * E + e0;
+  const float4* xr = h_s + grp;
+  for (int st = 0; st < n_st; ++st) {
+    if (stages == 4) asm volatile("cp.async.wait_group 2;" ::: "memory");
+    else asm volatile("cp.async.wait_group 1;" ::: "memory");
+    __syncthreads();  // stage st is there, and everybody has read stage st - 1: its place is free
+    load();
+    if (in_range == 0) {
+#pragma unroll
+      for (int t = 0; t < kRouterStreamTok; ++t)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[t][q] = 0.f;
+    }
+    const __half* w = w0 + at * kRouterStageElems;
+#pragma unroll
+    for (int b = 0; b < kRouterStageRows; ++b) {
+      const float4 x = xr[b * R];
+      const uint2 wv = *reinterpret_cast<const uint2*>(w + b * 2048);
+      const float2 wa = __half22float2(u32_as_half2(wv.x)), wb = __half22float2(u32_as_half2(wv.y));
+      const float xs[kRouterStreamTok] = {x.x, x.y, x.z, x.w}, ws[4] = {wa.x, wa.y, wb.x, wb.y};
+#pragma unroll
+      for (int t = 0; t < kRouterStreamTok; ++t)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[t][q] = fmaf(xs[t], ws[q], acc[t][q]);
+    }
+    xr += kRouterStageRows * R;
+    if (++at == stages) at = 0;
+    if (++in_range == per_range) {  // the range's chains are complete
+      in_range = 0;
+#pragma unroll
+      for (int t = 0; t < kRouterStreamTok; ++t)
+        *reinterpret_cast<float4*>(part + ((size_t)grp * kRouterStreamTok + t) * E + e0) = make_float4(acc[t][0], acc[t][1], acc[t][2], acc[t][3]);
+      __syncthreads();
+      for (int j = tid; j < kRouterStreamTok * E; j += kRouterStreamThreads) {
+        float v = 0.f;
+#pragma unroll 8
+        for (int g = 0; g < R; ++g) v += part[g * kRouterStreamTok * E + j];
+        logit[j] += v;  // (E >= 32 is a power of two: E = Epad)
+      }
+    }
+  }
+  __syncthreads();
+  const int t = tid >> 5;  // one warp per token
+  if (t < live) router_select(logit + t * Epad, m0 + t, E, Epad, k, renorm, ids, gates);
+}
+
 cudaError_t launch_router_topk(const __half* h, const __half* wr, int M, int H, int E, int k, int renorm, int32_t* ids,
                                float* gates, cudaStream_t st, uint64_t* n_launch, int pdl) {
   return launch_router_topk_norm(h, wr, M, H, E, k, renorm, ids, gates, nullptr, 0, nullptr, 0.f, st, n_launch, pdl);
@@ -1317,32 +1422,53 @@ cudaError_t launch_router_topk_norm(const __half* h, const __half* wr, int M, in
     const int L = E / 8, R = kRouterClThreads / L;
     const size_t smem_cl = ((size_t)H / kRouterCluster + (size_t)R * E + (size_t)(kRouterCluster + 1) * Epad) * sizeof(float);
     auto smem_tok = [&](int tok) { return (((size_t)H / kRouterCluster + 4) * tok + (size_t)tok * E) * sizeof(float) + (size_t)H / kRouterCluster * E * 2; };
-    constexpr size_t kMostTok = 227 * 1024 - 1024;
+    auto smem_stream = [&](int stages) {
+      return (size_t)stages * kRouterStageElems * 2 + ((size_t)4 * H + 2048 * kRouterStreamTok + (size_t)kRouterStreamTok * Epad) * sizeof(float);
+    };
+    constexpr size_t kMost = 227 * 1024 - 1024;
+    int tok = 0;
+    // Times in us, fitted to 20 matrices of 56 to 4096 tokens.  A cluster per token:
+    const double size = (double)H * E, Hc = H / kRouterCluster;
+    double best = 0.95 * (4.8 + 3e-6 * size + M * (0.125 + 1.2e-7 * size));
     if (M >= kRouterManyTokens && !norm_gain && E <= 256 && R % 4 == 0) {
-      // Tokens to a cluster: a cluster takes 10 us or, from 18 tokens on (128 experts of 2048), 0.315 more a token; 15 run at a time, and another 17
-      // beside them, in half as much again, where two CTAs fit an SM.
-      int tok = 0;
-      double best = 1e30;
+      // Clusters of t tokens, 15 at a time, and another 17 beside them, in half as much again, where two CTAs fit an SM.  A cluster takes a thread's
+      // way along its range of the rows (two experts to a thread up to 15 clusters, beyond that four), with an addition for each of the R chains, and the more the
+      // more threads there are: 4096 x 16, 56 tokens 17.6 where a cluster per token takes 12.5; 8192 x 16, 128 tokens 24.7 and 22.8.
       for (int t = 8; t <= 64; t += 8) {
-        if (smem_tok(t) > kMostTok) break;
+        if (smem_tok(t) > kMost) break;
         const int c = (M + t - 1) / t;
-        const double us = std::max(10.0, 4.3 + 0.315 * t * ((double)H * E / (2048 * 128)));
-        const double all = us * (c <= 15 ? 1.0 : smem_tok(t) <= kMostTok / 2 ? 1.5 * ((c + 31) / 32) : (double)((c + 14) / 15));
+        const double us = c <= 15 ? 6.0 + 0.0145 * Hc + 0.03 * R + 1.22e-6 * size * (t - 8) : 8.3 + 0.018 * Hc + 0.95e-6 * size * std::max(0, t - 16);
+        const double all = us * (c <= 15 ? 1.0 : smem_tok(t) <= kMost / 2 ? 1.5 * ((c + 31) / 32) : (double)((c + 14) / 15));
         if (all < best) best = all, tok = t;
       }
-      if (tok) {
-        const int clusters = (M + tok - 1) / tok;  // (up to 15 run at once with an SM to each CTA)
-        auto run = [&](auto kernel, int threads) {
-          static std::atomic<uint64_t> attr_done;
-          const cudaError_t e = smem_limit_once(&attr_done, {reinterpret_cast<const void*>(router_topk_tokens_kernel<2, 512>),
-                                                             reinterpret_cast<const void*>(router_topk_tokens_kernel<4, 256>)}, kMostTok);
-          if (e != cudaSuccess) return e;
-          ++*n_launch;
-          return launch_dep(kernel, dim3(clusters * kRouterCluster), dim3(threads), smem_tok(tok), st, pdl, kRouterCluster, h, wr, M, H, E, tok, k,
-                            renorm, ids, gates);
-        };
-        return clusters <= 15 ? run(router_topk_tokens_kernel<2, 512>, 512) : run(router_topk_tokens_kernel<4, 256>, 256);
+    }
+    // Streamed: chains of a multiple of eight rows, 2048 / E of them in each range.  A wave of CTAs takes as long whatever the tokens (2048 x 64 16.5 us,
+    // 2048 x 256 39, 4096 x 256 63, 5120 x 256 75).  Where clusters of tokens are not possible it is as fast as a cluster per token at 113 (1024 x 512) to 137
+    // tokens (2048 x 512), with 256 experts at 180.
+    if (M >= kRouterManyTokens && !norm_gain && E == Epad && 2048 % E == 0 && H / kRouterCluster % (kRouterStageRows * R) == 0 && smem_stream(3) <= kMost) {
+      const double us = (9.0 + 51.5e-6 * size) * ((M + 148 * kRouterStreamTok - 1) / (148 * kRouterStreamTok));
+      if (E > 256 ? M >= 128 : smem_tok(8) > kMost ? M >= 184 : us < best) {
+        const int stages = smem_stream(4) <= kMost ? 4 : 3;
+        static std::atomic<uint64_t> attr_done;
+        const cudaError_t e = smem_limit_once(&attr_done, {reinterpret_cast<const void*>(router_topk_stream_kernel)}, kMost);
+        if (e != cudaSuccess) return e;
+        ++*n_launch;
+        return launch_dep(router_topk_stream_kernel, dim3((M + kRouterStreamTok - 1) / kRouterStreamTok), dim3(kRouterStreamThreads), smem_stream(stages), st,
+                          pdl, 1, h, wr, M, H, E, Epad, k, renorm, stages, ids, gates);
       }
+    }
+    if (tok) {
+      const int clusters = (M + tok - 1) / tok;  // (up to 15 run at once with an SM to each CTA)
+      auto run = [&](auto kernel, int threads) {
+        static std::atomic<uint64_t> attr_done;
+        const cudaError_t e = smem_limit_once(&attr_done, {reinterpret_cast<const void*>(router_topk_tokens_kernel<2, 512>),
+                                                           reinterpret_cast<const void*>(router_topk_tokens_kernel<4, 256>)}, kMost);
+        if (e != cudaSuccess) return e;
+        ++*n_launch;
+        return launch_dep(kernel, dim3(clusters * kRouterCluster), dim3(threads), smem_tok(tok), st, pdl, kRouterCluster, h, wr, M, H, E, tok, k,
+                          renorm, ids, gates);
+      };
+      return clusters <= 15 ? run(router_topk_tokens_kernel<2, 512>, 512) : run(router_topk_tokens_kernel<4, 256>, 256);
     }
     constexpr size_t kMostCl = 160 * 1024;
     if (smem_cl <= kMostCl) {

@@ -35,3 +35,41 @@ def test_router_of_many_tokens_has_the_bits_of_the_router_of_few(hidden, E, k, M
     assert torch.equal(ids, torch.cat([p[0] for p in parts]))
     assert torch.equal(gates, torch.cat([p[1] for p in parts]))
     ctx.close()
+
+
+# The streamed form: matrices whose eighth does not fit beside the tokens (256 experts of 4096 and 5120, 512, 1024) or leaves room for too few (128 of
+# 4096), the fewest tokens it takes and one less, a last CTA of one to three tokens, two waves.
+@pytest.mark.parametrize("hidden,E,k,M", [(2048, 512, 8, 128), (2048, 512, 8, 127), (1024, 1024, 32, 131), (4096, 256, 8, 186), (4096, 256, 8, 183), (5120, 256, 8, 613),
+                                          (4096, 128, 8, 511)])
+def test_streamed_router_has_the_bits_of_the_router_of_few(hidden, E, k, M):
+    test_router_of_many_tokens_has_the_bits_of_the_router_of_few(hidden, E, k, M)
+
+
+# A wave of the streamed form takes as long for 512 tokens as for 200 (25 % are left for noise), a cluster per token more than twice as long.
+@pytest.mark.parametrize("hidden,E", [(2048, 512), (1024, 1024), (4096, 256), (5120, 256)])
+def test_a_wave_of_the_streamed_router_takes_as_long_whatever_the_tokens(hidden, E):
+    import torch
+    from paper_2607_10183_b200 import binding as B
+    rng = np.random.default_rng(5)
+    ctx = B.Context(4 * hidden * E + (8 << 20), workspace_bytes=1 << 20)
+    rid = ctx.register_f16((rng.standard_normal((hidden, E)) * 0.02).astype(np.float16))
+    ctx.set_placement([])
+    times = []
+    for M in (200, 512):
+        h = H.to_dev(rng.standard_normal((M, hidden)).astype(np.float16))
+        ids = torch.empty((M, 8), dtype=torch.int32, device="cuda")
+        gates = torch.empty((M, 8), dtype=torch.float32, device="cuda")
+        torch.cuda.synchronize()
+        passes = []
+        for _ in range(12):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record(ctx.compute)
+            for _ in range(10):
+                ctx.route_topk(rid, h, M, 8, ids, gates)
+            b.record(ctx.compute)
+            b.synchronize()
+            passes.append(a.elapsed_time(b) * 100)
+        times.append(sorted(passes[2:])[5])
+    ctx.close()
+    print(f"{hidden} x {E}: {times[0]:.1f} us for 200 tokens, {times[1]:.1f} for 512")
+    assert times[1] <= 1.25 * times[0]
