@@ -1029,6 +1029,9 @@ __device__ __forceinline__ void st_cluster_f32(const float* local_smem_ptr, uint
 // Optional RMSNorm prologue (gain != null): the token's row is xn (fp16 or fp32), every CTA of the cluster sums its
 // squares itself (the whole row is a few kilobytes), normalises its own eighth, h = rn16(x * g / sqrt(mean(x^2) + eps)),
 // uses it and writes it to h_out for the expert kernels that follow.
+// MANY: more than 256 experts.  Their few row groups (2 to 7) are not unrolled and multiply-adds are not paired (paired, 1024 experts of 1024, a token:
+// 35.1 -> 36.8 us, 512 of 2048, 32 tokens 28.0 -> 28.6; up to 256 experts it is the other way round).
+template <bool MANY>
 __global__ void __launch_bounds__(kRouterClThreads) router_topk_cluster_kernel(const __half* __restrict__ h,
                                                                                const __half* __restrict__ wr, int H, int E, int Epad,
                                                                                int k, int renorm, int32_t* __restrict__ ids,
@@ -1124,7 +1127,10 @@ __global__ void __launch_bounds__(kRouterClThreads) router_topk_cluster_kernel(c
         const float x = i < Hc ? h_s[i] : 0.f;
         const uint32_t ws[4] = {w[b].x, w[b].y, w[b].z, w[b].w};
 #pragma unroll
-        for (int q = 0; q < 4; ++q) acc[q] = fma_x2(make_float2(x, x), __half22float2(u32_as_half2(ws[q])), acc[q]);
+        for (int q = 0; q < 4; ++q) {
+          const float2 f = __half22float2(u32_as_half2(ws[q]));
+          acc[q] = MANY ? make_float2(fmaf(x, f.x, acc[q].x), fmaf(x, f.y, acc[q].y)) : fma_x2(make_float2(x, x), f, acc[q]);
+        }
       }
     }
 #pragma unroll
@@ -1134,14 +1140,14 @@ __global__ void __launch_bounds__(kRouterClThreads) router_topk_cluster_kernel(c
   for (int e = threadIdx.x; e < Epad; e += kRouterClThreads) {
     float t = 0.f;
     if (e < E) {
-#pragma unroll 8
+#pragma unroll (MANY ? 1 : 8)
       for (int g = 0; g < R; ++g) t += part[(size_t)g * E + e];
     }
     st_cluster_f32(cl + (size_t)rank * Epad + e, 0, t);  // into CTA 0's copy of cl
   }
   cluster_sync_all();
   if (rank != 0) return;
-  if (E <= 256) {  // one warp
+  if constexpr (!MANY) {  // one warp
     if (threadIdx.x >= 32) return;
     auto select = [&](auto per) {
       float v[decltype(per)::value];
@@ -1473,10 +1479,11 @@ cudaError_t launch_router_topk_norm(const __half* h, const __half* wr, int M, in
     constexpr size_t kMostCl = 160 * 1024;
     if (smem_cl <= kMostCl) {
       static std::atomic<uint64_t> attr_done;
-      const cudaError_t e = smem_limit_once(&attr_done, {reinterpret_cast<const void*>(router_topk_cluster_kernel)}, kMostCl);
+      const cudaError_t e = smem_limit_once(&attr_done, {reinterpret_cast<const void*>(router_topk_cluster_kernel<false>),
+                                                         reinterpret_cast<const void*>(router_topk_cluster_kernel<true>)}, kMostCl);
       if (e != cudaSuccess) return e;
       ++*n_launch;
-      return launch_dep(router_topk_cluster_kernel, dim3(kRouterCluster, M), dim3(kRouterClThreads), smem_cl, st, pdl, kRouterCluster,
+      return launch_dep(E > 256 ? router_topk_cluster_kernel<true> : router_topk_cluster_kernel<false>, dim3(kRouterCluster, M), dim3(kRouterClThreads), smem_cl, st, pdl, kRouterCluster,
                         h, wr, H, E, Epad, k, renorm, ids, gates, norm_x, norm_x_f32, norm_gain, eps, const_cast<__half*>(h));
     }
   }
