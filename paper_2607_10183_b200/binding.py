@@ -23,6 +23,8 @@ ATS_OUT_F32, ATS_OUT_F16 = 0, 1
 ATS_MODE_DECODE, ATS_MODE_PREFILL = 0, 1
 ATS_FLAG_POISON_SLOTS, ATS_FLAG_SKIP_SCALE_CHECK, ATS_FLAG_TIME_KERNELS, ATS_FLAG_NO_PDL, ATS_FLAG_MOE_RING_ONLY = 1, 2, 4, 8, 16
 ATS_FLAG_NO_GEMM_PAIR = 32
+ATS_FLAG_NO_GEMM_FEW = 64
+ATS_GEMM_PLAIN, ATS_GEMM_PAIRS, ATS_GEMM_FEW = 0, 1, 2
 ATS_LAYER_NO_TOPK_RENORM = 1
 ATS_STATS_LIST = 512
 EDGES = ("h", "q", "k", "v", "q_rot", "a", "o", "x1", "h2", "g", "u", "act", "d")
@@ -32,7 +34,7 @@ EXPORTS = (
     "ats_plan_placement", "ats_get_placement", "ats_linear", "ats_linear_static_scratch", "ats_route_topk", "ats_moe_linear", "ats_layer_decode", "ats_layer_decode_host", "ats_embed", "ats_lm_head",
     "ats_layer_prefill", "ats_workspace_bytes", "ats_dequantize", "ats_get_numerics", "ats_get_stats", "ats_set_flags", "ats_reset_stats",
     "ats_sync", "ats_measure_h2d", "ats_measure_hbm_read", "ats_debug_fail_copies", "ats_debug_gemv_wait", "ats_debug_skip_stages", "ats_register_host_buffer", "ats_unregister_host_buffer", "ats_debug_decode_buffer", "ats_debug_prefill_buffer", "ats_host_solve_placement", "ats_host_repack_q4",
-    "ats_host_unpack_q4", "ats_host_group_pairs", "ats_host_dynamic_transfer", "ats_host_transfer_latency", "ats_host_deviation",
+    "ats_host_unpack_q4", "ats_host_group_pairs", "ats_host_gemm_kernel", "ats_host_dynamic_transfer", "ats_host_transfer_latency", "ats_host_deviation",
     "ats_host_reschedule", "ats_profile_tensor", "ats_set_tensor_value",
 )
 
@@ -107,6 +109,7 @@ def _load():
         "ats_host_repack_q4": (i32, [vp, vp, vp, u32, u32]),
         "ats_host_unpack_q4": (i32, [vp, vp, vp, u32, u32]),
         "ats_host_group_pairs": (i32, [vp, u32, u32, vp, vp, vp, vp]),
+        "ats_host_gemm_kernel": (i32, [u32, u32, u32, u32, u32, u64, u32, P(i32), P(u32)]),
         "ats_profile_tensor": (i32, [vp, i32, vp, vp, u32, u32, P(C.c_double), P(C.c_double)]),
         "ats_set_tensor_value": (i32, [vp, i32, C.c_int64, C.c_int64]),
         "ats_host_dynamic_transfer": (i32, [vp, vp, vp, vp, vp, u32, vp, vp, P(C.c_double)]),
@@ -377,6 +380,15 @@ def host_group_pairs(ids, E):
 
 
 ATS_ROUND_START, ATS_NO_TRANSFER = -1, -2
+
+
+def host_gemm_kernel(fmt, n_out, k_in, T, flags=0, scratch_bytes=1 << 40, sm_count=148):
+    """(kernel, longest chain of k) of a prompt product of T rows."""
+    kernel, chain = C.c_int32(), C.c_uint32()
+    st = lib.ats_host_gemm_kernel(fmt, n_out, k_in, T, flags, scratch_bytes, sm_count, C.byref(kernel), C.byref(chain))
+    if st != ATS_OK:
+        raise AtsError(st, "no prompt product")
+    return kernel.value, chain.value
 
 
 def _f64(a):

@@ -380,7 +380,7 @@ struct GemmParams {
   int grp_max_rows;         // the largest expert's row count (sizes the grid)
   uint64_t grp_stride;
   const uint8_t* const* grp_tab[3];
-  // optional fused SwiGLU (launch_gemm_pair only): act[t][f] = rn16(silu(y[t][f]) * y[t][n_rows + f]) of segments gate, up;
+  // optional fused SwiGLU (launch_gemm_pair and launch_gemm_few): act[t][f] = rn16(silu(y[t][f]) * y[t][n_rows + f]) of segments gate, up;
   // y itself is written only where it is not null
   __half* act;
   int ldact;
@@ -394,6 +394,7 @@ struct GemmPairPlan {
   uint64_t scratch;
 };
 bool gemm_pair_eligible(const GemmParams& p, int sm_count, GemmPairPlan* plan);
+int gemm_pair_chain(const GemmParams& p, const GemmPairPlan& plan);  // the k that an accumulator adds up at most (not grouped)
 // the one of these two kernels that would take the product with all the scratch it wants: its time, and the k that it adds up in one accumulator
 struct GemmOther {
   double us;
@@ -407,6 +408,7 @@ struct GemmFewPlan {
   double us;
 };
 bool gemm_few_eligible(const GemmParams& p, int sm_count, GemmFewPlan* plan);
+int gemm_few_chain(const GemmParams& p, const GemmFewPlan& plan);
 cudaError_t launch_gemm_few(const GemmParams& p, const GemmFewPlan& plan, int sm_count, cudaStream_t st, uint64_t* n_launch, std::string* err);
 // the single-CTA kernel: scratch of its plan, the k that the plan adds up in one accumulator, its time
 uint64_t gemm_scratch_bytes(int T, int n_total, int K);

@@ -323,21 +323,27 @@ static int32_t run_gemv_group(ats_ctx* ctx, Operand* ops, int n, GemvParams p) {
   return ATS_OK;
 }
 
-// One GEMM launch: on the kernel for few tokens, on pairs of CTAs, or on the kernel of plain tiles (slice address tables).  Under
-// ATS_FLAG_NO_GEMM_PAIR nothing runs on pairs, and the grouped form (which the host has sorted then) on plain tiles.  A SwiGLU that was
-// asked for runs in the epilogue or as a launch of its own.
+// Which kernel takes a GEMM: the one for few tokens, pairs of CTAs, or plain tiles (slice address tables).  Under ATS_FLAG_NO_GEMM_PAIR nothing runs on
+// pairs, and the grouped form (which the host has sorted then) on plain tiles; under ATS_FLAG_NO_GEMM_FEW nothing on the first.
+static int choose_gemm(const GemmParams& p, uint32_t flags, int sm_count, GemmFewPlan* few, GemmPairPlan* pair) {
+  const bool pairs = !(flags & ATS_FLAG_NO_GEMM_PAIR);
+  if (!(flags & ATS_FLAG_NO_GEMM_FEW) && (pairs || !p.grp_off) && gemm_few_eligible(p, sm_count, few)) return ATS_GEMM_FEW;
+  return pairs && gemm_pair_eligible(p, sm_count, pair) ? ATS_GEMM_PAIRS : ATS_GEMM_PLAIN;
+}
+
+// One GEMM launch.  A SwiGLU that was asked for runs in the epilogue or as a launch of its own.
 static int32_t launch_gemm_any(ats_ctx* ctx, GemmParams p) {
   std::string err;
   cudaError_t e;
   __half* act = p.act;
   p.counters = reinterpret_cast<int*>(ctx->ws) + 64;  // (the attention's: zero between launches, and launches follow one another)
-  const bool pairs = !(ctx->cfg.flags & ATS_FLAG_NO_GEMM_PAIR);
   GemmPairPlan plan{};
   GemmFewPlan few{};
-  if ((pairs || !p.grp_off) && gemm_few_eligible(p, ctx->sm_count, &few)) {
+  const int kernel = choose_gemm(p, ctx->cfg.flags, ctx->sm_count, &few, &plan);
+  if (kernel == ATS_GEMM_FEW) {
     e = launch_gemm_few(p, few, ctx->sm_count, ctx->cs, &ctx->stats.kernel_launches, &err);
     act = nullptr;
-  } else if (pairs && gemm_pair_eligible(p, ctx->sm_count, &plan)) {
+  } else if (kernel == ATS_GEMM_PAIRS) {
     e = launch_gemm_pair(p, plan, ctx->sm_count, ctx->cs, &ctx->stats.kernel_launches, &err);
     act = nullptr;
   } else {
@@ -1272,6 +1278,35 @@ int32_t ats_dequantize(ats_ctx* ctx, int32_t id, int32_t expert, void* out_dev, 
   ATS_CUDA(launch_dequant(ptr, (int)t->d.n_out, (int)t->d.k_in, out_dev, out_fmt == ATS_OUT_F16, t->d.fmt == ATS_FMT_MXFP4, ctx->cs,
                           &ctx->stats.kernel_launches));
   if (f >= 0) ATS_TRY(release(ctx, f));
+  return ATS_OK;
+}
+
+int32_t ats_host_gemm_kernel(uint32_t fmt, uint32_t n_out, uint32_t k_in, uint32_t T, uint32_t flags, uint64_t scratch_bytes, uint32_t sm_count,
+                             int32_t* kernel, uint32_t* chain_k) {
+  const bool w16 = fmt == ATS_FMT_W16;
+  if (!kernel || (!w16 && fmt != ATS_FMT_Q4B32 && fmt != ATS_FMT_MXFP4)) return ATS_ERR_INVALID;
+  if (T <= 8 || T > 1u << 22 || n_out == 0 || n_out > 1u << 24 || k_in == 0 || k_in > 1u << 24 || k_in % (w16 ? 8 : 32) || sm_count == 0 || sm_count > 1024)
+    return ATS_ERR_SHAPE;
+  GemmParams p{};
+  uint8_t* const aligned = reinterpret_cast<uint8_t*>(16);
+  p.n_seg = 1;
+  p.seg[0] = GemvSeg{aligned, (int)n_out};
+  p.K = p.ldx = (int)k_in;
+  p.T = (int)T;
+  p.x = reinterpret_cast<const __half*>(aligned);
+  p.y = reinterpret_cast<__half*>(aligned);
+  p.ldy = (int)n_out;
+  p.w16 = w16;
+  p.mx = fmt == ATS_FMT_MXFP4;
+  p.scratch = scratch_bytes ? aligned : nullptr;
+  p.scratch_bytes = scratch_bytes;
+  p.counters = reinterpret_cast<int*>(aligned);
+  GemmFewPlan few{};
+  GemmPairPlan pair{};
+  *kernel = choose_gemm(p, flags, (int)sm_count, &few, &pair);
+  const int rows = (int)n_out;
+  if (chain_k)
+    *chain_k = (uint32_t)(*kernel == ATS_GEMM_FEW ? gemm_few_chain(p, few) : *kernel == ATS_GEMM_PAIRS ? gemm_pair_chain(p, pair) : gemm_chain(&rows, 1, p.T, p.K));
   return ATS_OK;
 }
 

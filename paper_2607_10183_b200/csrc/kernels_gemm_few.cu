@@ -851,6 +851,13 @@ GemmFewPlan plan_of(const GemmParams& g, int sm_count, int limit) {
 
 }  // namespace
 
+int gemm_few_chain(const GemmParams& g, const GemmFewPlan& pl) {
+  const int units = (g.K + kUnitK - 1) / kUnitK, per = (units + pl.parts - 1) / pl.parts, steps = pl.mode == kDeep ? 1 : 2;  // (of 128 k, a unit)
+  int n = per;
+  if (n > pl.max_units) n = (n + (n - 1) / pl.max_units) / ((n + pl.max_units - 1) / pl.max_units);
+  return std::min(g.K, (n * steps + pl.turns - 1) / pl.turns * 128);
+}
+
 bool gemm_few_eligible(const GemmParams& g, int sm_count, GemmFewPlan* plan) {
   if (g.w16 || g.n_seg < 1 || g.n_seg > 3 || g.K % 32 || g.K > (1 << 24) || g.ldx % 8) return false;
   if (reinterpret_cast<uintptr_t>(g.x) & 15) return false;

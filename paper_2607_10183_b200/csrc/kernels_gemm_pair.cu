@@ -955,20 +955,26 @@ bool gemm_pair_eligible(const GemmParams& g, int sm_count, GemmPairPlan* plan) {
   return pl.pairs > 0 && pl.us <= single;
 }
 
-GemmOther gemm_other(const GemmParams& g, int sm_count) {
-  GemmParams all = g;
-  all.scratch = reinterpret_cast<void*>(16);
-  all.scratch_bytes = ~0ull;
+int gemm_pair_chain(const GemmParams& g, const GemmPairPlan& pl) {
   int rows[3] = {0, 0, 0}, n_ft = 0;
   for (int i = 0; i < g.n_seg; ++i) rows[i] = g.seg[i].n_rows;
-  GemmPairPlan pl{};
-  if (!gemm_pair_eligible(all, sm_count, &pl)) return GemmOther{single_cta_us(g), gemm_chain(rows, g.n_seg, g.T, g.K)};
   for (int i = 0; i < g.n_seg; ++i) n_ft += feature_tiles(rows, i, g.act != nullptr);
   const int units = (g.K + kUnitK - 1) / kUnitK, split = n_ft * pl.n_tt - pl.n_whole;
   auto chain = [&](int n) { return !pl.own || n <= pl.max_units ? n : (n + (n - 1) / pl.max_units) / ((n + pl.max_units - 1) / pl.max_units); };
   int most = pl.n_whole ? chain(units) : 1;
   if (split) most = std::max(most, chain(std::min(units, (int)(((long long)split * units + pl.split_pairs - 1) / pl.split_pairs))));
-  return GemmOther{pl.us, std::min(g.K, most * kUnitK)};
+  return std::min(g.K, most * kUnitK);
+}
+
+GemmOther gemm_other(const GemmParams& g, int sm_count) {
+  GemmParams all = g;
+  all.scratch = reinterpret_cast<void*>(16);
+  all.scratch_bytes = ~0ull;
+  int rows[3] = {0, 0, 0};
+  for (int i = 0; i < g.n_seg; ++i) rows[i] = g.seg[i].n_rows;
+  GemmPairPlan pl{};
+  if (!gemm_pair_eligible(all, sm_count, &pl)) return GemmOther{single_cta_us(g), gemm_chain(rows, g.n_seg, g.T, g.K)};
+  return GemmOther{pl.us, gemm_pair_chain(g, pl)};
 }
 
 cudaError_t launch_gemm_pair(const GemmParams& g, const GemmPairPlan& pl, int sm_count, cudaStream_t st, uint64_t* n_launch, std::string* err) {
