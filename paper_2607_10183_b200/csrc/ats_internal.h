@@ -395,19 +395,20 @@ struct GemmPairPlan {
 };
 bool gemm_pair_eligible(const GemmParams& p, int sm_count, GemmPairPlan* plan);
 int gemm_pair_chain(const GemmParams& p, const GemmPairPlan& plan);  // the k that an accumulator adds up at most (not grouped)
-// the one of these two kernels that would take the product with all the scratch it wants: its time, and the k that it adds up in one accumulator
+// the one of these two kernels (without `pairs`, the single-CTA kernel) that would take the product with all the scratch it wants: its time, and the k that it
+// adds up in one accumulator
 struct GemmOther {
   double us;
   int chain;
 };
-GemmOther gemm_other(const GemmParams& p, int sm_count);
+GemmOther gemm_other(const GemmParams& p, int sm_count, bool pairs);
 cudaError_t launch_gemm_pair(const GemmParams& p, const GemmPairPlan& plan, int sm_count, cudaStream_t st, uint64_t* n_launch, std::string* err);
 // GEMMs of few tokens, 4-bit formats, on single CTAs (kernels_gemm_few.cu)
 struct GemmFewPlan {
   int mode, nt, n_tt, n_ft, parts, turns, max_units;
   double us;
 };
-bool gemm_few_eligible(const GemmParams& p, int sm_count, GemmFewPlan* plan);
+bool gemm_few_eligible(const GemmParams& p, int sm_count, bool pairs, GemmFewPlan* plan);  // (pairs: they may take it otherwise)
 int gemm_few_chain(const GemmParams& p, const GemmFewPlan& plan);
 cudaError_t launch_gemm_few(const GemmParams& p, const GemmFewPlan& plan, int sm_count, cudaStream_t st, uint64_t* n_launch, std::string* err);
 // the single-CTA kernel: scratch of its plan, the k that the plan adds up in one accumulator, its time

@@ -327,7 +327,7 @@ static int32_t run_gemv_group(ats_ctx* ctx, Operand* ops, int n, GemvParams p) {
 // pairs, and the grouped form (which the host has sorted then) on plain tiles; under ATS_FLAG_NO_GEMM_FEW nothing on the first.
 static int choose_gemm(const GemmParams& p, uint32_t flags, int sm_count, GemmFewPlan* few, GemmPairPlan* pair) {
   const bool pairs = !(flags & ATS_FLAG_NO_GEMM_PAIR);
-  if (!(flags & ATS_FLAG_NO_GEMM_FEW) && (pairs || !p.grp_off) && gemm_few_eligible(p, sm_count, few)) return ATS_GEMM_FEW;
+  if (!(flags & ATS_FLAG_NO_GEMM_FEW) && (pairs || !p.grp_off) && gemm_few_eligible(p, sm_count, pairs, few)) return ATS_GEMM_FEW;
   return pairs && gemm_pair_eligible(p, sm_count, pair) ? ATS_GEMM_PAIRS : ATS_GEMM_PLAIN;
 }
 

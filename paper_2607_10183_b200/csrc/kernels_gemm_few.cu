@@ -858,7 +858,7 @@ int gemm_few_chain(const GemmParams& g, const GemmFewPlan& pl) {
   return std::min(g.K, (n * steps + pl.turns - 1) / pl.turns * 128);
 }
 
-bool gemm_few_eligible(const GemmParams& g, int sm_count, GemmFewPlan* plan) {
+bool gemm_few_eligible(const GemmParams& g, int sm_count, bool pairs, GemmFewPlan* plan) {
   if (g.w16 || g.n_seg < 1 || g.n_seg > 3 || g.K % 32 || g.K > (1 << 24) || g.ldx % 8) return false;
   if (reinterpret_cast<uintptr_t>(g.x) & 15) return false;
   if ((g.res != nullptr) != (g.y2 != nullptr)) return false;
@@ -873,7 +873,7 @@ bool gemm_few_eligible(const GemmParams& g, int sm_count, GemmFewPlan* plan) {
   // 94 -> 88; 1500 through 4 of 64, 94 rows, 218 -> 217; 2048 through 8 of 128, 128 rows, 346 -> 366)
   if (g.grp_off) return g.n_groups > 0 && g.T <= 80 * g.n_groups && (g.n_seg == 1 || g.act) && g.grp_stride % 16 == 0 && !g.res;
   // (against the best of all ways and kernels the choice loses 1.5 %: both models are off by about 5 %)
-  const GemmOther other = gemm_other(g, sm_count);
+  const GemmOther other = gemm_other(g, sm_count, pairs);
   const GemmFewPlan pl = *plan = plan_of(g, sm_count, other.chain);
   return pl.parts && pl.us <= 0.96 * other.us;
 }

@@ -966,14 +966,14 @@ int gemm_pair_chain(const GemmParams& g, const GemmPairPlan& pl) {
   return std::min(g.K, most * kUnitK);
 }
 
-GemmOther gemm_other(const GemmParams& g, int sm_count) {
+GemmOther gemm_other(const GemmParams& g, int sm_count, bool pairs) {
   GemmParams all = g;
   all.scratch = reinterpret_cast<void*>(16);
   all.scratch_bytes = ~0ull;
   int rows[3] = {0, 0, 0};
   for (int i = 0; i < g.n_seg; ++i) rows[i] = g.seg[i].n_rows;
   GemmPairPlan pl{};
-  if (!gemm_pair_eligible(all, sm_count, &pl)) return GemmOther{single_cta_us(g), gemm_chain(rows, g.n_seg, g.T, g.K)};
+  if (!pairs || !gemm_pair_eligible(all, sm_count, &pl)) return GemmOther{single_cta_us(g), gemm_chain(rows, g.n_seg, g.T, g.K)};
   return GemmOther{pl.us, gemm_pair_chain(g, pl)};
 }
 

@@ -60,3 +60,21 @@ def test_flags_and_sizes():
             B.host_gemm_kernel(B.ATS_FMT_Q4B32, *bad)
     with pytest.raises(B.AtsError):
         B.host_gemm_kernel(B.ATS_FMT_F16, 4096, 4096, 9)
+
+
+def test_without_pairs_the_kernel_for_few_tokens_is_compared_with_plain_tiles():
+    """Its chains are no longer than theirs (a unit of 256 k at least), and it takes what it is faster at than they are."""
+    import random
+    B = _binding()
+    rng = random.Random(3)
+    taken = 0
+    for _ in range(3000):
+        n, k, T = int(2 ** rng.uniform(0, 14.8)), 32 * int(2 ** rng.uniform(0, 9)), int(2 ** rng.uniform(3.3, 12))
+        fmt = rng.choice([B.ATS_FMT_Q4B32, B.ATS_FMT_MXFP4])
+        kernel, chain = B.host_gemm_kernel(fmt, n, k, T, B.ATS_FLAG_NO_GEMM_PAIR)
+        if kernel == B.ATS_GEMM_FEW:
+            taken += 1
+            assert chain <= max(256, B.host_gemm_kernel(fmt, n, k, T, B.ATS_FLAG_NO_GEMM_PAIR | B.ATS_FLAG_NO_GEMM_FEW)[1]), (n, k, T)
+    assert taken > 2000
+    for fmt, n, k, T in ((B.ATS_FMT_Q4B32, 13392, 4896, 1391), (B.ATS_FMT_MXFP4, 5983, 13344, 114), (B.ATS_FMT_MXFP4, 11047, 11968, 174)):
+        assert B.host_gemm_kernel(fmt, n, k, T, B.ATS_FLAG_NO_GEMM_PAIR)[0] == B.ATS_GEMM_FEW
