@@ -307,10 +307,10 @@ int attn_decode_splits(int n_ctx);
 size_t attn_decode_scratch_floats(int n_q, int d, int n_ctx);
 cudaError_t launch_attn_decode_fused(AttnDecodeParams p, int d, int pdl, cudaStream_t st, uint64_t* n_launch);
 cudaError_t launch_router_topk(const __half* h, const __half* wr, int M, int H, int E, int k, int renorm, int32_t* ids,
-                               float* gates, cudaStream_t st, uint64_t* n_launch, int pdl = 0);
+                               float* gates, int sm_count, cudaStream_t st, uint64_t* n_launch, int pdl = 0);
 cudaError_t launch_router_topk_norm(const __half* h, const __half* wr, int M, int H, int E, int k, int renorm, int32_t* ids,
                                     float* gates, const void* norm_x, int norm_x_f32, const __half* norm_gain, float eps,
-                                    cudaStream_t st, uint64_t* n_launch, int pdl = 0);
+                                    int sm_count, cudaStream_t st, uint64_t* n_launch, int pdl = 0);
 // y16[m] = rn16(res[m] + sum_j gates[m][j] * d32[m*k + j])   (res fp16 or fp32)
 cudaError_t launch_moe_combine(const void* res, int res_is_f32, const float* gates, const float* d32, __half* y16,
                                int M, int k, int H, cudaStream_t st, uint64_t* n_launch, int pdl = 0);
@@ -330,7 +330,7 @@ cudaError_t launch_attn_prefill(const __half* q_rot16, const __half* kc, const _
 // the same on tcgen05 (kernels_attn_prefill.cu): chunks and buffers it takes, and its launcher
 bool attn_prefill_tc_eligible(const __half* q_rot16, const __half* kc, const __half* vc, const __half* a16, int T, int d);
 cudaError_t launch_attn_prefill_tc(const __half* q_rot16, const __half* kc, const __half* vc, __half* a16, int T, int n_q, int n_kv, int d,
-                                   int cap, int pos0, int* status, cudaStream_t st, uint64_t* n_launch, int pdl = 0);
+                                   int cap, int pos0, int* status, int sm_count, cudaStream_t st, uint64_t* n_launch, int pdl = 0);
 // MoE prefill helpers (kernels_prefill.cu): rows gathered in expert order, and the gated sum back in token order
 cudaError_t launch_moe_sort_gather(const int32_t* ids, int P, int E, int k, int H, const __half* h, int* order, int* pos, int* off, __half* xs,
                                    int* status, int* done, int seq, int sm_count, cudaStream_t st, uint64_t* n_launch, int pdl);
@@ -405,7 +405,7 @@ GemmOther gemm_other(const GemmParams& p, int sm_count, bool pairs);
 cudaError_t launch_gemm_pair(const GemmParams& p, const GemmPairPlan& plan, int sm_count, cudaStream_t st, uint64_t* n_launch, std::string* err);
 // GEMMs of few tokens, 4-bit formats, on single CTAs (kernels_gemm_few.cu)
 struct GemmFewPlan {
-  int mode, nt, n_tt, n_ft, parts, turns, max_units;
+  int mode, nt, n_tt, parts, turns, max_units;
   double us;
 };
 bool gemm_few_eligible(const GemmParams& p, int sm_count, bool pairs, GemmFewPlan* plan);  // (pairs: they may take it otherwise)

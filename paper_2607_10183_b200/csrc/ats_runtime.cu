@@ -1320,7 +1320,7 @@ int32_t ats_route_topk(ats_ctx* ctx, int32_t router_id, const void* h, uint32_t 
   if (k == 0 || k > 32 || k > E || E > 1024) return fail(ctx, ATS_ERR_SHAPE, "top-k %u of %u experts unsupported", k, E);
   if (M == 0) return ATS_OK;
   ATS_CUDA(launch_router_topk((const __half*)h, (const __half*)t->f16_dev, (int)M, (int)t->d.k_in, (int)E, (int)k, 1,
-                              ids_dev, gates_dev, ctx->cs, &ctx->stats.kernel_launches));
+                              ids_dev, gates_dev, ctx->sm_count, ctx->cs, &ctx->stats.kernel_launches));
   return ATS_OK;
 }
 
@@ -1532,7 +1532,7 @@ int32_t ats_layer_decode(ats_ctx* ctx, const ats_layer_desc* L, const void* x_in
   if (!(mskip & 32))
     ATS_CUDA(launch_router_topk_norm(w.h2_16, (const __half*)ctx->tensors[L->router].f16_dev, (int)M, H, E, k,
                                      (L->flags & ATS_LAYER_NO_TOPK_RENORM) ? 0 : 1, w.ids, w.gates, attn ? (const void*)w.x1_32 : x_in,
-                                     attn ? 1 : 0, (const __half*)ctx->tensors[L->ffn_norm].f16_dev, L->rms_eps, ctx->cs, nl, pdl));
+                                     attn ? 1 : 0, (const __half*)ctx->tensors[L->ffn_norm].f16_dev, L->rms_eps, ctx->sm_count, ctx->cs, nl, pdl));
   const Tensor &tg = ctx->tensors[L->w_gate], &tu = ctx->tensors[L->w_up], &td = ctx->tensors[L->w_down];
   bool implicit = tg.contiguous_dev && tu.contiguous_dev && td.contiguous_dev;
   if (!implicit && M == 1 && !(ctx->cfg.flags & ATS_FLAG_MOE_RING_ONLY) && tg.slice_tab_dev && tu.slice_tab_dev && td.slice_tab_dev) {
@@ -1766,7 +1766,7 @@ int32_t ats_layer_prefill(ats_ctx* ctx, const ats_layer_desc* L, const void* x_i
                                         (int)L->kv_capacity, (int)pos0, rope_freq(ctx, L->rope_theta, d), ctx->cs, nl, pdl));
     if (attn_prefill_tc_eligible(w.qrot16, (const __half*)k_cache, (const __half*)v_cache, w.a16, (int)T, d))
       ATS_CUDA(launch_attn_prefill_tc(w.qrot16, (const __half*)k_cache, (const __half*)v_cache, w.a16, (int)T, nq, nkv, d,
-                                      (int)L->kv_capacity, (int)pos0, ctx->dev_status, ctx->cs, nl, pdl));
+                                      (int)L->kv_capacity, (int)pos0, ctx->dev_status, ctx->sm_count, ctx->cs, nl, pdl));
     else
       ATS_CUDA(launch_attn_prefill(w.qrot16, (const __half*)k_cache, (const __half*)v_cache, w.a16, (int)T, nq, nkv, d,
                                    (int)L->kv_capacity, (int)pos0, ctx->cs, nl, pdl));
@@ -1800,7 +1800,7 @@ int32_t ats_layer_prefill(ats_ctx* ctx, const ats_layer_desc* L, const void* x_i
       if (capturing != cudaStreamCaptureStatusNone) ATS_CUDA(cudaErrorStreamCaptureUnsupported);
     }
     ATS_CUDA(launch_router_topk(w.h2_16, (const __half*)ctx->tensors[L->router].f16_dev, (int)T, H, E, k,
-                                (L->flags & ATS_LAYER_NO_TOPK_RENORM) ? 0 : 1, w.ids, w.gates, ctx->cs, nl, pdl));
+                                (L->flags & ATS_LAYER_NO_TOPK_RENORM) ? 0 : 1, w.ids, w.gates, ctx->sm_count, ctx->cs, nl, pdl));
     // the sort's arrays, laid out as the workspace has them, so that one copy takes all three
     int32_t* order_h = ctx->ids_host + kMaxPairs;              // sorted position -> pair
     int32_t* pos_h = order_h + (w.pos - w.order);              // pair -> sorted position

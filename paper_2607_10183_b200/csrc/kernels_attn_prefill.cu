@@ -394,7 +394,7 @@ bool attn_prefill_tc_eligible(const __half* q_rot16, const __half* kc, const __h
 }
 
 cudaError_t launch_attn_prefill_tc(const __half* q_rot16, const __half* kc, const __half* vc, __half* a16, int T, int n_q, int n_kv, int d,
-                                   int cap, int pos0, int* status, cudaStream_t st, uint64_t* n_launch, int pdl) {
+                                   int cap, int pos0, int* status, int sm_count, cudaStream_t st, uint64_t* n_launch, int pdl) {
   // rows beyond the context (and query rows beyond T) read as zeros: the cache may hold anything there
   CUtensorMap qm, km, vm;
   const uint64_t row = (uint64_t)d * 2;
@@ -411,7 +411,7 @@ cudaError_t launch_attn_prefill_tc(const __half* q_rot16, const __half* kc, cons
   // One tile to a CTA, its key blocks in two, where all such CTAs run at once and there are blocks enough for the merge (2 us) to pay.  Layers of 4096,
   // 130 tokens after 2000: 152.9 -> 139.2 us, 300 after 1500 184.5 -> 175.1; of 2048, 1000 after 300: 143.0 -> 131.9; 700 tokens of 24 heads of 64
   // 81.3 -> 78.3.  With four blocks (400 tokens of 40 heads, 228.7) it was 2 us slower.
-  const bool split = (T + kQRows - 1) / kQRows * n_q <= 148 && (pos0 + T + kKeys - 1) / kKeys >= 6;
+  const bool split = (T + kQRows - 1) / kQRows * n_q <= sm_count && (pos0 + T + kKeys - 1) / kKeys >= 6;
   p.pair_heads = p.group % 2 == 0 && !split;
   const int tokens = p.pair_heads || split ? kQRows : 2 * kQRows;
   p.n_tb = (T + tokens - 1) / tokens;

@@ -1413,15 +1413,15 @@ __global__ void __launch_bounds__(kRouterStreamThreads) router_topk_stream_kerne
 }
 
 cudaError_t launch_router_topk(const __half* h, const __half* wr, int M, int H, int E, int k, int renorm, int32_t* ids,
-                               float* gates, cudaStream_t st, uint64_t* n_launch, int pdl) {
-  return launch_router_topk_norm(h, wr, M, H, E, k, renorm, ids, gates, nullptr, 0, nullptr, 0.f, st, n_launch, pdl);
+                               float* gates, int sm_count, cudaStream_t st, uint64_t* n_launch, int pdl) {
+  return launch_router_topk_norm(h, wr, M, H, E, k, renorm, ids, gates, nullptr, 0, nullptr, 0.f, sm_count, st, n_launch, pdl);
 }
 
 // With norm_gain: h = RMSNorm(norm_x; norm_gain) is computed first and written to h (which the kernels after the router
 // read); one launch where the cluster kernel takes the shape, else the stand-alone norm and then the router.
 cudaError_t launch_router_topk_norm(const __half* h, const __half* wr, int M, int H, int E, int k, int renorm, int32_t* ids,
                                     float* gates, const void* norm_x, int norm_x_f32, const __half* norm_gain, float eps,
-                                    cudaStream_t st, uint64_t* n_launch, int pdl) {
+                                    int sm_count, cudaStream_t st, uint64_t* n_launch, int pdl) {
   int Epad = 32;
   while (Epad < E) Epad <<= 1;
   if (E % 8 == 0 && H % (8 * kRouterCluster) == 0 && H <= 8 * kRouterClThreads * kRouterCluster && (((uintptr_t)wr | (uintptr_t)h) & 15) == 0) {
@@ -1452,7 +1452,7 @@ cudaError_t launch_router_topk_norm(const __half* h, const __half* wr, int M, in
     // 2048 x 256 39, 4096 x 256 63, 5120 x 256 75).  Where clusters of tokens are not possible it is as fast as a cluster per token at 113 (1024 x 512) to 137
     // tokens (2048 x 512), with 256 experts at 180.
     if (M >= kRouterManyTokens && !norm_gain && E == Epad && 2048 % E == 0 && H / kRouterCluster % (kRouterStageRows * R) == 0 && smem_stream(3) <= kMost) {
-      const double us = (9.0 + 51.5e-6 * size) * ((M + 148 * kRouterStreamTok - 1) / (148 * kRouterStreamTok));
+      const double us = (9.0 + 51.5e-6 * size) * ((M + sm_count * kRouterStreamTok - 1) / (sm_count * kRouterStreamTok));
       if (E > 256 ? M >= 128 : smem_tok(8) > kMost ? M >= 184 : us < best) {
         const int stages = smem_stream(4) <= kMost ? 4 : 3;
         static std::atomic<uint64_t> attr_done;

@@ -791,12 +791,12 @@ FewRings rings_of(int mode, int nt, int parts, bool lines, size_t list) {
 // Time in us of one way to divide the work: launch and first loads, waves of units (expansion or MMAs, whichever is longer, and what the CTAs take
 // from each other in the L2 cache), accumulators in turn, the cluster's exchange, sums that are handed over.  Fitted to 2939 launches back to
 // back on new weights (21 products, 12 to 640 tokens; 5 % rms within 1.15 times the best way; the way chosen is 1.3 % slower than the best one);
-// long launches run at the power limit.
-double few_us(const GemmParams& g, int rows, int mode, int nt, int n_tt, int active, int waves, int units, int parts, int turns, int handed) {
+// long launches run at the power limit.  `active`: the part of the SMs that have a CTA.
+double few_us(const GemmParams& g, int rows, int mode, int nt, int n_tt, double active, int waves, int units, int parts, int turns, int handed) {
   const bool deep = mode == kDeep;
   const double e = (deep ? 0.407 : 0.933) * (g.mx ? 1.0 : 1.056), m = (deep ? 0.0042 : 0.0093) * nt;
-  const double unit = std::pow(e * e * e * e + m * m * m * m, 0.25) + (deep ? 0.00063 : 0.0) * nt * active / 148;
-  const double us = 0.78 + 3.15 * active / 148 + 0.0157 * nt + waves * units * unit + (parts > 1 || turns > 1 || handed ? 0.72 : 0.0) + 0.22 * (turns - 1) +
+  const double unit = std::pow(e * e * e * e + m * m * m * m, 0.25) + (deep ? 0.00063 : 0.0) * nt * active;
+  const double us = 0.78 + 3.15 * active + 0.0157 * nt + waves * units * unit + (parts > 1 || turns > 1 || handed ? 0.72 : 0.0) + 0.22 * (turns - 1) +
                     (parts > 1 ? 0.02 * nt + 0.44 * parts : 0.0) + waves * handed * (nt <= 64 ? 0.23 : 0.48 + 0.0147 * nt);
   return std::max(us, 1.0 + 2e-6 / 1286 * nt * n_tt * rows * g.K);
 }
@@ -841,8 +841,8 @@ GemmFewPlan plan_of(const GemmParams& g, int sm_count, int limit) {
           if (own > scratch) continue;
         }
         const int handed = (per + max_units - 1) / max_units - 1;
-        const double us = few_us(g, n, mode, nt, n_tt, active, waves, per, parts, turns, handed);
-        if (us < best.us) best = GemmFewPlan{mode, nt, n_tt, n_ft, parts, turns, max_units, us};
+        const double us = few_us(g, n, mode, nt, n_tt, (double)active / sm_count, waves, per, parts, turns, handed);
+        if (us < best.us) best = GemmFewPlan{mode, nt, n_tt, parts, turns, max_units, us};
       }
     }
   }
