@@ -170,13 +170,15 @@ struct W16Params {
   int ldres;
   int ksplit;  // warps that share one pair of rows, each on its own part of K: 1, 2, 4 or 8
 };
-template <int M>
+// UNIFORM: the warp number is known to be the same for the warp, which takes fewer registers.  With six and seven rows the kernel is faster for it
+// (14336 x 4096, seven rows 61.4 -> 57.3 us); with one, three and eight it is not.  With two, four and five rows an SM holds one CTA more, but a CTA
+// takes longer: see the launcher.
+template <int M, bool UNIFORM>
 __global__ void __launch_bounds__(256) gemv_w16_kernel(const W16Params p) {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   bool waited = false;  // x and the residual come from the preceding kernel; the first weight loads need not wait for it
   __shared__ float red_s[8][2][M];
-  // (several rows: a warp number that is known to be the same for the warp, 14336 x 4096 over five rows 37.4 -> 33.7 us; one row 7.75 -> 7.85)
-  const int lane = threadIdx.x & 31, w = M > 1 ? __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0) : (int)(threadIdx.x >> 5);
+  const int lane = threadIdx.x & 31, w = UNIFORM ? __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0) : (int)(threadIdx.x >> 5);
   const int K = p.K, nch = K / 8;  // 16-byte pieces per row
   const bool sw = p.mode == GEMV_SWIGLU_F16;
   int n_rows = 0;  // weight rows side by side (SwiGLU: outputs, each fed by one gate row and one up row)
@@ -314,15 +316,21 @@ cudaError_t launch_gemv_w16(const GemvParams& g, cudaStream_t st, uint64_t* n_la
   const int upc = 8 / ks;
   const dim3 grid(std::max(1, std::min((n_units + upc - 1) / upc, 148 * 8))), block(256);
   ++*n_launch;
+  // (CTAs to an SM.  Five rows, plain -> uniform, us: 14336 x 4096 47.1 -> 45.1, 1536 x 8192 equal, 777 x 15008 22.5 -> 18.4, where there are fewer waves;
+  // 512 x 16384 15.8 -> 17.9, 1024 x 16384 22.6 -> 26.2, where there are not; four rows 777 x 15008 16.9 -> 17.4, 1024 x 16384 23.3 -> 18.4)
+  auto run = [&](auto* plain, auto* uniform, int plain_ctas, int uniform_ctas) {
+    auto waves = [&](int ctas) { return ((int)grid.x + ctas * 148 - 1) / (ctas * 148); };
+    return launch_dep(waves(uniform_ctas) < waves(plain_ctas) ? uniform : plain, grid, block, 0, st, g.pdl, 1, p);
+  };
   switch (g.M) {
-    case 1: return launch_dep(gemv_w16_kernel<1>, grid, block, 0, st, g.pdl, 1, p);
-    case 2: return launch_dep(gemv_w16_kernel<2>, grid, block, 0, st, g.pdl, 1, p);
-    case 3: return launch_dep(gemv_w16_kernel<3>, grid, block, 0, st, g.pdl, 1, p);
-    case 4: return launch_dep(gemv_w16_kernel<4>, grid, block, 0, st, g.pdl, 1, p);
-    case 5: return launch_dep(gemv_w16_kernel<5>, grid, block, 0, st, g.pdl, 1, p);
-    case 6: return launch_dep(gemv_w16_kernel<6>, grid, block, 0, st, g.pdl, 1, p);
-    case 7: return launch_dep(gemv_w16_kernel<7>, grid, block, 0, st, g.pdl, 1, p);
-    default: return launch_dep(gemv_w16_kernel<8>, grid, block, 0, st, g.pdl, 1, p);
+    case 1: return launch_dep(gemv_w16_kernel<1, false>, grid, block, 0, st, g.pdl, 1, p);
+    case 2: return run(gemv_w16_kernel<2, false>, gemv_w16_kernel<2, true>, 3, 4);
+    case 3: return launch_dep(gemv_w16_kernel<3, false>, grid, block, 0, st, g.pdl, 1, p);
+    case 4: return run(gemv_w16_kernel<4, false>, gemv_w16_kernel<4, true>, 3, 4);
+    case 5: return run(gemv_w16_kernel<5, false>, gemv_w16_kernel<5, true>, 2, 3);
+    case 6: return launch_dep(gemv_w16_kernel<6, true>, grid, block, 0, st, g.pdl, 1, p);
+    case 7: return launch_dep(gemv_w16_kernel<7, true>, grid, block, 0, st, g.pdl, 1, p);
+    default: return launch_dep(gemv_w16_kernel<8, false>, grid, block, 0, st, g.pdl, 1, p);
   }
 }
 
