@@ -1791,8 +1791,8 @@ int32_t ats_layer_prefill(ats_ctx* ctx, const ats_layer_desc* L, const void* x_i
     // (every slice once per 128 of its rows).
     const int k = (int)L->top_k, E = (int)L->n_experts, P = (int)T * k, F = (int)L->ffn;
     const Tensor &tg = ctx->tensors[L->w_gate], &tu = ctx->tensors[L->w_up], &td = ctx->tensors[L->w_down];
-    // (on the device nobody tells the host how many rows an expert has at most, which the single-CTA kernel's grouped form has to know: the
-    // pairs take what has contiguous experts, `hidden` and `ffn` being multiples of 32)
+    // (on the device nobody tells the host how many rows an expert has at most, which the grouped form of the plain tiles has to know: the kernel for few
+    // tokens or the pairs take what has contiguous experts, `hidden` and `ffn` being multiples of 32)
     const bool on_device = tg.contiguous_dev && tu.contiguous_dev && td.contiguous_dev && ctx->done_dev && !(ctx->cfg.flags & ATS_FLAG_NO_GEMM_PAIR);
     if (on_device) {  // (a wait for the router cannot be captured)
       cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;

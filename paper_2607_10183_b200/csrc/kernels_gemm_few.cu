@@ -18,7 +18,8 @@
 // steps go to up to four accumulators in turn where a CTA has one tile and tensor memory has room, or an accumulator is handed over and the
 // sums so far wait in the scratch.
 //
-// What bounds it: up to 64 tokens expansion and HBM (148 CTAs of 256 features: 6.3 TB/s of weights), with 128 the MMAs at the power limit (1.3 to
+// What bounds it: up to 64 tokens HBM where every SM has a CTA (6.3 TB/s of weights; an SM's share of the rate is 396 cycles for 128 k of 128 features,
+// the expansion stays just under it), with 128 the MMAs at the power limit (1.3 to
 // 1.4 PFLOP/s); products of few tiles launch, first loads and output (2.5 to 4 us) and the exchange.  Back to back on new weights, before (pairs or
 // gemm_q4_kernel) -> now, us:
 //   1024 x 1024, 16 tokens Q4       5.8 -> 3.3      4096 x 4096, 16 / 77 / 512 tokens MXFP4   10.8 / 13.9 / 21.5 -> 7.2 / 10.6 / 17.5
