@@ -711,7 +711,7 @@ def test_gate_up_both_streamed_needs_two_slots(B, torch):
 
 
 # ------------------------------------------------------------------------------------------------- a4 routing, a5 MoE
-# (hidden, experts, k): the cluster kernel with the selection by counting ranks (up to 256 experts, incl. exactly 256), the
+# (hidden, experts, k): the cluster kernel with the selection by integer keys (up to 256 experts, incl. exactly 256), the
 # cluster kernel with the warp argmax (more experts), the one-CTA kernel (shapes the cluster form does not take), and the
 # largest router the library accepts
 @pytest.mark.parametrize("Hd,E,k", [(128, 48, 6), (128, 256, 8), (128, 264, 8), (100, 50, 6), (256, 1024, 32)])
@@ -751,8 +751,8 @@ def test_attention_merge_round_trips(B, torch, d, group, pos):
     H.assert_close(ys[0], want, what=f"layer, {pos + 1} positions")
 
 
-# Many tokens (the kernel that takes four tokens per CTA): the last CTA with one to four tokens, the shortest chains it takes (eight
-# rows), 32 experts and as many as 1024, three stages instead of four; and the neighbours it leaves to the cluster kernel.
+# Many tokens (clusters of tokens, or four tokens per CTA where the matrix is streamed): a last CTA or cluster with few tokens, short chains, 32
+# experts and as many as 1024, rows of 6144.
 @pytest.mark.parametrize("Hd,E,k,M", [(512, 256, 8, 128), (2048, 128, 8, 129), (4096, 32, 4, 130), (4096, 64, 6, 131), (256, 1024, 32, 132),
                                       (6144, 128, 8, 128), (2048, 128, 8, 127), (2048, 96, 8, 128)])
 def test_route_topk_many_tokens(B, torch, Hd, E, k, M):

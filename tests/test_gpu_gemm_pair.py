@@ -1,4 +1,5 @@
-"""The GEMMs on pairs of CTAs at the edges of their tiles, units and work ranges, against the oracle."""
+"""The GEMMs on pairs of CTAs at the edges of their tiles, units and work ranges, against the oracle.  The kernel for few tokens takes most of the 4-bit
+products here; tests/test_gpu_gemm_pair_4bit.py runs these tests without it."""
 import numpy as np
 import pytest
 
@@ -89,7 +90,7 @@ def test_tiles_of_several_contributors_match_oracle(fmt, N, K, T):
         ctx.linear(tid, xd, y, T)
         ctx.sync()
         outs.append(y.cpu().numpy().view(np.uint16))
-    assert ctx.stats().kernel_launches == 3  # (the sum needs no launch of its own: this is the kernel on pairs)
+    assert ctx.stats().kernel_launches == 3  # (the sum needs no launch of its own)
     ctx.close()
     w = torch.from_numpy(weights[0] if fmt == "w16" else O.dequantize(*weights, O.WEIGHT_F16).astype(np.float32)).cuda().double()
     want = (xd.double() @ w.t()).cpu().numpy()  # all rows, in 64 bits
@@ -219,8 +220,8 @@ def test_gemm_with_the_least_workspace_keeps_the_chains_short():
     assert ws > 1024 and differ <= 0.0065 * limit / 1000
 
 
-# Which kernel takes a product: the pairs where they are the faster ones, else the single-CTA kernel (few tiles: it splits K and adds the
-# parts up in a launch of its own), whose results those are then bit for bit.
+# Which kernel takes a product (fp16, or without the kernel for few tokens): the pairs where they are the faster ones, else the single-CTA kernel (few
+# tiles: it splits K and adds the parts up in a launch of its own), whose results those are then bit for bit.
 @pytest.mark.parametrize("fmt,N,K,T,pairs", [("w16", 4096, 4096, 256, False), ("w16", 1024, 8192, 1000, False), ("w16", 640, 5120, 128, False),
                                              ("q4", 1024, 8192, 100, False), ("q4", 640, 5120, 128, False), ("mxfp4", 640, 5120, 512, False),
                                              ("q4", 6144, 2048, 33, True), ("w16", 8192, 2048, 128, True), ("q4", 333, 4096, 100, True)])

@@ -527,6 +527,6 @@ def test_moe_prefill_sorted_on_the_device_has_the_bits_of_the_host_sort(B, torch
 
 @pytest.mark.parametrize("E,k,T,skew", [(16, 8, 513, 0.0), (128, 8, 700, 0.0), (264, 8, 601, 0.0), (8, 8, 4097, 4.0), (8, 8, 8192, 0.0)])
 def test_moe_prefill_sort_of_more_pairs_than_the_first_votes_hold(B, torch, E, k, T, skew):
-    """More than 4096 pairs: a warp's part is longer than the votes that it keeps in registers.  264 experts of 18 rows; 8 experts of
+    """More than 4096 pairs: a thread's part is longer than the ids that it keeps in registers.  264 experts of 18 rows; 8 experts of
     4097 rows (more than 128 blocks of 256 rows) and of 8192 (more than 255: the outputs are staged in halves)."""
     test_moe_prefill_sorted_on_the_device_has_the_bits_of_the_host_sort(B, torch, E, k, T, skew)
