@@ -415,6 +415,8 @@ int32_t ats_host_solve_placement(const int64_t* s, const int64_t* r, const int64
  * position of expert e, off[E] = P; *max_rows = the largest expert's row count.  ATS_ERR_INVALID for an id out of range. */
 int32_t ats_host_group_pairs(const int32_t* ids, uint32_t P, uint32_t E, int32_t* order, int32_t* pos, int32_t* off,
                              int32_t* max_rows);
+int32_t ats_host_repack_q4(const void* codes, const void* scales, void* out_slice, uint32_t n_out, uint32_t k_in);
+int32_t ats_host_unpack_q4(const void* slice, void* out_codes, void* out_scales, uint32_t n_out, uint32_t k_in);
 /* Which kernel the prompt product of ats_linear runs on (host only; T rows, more than 8, of a dense tensor), under the flags of a context, with
  * scratch_bytes for partial sums, 16-byte aligned operands and a GPU of sm_count SMs: ATS_GEMM_PLAIN (128 x 128 and wider tiles on single CTAs),
  * ATS_GEMM_PAIRS or ATS_GEMM_FEW; *chain_k (optional) = the k that it adds up in one accumulator at most.  ATS_ERR_SHAPE for sizes that ats_linear
@@ -422,8 +424,6 @@ int32_t ats_host_group_pairs(const int32_t* ids, uint32_t P, uint32_t E, int32_t
 enum { ATS_GEMM_PLAIN = 0, ATS_GEMM_PAIRS = 1, ATS_GEMM_FEW = 2 };
 int32_t ats_host_gemm_kernel(uint32_t fmt, uint32_t n_out, uint32_t k_in, uint32_t T, uint32_t flags, uint64_t scratch_bytes, uint32_t sm_count,
                              int32_t* kernel, uint32_t* chain_k);
-int32_t ats_host_repack_q4(const void* codes, const void* scales, void* out_slice, uint32_t n_out, uint32_t k_in);
-int32_t ats_host_unpack_q4(const void* slice, void* out_codes, void* out_scales, uint32_t n_out, uint32_t k_in);
 
 /* Load-aware dynamic transfer (Section 4.4), host only.  A round runs tensors 0..n-1 in order; b[i] (ATS_HOST / ATS_GPU) is
  * the default backend from static placement, t_gpu[i] / t_host[i] the current execution times of tensor i's operator on the
