@@ -396,7 +396,7 @@ struct GemmPairPlan {
 bool gemm_pair_eligible(const GemmParams& p, int sm_count, GemmPairPlan* plan);
 int gemm_pair_chain(const GemmParams& p, const GemmPairPlan& plan);  // the k that an accumulator adds up at most (not grouped)
 // the one of these two kernels (without `pairs`, the single-CTA kernel) that would take the product with all the scratch it wants: its time, and the k that it
-// adds up in one accumulator, whichever of its two plans the scratch holds
+// adds up in one accumulator
 struct GemmOther {
   double us;
   int chain;

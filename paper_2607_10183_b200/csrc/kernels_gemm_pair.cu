@@ -970,15 +970,11 @@ GemmOther gemm_other(const GemmParams& g, int sm_count, bool pairs) {
   GemmParams all = g;
   all.scratch = reinterpret_cast<void*>(16);
   all.scratch_bytes = ~0ull;
-  int rows[3] = {0, 0, 0}, n = 0;
-  for (int i = 0; i < g.n_seg; ++i) n += rows[i] = g.seg[i].n_rows;
+  int rows[3] = {0, 0, 0};
+  for (int i = 0; i < g.n_seg; ++i) rows[i] = g.seg[i].n_rows;
   GemmPairPlan pl{};
   if (!pairs || !gemm_pair_eligible(all, sm_count, &pl)) return GemmOther{single_cta_us(g), gemm_chain(rows, g.n_seg, g.T, g.K)};
-  GemmOther other{pl.us, gemm_pair_chain(g, pl)};
-  all.scratch_bytes = gemm_scratch_bytes(g.T, n, g.K);
-  if (pl.scratch > all.scratch_bytes)  // (a caller without that scratch has the other plan, see plan_of)
-    other.chain = std::min(other.chain, gemm_pair_eligible(all, sm_count, &pl) ? gemm_pair_chain(g, pl) : gemm_chain(rows, g.n_seg, g.T, g.K));
-  return other;
+  return GemmOther{pl.us, gemm_pair_chain(g, pl)};
 }
 
 cudaError_t launch_gemm_pair(const GemmParams& g, const GemmPairPlan& pl, int sm_count, cudaStream_t st, uint64_t* n_launch, std::string* err) {

@@ -78,22 +78,3 @@ def test_without_pairs_the_kernel_for_few_tokens_is_compared_with_plain_tiles():
     assert taken > 2000
     for fmt, n, k, T in ((B.ATS_FMT_Q4B32, 13392, 4896, 1391), (B.ATS_FMT_MXFP4, 5983, 13344, 114), (B.ATS_FMT_MXFP4, 11047, 11968, 174)):
         assert B.host_gemm_kernel(fmt, n, k, T, B.ATS_FLAG_NO_GEMM_PAIR)[0] == B.ATS_GEMM_FEW
-
-
-def test_chains_of_few_tokens_are_no_longer_than_the_other_kernels_whatever_the_scratch():
-    """The pairs have two plans, and the caller's scratch decides between them."""
-    import random
-    B = _binding()
-    rng = random.Random(5)
-    taken = 0
-    for i in range(4000):
-        n, k, T = int(2 ** rng.uniform(9, 14)), 32 * int(2 ** rng.uniform(4, 9)), int(2 ** rng.uniform(3.3, 12))
-        fmt = rng.choice([B.ATS_FMT_Q4B32, B.ATS_FMT_MXFP4])
-        if i < 4:
-            fmt, n, k, T = ((B.ATS_FMT_Q4B32, 4549, 9888, 121), (B.ATS_FMT_MXFP4, 3906, 10368, 25), (B.ATS_FMT_Q4B32, 3744, 10304, 25), (B.ATS_FMT_MXFP4, 601, 10336, 100))[i]
-        for scratch in (32 * n * T, 1 << 40):
-            kernel, chain = B.host_gemm_kernel(fmt, n, k, T, 0, scratch)
-            if kernel == B.ATS_GEMM_FEW:
-                taken += 1
-                assert chain <= max(256, B.host_gemm_kernel(fmt, n, k, T, B.ATS_FLAG_NO_GEMM_FEW, scratch)[1]), (n, k, T, scratch)
-    assert taken > 5000
