@@ -78,3 +78,20 @@ def test_without_pairs_the_kernel_for_few_tokens_is_compared_with_plain_tiles():
     assert taken > 2000
     for fmt, n, k, T in ((B.ATS_FMT_Q4B32, 13392, 4896, 1391), (B.ATS_FMT_MXFP4, 5983, 13344, 114), (B.ATS_FMT_MXFP4, 11047, 11968, 174)):
         assert B.host_gemm_kernel(fmt, n, k, T, B.ATS_FLAG_NO_GEMM_PAIR)[0] == B.ATS_GEMM_FEW
+
+
+def test_chains_of_few_tokens_are_no_longer_than_the_other_kernels():
+    """With all the scratch that these want; with less, by no more than a quarter (see the kernel)."""
+    import random
+    B = _binding()
+    rng = random.Random(5)
+    taken = 0
+    for _ in range(4000):
+        n, k, T = int(2 ** rng.uniform(9, 14)), 32 * int(2 ** rng.uniform(4, 9)), int(2 ** rng.uniform(3.3, 12))
+        fmt = rng.choice([B.ATS_FMT_Q4B32, B.ATS_FMT_MXFP4])
+        for scratch, more in ((1 << 40, 1.0), (32 * n * T, 1.25)):
+            kernel, chain = B.host_gemm_kernel(fmt, n, k, T, 0, scratch)
+            if kernel == B.ATS_GEMM_FEW:
+                taken += 1
+                assert chain <= max(256, more * B.host_gemm_kernel(fmt, n, k, T, B.ATS_FLAG_NO_GEMM_FEW, scratch)[1]), (n, k, T, scratch)
+    assert taken > 5000
