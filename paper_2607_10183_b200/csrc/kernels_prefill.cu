@@ -321,7 +321,7 @@ cudaError_t launch_swiglu16(const __half* gu, int ld, int ffn, __half* act, int 
 // Every CTA counts the pairs for itself (16 KB of ids for 4096 pairs), finds those of its expert and run in the order of its threads' contiguous parts,
 // places them and copies their rows.  The completion word tells the host that the router has run.
 //   DEALT   an expert has as many CTAs as it has runs of `share` rows, so that none copies more than those however the tokens are routed
-//   else    an expert has 1 << shift CTAs, which need not know the other experts' counts: 0.6 to 1 us less
+//   else    an expert has 1 << shift CTAs, which need not know the other experts' counts: 0.6 to 1.2 us less
 // Bound by latencies (ids twice, a sum over the CTA, or two, rows) and the copies (4096 rows of 4 KB written: 2.6 us).
 constexpr int kSortThreads = 256, kSortShare = 512;
 template <bool DEALT>
@@ -464,10 +464,12 @@ cudaError_t launch_moe_sort_gather(const int32_t* ids, int P, int E, int k, int 
   // Four CTAs to an SM (with even routings one took 19.8 us, two 14.0, four 11.2, eight 12.9: copies in flight against ids read).
   int shift = 0;
   while ((2 << shift) * E <= 4 * sm_count) ++shift;
-  // An expert has at most a row of each token: where that is at most 16 to each of its 1 << shift CTAs there is nothing to deal.  (Layers, every token
-  // to other experts / all tokens to the same, us.  19 rows, 300 tokens through 4 of 32: fixed 126.4 / 129, dealt 127.1 / 125.5; 128 rows, 512 tokens through
-  // 8 of 128: 145 / 129, 143 / 101; 1024 rows, 4096 tokens: 588 / 884, 581 / 511.  1024 tokens through 8 of 1024 654 / 837, 658 / 585.)
-  if (P / k <= 16 << shift && k <= 32)
+  // An expert has at most a row of each token: where that is at most 16 to each of its 1 << shift CTAs, or 40 of few pairs, there is not much to deal.
+  // (Layers, every token to other experts / all tokens to the same, us.  37 rows, 150 tokens through 2 of 128: fixed 70.9, dealt 72.1; 19 rows, 300
+  // through 4 of 32: fixed 126.4 / 129, dealt 127.1 / 125.5; 128 rows, 512 through 8 of 128: 145 / 129, 143 / 101; 1024 rows, 4096 tokens: 588 / 884,
+  // 581 / 511.  1024 tokens through 8 of 1024 654 / 837, 658 / 585.  With 1400 pairs and more dealing is 1 to 2.5 % faster for even routings too.)
+  const int T = P / k;
+  if (P <= kSortShare << shift && (T <= 16 << shift || (P <= 1280 && T <= 40 << shift)))  // (the list holds kSortShare rows)
     return launch_dep(moe_sort_gather_kernel<false>, dim3(E << shift), dim3(kSortThreads), 0, st, pdl, 1, ids, P, E, 0, 0u, shift, k, H, h, order, pos, off, xs,
                       status, done, seq);
   // A run that is not full can end each expert, so as many CTAs as there are experts (or rows) are on top of the P / share: many experts make it up to

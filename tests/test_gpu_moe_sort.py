@@ -11,7 +11,7 @@ MB = 1 << 20
 
 # Runs of rows per expert: one expert with hundreds of them, all rows in one expert, more experts than four to an SM, most of them without
 # rows, the most experts; a last run of one row and full ones; ids beyond the sixteen that a thread keeps.
-@pytest.mark.parametrize("E,k,T,skew", [(128, 8, 513, 6.0), (264, 8, 1100, 4.0), (600, 4, 301, 6.0), (1024, 8, 70, 0.0), (8, 1, 3000, 30.0), (4, 1, 129, 0.0), (128, 8, 1024, 0.0)])
+@pytest.mark.parametrize("E,k,T,skew", [(128, 8, 513, 6.0), (264, 8, 1100, 4.0), (600, 4, 301, 6.0), (1024, 8, 70, 0.0), (8, 1, 3000, 30.0), (4, 1, 129, 0.0), (128, 8, 1024, 0.0), (128, 8, 160, 6.0), (128, 8, 161, 6.0), (32, 4, 320, 30.0)])
 def test_rows_of_any_routing_have_the_bits_of_the_host_sort(E, k, T, skew):
     import torch
     from paper_2607_10183_b200 import binding as B
